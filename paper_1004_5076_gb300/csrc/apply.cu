@@ -68,24 +68,20 @@ __device__ __forceinline__ void axpy2(cx<double>& a, double s, cx<double> b) { a
 // current summaries of t (as k_summ; written by the thread of point 0) and
 // the point's weighted sources qsrc[Qi*12 + set*4 + {x, y, z, div}] of the
 // exterior J, interior J and exterior M sets (J(r) = a (r - c) - beta,
-// div J = 2a, times the quadrature weight); it also zeroes the output y.
+// div J = 2a, times the quadrature weight).
 template <typename R>
 __global__ void k_sources(const cx<R>* __restrict__ x, const int32_t* __restrict__ unk,
                           const double* __restrict__ cX, const double* __restrict__ tri,
                           const double* __restrict__ qp, const double* __restrict__ qw, int64_t Q, int q,
-                          cx<R>* __restrict__ summ, cx<R>* __restrict__ qsrc, cx<R>* __restrict__ y, int64_t N,
-                          int64_t ldx, int64_t ldy) {
+                          cx<R>* __restrict__ summ, cx<R>* __restrict__ qsrc, int64_t ldx) {
   const int64_t Qi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (Qi >= Q) return;
   {  // right-hand side blockIdx.y of a batch: its columns and workspaces
     const int64_t c = blockIdx.y;
     x += c * ldx;
-    y += c * ldy;
     summ += c * (Q / q) * 12;
     qsrc += c * Q * 12;
   }
-  // y is summed into by k_points (two terms per row)
-  for (int64_t r = Qi; r < N; r += Q) y[r] = czero<R>();
   const int64_t t = Qi / q;
   const int a = (int)(Qi - t * q);
   const double* g = tri + 16 * t;
@@ -418,26 +414,19 @@ __device__ __forceinline__ cx<R> dot3(const R* X, const cx<R>* V) {
 // edge kk of triangle t, from the point's records (recs[medium*NREC]):
 // type 0 <X, E_e - E_i>, 1 <X, H_e - H_i> (weak forms), 2 Eq. 13, 3 Eq. 14.
 template <typename R>
-__device__ __forceinline__ void test_point(const cx<R>* recs, const cx<R>* __restrict__ summ,
-                                           const double* __restrict__ tri, const R* __restrict__ tp,
-                                           const R* __restrict__ sig, int64_t t, int kk, int a, int q, R ke, R ki,
-                                           R ze, R zi, cx<R>* out) {
+__device__ __forceinline__ void test_point(const cx<R>* recs, const double* __restrict__ tri,
+                                           const R* __restrict__ tp, const R* __restrict__ sig, int64_t t, int kk,
+                                           int a, int q, R ke, R ki, R ze, R zi, cx<R>* out) {
   const double* g = tri + 16 * t;
   const R nrm[3] = {(R)g[12], (R)g[13], (R)g[14]};
-  const cx<R>* se = summ + (3 * t + 0) * 4;
-  const cx<R>* si = summ + (3 * t + 1) * 4;
-  const cx<R>* sM = summ + (3 * t + 2) * 4;
   const R kl[2] = {ke, ki}, zl[2] = {ze, zi};
   const int64_t Qa = t * q + a;
   const R* tq = tp + 16 * Qa;
   const R w = tq[3];
   const R sg = sig[Qa];
   const R divX = tq[13 + kk];
-  R X[3], rel[3];
-  for (int c = 0; c < 3; ++c) {
-    X[c] = tq[4 + 3 * kk + c];
-    rel[c] = tq[c];
-  }
+  R X[3];
+  for (int c = 0; c < 3; ++c) X[c] = tq[4 + 3 * kk + c];
   cx<R> WE[3], WH[3], E[2][3];
   cx<R> wE = czero<R>(), wH = czero<R>();
   for (int c = 0; c < 3; ++c) WE[c] = WH[c] = czero<R>();
@@ -456,28 +445,12 @@ __device__ __forceinline__ void test_point(const cx<R>* recs, const cx<R>* __res
       E[m][c] = -z * (k * jA + (R(1) / k) * mulj(gphi)) - cF;
     }
   }
-  cx<R> Js[3], M[3];  // J_e + J_i and M of this triangle at the point
-  for (int c = 0; c < 3; ++c) {
-    Js[c] = rel[c] * se[0] - se[1 + c] + rel[c] * si[0] - si[1 + c];
-    M[c] = rel[c] * sM[0] - sM[1 + c];
-  }
-  // n x (J_e + J_i), n x M and n x X
-  cx<R> nJ[3], nM[3];
-  nJ[0] = nrm[1] * Js[2] - nrm[2] * Js[1];
-  nJ[1] = nrm[2] * Js[0] - nrm[0] * Js[2];
-  nJ[2] = nrm[0] * Js[1] - nrm[1] * Js[0];
-  nM[0] = nrm[1] * M[2] - nrm[2] * M[1];
-  nM[1] = nrm[2] * M[0] - nrm[0] * M[2];
-  nM[2] = nrm[0] * M[1] - nrm[1] * M[0];
   const R nX[3] = {nrm[1] * X[2] - nrm[2] * X[1], nrm[2] * X[0] - nrm[0] * X[2], nrm[0] * X[1] - nrm[1] * X[0]};
-  const cx<R> XJ = dot3(X, Js), XnM = dot3(X, nM);
   const cx<R> hterm = dot3(X, WH) + divX * wH;
   out[0] = w * (dot3(X, WE) + divX * wE);
   out[1] = w * hterm;
-  // Eq. 13: <X, dH> - <sigma n x X, E_e^+>, side limits (J_e+J_i) x n / 2 and sigma M / 2
-  out[2] = w * (hterm - R(0.5) * dot3(X, nJ) - sg * dot3(nX, E[0]) - (R(0.5) * sg) * dot3(X, M));
-  // Eq. 14: <X, J_e + J_i> - <sigma X, E_i^->, side limit n x M / 2
-  out[3] = w * (XJ - sg * dot3(X, E[1]) - (R(0.5) * sg) * XnM);
+  out[2] = w * (hterm - sg * dot3(nX, E[0]));  // Eq. 13: <X, dH> - <sigma n x X, E_e>
+  out[3] = (-w * sg) * dot3(X, E[1]);          // Eq. 14: -<sigma X, E_i>
 }
 
 // d out / d sg of the Eq. 13 and Eq. 14 tested values of local edge kk at
@@ -618,8 +591,9 @@ __host__ __device__ constexpr size_t pt_smem_bytes(int q, size_t csize) {
   return (size_t)PT_WARPS * pt_warp_complex(q) * csize + (size_t)PT_WARPS * PT_NSTG * sizeof(uint64_t);
 }
 
-// SENS = true (conductivity sensitivity): instead of testing into y, the
-// kernel writes hs[t q + a] = eta0 sum_kk (lam_row2 d2 + lam_row3 d3), the
+// SENS = true (conductivity sensitivity): the near corrections are added at
+// the points, and instead of the tested values val[t][kk][type] the kernel
+// writes hs[t q + a] = eta0 sum_kk (lam_row2 d2 + lam_row3 d3), the
 // derivative of lam^T A x with respect to the conductivity [S] at the point.
 //
 // QT > 0 fixes q at compile time (then every shared-memory offset of a record
@@ -632,13 +606,14 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
     const R* __restrict__ dL, const cx<R>* __restrict__ corr, const int32_t* __restrict__ noff,
     const int32_t* __restrict__ nsrc, const cx<R>* __restrict__ summ, const double* __restrict__ tri,
     const R* __restrict__ tp, const R* __restrict__ sig, int64_t nt, int q_arg, int n0, int n1, int n2, R ke, R ki,
-    R ze, R zi, int has_near, const int32_t* __restrict__ valrow, cx<R>* __restrict__ y, int* __restrict__ tmo,
-    const cx<R>* __restrict__ lam, cx<R>* __restrict__ hs) {
+    R ze, R zi, int has_near, const int32_t* __restrict__ valrow, cx<R>* __restrict__ val, int* __restrict__ tmo,
+    const cx<R>* __restrict__ lam, cx<R>* __restrict__ hs, int64_t cs_grid, int64_t cs_val) {
   const int q = QT > 0 ? QT : q_arg;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = (int64_t)blockIdx.x * PT_WARPS + warp;
   if (t >= nt) return;  // whole warp; no CTA-wide barrier below
+  grids += blockIdx.y * cs_grid;  // right-hand side blockIdx.y of a batch
   const int pairc = NCORR * 2 * q;  // complex per pair: [point][medium][component]
   cx<R>* ring = reinterpret_cast<cx<R>*>(smem_raw) + (int64_t)warp * pt_warp_complex(q);
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<cx<R>*>(smem_raw) + PT_WARPS * pt_warp_complex(q)) +
@@ -648,7 +623,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
 
   const bool act = lane < 4 * q;
   const int a = min(lane >> 2, q - 1), med = (lane >> 1) & 1, h = lane & 1;
-  const int j0 = has_near ? noff[t] : 0, j1 = has_near ? noff[t + 1] : 0;
+  const int j0 = SENS && has_near ? noff[t] : 0, j1 = SENS && has_near ? noff[t + 1] : 0;
   const int nst = (j1 - j0 + PT_KP - 1) / PT_KP;
   const unsigned pair_bytes = (unsigned)(pairc * sizeof(cx<R>));
   // stage st -> slot st % PT_NSTG, issued by lane 0
@@ -659,7 +634,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
     bulk_load(ring + (st % PT_NSTG) * PT_KP * pairc, corr + (int64_t)pj * pairc, np * pair_bytes,
               bars + st % PT_NSTG);
   };
-  if (nst > 0) {
+  if (SENS && nst > 0) {
     if (lane == 0) {
 #pragma unroll
       for (int i = 0; i < PT_NSTG; ++i) mbar_init(bars + i, 1);
@@ -673,7 +648,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
   int src_nxt = lane < npair ? nsrc[j0 + lane] : 0, src_cur = 0;
   cx<R> acc[NREC / 2];
   interp_group<R, P>(grids, base, L, dL, t * q + a, med, h, n1, n2, acc);
-  if (nst > 0) {
+  if (SENS && nst > 0) {
     const int set = h ? 2 : med;  // source J of this medium, or M
     // the interior medium sees -M: accumulate -acc + sum, then negate back
     const bool neg = h && med;
@@ -742,7 +717,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
   if (lane < 3 * q) {
     const int kk = lane / q, pa = lane - kk * q;
     cx<R> o[4];
-    test_point(recs + pa * 2 * NREC, summ, tri, tp, sig, t, kk, pa, q, ke, ki, ze, zi, o);
+    test_point(recs + pa * 2 * NREC, tri, tp, sig, t, kk, pa, q, ke, ki, ze, zi, o);
     cx<R>* d = part + (kk * q + pa) * 4;
 #pragma unroll
     for (int c = 0; c < 4; ++c) d[c] = o[c];
@@ -753,166 +728,10 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
     const cx<R>* sp = part + kk * q * 4 + c;
     cx<R> v = czero<R>();
     for (int pa = 0; pa < q; ++pa) v += sp[pa * 4];
-    // each row is the sum of exactly two such values (the edge's two
-    // triangles) added to a zeroed word, so the result does not depend on
-    // which arrives first
-    const int row = valrow[(t * 3 + kk) * 4 + c];
-    if (row >= 0) {
-      atomicAdd(&y[row].re, v.re);
-      atomicAdd(&y[row].im, v.im);
-    }
+    val[blockIdx.y * cs_val + t * 12 + lane] = v;
   }
 }
 
-
-// K6-8 for a batch of ncol right-hand sides: one CTA per target triangle
-// t = blockIdx.x.  Thread T works on column T / 4q as lane (point, medium,
-// group) T mod 4q of k_points would, so the 4q lanes of each column are
-// packed back to back (8 columns x 24 lanes = 6 full warps for q = 6, where
-// a warp per column would leave 8 lanes of every warp idle).  The near
-// records of t stream once through one ring shared by all threads (PB_NSTG
-// stages of PB_KP pairs, filled by thread 0 with bulk copies), so each record
-// leaves HBM once for all columns.  After consuming a stage every thread
-// joins a CTA barrier that also combines the bounded waits' results: the
-// slot is then free for the next copy, and all threads leave the stage loop
-// together when a wait expired.  Testing (3q tasks per column) and the row
-// sums (12 per column) are packed the same way, on a per-column area beside
-// the ring.
-constexpr int PB_NSTG = 2;  // 2 stages of 8 pairs: half the CTA barriers and waits of 4 stages of 4
-constexpr int PB_KP = 8;
-
-__host__ __device__ constexpr int pb_ring_complex(int q) { return PB_NSTG * PB_KP * NCORR * 2 * q; }
-__host__ __device__ constexpr int pb_col_complex(int q) { return 2 * q * NREC + 3 * q * 4; }
-__host__ __device__ constexpr size_t pb_smem_bytes(int q, int kc, size_t csize) {
-  return ((size_t)pb_ring_complex(q) + (size_t)kc * pb_col_complex(q)) * csize + PB_NSTG * sizeof(uint64_t);
-}
-__host__ __device__ constexpr int pb_threads(int q, int ncol) { return (4 * q * ncol + 31) / 32 * 32; }
-
-template <typename R, int P, int QT = 0>
-__global__ void __launch_bounds__(KBATCH * 32, sizeof(R) == 4 ? (P == 4 ? 2 : 3) : 1) k_points_batch(
-    const cx<R>* __restrict__ grids, const int32_t* __restrict__ base, const R* __restrict__ L,
-    const R* __restrict__ dL, const cx<R>* __restrict__ corr, const int32_t* __restrict__ noff,
-    const int32_t* __restrict__ nsrc, const cx<R>* __restrict__ summ, const double* __restrict__ tri,
-    const R* __restrict__ tp, const R* __restrict__ sig, int64_t nt, int q_arg, int n0, int n1, int n2, R ke, R ki,
-    R ze, R zi, int has_near, const int32_t* __restrict__ valrow, cx<R>* __restrict__ y, int* __restrict__ tmo,
-    int64_t cs_grid, int64_t cs_summ, int64_t ldy, int ncol) {
-  const int q = QT > 0 ? QT : q_arg;  // as in k_points
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int T = threadIdx.x, lane = T & 31;
-  const int nl = 4 * q;                    // phase-1 tasks per column
-  const bool act = T < ncol * nl;          // threads past them repeat a task of the last column, unstored
-  const int col = act ? T / nl : ncol - 1;
-  const int task = act ? T - col * nl : nl - 1;
-  const int64_t t = blockIdx.x;
-  const int pairc = NCORR * 2 * q;
-  cx<R>* ring = reinterpret_cast<cx<R>*>(smem_raw);
-  cx<R>* area = ring + pb_ring_complex(q);  // per column: recs [q][2][NREC], then part [3][q][4]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(area + (int64_t)ncol * pb_col_complex(q));
-
-  const int a = task >> 2, med = (task >> 1) & 1, h = task & 1;
-  const int j0 = has_near ? noff[t] : 0, j1 = has_near ? noff[t + 1] : 0;
-  const int nst = (j1 - j0 + PB_KP - 1) / PB_KP;  // the same for every thread of the CTA
-  const unsigned pair_bytes = (unsigned)(pairc * sizeof(cx<R>));
-  auto issue = [&](int st) {  // thread 0 only
-    const int pj = j0 + st * PB_KP;
-    const int np = min(PB_KP, j1 - pj);
-    fence_proxy_async();
-    bulk_load(ring + (st % PB_NSTG) * PB_KP * pairc, corr + (int64_t)pj * pairc, np * pair_bytes,
-              bars + st % PB_NSTG);
-  };
-  if (nst > 0) {
-    if (T == 0) {
-#pragma unroll
-      for (int i = 0; i < PB_NSTG; ++i) mbar_init(bars + i, 1);
-      mbar_init_fence();
-      for (int st = 0; st < PB_NSTG - 1 && st < nst; ++st) issue(st);
-    }
-    __syncthreads();  // the barriers are initialised before anyone waits on them
-  }
-  const int npair = j1 - j0;
-  const cx<R>* summ_c = summ + col * cs_summ;
-  int src_nxt = lane < npair ? nsrc[j0 + lane] : 0, src_cur = 0;
-  cx<R> acc[NREC / 2];
-  interp_group<R, P>(grids + col * cs_grid, base, L, dL, t * q + a, med, h, n1, n2, acc);
-  if (nst > 0) {
-    const int set = h ? 2 : med;
-    const bool neg = h && med;
-    if (neg)
-#pragma unroll
-      for (int c = 0; c < NREC / 2; ++c) acc[c] = -acc[c];
-    NearAcc<R> na;
-    na.begin(acc);
-    int st = 0;
-    bool ok = true;
-    for (; st < nst; ++st) {
-      // slot (st - 1) % PB_NSTG was released by every thread at the barrier ending stage st - 1
-      if (T == 0 && st + PB_NSTG - 1 < nst) issue(st + PB_NSTG - 1);
-      const bool here = __all_sync(0xffffffffu, mbar_wait(bars + st % PB_NSTG, (st / PB_NSTG) & 1));
-      if (here) {
-        const cx<R>* rs = ring + (st % PB_NSTG) * PB_KP * pairc + (a * 2 + med) * NCORR;
-#pragma unroll
-        for (int k = 0; k < PB_KP; ++k) {
-          const int jj = st * PB_KP + k;
-          if (jj < npair) {
-            if ((jj & 31) == 0) {
-              src_cur = src_nxt;
-              src_nxt = jj + 32 + lane < npair ? nsrc[j0 + jj + 32 + lane] : 0;
-            }
-            const int64_t sj = __shfl_sync(0xffffffffu, src_cur, jj & 31);
-            cx<R> d[NCORR], sv[4];
-            load_group(summ_c + (3 * sj + set) * 4, sv);
-#pragma unroll
-            for (int c = 0; c < NCORR; c += 2) load_pair_smem(rs + k * pairc + c, d + c);
-            na.add(d, sv);
-          }
-        }
-      }
-      ok = __syncthreads_and(here) != 0;
-      if (!ok) break;
-    }
-    if (!ok && T == 0) {
-      // stages st .. min(st + PB_NSTG - 1, nst - 1) may still be in flight: let them land
-      for (int s2 = st; s2 < nst && s2 < st + PB_NSTG; ++s2)
-        (void)mbar_wait(bars + s2 % PB_NSTG, (s2 / PB_NSTG) & 1);
-      atomicOr(tmo, 1);
-    }
-    na.end(acc);
-    if (neg)
-#pragma unroll
-      for (int c = 0; c < NREC / 2; ++c) acc[c] = -acc[c];
-  }
-  // the ring is dead from here on: every thread passed the last stage's barrier
-  if (act) {
-    cx<R>* o = area + (int64_t)col * pb_col_complex(q) + (a * 2 + med) * NREC + 10 * h;
-#pragma unroll
-    for (int c = 0; c < NREC / 2; ++c) o[c] = acc[c];
-  }
-  __syncthreads();
-  if (T < ncol * 3 * q) {
-    const int c2 = T / (3 * q), r = T - c2 * 3 * q;
-    const int kk = r / q, pa = r - kk * q;
-    cx<R>* ar = area + (int64_t)c2 * pb_col_complex(q);
-    cx<R> o[4];
-    test_point(ar + pa * 2 * NREC, summ + c2 * cs_summ, tri, tp, sig, t, kk, pa, q, ke, ki, ze, zi, o);
-    cx<R>* d = ar + 2 * q * NREC + (kk * q + pa) * 4;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) d[c] = o[c];
-  }
-  __syncthreads();
-  for (int u = T; u < ncol * 12; u += blockDim.x) {  // more tasks than threads when q = 1
-    const int c2 = u / 12, r = u - c2 * 12;
-    const int kk = r >> 2, c = r & 3;
-    const cx<R>* sp = area + (int64_t)c2 * pb_col_complex(q) + 2 * q * NREC + kk * q * 4 + c;
-    cx<R> v = czero<R>();
-    for (int pa = 0; pa < q; ++pa) v += sp[pa * 4];
-    const int row = valrow[(t * 3 + kk) * 4 + c];
-    if (row >= 0) {
-      cx<R>* yc = y + c2 * ldy;
-      atomicAdd(&yc[row].re, v.re);
-      atomicAdd(&yc[row].im, v.im);
-    }
-  }
-}
 
 // ================================================================ transposed apply
 // x_bar = A^T y_bar: the stages of the apply in reverse order, each the
@@ -1329,7 +1148,7 @@ __global__ void k_x_adj(const cx<R>* __restrict__ stot, const int32_t* __restric
 template <typename R>
 using PointsFn = void (*)(const cx<R>*, const int32_t*, const R*, const R*, const cx<R>*, const int32_t*,
                           const int32_t*, const cx<R>*, const double*, const R*, const R*, int64_t, int, int, int,
-                          int, R, R, R, R, int, const int32_t*, cx<R>*, int*, const cx<R>*, cx<R>*);
+                          int, R, R, R, R, int, const int32_t*, cx<R>*, int*, const cx<R>*, cx<R>*, int64_t, int64_t);
 
 template <typename R>
 PrecData<R>& pdata(scabem_op* op);
@@ -1345,47 +1164,6 @@ PrecData<double>& pdata<double>(scabem_op* op) {
 }  // namespace
 
 template <typename R>
-int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s) {
-  PrecData<R>& pd = pdata<R>(op);
-  const int64_t nt = op->nt, Q = op->Q;
-  const int n0 = op->n[0], n1 = op->n[1], n2 = op->n[2];
-  const int64_t ng = (int64_t)n0 * n1 * n2;
-  prof_mark(op, s);
-  k_sources<R><<<(int)cdiv(Q, 128), 128, 0, s>>>(x, op->unk, op->cX, op->tri, op->qp, op->qw, Q, op->q, pd.summ,
-                                                 pd.qsrc, y, op->N, 0, 0);
-  CK(cudaGetLastError());
-  prof_mark(op, s);
-  if (op->ngnz > 0) {
-    k_gather<R><<<(int)cdiv(op->ngnz * 32, 256), 256, 0, s>>>(pd.qsrc, op->gpt, op->goff, op->gent,
-                                                              gather_weights<R>(op), op->ngnz, ng, pd.src, 0, 0);
-    CK(cudaGetLastError());
-  }
-  prof_mark(op, s);
-  int rc = fft_conv<R>(op, pd, s, false);
-  if (rc) return rc;
-  prof_mark(op, s);
-  {
-    const size_t sm = pt_smem_bytes(op->q, sizeof(cx<R>));
-    PointsFn<R> fn = op->q == 6 ? (op->p == 2 ? k_points<R, 2, false, 6> : op->p == 3 ? k_points<R, 3, false, 6>
-                                                                                   : k_points<R, 4, false, 6>)
-                                : (op->p == 2 ? k_points<R, 2> : op->p == 3 ? k_points<R, 3> : k_points<R, 4>);
-    if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
-    fn<<<(int)cdiv(nt, PT_WARPS), PT_WARPS * 32, sm, s>>>(pd.grid, op->base, pd.L, pd.dL, pd.near, op->noff, op->nsrc, pd.summ,
-                                                  op->tri, pd.tp, pd.sig, nt, op->q, n0, n1, n2, (R)op->ke, (R)op->ki,
-                                                  (R)op->ze, (R)op->zi, op->npairs > 0 ? 1 : 0, op->valrow, y,
-                                                  op->tmo_d, nullptr, nullptr);
-    CK(cudaGetLastError());
-  }
-  prof_mark(op, s);
-  return SCABEM_OK;
-}
-
-template <typename R>
-using PointsBatchFn = void (*)(const cx<R>*, const int32_t*, const R*, const R*, const cx<R>*, const int32_t*,
-                               const int32_t*, const cx<R>*, const double*, const R*, const R*, int64_t, int, int, int,
-                               int, R, R, R, R, int, const int32_t*, cx<R>*, int*, int64_t, int64_t, int64_t, int);
-
-template <typename R>
 int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int k, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
   if (k < 1 || k > KBATCH || k > pd.kcap) {
@@ -1397,7 +1175,7 @@ int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
   const int64_t ng = (int64_t)n0 * n1 * n2;
   prof_mark(op, s);
   k_sources<R><<<dim3((unsigned)cdiv(Q, 128), k), 128, 0, s>>>(x, op->unk, op->cX, op->tri, op->qp, op->qw, Q,
-                                                               op->q, pd.summ, pd.qsrc, y, op->N, ldx, ldy);
+                                                               op->q, pd.summ, pd.qsrc, ldx);
   CK(cudaGetLastError());
   prof_mark(op, s);
   if (op->ngnz > 0) {
@@ -1411,20 +1189,25 @@ int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
   if (rc) return rc;
   prof_mark(op, s);
   {
-    const size_t sm = pb_smem_bytes(op->q, k, sizeof(cx<R>));
-    PointsBatchFn<R> fn =
-        op->q == 6 ? (op->p == 2 ? k_points_batch<R, 2, 6> : op->p == 3 ? k_points_batch<R, 3, 6> : k_points_batch<R, 4, 6>)
-                   : (op->p == 2 ? k_points_batch<R, 2> : op->p == 3 ? k_points_batch<R, 3> : k_points_batch<R, 4>);
-    if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)pb_smem_bytes(op->q, KBATCH, sizeof(cx<R>))))
-      return rc_;
-    fn<<<(unsigned)nt, pb_threads(op->q, k), sm, s>>>(
+    const size_t sm = pt_smem_bytes(op->q, sizeof(cx<R>));
+    PointsFn<R> fn = op->q == 6 ? (op->p == 2 ? k_points<R, 2, false, 6> : op->p == 3 ? k_points<R, 3, false, 6>
+                                                                                   : k_points<R, 4, false, 6>)
+                                : (op->p == 2 ? k_points<R, 2> : op->p == 3 ? k_points<R, 3> : k_points<R, 4>);
+    if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
+    fn<<<dim3((unsigned)cdiv(nt, PT_WARPS), k), PT_WARPS * 32, sm, s>>>(
         pd.grid, op->base, pd.L, pd.dL, pd.near, op->noff, op->nsrc, pd.summ, op->tri, pd.tp, pd.sig, nt, op->q, n0,
-        n1, n2, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi, op->npairs > 0 ? 1 : 0, op->valrow, y, op->tmo_d,
-        col_stride_grid(op), col_stride_summ(op), ldy, k);
+        n1, n2, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi, 0, op->valrow, pd.val, op->tmo_d, nullptr, nullptr,
+        col_stride_grid(op), col_stride_val(op));
     CK(cudaGetLastError());
   }
+  if ((rc = near_rows<R>(op, x, ldx, y, ldy, k, s))) return rc;
   prof_mark(op, s);
   return SCABEM_OK;
+}
+
+template <typename R>
+int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s) {
+  return apply_batch<R>(op, x, op->N, y, op->N, 1, s);
 }
 
 template <typename R>
@@ -1480,16 +1263,15 @@ int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_
 
 // hs[p] = d(lam^T A x)/d sigma_p [per S] at every quadrature point
 // (complex128): the apply's stages up to the records, then the derivative
-// of the sigma-weighted testing (k_points in its sensitivity mode).  yscr:
-// N complex of scratch.
+// of the sigma-weighted testing (k_points in its sensitivity mode).
 int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* lam, cx<double>* hs,
-                         cx<double>* yscr, cudaStream_t s) {
+                         cudaStream_t s) {
   PrecData<double>& pd = op->d;
   const int64_t nt = op->nt, Q = op->Q;
   const int n0 = op->n[0], n1 = op->n[1], n2 = op->n[2];
   const int64_t ng = (int64_t)n0 * n1 * n2;
   k_sources<double><<<(int)cdiv(Q, 128), 128, 0, s>>>(x, op->unk, op->cX, op->tri, op->qp, op->qw, Q, op->q,
-                                                      pd.summ, pd.qsrc, yscr, op->N, 0, 0);
+                                                      pd.summ, pd.qsrc, op->N);
   CK(cudaGetLastError());
   if (op->ngnz > 0) {
     k_gather<double><<<(int)cdiv(op->ngnz * 32, 256), 256, 0, s>>>(pd.qsrc, op->gpt, op->goff, op->gent, op->gwd,
@@ -1505,7 +1287,7 @@ int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* l
   fn<<<(int)cdiv(nt, PT_WARPS), PT_WARPS * 32, sm, s>>>(pd.grid, op->base, pd.L, pd.dL, pd.near, op->noff, op->nsrc,
                                                         pd.summ, op->tri, pd.tp, pd.sig, nt, op->q, n0, n1, n2, op->ke,
                                                         op->ki, op->ze, op->zi, op->npairs > 0 ? 1 : 0, op->valrow,
-                                                        yscr, op->tmo_d, lam, hs);
+                                                        nullptr, op->tmo_d, lam, hs, 0, 0);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }

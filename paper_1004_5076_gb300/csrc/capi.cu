@@ -98,6 +98,9 @@ void free_prec(PrecData<R>& pd) {
   cudaFree(pd.val);
   cudaFree(pd.recb);
   cudaFree(pd.nadj);
+  cudaFree(pd.nmv);
+  cudaFree(pd.nmt);
+  cudaFree(pd.gram);
   cudaFree(pd.sbar);
   cudaFree(pd.xs);
   cudaFree(pd.ys);
@@ -161,11 +164,12 @@ int ensure_batch(scabem_op* op, int k, cudaStream_t s) {
   }
   if (k <= pd.kcap) return SCABEM_OK;
   CK(cudaStreamSynchronize(s));  // nothing in flight uses the old buffers
-  cx<R>* nb[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  cx<R>** cur[6] = {&pd.summ, &pd.qsrc, &pd.src, &pd.stA, &pd.stB, &pd.grid};
-  const int64_t cs[6] = {col_stride_summ(op), col_stride_qsrc(op), col_stride_grid(op), col_stride_st(op),
-                         col_stride_st(op), col_stride_grid(op)};
-  for (int i = 0; i < 6; ++i) {
+  constexpr int NB = 7;
+  cx<R>* nb[NB] = {};
+  cx<R>** cur[NB] = {&pd.summ, &pd.qsrc, &pd.src, &pd.stA, &pd.stB, &pd.grid, &pd.val};
+  const int64_t cs[NB] = {col_stride_summ(op), col_stride_qsrc(op), col_stride_grid(op), col_stride_st(op),
+                          col_stride_st(op), col_stride_grid(op), col_stride_val(op)};
+  for (int i = 0; i < NB; ++i) {
     int rc = dalloc(&nb[i], cs[i] * k);
     if (rc) {
       for (int j = 0; j < i; ++j) cudaFree(nb[j]);
@@ -173,12 +177,12 @@ int ensure_batch(scabem_op* op, int k, cudaStream_t s) {
     }
   }
   // column 0 keeps its contents (the single-column paths use it); the others start at zero
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < NB; ++i) {
     CK(cudaMemcpyAsync(nb[i], *cur[i], sizeof(cx<R>) * cs[i], cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(nb[i] + cs[i], 0, sizeof(cx<R>) * cs[i] * (k - 1), s));
   }
   CK(cudaStreamSynchronize(s));
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < NB; ++i) {
     cudaFree(*cur[i]);
     *cur[i] = nb[i];
   }
@@ -608,6 +612,18 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
       eunk[3 * e + 2] = (int32_t)(2 * nL + 2 * nR + ci);
     }
   }
+  // the edges in class order (plain, then absorber) and each triangle's edges in it
+  std::vector<int32_t> rtk(4 * m->ne), tedge(3 * m->nt);
+  for (int64_t e = 0; e < m->ne; ++e) {
+    const int64_t r = (m->eclass[e] == 0 ? 0 : nL) + m->ecidx[e];
+    for (int c = 0; c < 4; ++c) rtk[4 * r + c] = etk[4 * e + c];
+  }
+  for (int64_t i = 0; i < 3 * m->nt; ++i) {
+    const int32_t e = m->tri_edge[i];
+    tedge[i] = (int32_t)((m->eclass[e] == 0 ? 0 : nL) + m->ecidx[e]);
+  }
+  TRY(dalloc(&op->rtk, 4 * op->ne));
+  TRY(dalloc(&op->tedge, 3 * op->nt));
   TRY(dalloc(&op->etk, 4 * op->ne));
   TRY(dalloc(&op->ecls, op->ne));
   TRY(dalloc(&op->eunk, 3 * op->ne));
@@ -640,6 +656,8 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
   TRY(upload(op->xsrc, xsrc.data(), sizeof(int32_t) * xsrc.size()));
   TRY(upload(op->region, m->region.data(), sizeof(int32_t) * m->nt));
   TRY(upload(op->etk, etk.data(), sizeof(int32_t) * etk.size()));
+  TRY(upload(op->rtk, rtk.data(), sizeof(int32_t) * rtk.size()));
+  TRY(upload(op->tedge, tedge.data(), sizeof(int32_t) * tedge.size()));
   TRY(upload(op->ecls, ecls.data(), sizeof(int32_t) * ecls.size()));
   TRY(upload(op->eunk, eunk.data(), sizeof(int32_t) * eunk.size()));
   TRY(setup_geometry(op, m, s));
@@ -649,6 +667,7 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
   TRY(alloc_st(op, op->f, s));
   TRY(setup_green(op, s));
   TRY(setup_near(op, s));
+  TRY(setup_near_matrix(op, s));
   TRY(setup_sigma_monomial(op, 0, nullptr, s));
   *out = op;
   return SCABEM_OK;
@@ -801,6 +820,15 @@ void scabem_op_destroy(scabem_op_t op) {
   cudaFree(op->roff);
   cudaFree(op->rpair);
   cudaFree(op->xsrc);
+  cudaFree(op->rtk);
+  cudaFree(op->tedge);
+  cudaFree(op->nm_off);
+  cudaFree(op->nm_nl);
+  cudaFree(op->nm_col);
+  cudaFree(op->nm_tpos);
+  cudaFree(op->nm_vo);
+  cudaFree(op->nm_vt);
+  cudaFree(op->nm_gcol);
   cudaFree(op->acoord);
   if (op->tmo_h) cudaFreeHost(op->tmo_h);
   free_prec(op->f);

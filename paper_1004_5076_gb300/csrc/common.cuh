@@ -150,7 +150,10 @@ struct PrecData {
   cx<R>* nadj = nullptr;  // npairs * 12: per-pair near contributions (transposed apply)
   cx<R>* stB = nullptr;   // 16 * P0 * cst
   cx<R>* grid = nullptr;  // n0 n1 n2 * 16, point-major: [point][medium][J, M set][A or F (3), phi or psi]
-  cx<R>* val = nullptr;   // nt * 3 * 4
+  cx<R>* val = nullptr;   // nt * 3 * 4 tested values of the grid part
+  cx<R>* nmv = nullptr;   // near matrix, row-wise (near.cu)
+  cx<R>* nmt = nullptr;   // near matrix, transposed
+  R* gram = nullptr;      // nR * 5: <X_r, X_m> of absorber edges sharing a triangle
   cx<R>* xs = nullptr;    // staging for host x/y: N * nrhs_cap
   cx<R>* ys = nullptr;
   int64_t stage_cap = 0;
@@ -229,6 +232,21 @@ struct scabem_op {
   int64_t npairs = 0;
   int32_t* noff = nullptr;  // nt + 1
   int32_t* nsrc = nullptr;  // npairs
+  // near matrix over pairs of edges in class order (near.cu): row r's columns
+  // nm_col[nm_off[r] .. nm_off[r+1]), the nm_nl[r] plain ones first; nm_tpos =
+  // position of r among the columns of nm_col[i]; values of row r from
+  // nm_vo[r] (row-wise) and nm_vt[r] (transposed)
+  int32_t* rtk = nullptr;    // ne * 4: T+, k+, T-, k- of the edges in class order
+  int32_t* tedge = nullptr;  // nt * 3: class-order number of each local edge
+  int64_t nm_nnz = 0;
+  int32_t* nm_off = nullptr;
+  int32_t* nm_nl = nullptr;
+  int32_t* nm_col = nullptr;
+  int32_t* nm_tpos = nullptr;
+  int64_t* nm_vo = nullptr;
+  int64_t* nm_vt = nullptr;
+  int32_t* nm_gcol = nullptr;  // nR * 5 columns of gram, -1 past the last
+  bool nm_ready = false;       // values formed for all rows
   // reverse list: pairs rpair[roff[s] .. roff[s+1]) have source triangle s
   int32_t* roff = nullptr;   // nt + 1
   int32_t* rpair = nullptr;  // npairs
@@ -260,6 +278,7 @@ inline int64_t col_stride_grid(const scabem_op* op) {  // src and grid
 inline int64_t col_stride_st(const scabem_op* op) {  // stA and stB
   return (int64_t)NFIELD_OUT * op->P[0] * op->cst;
 }
+inline int64_t col_stride_val(const scabem_op* op) { return op->nt * 12; }
 inline int64_t col_stride_summ(const scabem_op* op) { return op->nt * 12; }
 inline int64_t col_stride_qsrc(const scabem_op* op) { return op->Q * 12; }
 // Right-hand sides the batched apply handles per pass (one CTA of that many
@@ -315,6 +334,12 @@ int setup_circulant(scabem_op* op, const scabem_mesh* mesh, const scabem_circula
 int circulant_apply(scabem_op* op, const cx<double>* in, cx<double>* out, int k, int64_t cs_in, int64_t cs_out,
                     cudaStream_t s);
 void circulant_release(scabem_op* op);
+// near.cu
+int setup_near_matrix(scabem_op* op, cudaStream_t s);
+int near_matrix_update(scabem_op* op, cudaStream_t s);
+// y_c = near part of A x_c + row sums of the tested values pd.val (column c), c < kc <= KBATCH
+template <typename R>
+int near_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s);
 // apply.cu
 template <typename R>
 int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s);
@@ -328,7 +353,7 @@ template <typename R>
 int ensure_batch(scabem_op* op, int k, cudaStream_t s);
 // hs[p] = d(lam^T A x)/d sigma_p [per S] at every quadrature point (complex128)
 int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* lam, cx<double>* hs,
-                         cx<double>* yscr, cudaStream_t s);
+                         cudaStream_t s);
 // x_bar = A^T y_bar (transpose, no conjugation)
 template <typename R>
 int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_t s);

@@ -1,0 +1,657 @@
+// Near-field precorrection and local terms as a sparse Galerkin matrix.
+//
+// The precorrection of the precorrected-FFT method (Appendix B's near data at
+// the target quadrature points, exact minus grid moments) reaches the rows
+// only through the Galerkin testing of Eqs. 1-3, 13 and 14, and its sources
+// only through the RWG expansion.  Both are linear and fixed while the
+// conductivity is, so the product of testing, near records and expansion is
+// formed once (set-up, and again for the absorber rows on every
+// scabem_set_sigma): one small block per pair of edges of which some pair of
+// triangles is near, together with the side-limit terms of the triangles the
+// two edges share.  With J_i = -J_e on plain (L) edges and the same panel
+// moments in the rows of E and H, the block of an edge pair holds
+//
+//   row L, col L (3):  U  G  V
+//     E: U xJ - G xM                     H: G xJ + V xM
+//   row L, col R (5):  Ue Ui ge gi V
+//     E: Ue Je - Ui Ji - (ge + gi) M     H: ge Je - gi Ji + V M
+//   row R, col L (6):  U  G  G13 V13 P Q
+//     Eq. 3: U xJ - G xM   Eq. 13: G13 xJ + V13 xM   Eq. 14: P xJ + Q xM
+//   row R, col R (8):  Ue Ui e13 i13 G V13 P Q
+//     Eq. 3: Ue Je - Ui Ji - G M   Eq. 13: e13 Je + i13 Ji + V13 M
+//     Eq. 14: P Ji + Q M (+ <X, X'> Je of edges sharing a triangle)
+//
+// where U = j (z/k phi - z k alpha), V = j (phi/(k z) - (k/z) alpha),
+// alpha = <X, A>, phi = <div X, phi>, g = <X, curl A> of the unit current
+// of the column edge, summed over media without a subscript, and the 13 / P /
+// Q entries carry the sigma-weighted and side-limit terms of their rows.
+//
+// Edges are numbered by class here: row or column r < nL is the plain edge of
+// class index r, r >= nL the absorber edge r - nL.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "common.cuh"
+
+namespace {
+
+using cd = cx<double>;
+
+// values per edge pair, by (row class, column class)
+__host__ __device__ constexpr int nm_words(bool rowR, bool colR) {
+  return rowR ? (colR ? 8 : 6) : (colR ? 5 : 3);
+}
+
+// index of near pair (t, s) in t's ascending source list, -1 if absent
+__device__ __forceinline__ int find_pair(const int32_t* __restrict__ noff, const int32_t* __restrict__ nsrc, int t,
+                                         int s) {
+  int lo = noff[t], hi = noff[t + 1];
+  const int end = hi;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (nsrc[mid] < s)
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  return lo < end && nsrc[lo] == s ? lo : -1;
+}
+__device__ __forceinline__ bool near_or_same(const int32_t* __restrict__ noff, const int32_t* __restrict__ nsrc, int t,
+                                             int s) {
+  return t == s || find_pair(noff, nsrc, t, s) >= 0;
+}
+
+// Columns of every row, one warp per row: the edges of the near (or same)
+// triangles s of the row's two triangles.  An edge met through several
+// triangle pairs is kept at the first of them (T+ before T-, then the lower
+// source triangle), which needs two look-ups and no sorting.  cnt != null
+// counts (cnt[r] all, nl[r] plain columns); else the columns are written,
+// plain ones first.
+__global__ void __launch_bounds__(128) k_near_pattern(const int32_t* __restrict__ rtk, const int32_t* __restrict__ tedge,
+                                                      const int32_t* __restrict__ noff,
+                                                      const int32_t* __restrict__ nsrc, int64_t ne, int64_t nL,
+                                                      int32_t* __restrict__ cnt, int32_t* __restrict__ nl,
+                                                      const int32_t* __restrict__ off, int32_t* __restrict__ col) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (r >= ne) return;
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1;
+  const int T0 = rtk[4 * r];
+  int cl = 0, cr = 0;
+  const int64_t bl = cnt ? 0 : off[r], br = cnt ? 0 : bl + nl[r];
+  for (int it = 0; it < 2; ++it) {
+    const int t = rtk[4 * r + 2 * it];
+    const int n0 = noff[t], len = noff[t + 1] - n0;
+    const int total = len > 0 ? 3 * len : 3;  // without near data: the triangle itself
+    for (int i0 = 0; i0 < total; i0 += 32) {
+      const int i = i0 + lane;
+      bool keep = i < total;
+      int m = 0;
+      if (keep) {
+        const int s = len > 0 ? nsrc[n0 + i / 3] : t;
+        m = tedge[3 * (int64_t)s + i % 3];
+        const int s2 = rtk[4 * (int64_t)m] == s ? rtk[4 * (int64_t)m + 2] : rtk[4 * (int64_t)m];
+        if (s2 < s && near_or_same(noff, nsrc, t, s2)) keep = false;
+        if (keep && it == 1 && (near_or_same(noff, nsrc, T0, s) || near_or_same(noff, nsrc, T0, s2))) keep = false;
+      }
+      const unsigned ml = __ballot_sync(0xffffffffu, keep && m < nL), mr = __ballot_sync(0xffffffffu, keep && m >= nL);
+      if (!cnt && keep) {
+        if (m < nL)
+          col[bl + cl + __popc(ml & below)] = m;
+        else
+          col[br + cr + __popc(mr & below)] = m;
+      }
+      cl += __popc(ml);
+      cr += __popc(mr);
+    }
+  }
+  if (cnt && lane == 0) {
+    cnt[r] = cl + cr;
+    nl[r] = cl;
+  }
+}
+
+// tpos[i] = position of row r among the columns of row m = col[i] (the
+// pattern is symmetric), one warp per row r
+__global__ void __launch_bounds__(128) k_near_tpos(const int32_t* __restrict__ off, const int32_t* __restrict__ nl,
+                                                   const int32_t* __restrict__ col, int64_t ne, int64_t nL,
+                                                   int32_t* __restrict__ tpos) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (r >= ne) return;
+  for (int i = off[r] + (threadIdx.x & 31); i < off[r + 1]; i += 32) {
+    const int m = col[i];
+    const int b = off[m], e0 = r < nL ? b : b + nl[m], e1 = r < nL ? b + nl[m] : off[m + 1];
+    int p = 0;
+    for (int k = e0; k < e1; ++k)
+      if (col[k] == r) p = k - b;
+    tpos[i] = p;
+  }
+}
+
+// Values of the rows r0 .. ne - 1, one warp per row, one lane per column:
+// sums over the (at most four) near triangle pairs of the edge pair and the
+// target points, in FP64, from the near records of type RG.  Written to the
+// row-wise (f) and the transposed (t) copies of each precision that is built.
+template <typename RG>
+__global__ void __launch_bounds__(128)
+    k_near_values(int64_t r0, int64_t ne, int64_t nL, const int32_t* __restrict__ off, const int32_t* __restrict__ nl,
+                  const int32_t* __restrict__ col, const int32_t* __restrict__ tpos, const int64_t* __restrict__ vo,
+                  const int64_t* __restrict__ vt, const int32_t* __restrict__ rtk, const int32_t* __restrict__ noff,
+                  const int32_t* __restrict__ nsrc, const cx<RG>* __restrict__ rec, const double* __restrict__ tri,
+                  const double* __restrict__ cX, const double* __restrict__ tp, const double* __restrict__ sig, int q,
+                  double ke, double ki, double ze, double zi, cd* __restrict__ fd, cd* __restrict__ td,
+                  cx<float>* __restrict__ ff, cx<float>* __restrict__ tf) {
+  const int64_t r = r0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  if (r >= ne) return;
+  const bool rowR = r >= nL;
+  const int cl = nl[r], c0 = off[r], cnt = off[r + 1] - c0;
+  for (int j = threadIdx.x & 31; j < cnt; j += 32) {
+    const int m = col[c0 + j];
+    const bool colR = m >= nL;
+    cd al[2], ph[2], ga[2];  // alpha, phi, gamma per medium
+    for (int i = 0; i < 2; ++i) al[i] = ph[i] = ga[i] = mk(0.0, 0.0);
+    cd s13J = mk(0.0, 0.0), s13M = s13J, s14J = s13J, s14M = s13J;  // sigma-weighted, without the factor j of J
+    double xx = 0.0, xnx = 0.0, sxx = 0.0, sxnx = 0.0;              // shared-triangle terms
+    for (int pr = 0; pr < 4; ++pr) {
+      const int t = rtk[4 * r + 2 * (pr >> 1)], k = rtk[4 * r + 2 * (pr >> 1) + 1];
+      const int s = rtk[4 * (int64_t)m + 2 * (pr & 1)], l = rtk[4 * (int64_t)m + 2 * (pr & 1) + 1];
+      const int p = find_pair(noff, nsrc, t, s);
+      if (p < 0 && t != s) continue;
+      const double* n = tri + 16 * (int64_t)t + 12;
+      const double* gs = tri + 16 * (int64_t)s;
+      const double a0 = cX[3 * (int64_t)s + l];
+      const double be[3] = {a0 * (gs[3 * l] - gs[9]), a0 * (gs[3 * l + 1] - gs[10]), a0 * (gs[3 * l + 2] - gs[11])};
+      for (int a = 0; a < q; ++a) {
+        const int64_t Qa = (int64_t)t * q + a;
+        const double* tq = tp + 16 * Qa;
+        const double w = tq[3], sg = rowR ? w * sig[Qa] : 0.0, dv = w * tq[13 + k];
+        const double X[3] = {tq[4 + 3 * k], tq[5 + 3 * k], tq[6 + 3 * k]};
+        const double nX[3] = {n[1] * X[2] - n[2] * X[1], n[2] * X[0] - n[0] * X[2], n[0] * X[1] - n[1] * X[0]};
+        if (t == s) {
+          const double* Y = tq + 4 + 3 * l;
+          const double d = X[0] * Y[0] + X[1] * Y[1] + X[2] * Y[2];
+          const double c = -(nX[0] * Y[0] + nX[1] * Y[1] + nX[2] * Y[2]);  // X . (n x Y)
+          xx += w * d;
+          xnx += w * c;
+          sxx += sg * d;
+          sxnx += sg * c;
+        }
+        if (p < 0) continue;
+        // X . (Q x be) = Q . (be x X)
+        const double bX[3] = {be[1] * X[2] - be[2] * X[1], be[2] * X[0] - be[0] * X[2], be[0] * X[1] - be[1] * X[0]};
+        const double Xb = X[0] * be[0] + X[1] * be[1] + X[2] * be[2];
+#pragma unroll
+        for (int med = 0; med < 2; ++med) {
+          const cx<RG>* dp = rec + (((int64_t)p * q + a) * 2 + med) * NCORR;
+          cd d[NCORR];
+#pragma unroll
+          for (int c = 0; c < NCORR; ++c) d[c] = mk((double)dp[c].re, (double)dp[c].im);
+          cd xa = mk(0.0, 0.0), xc = xa;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            axpy(xa, a0 * X[c], d[1 + c]);
+            axpy(xc, a0 * X[c], d[7 + c]);
+            axpy(xc, -bX[c], d[4 + c]);
+          }
+          axpy(xa, -Xb, d[0]);
+          axpy(al[med], w, xa);
+          axpy(ph[med], 2.0 * a0 * dv, d[0]);
+          axpy(ga[med], w, xc);
+          if (rowR) {
+            const double k_ = med ? ki : ke, z = med ? zi : ze;
+            if (med == 0) {
+              const double nb = nX[0] * be[0] + nX[1] * be[1] + nX[2] * be[2];
+              const double bn[3] = {be[1] * nX[2] - be[2] * nX[1], be[2] * nX[0] - be[0] * nX[2],
+                                    be[0] * nX[1] - be[1] * nX[0]};
+              cd na = mk(0.0, 0.0), ng = na, nc = na;
+#pragma unroll
+              for (int c = 0; c < 3; ++c) {
+                axpy(na, a0 * nX[c], d[1 + c]);
+                axpy(ng, 2.0 * a0 * nX[c], d[4 + c]);
+                axpy(nc, a0 * nX[c], d[7 + c]);
+                axpy(nc, -bn[c], d[4 + c]);
+              }
+              axpy(na, -nb, d[0]);
+              axpy(s13J, sg * z * k_, na);
+              axpy(s13J, sg * z / k_, ng);
+              axpy(s13M, sg, nc);
+            } else {
+              cd xg = mk(0.0, 0.0);
+#pragma unroll
+              for (int c = 0; c < 3; ++c) axpy(xg, 2.0 * a0 * X[c], d[4 + c]);
+              axpy(s14J, sg * z * k_, xa);
+              axpy(s14J, sg * z / k_, xg);
+              axpy(s14M, -sg, xc);
+            }
+          }
+        }
+      }
+    }
+    const cd Ue = mulj((ze / ke) * ph[0] - (ze * ke) * al[0]), Ui = mulj((zi / ki) * ph[1] - (zi * ki) * al[1]);
+    const cd V = mulj((1.0 / (ke * ze)) * ph[0] - (ke / ze) * al[0] + (1.0 / (ki * zi)) * ph[1] - (ki / zi) * al[1]);
+    const cd G = ga[0] + ga[1];
+    cd v[8];
+    if (!rowR) {
+      if (!colR) {
+        v[0] = Ue + Ui;
+        v[1] = G;
+        v[2] = V;
+      } else {
+        v[0] = Ue;
+        v[1] = Ui;
+        v[2] = ga[0];
+        v[3] = ga[1];
+        v[4] = V;
+      }
+    } else {
+      const cd V13 = V + s13M - mk(0.5 * sxx, 0.0), Q = s14M - mk(0.5 * sxnx, 0.0);
+      if (!colR) {
+        v[0] = Ue + Ui;
+        v[1] = G;
+        v[2] = G + mulj(s13J);
+        v[3] = V13;
+        v[4] = -mulj(s14J);
+        v[5] = Q;
+      } else {
+        v[0] = Ue;
+        v[1] = Ui;
+        v[2] = ga[0] + mulj(s13J) - mk(0.5 * xnx, 0.0);
+        v[3] = -ga[1] - mk(0.5 * xnx, 0.0);
+        v[4] = G;
+        v[5] = V13;
+        v[6] = mulj(s14J) + mk(xx, 0.0);
+        v[7] = Q;
+      }
+    }
+    const int words = nm_words(rowR, colR);
+    // row-wise: [plain columns][word][column], [absorber columns][word][column]
+    const int64_t fb = vo[r] + (colR ? (int64_t)nm_words(rowR, false) * cl + (j - cl) : j);
+    const int fs = colR ? cnt - cl : cl;
+    // transposed: row m, its neighbours' position of r
+    const int tl = nl[m], tc = off[m + 1] - off[m], tj = tpos[c0 + j];
+    const int64_t tb = vt[m] + (rowR ? (int64_t)nm_words(false, colR) * tl + (tj - tl) : tj);
+    const int ts = rowR ? tc - tl : tl;
+    for (int e = 0; e < words; ++e) {
+      if (fd) fd[fb + (int64_t)e * fs] = v[e];
+      if (ff) ff[fb + (int64_t)e * fs] = cvt<float>(v[e]);
+      if (td) td[tb + (int64_t)e * ts] = v[e];
+      if (tf) tf[tb + (int64_t)e * ts] = cvt<float>(v[e]);
+    }
+  }
+}
+
+// <X_r, X_m> of absorber edge r with the absorber edges m of its two
+// triangles (at most five): the Eq. 14 coefficient of J_e
+__global__ void k_near_gram(const int32_t* __restrict__ rtk, const int32_t* __restrict__ tedge,
+                            const double* __restrict__ tp, int64_t ne, int64_t nL, int q, int32_t* __restrict__ gcol,
+                            double* __restrict__ gd, float* __restrict__ gf) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= ne - nL) return;
+  const int64_t r = nL + i;
+  int col[5];
+  double val[5];
+  int n = 0;
+  for (int it = 0; it < 2; ++it) {
+    const int64_t t = rtk[4 * r + 2 * it];
+    const int k = rtk[4 * r + 2 * it + 1];
+    for (int l = 0; l < 3; ++l) {
+      const int m = tedge[3 * t + l];
+      if (m < nL) continue;
+      double s = 0.0;
+      for (int a = 0; a < q; ++a) {
+        const double* tq = tp + 16 * (t * q + a);
+        for (int c = 0; c < 3; ++c) s += tq[3] * tq[4 + 3 * k + c] * tq[4 + 3 * l + c];
+      }
+      int f = 0;
+      while (f < n && col[f] != m) ++f;
+      if (f == n) {
+        if (n == 5) continue;
+        col[n] = m;
+        val[n++] = 0.0;
+      }
+      val[f] += s;
+    }
+  }
+  for (int f = 0; f < 5; ++f) {
+    gcol[5 * i + f] = f < n ? col[f] : -1;
+    gd[5 * i + f] = f < n ? val[f] : 0.0;
+    gf[5 * i + f] = f < n ? (float)val[f] : 0.f;
+  }
+}
+
+// ---------------------------------------------------------------- products
+template <typename R>
+__device__ __forceinline__ void cmac(cx<R>& a, cx<R> v, cx<R> x) {
+  cfma(a, v, x);
+}
+template <>
+__device__ __forceinline__ void cmac(cx<float>& a, cx<float> v, cx<float> x) {
+  // two packed FP32x2 FMAs: a + v.re (x.re, x.im) + v.im (-x.im, x.re)
+  float2 r = __ffma2_rn(make_float2(v.re, v.re), make_float2(x.re, x.im), make_float2(a.re, a.im));
+  r = __ffma2_rn(make_float2(v.im, v.im), make_float2(-x.im, x.re), r);
+  a = mk(r.x, r.y);
+}
+template <typename R>
+__device__ __forceinline__ cx<R> ldstream(const cx<R>* p) {
+  return *p;
+}
+
+// One row of the matrix (T = false) or of its transpose (T = true) against
+// the kc <= K columns of x: the row's three (two for a plain edge) sums in
+// acc, each lane of the NM_LANES sharing the row taking every NM_LANES-th
+// column.  x holds the unknowns (or, transposed, the rows) of an edge m at m,
+// nL + m (plain) or nL + m, nL + m + nR, nL + m + 2 nR (absorber).
+constexpr int NM_LANES = 16;
+constexpr int NM_THREADS = 128;
+
+template <typename R, int K, bool T>
+__device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, const int32_t* __restrict__ off,
+                                         const int32_t* __restrict__ nl, const int32_t* __restrict__ col,
+                                         const int64_t* __restrict__ vo, const cx<R>* __restrict__ val,
+                                         const cx<R>* __restrict__ x, int64_t ldx, int kc, int lane, cx<R> acc[3][K]) {
+  const bool isR = r >= nL;
+  const int c0 = off[r], cl = nl[r], cr = off[r + 1] - c0 - cl;
+  const cx<R>* v0 = val + vo[r];
+  if (!isR) {
+    for (int j = lane; j < cl; j += NM_LANES) {
+      const int m = col[c0 + j];
+      const cx<R> U = v0[j], G = v0[cl + j], V = v0[2 * cl + j];
+      const cx<R>* xm = x + m;
+#pragma unroll
+      for (int c = 0; c < K; ++c)
+        if (c < kc) {
+          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nL];
+          if (!T) {
+            cmac(acc[0][c], U, a);
+            cmac(acc[0][c], -G, b);
+            cmac(acc[1][c], G, a);
+            cmac(acc[1][c], V, b);
+          } else {
+            cmac(acc[0][c], U, a);
+            cmac(acc[0][c], G, b);
+            cmac(acc[1][c], -G, a);
+            cmac(acc[1][c], V, b);
+          }
+        }
+    }
+    v0 += (int64_t)nm_words(false, false) * cl;
+    for (int j = lane; j < cr; j += NM_LANES) {
+      const int m = col[c0 + cl + j];
+      cx<R> v[6];
+#pragma unroll
+      for (int e = 0; e < (T ? 6 : 5); ++e) v[e] = v0[(int64_t)e * cr + j];
+      const cx<R>* xm = x + nL + m;
+#pragma unroll
+      for (int c = 0; c < K; ++c)
+        if (c < kc) {
+          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nR], d = xm[c * ldx + 2 * nR];
+          if (!T) {  // Ue Ui ge gi V
+            cmac(acc[0][c], v[0], a);
+            cmac(acc[0][c], -v[1], b);
+            cmac(acc[0][c], -(v[2] + v[3]), d);
+            cmac(acc[1][c], v[2], a);
+            cmac(acc[1][c], -v[3], b);
+            cmac(acc[1][c], v[4], d);
+          } else {  // U G G13 V13 P Q against the rows of Eqs. 3, 13, 14
+            cmac(acc[0][c], v[0], a);
+            cmac(acc[0][c], v[2], b);
+            cmac(acc[0][c], v[4], d);
+            cmac(acc[1][c], -v[1], a);
+            cmac(acc[1][c], v[3], b);
+            cmac(acc[1][c], v[5], d);
+          }
+        }
+    }
+  } else {
+    for (int j = lane; j < cl; j += NM_LANES) {
+      const int m = col[c0 + j];
+      cx<R> v[6];
+#pragma unroll
+      for (int e = 0; e < (T ? 5 : 6); ++e) v[e] = v0[(int64_t)e * cl + j];
+      const cx<R>* xm = x + m;
+#pragma unroll
+      for (int c = 0; c < K; ++c)
+        if (c < kc) {
+          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nL];
+          if (!T) {
+            cmac(acc[0][c], v[0], a);
+            cmac(acc[0][c], -v[1], b);
+            cmac(acc[1][c], v[2], a);
+            cmac(acc[1][c], v[3], b);
+            cmac(acc[2][c], v[4], a);
+            cmac(acc[2][c], v[5], b);
+          } else {
+            cmac(acc[0][c], v[0], a);
+            cmac(acc[0][c], v[2], b);
+            cmac(acc[1][c], -v[1], a);
+            cmac(acc[1][c], -v[3], b);
+            cmac(acc[2][c], -(v[2] + v[3]), a);
+            cmac(acc[2][c], v[4], b);
+          }
+        }
+    }
+    v0 += (int64_t)(T ? 5 : 6) * cl;
+    for (int j = lane; j < cr; j += NM_LANES) {
+      const int m = col[c0 + cl + j];
+      cx<R> v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = v0[(int64_t)e * cr + j];
+      const cx<R>* xm = x + nL + m;
+#pragma unroll
+      for (int c = 0; c < K; ++c)
+        if (c < kc) {
+          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nR], d = xm[c * ldx + 2 * nR];
+          if (!T) {
+            cmac(acc[0][c], v[0], a);
+            cmac(acc[0][c], -v[1], b);
+            cmac(acc[0][c], -v[4], d);
+            cmac(acc[1][c], v[2], a);
+            cmac(acc[1][c], v[3], b);
+            cmac(acc[1][c], v[5], d);
+            cmac(acc[2][c], v[6], b);
+            cmac(acc[2][c], v[7], d);
+          } else {
+            cmac(acc[0][c], v[0], a);
+            cmac(acc[0][c], v[2], b);
+            cmac(acc[1][c], -v[1], a);
+            cmac(acc[1][c], v[3], b);
+            cmac(acc[1][c], v[6], d);
+            cmac(acc[2][c], -v[4], a);
+            cmac(acc[2][c], v[5], b);
+            cmac(acc[2][c], v[7], d);
+          }
+        }
+    }
+  }
+}
+
+// y = near part + the tested values of the grid part (val, summed per row
+// over the edge's two triangles): the last launch of an apply.  Every row is
+// written once, from sums in a fixed order.
+template <typename R, int K>
+__global__ void __launch_bounds__(NM_THREADS)
+    k_near_rows(const int32_t* __restrict__ off, const int32_t* __restrict__ nl, const int32_t* __restrict__ col,
+                const int64_t* __restrict__ vo, const cx<R>* __restrict__ nmv, const int32_t* __restrict__ gcol,
+                const R* __restrict__ gval, const int32_t* __restrict__ rtk, int64_t ne, int64_t nL,
+                const cx<R>* __restrict__ val, int64_t cs_val, const cx<R>* __restrict__ x, int64_t ldx,
+                cx<R>* __restrict__ y, int64_t ldy, int kc) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / NM_LANES;
+  const int lane = threadIdx.x % NM_LANES;
+  const int64_t nR = ne - nL;
+  cx<R> acc[3][K];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int c = 0; c < K; ++c) acc[i][c] = czero<R>();
+  if (r < ne) {
+    near_row<R, K, false>(r, nL, nR, off, nl, col, vo, nmv, x, ldx, kc, lane, acc);
+    if (r >= nL && lane < 5) {
+      const int g = gcol[5 * (r - nL) + lane];
+      if (g >= 0) {
+        const R s = gval[5 * (r - nL) + lane];
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+          if (c < kc) axpy(acc[2][c], s, x[c * ldx + nL + g]);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = NM_LANES / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        acc[i][c].re += __shfl_xor_sync(0xffffffffu, acc[i][c].re, o);
+        acc[i][c].im += __shfl_xor_sync(0xffffffffu, acc[i][c].im, o);
+      }
+  if (r >= ne || lane >= kc) return;
+  // lane c finishes column c
+  const int64_t v0 = ((int64_t)rtk[4 * r] * 3 + rtk[4 * r + 1]) * 4, v1 = ((int64_t)rtk[4 * r + 2] * 3 + rtk[4 * r + 3]) * 4;
+  const cx<R>* vc = val + lane * cs_val;
+  cx<R>* yc = y + lane * ldy;
+  cx<R> s[3];
+#pragma unroll
+  for (int c = 0; c < K; ++c)
+    if (c == lane)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) s[i] = acc[i][c];
+  if (r < nL) {
+    yc[r] = s[0] + (vc[v0] + vc[v1]);
+    yc[nL + r] = s[1] + (vc[v0 + 1] + vc[v1 + 1]);
+  } else {
+    yc[nL + r] = s[0] + (vc[v0] + vc[v1]);
+    yc[nL + r + nR] = s[1] + (vc[v0 + 2] + vc[v1 + 2]);
+    yc[nL + r + 2 * nR] = s[2] + (vc[v0 + 3] + vc[v1 + 3]);
+  }
+}
+
+template <typename R>
+PrecData<R>& pdata(scabem_op* op);
+template <>
+PrecData<float>& pdata<float>(scabem_op* op) {
+  return op->f;
+}
+template <>
+PrecData<double>& pdata<double>(scabem_op* op) {
+  return op->d;
+}
+
+template <typename R, int K>
+int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
+  PrecData<R>& pd = pdata<R>(op);
+  k_near_rows<R, K><<<(unsigned)cdiv(op->ne * NM_LANES, NM_THREADS), NM_THREADS, 0, s>>>(
+      op->nm_off, op->nm_nl, op->nm_col, op->nm_vo, pd.nmv, op->nm_gcol, pd.gram, op->rtk, op->ne, op->nL, pd.val,
+      op->nt * 12, x, ldx, y, ldy, kc);
+  CK(cudaGetLastError());
+  return SCABEM_OK;
+}
+
+}  // namespace
+
+// y_c = near part of A x_c + the row sums of pd.val's column c, c < kc <= KBATCH
+template <typename R>
+int near_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
+  switch (kc) {
+    case 1: return launch_rows<R, 1>(op, x, ldx, y, ldy, kc, s);
+    case 2: return launch_rows<R, 2>(op, x, ldx, y, ldy, kc, s);
+    case 3: return launch_rows<R, 3>(op, x, ldx, y, ldy, kc, s);
+    case 4: return launch_rows<R, 4>(op, x, ldx, y, ldy, kc, s);
+    case 5:
+    case 6: return launch_rows<R, 6>(op, x, ldx, y, ldy, kc, s);
+    default: return launch_rows<R, 8>(op, x, ldx, y, ldy, kc, s);
+  }
+}
+template int near_rows<float>(scabem_op*, const cx<float>*, int64_t, cx<float>*, int64_t, int, cudaStream_t);
+template int near_rows<double>(scabem_op*, const cx<double>*, int64_t, cx<double>*, int64_t, int, cudaStream_t);
+
+// Pattern and storage of the matrix (after the near list); its values follow
+// with the first conductivity.
+int setup_near_matrix(scabem_op* op, cudaStream_t s) {
+  const int64_t ne = op->ne, nL = op->nL, nR = op->nR;
+  const unsigned gw = (unsigned)cdiv(ne * 32, 128);
+  int32_t* cnt = nullptr;
+  CK(cudaMalloc(&op->nm_nl, sizeof(int32_t) * ne));
+  CK(cudaMalloc(&op->nm_off, sizeof(int32_t) * (ne + 1)));
+  CK(cudaMalloc(&op->nm_vo, sizeof(int64_t) * (ne + 1)));
+  CK(cudaMalloc(&op->nm_vt, sizeof(int64_t) * (ne + 1)));
+  cnt = op->nm_off;  // counts first, offsets afterwards
+  k_near_pattern<<<gw, 128, 0, s>>>(op->rtk, op->tedge, op->noff, op->nsrc, ne, nL, cnt, op->nm_nl, nullptr, nullptr);
+  CK(cudaGetLastError());
+  std::vector<int32_t> hc(ne + 1), hl(ne);
+  CK(cudaMemcpyAsync(hc.data(), cnt, sizeof(int32_t) * ne, cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(hl.data(), op->nm_nl, sizeof(int32_t) * ne, cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  std::vector<int64_t> vo(ne + 1), vt(ne + 1);
+  int64_t acc = 0, av = 0, at = 0;
+  for (int64_t r = 0; r < ne; ++r) {
+    const int64_t n = hc[r], l = hl[r];
+    hc[r] = (int32_t)acc;
+    vo[r] = av;
+    vt[r] = at;
+    acc += n;
+    av += nm_words(r >= nL, false) * l + nm_words(r >= nL, true) * (n - l);
+    at += nm_words(false, r >= nL) * l + nm_words(true, r >= nL) * (n - l);
+    if (acc > INT32_MAX) {
+      set_error("near list too long: reduce r_near");
+      return SCABEM_E_ARG;
+    }
+  }
+  hc[ne] = (int32_t)acc;
+  vo[ne] = av;
+  vt[ne] = at;
+  op->nm_nnz = acc;
+  CK(cudaMemcpyAsync(op->nm_off, hc.data(), sizeof(int32_t) * (ne + 1), cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(op->nm_vo, vo.data(), sizeof(int64_t) * (ne + 1), cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(op->nm_vt, vt.data(), sizeof(int64_t) * (ne + 1), cudaMemcpyHostToDevice, s));
+  CK(cudaMalloc(&op->nm_col, sizeof(int32_t) * acc));
+  CK(cudaMalloc(&op->nm_tpos, sizeof(int32_t) * acc));
+  k_near_pattern<<<gw, 128, 0, s>>>(op->rtk, op->tedge, op->noff, op->nsrc, ne, nL, nullptr, op->nm_nl, op->nm_off,
+                                    op->nm_col);
+  CK(cudaGetLastError());
+  k_near_tpos<<<gw, 128, 0, s>>>(op->nm_off, op->nm_nl, op->nm_col, ne, nL, op->nm_tpos);
+  CK(cudaGetLastError());
+  if (op->f.built) {
+    CK(cudaMalloc(&op->f.nmv, sizeof(cx<float>) * av));
+    CK(cudaMalloc(&op->f.nmt, sizeof(cx<float>) * at));
+  }
+  if (op->d.built) {
+    CK(cudaMalloc(&op->d.nmv, sizeof(cd) * av));
+    CK(cudaMalloc(&op->d.nmt, sizeof(cd) * at));
+  }
+  const int64_t ng = std::max<int64_t>(nR, 1) * 5;
+  CK(cudaMalloc(&op->nm_gcol, sizeof(int32_t) * ng));
+  CK(cudaMalloc(&op->d.gram, sizeof(double) * ng));
+  CK(cudaMalloc(&op->f.gram, sizeof(float) * ng));
+  if (nR > 0) {
+    k_near_gram<<<(unsigned)cdiv(nR, 128), 128, 0, s>>>(op->rtk, op->tedge, op->d.tp, ne, nL, op->q, op->nm_gcol,
+                                                        op->d.gram, op->f.gram);
+    CK(cudaGetLastError());
+  }
+  CK(cudaStreamSynchronize(s));
+  op->nm_ready = false;
+  return SCABEM_OK;
+}
+
+// Values for the operator's current conductivity: all rows the first time,
+// the absorber rows (the only ones that hold it) after that.
+int near_matrix_update(scabem_op* op, cudaStream_t s) {
+  const int64_t r0 = op->nm_ready ? op->nL : 0, nr = op->ne - r0;
+  if (nr > 0) {
+    const unsigned g = (unsigned)cdiv(nr * 32, 128);
+    if (op->d.near)
+      k_near_values<double><<<g, 128, 0, s>>>(r0, op->ne, op->nL, op->nm_off, op->nm_nl, op->nm_col, op->nm_tpos,
+                                              op->nm_vo, op->nm_vt, op->rtk, op->noff, op->nsrc, op->d.near, op->tri,
+                                              op->cX, op->d.tp, op->sig64, op->q, op->ke, op->ki, op->ze, op->zi,
+                                              op->d.nmv, op->d.nmt, op->f.nmv, op->f.nmt);
+    else
+      k_near_values<float><<<g, 128, 0, s>>>(r0, op->ne, op->nL, op->nm_off, op->nm_nl, op->nm_col, op->nm_tpos,
+                                             op->nm_vo, op->nm_vt, op->rtk, op->noff, op->nsrc, op->f.near, op->tri,
+                                             op->cX, op->d.tp, op->sig64, op->q, op->ke, op->ki, op->ze, op->zi,
+                                             op->d.nmv, op->d.nmt, op->f.nmv, op->f.nmt);
+    CK(cudaGetLastError());
+  }
+  op->nm_ready = true;
+  return SCABEM_OK;
+}

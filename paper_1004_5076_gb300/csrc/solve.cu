@@ -1488,8 +1488,8 @@ int rhs_impl(scabem_op* op, const scabem_source* src, int nsrc, void* b, int64_t
 // (x, lam: device complex128, N each).  g_out: host, 2 * entries doubles.
 int sigma_gradient_impl(scabem_op* op, const cd* x, const cd* lam, const scabem_source* src, int nsrc,
                         const scabem_sigma* basis, double* g_out, cudaStream_t s) {
-  const int64_t Q = op->Q, N = op->N;
-  cd *hs = nullptr, *yscr = nullptr, *g = nullptr;
+  const int64_t Q = op->Q;
+  cd *hs = nullptr, *g = nullptr;
   double* dseg = nullptr;
   int64_t ng = basis->kind == SCABEM_SIGMA_PER_QPOINT ? Q
                : basis->kind == SCABEM_SIGMA_BSPLINE   ? basis->ncoef
@@ -1498,9 +1498,8 @@ int sigma_gradient_impl(scabem_op* op, const cd* x, const cd* lam, const scabem_
   auto fail = [&](cudaError_t e, const char* what) { rc = cuda_fail(e, what); };
   cudaError_t e;
   if ((e = cudaMalloc(&hs, sizeof(cd) * Q)) != cudaSuccess) fail(e, "cudaMalloc");
-  if (!rc && (e = cudaMalloc(&yscr, sizeof(cd) * N)) != cudaSuccess) fail(e, "cudaMalloc");
   if (!rc && (e = cudaMalloc(&g, sizeof(cd) * (ng > 0 ? ng : 1))) != cudaSuccess) fail(e, "cudaMalloc");
-  if (!rc) rc = sigma_sensitivity_op(op, x, lam, hs, yscr, s);
+  if (!rc) rc = sigma_sensitivity_op(op, x, lam, hs, s);
   for (int i = 0; !rc && i < nsrc; ++i) {
     const double k = src[i].side == 0 ? op->ki : op->ke, z = src[i].side == 0 ? op->zi : op->ze;
     k_rhs_sens<<<(int)cdiv(Q, 256), 256, 0, s>>>(src[i], op->tri, op->cX, op->qp, op->qw, op->valrow, lam, Q,
@@ -1529,7 +1528,6 @@ int sigma_gradient_impl(scabem_op* op, const cd* x, const cd* lam, const scabem_
   }
   if (!rc && (e = cudaStreamSynchronize(s)) != cudaSuccess) fail(e, "cudaStreamSynchronize");
   cudaFree(hs);
-  cudaFree(yscr);
   cudaFree(g);
   cudaFree(dseg);
   return rc;
