@@ -1,20 +1,19 @@
 // The matvec y = A x of the grid-accelerated operator (one right-hand side).
 //
-//  K1 k_sources  RWG coefficients -> per-triangle current summaries
+//  K1 k_summ     RWG coefficients -> per-triangle current summaries
 //                J(r) = a (r - c_t) - beta for the exterior J, interior J and
-//                exterior M sets (current reduction, Eqs. 10-12), and the
-//                weighted point sources at the quadrature points
-//  K2 k_gather   point sources spread onto the grid by the Lagrange stencils
-//                (12 fields), as a gather over the covered grid points
+//                exterior M sets (current reduction, Eqs. 10-12)
+//  K2 k_project  summaries spread onto the grid by the triangles' stencil
+//                moments (moments.cu; 12 fields), as a gather over the covered
+//                grid points
 //  K3-5          fft_conv (fft.cu): 12 -> 16 grid potentials (A, phi, F, psi
 //                of each medium, Eqs. 15-16)
-//  K6-8 k_points per target triangle: potentials, gradients and curls at its
-//                quadrature points (interpolation), plus the near-field
-//                precorrection (exact minus grid panel moments), then the
-//                Galerkin testing of Eqs. 1-3 (weak form), Eq. 13 and Eq. 14
-//                (sigma-weighted, with the side-limit terms)
-//                and the per-edge sums of the two triangles' tested values
-//                into the rows
+//  K6 k_test     the potentials, gradients and curls tested per triangle by the
+//                same moments: Galerkin rows of Eqs. 1-3 (weak form), Eq. 13 and
+//                Eq. 14 (sigma-weighted)
+//  K7 k_near_rows  (near.cu) near-field precorrection (exact minus grid panel
+//                interaction) and side-limit terms as a sparse matrix over
+//                edges, plus the row sums of the tested values
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -28,35 +27,6 @@ __device__ __forceinline__ cx<R> coef_of(const cx<R>* __restrict__ x, int32_t co
   return czero<R>();
 }
 
-// K1: one thread per triangle.  summ[(t*3+set)*4 + {a, bx, by, bz}]
-template <typename R>
-__global__ void k_summ(const cx<R>* __restrict__ x, const int32_t* __restrict__ unk, const double* __restrict__ cX,
-                       const double* __restrict__ tri, int64_t nt, cx<R>* __restrict__ summ) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= nt) return;
-  const double* g = tri + 16 * t;
-  R rel[3][3];
-  for (int k = 0; k < 3; ++k)
-    for (int c = 0; c < 3; ++c) rel[k][c] = (R)(g[3 * k + c] - g[9 + c]);
-  R ck[3];
-  for (int k = 0; k < 3; ++k) ck[k] = (R)cX[3 * t + k];
-  for (int set = 0; set < 3; ++set) {
-    cx<R> a = czero<R>(), b0 = a, b1 = a, b2 = a;
-    for (int k = 0; k < 3; ++k) {
-      const cx<R> j = ck[k] * coef_of(x, unk[(3 * t + k) * 3 + set]);
-      a += j;
-      b0 += rel[k][0] * j;
-      b1 += rel[k][1] * j;
-      b2 += rel[k][2] * j;
-    }
-    cx<R>* o = summ + (3 * t + set) * 4;
-    o[0] = a;
-    o[1] = b0;
-    o[2] = b1;
-    o[3] = b2;
-  }
-}
-
 // a += s * b on (re, im) as one packed FP32x2 FMA in complex64.
 __device__ __forceinline__ void axpy2(cx<float>& a, float s, cx<float> b) {
   const float2 r = __ffma2_rn(make_float2(s, s), make_float2(b.re, b.im), make_float2(a.re, a.im));
@@ -64,130 +34,145 @@ __device__ __forceinline__ void axpy2(cx<float>& a, float s, cx<float> b) {
 }
 __device__ __forceinline__ void axpy2(cx<double>& a, double s, cx<double> b) { axpy(a, s, b); }
 
-// K1+K2a: one thread per quadrature point (point a of triangle t): the
-// current summaries of t (as k_summ; written by the thread of point 0) and
-// the point's weighted sources qsrc[Qi*12 + set*4 + {x, y, z, div}] of the
-// exterior J, interior J and exterior M sets (J(r) = a (r - c) - beta,
-// div J = 2a, times the quadrature weight).
-template <typename R>
-__global__ void k_sources(const cx<R>* __restrict__ x, const int32_t* __restrict__ unk,
-                          const double* __restrict__ cX, const double* __restrict__ tri,
-                          const double* __restrict__ qp, const double* __restrict__ qw, int64_t Q, int q,
-                          cx<R>* __restrict__ summ, cx<R>* __restrict__ qsrc, int64_t ldx) {
-  const int64_t Qi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (Qi >= Q) return;
-  {  // right-hand side blockIdx.y of a batch: its columns and workspaces
-    const int64_t c = blockIdx.y;
-    x += c * ldx;
-    summ += c * (Q / q) * 12;
-    qsrc += c * Q * 12;
-  }
-  const int64_t t = Qi / q;
-  const int a = (int)(Qi - t * q);
-  const double* g = tri + 16 * t;
-  R rel[3][3];
-  for (int k = 0; k < 3; ++k)
-    for (int c = 0; c < 3; ++c) rel[k][c] = (R)(g[3 * k + c] - g[9 + c]);
-  R ck[3];
-  for (int k = 0; k < 3; ++k) ck[k] = (R)cX[3 * t + k];
-  const R w = (R)qw[Qi];
-  const R rq[3] = {(R)(qp[3 * Qi] - g[9]), (R)(qp[3 * Qi + 1] - g[10]), (R)(qp[3 * Qi + 2] - g[11])};
-  cx<R>* o = qsrc + Qi * NFIELD_IN;
+// The four potentials of one (grid point, medium, group), or the summary (a,
+// beta) of one (triangle, set): 32 contiguous bytes in complex64.
+__device__ __forceinline__ void load_group(const cx<float>* p, cx<float>* v) {
+  const float4 u0 = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 u1 = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  v[0] = mk(u0.x, u0.y);
+  v[1] = mk(u0.z, u0.w);
+  v[2] = mk(u1.x, u1.y);
+  v[3] = mk(u1.z, u1.w);
+}
+__device__ __forceinline__ void load_group(const cx<double>* p, cx<double>* v) {
 #pragma unroll
-  for (int set = 0; set < 3; ++set) {
-    cx<R> al = czero<R>(), b0 = al, b1 = al, b2 = al;
-    for (int k = 0; k < 3; ++k) {
-      const cx<R> j = ck[k] * coef_of(x, unk[(3 * t + k) * 3 + set]);
-      al += j;
-      b0 += rel[k][0] * j;
-      b1 += rel[k][1] * j;
-      b2 += rel[k][2] * j;
-    }
-    if (a == 0) {
-      cx<R>* so = summ + (3 * t + set) * 4;
-      so[0] = al;
-      so[1] = b0;
-      so[2] = b1;
-      so[3] = b2;
-    }
-    o[set * 4 + 0] = w * (rq[0] * al - b0);
-    o[set * 4 + 1] = w * (rq[1] * al - b1);
-    o[set * 4 + 2] = w * (rq[2] * al - b2);
-    o[set * 4 + 3] = (R(2) * w) * al;
+  for (int f = 0; f < 4; ++f) {
+    const double2 u = __ldg(reinterpret_cast<const double2*>(p) + f);
+    v[f] = mk(u.x, u.y);
   }
 }
-
-// K2b: projection as a gather.  One warp per grid point that some stencil
-// covers: lane = portion * SL + slot reads 16-byte portion `portion` of the
-// rows qsrc[point] of entries slot, slot + SL, ... (SL rows per load
-// instruction, GATHER_INFLIGHT in flight), weighted by W_slot(point); the SL slot sums
-// of a portion are then added by shuffles and the slot-0 lanes write their
-// portion.  Points no stencil covers stay zero from set-up.  The sum order
-// is fixed, so the result does not depend on thread timing.
-constexpr int GATHER_INFLIGHT = 4;
-
-template <typename R>
-__device__ __forceinline__ void load_portion(const cx<R>* p, cx<R>* v);
-template <>
-__device__ __forceinline__ void load_portion<float>(const cx<float>* p, cx<float>* v) {
+// Four reals starting on a 16-byte boundary
+__device__ __forceinline__ void load4(const float* p, float* v) {
   const float4 u = __ldg(reinterpret_cast<const float4*>(p));
-  v[0] = mk(u.x, u.y);
-  v[1] = mk(u.z, u.w);
+  v[0] = u.x;
+  v[1] = u.y;
+  v[2] = u.z;
+  v[3] = u.w;
 }
-template <>
-__device__ __forceinline__ void load_portion<double>(const cx<double>* p, cx<double>* v) {
-  v[0] = p[0];
+__device__ __forceinline__ void load4(const double* p, double* v) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  v[3] = b.y;
+}
+__device__ __forceinline__ void load2(const float* p, float* v) {
+  const float2 u = __ldg(reinterpret_cast<const float2*>(p));
+  v[0] = u.x;
+  v[1] = u.y;
+}
+__device__ __forceinline__ void load2(const double* p, double* v) {
+  const double2 u = __ldg(reinterpret_cast<const double2*>(p));
+  v[0] = u.x;
+  v[1] = u.y;
 }
 
+// v[t] of a pair of lanes that differ in lane bit `o`: the lower one keeps
+// v[0 .. half), the upper one v[half .. 2 half), each adding the other's part
+// (the halving step of a reduction over several values).
 template <typename R>
-__global__ void k_gather(const cx<R>* __restrict__ qsrc, const int32_t* __restrict__ gpt,
-                         const int32_t* __restrict__ goff, const int32_t* __restrict__ gq, const R* __restrict__ gw,
-                         int64_t ngnz, int64_t ng, cx<R>* __restrict__ grids, int64_t cs_q, int64_t cs_g) {
-  constexpr int CPP = 16 / (int)sizeof(cx<R>);  // complex per 16-byte portion
-  qsrc += blockIdx.y * cs_q;  // right-hand side blockIdx.y of a batch
+__device__ __forceinline__ void halve(cx<R>* v, int half, int lane, int o) {
+  const bool up = (lane & o) != 0;
+#pragma unroll
+  for (int t = 0; t < half; ++t) {
+    const cx<R> send = up ? v[t] : v[t + half], keep = up ? v[t + half] : v[t];
+    v[t] = keep + mk(__shfl_xor_sync(0xffffffffu, send.re, o), __shfl_xor_sync(0xffffffffu, send.im, o));
+  }
+}
+template <typename R>
+__device__ __forceinline__ cx<R> xadd(cx<R> v, int o) {
+  return v + mk(__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o));
+}
+
+// K1: one thread per (triangle, set): the current summary
+// summ[(t*3+set)*4 + {a, bx, by, bz}], J(r) = a (r - c_t) - beta, of the
+// exterior J, interior J and exterior M sets.
+template <typename R>
+__global__ void k_summ(const cx<R>* __restrict__ x, const int32_t* __restrict__ unk, const R* __restrict__ geo,
+                       int64_t nt, cx<R>* __restrict__ summ, int64_t ldx) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= 3 * nt) return;
+  x += blockIdx.y * ldx;  // right-hand side blockIdx.y of a batch
+  summ += blockIdx.y * 12 * nt;
+  const int64_t t = i / 3;
+  const int set = (int)(i - 3 * t);
+  cx<R> a = czero<R>(), b0 = a, b1 = a, b2 = a;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    R g[4];
+    load4(geo + 16 * t + 4 * k, g);
+    const cx<R> j = g[0] * coef_of(x, unk[(3 * t + k) * 3 + set]);
+    a += j;
+    axpy2(b0, g[1], j);
+    axpy2(b1, g[2], j);
+    axpy2(b2, g[3], j);
+  }
+  cx<R>* o = summ + 4 * i;
+  o[0] = a;
+  o[1] = b0;
+  o[2] = b1;
+  o[3] = b2;
+}
+
+// K2: projection as a gather over the triangles.  One warp per grid point
+// that some stencil covers: lane = set * 8 + slot takes entries slot, slot + 8,
+// ... of the point, each one triangle's summary of that set (32 bytes in
+// complex64) against its moments m0, m1: a m1 - beta m0 and 2 a m0.  The slot
+// sums meet by halving exchanges.  Points no stencil covers stay zero from
+// set-up.  The sum order is fixed, so the result does not depend on thread
+// timing.  Bound by the latency of the (triangle -> summary) loads out of L2:
+// two entries per lane are in flight.
+constexpr int PJ_INFLIGHT = 2;
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_project(const cx<R>* __restrict__ summ, const int32_t* __restrict__ gpt,
+                                                 const int32_t* __restrict__ eoff, const int32_t* __restrict__ gtri,
+                                                 const R* __restrict__ gA, int64_t ngnz, int64_t ng,
+                                                 cx<R>* __restrict__ grids, int64_t cs_s, int64_t cs_g) {
+  summ += blockIdx.y * cs_s;  // right-hand side blockIdx.y of a batch
   grids += blockIdx.y * cs_g;
-  constexpr int NPOR = NFIELD_IN / CPP;          // portions per row: 6 or 12
-  constexpr int SL = 24 / NPOR;                  // rows per load instruction: 4 or 2
   const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int por = lane / SL, slot = lane - por * SL;
-  const bool act = lane < NPOR * SL && i < ngnz;
-  cx<R> acc[CPP];
+  if (i >= ngnz) return;  // whole warp
+  const int lane = threadIdx.x & 31, set = min(lane >> 3, 2), slot = lane & 7;
+  cx<R> acc[4];
 #pragma unroll
-  for (int c = 0; c < CPP; ++c) acc[c] = czero<R>();
-  if (act) {
-    const int e1 = goff[i + 1];
-    for (int e = goff[i] + slot; e < e1; e += GATHER_INFLIGHT * SL) {
-      int qe[GATHER_INFLIGHT];
-      R we[GATHER_INFLIGHT];
+  for (int c = 0; c < 4; ++c) acc[c] = czero<R>();
+  const int e1 = lane < 24 ? eoff[i + 1] : 0;
+  for (int e = eoff[i] + slot; e < e1; e += 8 * PJ_INFLIGHT) {
+    R w[PJ_INFLIGHT][4];
+    cx<R> v[PJ_INFLIGHT][4];
 #pragma unroll
-      for (int u = 0; u < GATHER_INFLIGHT; ++u) {
-        const int eu = e + u * SL;
-        qe[u] = eu < e1 ? gq[eu] : gq[e];
-        we[u] = eu < e1 ? gw[eu] : R(0);
+    for (int u = 0; u < PJ_INFLIGHT; ++u) {
+      const int eu = e + 8 * u < e1 ? e + 8 * u : e;
+      load4(gA + 4 * (int64_t)eu, w[u]);
+      load_group(summ + (3 * (int64_t)gtri[eu] + set) * 4, v[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < PJ_INFLIGHT; ++u) {
+      const R on = e + 8 * u < e1 ? R(1) : R(0);
+      const R m0 = on * w[u][0];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        axpy2(acc[c], on * w[u][1 + c], v[u][0]);
+        axpy2(acc[c], -m0, v[u][1 + c]);
       }
-      cx<R> v[GATHER_INFLIGHT][CPP];
-#pragma unroll
-      for (int u = 0; u < GATHER_INFLIGHT; ++u) load_portion<R>(qsrc + (int64_t)qe[u] * NFIELD_IN + por * CPP, v[u]);
-#pragma unroll
-      for (int u = 0; u < GATHER_INFLIGHT; ++u)
-#pragma unroll
-        for (int c = 0; c < CPP; ++c) axpy2(acc[c], we[u], v[u][c]);
+      axpy2(acc[3], m0 + m0, v[u][0]);
     }
   }
-  // every lane reaches the shuffles (no early exit above)
-#pragma unroll
-  for (int o = 1; o < SL; o <<= 1)
-#pragma unroll
-    for (int c = 0; c < CPP; ++c) {
-      acc[c].re += __shfl_xor_sync(0xffffffffu, acc[c].re, o);
-      acc[c].im += __shfl_xor_sync(0xffffffffu, acc[c].im, o);
-    }
-  if (act && slot == 0) {
-    const int64_t g = gpt[i];
-#pragma unroll
-    for (int c = 0; c < CPP; ++c) grids[(int64_t)(por * CPP + c) * ng + g] = acc[c];
-  }
+  halve(acc, 2, lane, 4);
+  halve(acc, 1, lane, 2);
+  acc[0] = xadd(acc[0], 1);
+  if (lane < 24 && !(lane & 1)) grids[(int64_t)(set * 4 + ((lane >> 1) & 1) + ((lane >> 1) & 2)) * ng + gpt[i]] = acc[0];
 }
 
 template <typename R>
@@ -210,21 +195,6 @@ const float* gather_weights<float>(scabem_op* op) {
 template <>
 const double* gather_weights<double>(scabem_op* op) {
   return op->gwd;
-}
-
-// The four potentials of one (grid point, medium, group) (32 contiguous bytes
-// in complex64).
-__device__ __forceinline__ void load_group(const cx<float>* p, cx<float>* v) {
-  const float4 u0 = __ldg(reinterpret_cast<const float4*>(p));
-  const float4 u1 = __ldg(reinterpret_cast<const float4*>(p) + 1);
-  v[0] = mk(u0.x, u0.y);
-  v[1] = mk(u0.z, u0.w);
-  v[2] = mk(u1.x, u1.y);
-  v[3] = mk(u1.z, u1.w);
-}
-__device__ __forceinline__ void load_group(const cx<double>* p, cx<double>* v) {
-#pragma unroll
-  for (int f = 0; f < 4; ++f) v[f] = p[f];
 }
 
 // Two consecutive complex values of shared memory on a 16-byte boundary.
@@ -303,73 +273,6 @@ __device__ __forceinline__ void interp_group(const cx<R>* __restrict__ grids, co
   r[9] = gx[1] - gy[0];
 }
 
-// The same sums in complex64 with the accumulator split as acc = P + j Q:
-// x s adds (s.re, s.re) * (x.re, x.im) to P and (s.im, s.im) * (x.re, x.im)
-// to Q, so that every record value enters the packed FMAs as the (re, im)
-// pair it is loaded as, and only the few source factors are duplicated.
-__device__ __forceinline__ void near_pq(const cx<float>* d, const cx<float>* sv, float2* P, float2* Q) {
-  float2 x[NCORR];
-#pragma unroll
-  for (int c = 0; c < NCORR; ++c) x[c] = make_float2(d[c].re, d[c].im);
-  const float2 ar = make_float2(sv[0].re, sv[0].re), ai = make_float2(sv[0].im, sv[0].im);
-  const float2 a2r = make_float2(2.f * sv[0].re, 2.f * sv[0].re), a2i = make_float2(2.f * sv[0].im, 2.f * sv[0].im);
-  float2 br[3], bi[3], nbr[3], nbi[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    br[c] = make_float2(sv[1 + c].re, sv[1 + c].re);
-    bi[c] = make_float2(sv[1 + c].im, sv[1 + c].im);
-    nbr[c] = make_float2(-sv[1 + c].re, -sv[1 + c].re);
-    nbi[c] = make_float2(-sv[1 + c].im, -sv[1 + c].im);
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    P[c] = __ffma2_rn(x[1 + c], ar, P[c]);  // A += a dP1 - beta dP0
-    Q[c] = __ffma2_rn(x[1 + c], ai, Q[c]);
-    P[c] = __ffma2_rn(x[0], nbr[c], P[c]);
-    Q[c] = __ffma2_rn(x[0], nbi[c], Q[c]);
-    P[4 + c] = __ffma2_rn(x[4 + c], a2r, P[4 + c]);  // grad phi += 2a dQ
-    Q[4 + c] = __ffma2_rn(x[4 + c], a2i, Q[4 + c]);
-    P[7 + c] = __ffma2_rn(x[7 + c], ar, P[7 + c]);  // curl A += a dC
-    Q[7 + c] = __ffma2_rn(x[7 + c], ai, Q[7 + c]);
-  }
-  P[3] = __ffma2_rn(x[0], a2r, P[3]);  // phi += 2a dP0
-  Q[3] = __ffma2_rn(x[0], a2i, Q[3]);
-  // curl A -= dQ x beta
-  P[7] = __ffma2_rn(x[5], nbr[2], P[7]);
-  Q[7] = __ffma2_rn(x[5], nbi[2], Q[7]);
-  P[7] = __ffma2_rn(x[6], br[1], P[7]);
-  Q[7] = __ffma2_rn(x[6], bi[1], Q[7]);
-  P[8] = __ffma2_rn(x[6], nbr[0], P[8]);
-  Q[8] = __ffma2_rn(x[6], nbi[0], Q[8]);
-  P[8] = __ffma2_rn(x[4], br[2], P[8]);
-  Q[8] = __ffma2_rn(x[4], bi[2], Q[8]);
-  P[9] = __ffma2_rn(x[4], nbr[1], P[9]);
-  Q[9] = __ffma2_rn(x[4], nbi[1], Q[9]);
-  P[9] = __ffma2_rn(x[5], br[0], P[9]);
-  Q[9] = __ffma2_rn(x[5], bi[0], Q[9]);
-}
-
-// Near-field accumulation state of one lane: complex64 keeps acc = P + j Q
-// through the near loop (near_pq); complex128 keeps acc itself (near_part).
-template <typename R>
-struct NearAcc;
-template <>
-struct NearAcc<float> {
-  float2 P[NREC / 2], Q[NREC / 2];
-  __device__ __forceinline__ void begin(const cx<float>* acc) {
-#pragma unroll
-    for (int c = 0; c < NREC / 2; ++c) {
-      P[c] = make_float2(acc[c].re, acc[c].im);
-      Q[c] = make_float2(0.f, 0.f);
-    }
-  }
-  __device__ __forceinline__ void add(const cx<float>* d, const cx<float>* sv) { near_pq(d, sv, P, Q); }
-  __device__ __forceinline__ void end(cx<float>* acc) const {
-#pragma unroll
-    for (int c = 0; c < NREC / 2; ++c) acc[c] = mk(P[c].x - Q[c].y, P[c].y + Q[c].x);
-  }
-};
-
 // One near record (dP0, dP1, dQ, dC) applied to source summary sv (a, beta):
 // A += a dP1 - beta dP0, phi += 2a dP0, grad phi += 2a dQ,
 // curl A += a dC - dQ x beta (the same for F, psi of an M source).
@@ -391,66 +294,9 @@ __device__ __forceinline__ void near_part(const cx<R>* d, const cx<R>* sv, cx<R>
   acc[9] -= d[4] * be[1] - d[5] * be[0];
 }
 
-template <>
-struct NearAcc<double> {
-  cx<double> a[NREC / 2];
-  __device__ __forceinline__ void begin(const cx<double>* acc) {
-#pragma unroll
-    for (int c = 0; c < NREC / 2; ++c) a[c] = acc[c];
-  }
-  __device__ __forceinline__ void add(const cx<double>* d, const cx<double>* sv) { near_part(d, sv, a); }
-  __device__ __forceinline__ void end(cx<double>* acc) const {
-#pragma unroll
-    for (int c = 0; c < NREC / 2; ++c) acc[c] = a[c];
-  }
-};
-
 template <typename R>
 __device__ __forceinline__ cx<R> dot3(const R* X, const cx<R>* V) {
   return X[0] * V[0] + X[1] * V[1] + X[2] * V[2];
-}
-
-// Weighted contributions of quadrature point a to the tested values of local
-// edge kk of triangle t, from the point's records (recs[medium*NREC]):
-// type 0 <X, E_e - E_i>, 1 <X, H_e - H_i> (weak forms), 2 Eq. 13, 3 Eq. 14.
-template <typename R>
-__device__ __forceinline__ void test_point(const cx<R>* recs, const double* __restrict__ tri,
-                                           const R* __restrict__ tp, const R* __restrict__ sig, int64_t t, int kk,
-                                           int a, int q, R ke, R ki, R ze, R zi, cx<R>* out) {
-  const double* g = tri + 16 * t;
-  const R nrm[3] = {(R)g[12], (R)g[13], (R)g[14]};
-  const R kl[2] = {ke, ki}, zl[2] = {ze, zi};
-  const int64_t Qa = t * q + a;
-  const R* tq = tp + 16 * Qa;
-  const R w = tq[3];
-  const R sg = sig[Qa];
-  const R divX = tq[13 + kk];
-  R X[3];
-  for (int c = 0; c < 3; ++c) X[c] = tq[4 + 3 * kk + c];
-  cx<R> WE[3], WH[3], E[2][3];
-  cx<R> wE = czero<R>(), wH = czero<R>();
-  for (int c = 0; c < 3; ++c) WE[c] = WH[c] = czero<R>();
-  for (int m = 0; m < 2; ++m) {
-    const cx<R>* r = recs + m * NREC;
-    const R k = kl[m], z = zl[m];
-    const R sgm = m == 0 ? R(1) : R(-1);
-    const cx<R> phi = r[3], psi = r[13];
-    wE += (sgm * z / k) * mulj(phi);
-    wH += (sgm / (k * z)) * mulj(psi);
-    for (int c = 0; c < 3; ++c) {
-      const cx<R> A = r[c], gphi = r[4 + c], cA = r[7 + c], F = r[10 + c], cF = r[17 + c];
-      const cx<R> jA = mulj(A), jF = mulj(F);
-      WE[c] += sgm * ((-z * k) * jA - cF);
-      WH[c] += sgm * (cA - (k / z) * jF);
-      E[m][c] = -z * (k * jA + (R(1) / k) * mulj(gphi)) - cF;
-    }
-  }
-  const R nX[3] = {nrm[1] * X[2] - nrm[2] * X[1], nrm[2] * X[0] - nrm[0] * X[2], nrm[0] * X[1] - nrm[1] * X[0]};
-  const cx<R> hterm = dot3(X, WH) + divX * wH;
-  out[0] = w * (dot3(X, WE) + divX * wE);
-  out[1] = w * hterm;
-  out[2] = w * (hterm - sg * dot3(nX, E[0]));  // Eq. 13: <X, dH> - <sigma n x X, E_e>
-  out[3] = (-w * sg) * dot3(X, E[1]);          // Eq. 14: -<sigma X, E_i>
 }
 
 // d out / d sg of the Eq. 13 and Eq. 14 tested values of local edge kk at
@@ -563,8 +409,8 @@ __global__ void k_wait_selftest(int* __restrict__ tmo) {
   if (!ok && threadIdx.x == 0) atomicOr(tmo, 1);
 }
 
-// K6-8: one warp per target triangle t, PT_WARPS triangles per CTA; warps
-// never wait on one another.
+// Conductivity sensitivity, one warp per target triangle t, PT_WARPS triangles
+// per CTA; warps never wait on one another.
 //  Phase 1: lane (point a, medium, record group h), 4q lanes, interpolates
 //    its 10 record values, then adds the near corrections.  The triangle's
 //    near records are one contiguous run (pairs noff[t] .. noff[t+1]); they
@@ -573,9 +419,10 @@ __global__ void k_wait_selftest(int* __restrict__ tmo) {
 //    one is consumed (the first ones during the interpolation).  A stage
 //    that does not arrive within the wait limit sets *tmo and ends the
 //    triangle's near loop after its copies in flight have landed.
-//  Phase 2: lane (local edge kk, point a), 3q lanes, forms the point's
-//    weighted tested values; phase 3: lane (kk, value type) sums them over the
-//    points in point order.
+//  Phase 2: lane (local edge kk, point a), 3q lanes, differentiates the point's
+//    sigma-weighted tested values; they are summed over kk into
+//    hs[t q + a] = eta0 sum_kk (lam_row2 d2 + lam_row3 d3), the derivative of
+//    lam^T A x with respect to the conductivity [S] at the point.
 constexpr int PT_WARPS = 4;
 constexpr int PT_NSTG = 2;  // 2 stages of 4 pairs: the bytes in flight of 4 stages of 2, with half the
 constexpr int PT_KP = 4;    // stages' waits, fences and copy issues per pair
@@ -591,29 +438,19 @@ __host__ __device__ constexpr size_t pt_smem_bytes(int q, size_t csize) {
   return (size_t)PT_WARPS * pt_warp_complex(q) * csize + (size_t)PT_WARPS * PT_NSTG * sizeof(uint64_t);
 }
 
-// SENS = true (conductivity sensitivity): the near corrections are added at
-// the points, and instead of the tested values val[t][kk][type] the kernel
-// writes hs[t q + a] = eta0 sum_kk (lam_row2 d2 + lam_row3 d3), the
-// derivative of lam^T A x with respect to the conductivity [S] at the point.
-//
-// QT > 0 fixes q at compile time (then every shared-memory offset of a record
-// is an immediate); QT = 0 takes the argument.  Lanes past the 4q of phase 1
-// repeat lane 4q - 4 .. 4q - 1's work without storing it, so that the near
-// loop runs without divergence.
-template <typename R, int P, bool SENS = false, int QT = 0>
-__global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 6) : 3) k_points(
+// Lanes past the 4q of phase 1 repeat lane 4q - 4 .. 4q - 1's work without
+// storing it, so that the near loop runs without divergence.
+template <typename R, int P>
+__global__ void __launch_bounds__(PT_WARPS * 32, 3) k_points_sens(
     const cx<R>* __restrict__ grids, const int32_t* __restrict__ base, const R* __restrict__ L,
     const R* __restrict__ dL, const cx<R>* __restrict__ corr, const int32_t* __restrict__ noff,
     const int32_t* __restrict__ nsrc, const cx<R>* __restrict__ summ, const double* __restrict__ tri,
-    const R* __restrict__ tp, const R* __restrict__ sig, int64_t nt, int q_arg, int n0, int n1, int n2, R ke, R ki,
-    R ze, R zi, int has_near, const int32_t* __restrict__ valrow, cx<R>* __restrict__ val, int* __restrict__ tmo,
-    const cx<R>* __restrict__ lam, cx<R>* __restrict__ hs, int64_t cs_grid, int64_t cs_val) {
-  const int q = QT > 0 ? QT : q_arg;
+    const R* __restrict__ tp, int64_t nt, int q, int n1, int n2, R ke, R ki, R ze, R zi, int has_near,
+    const int32_t* __restrict__ valrow, int* __restrict__ tmo, const cx<R>* __restrict__ lam, cx<R>* __restrict__ hs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = (int64_t)blockIdx.x * PT_WARPS + warp;
   if (t >= nt) return;  // whole warp; no CTA-wide barrier below
-  grids += blockIdx.y * cs_grid;  // right-hand side blockIdx.y of a batch
   const int pairc = NCORR * 2 * q;  // complex per pair: [point][medium][component]
   cx<R>* ring = reinterpret_cast<cx<R>*>(smem_raw) + (int64_t)warp * pt_warp_complex(q);
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<cx<R>*>(smem_raw) + PT_WARPS * pt_warp_complex(q)) +
@@ -623,7 +460,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
 
   const bool act = lane < 4 * q;
   const int a = min(lane >> 2, q - 1), med = (lane >> 1) & 1, h = lane & 1;
-  const int j0 = SENS && has_near ? noff[t] : 0, j1 = SENS && has_near ? noff[t + 1] : 0;
+  const int j0 = has_near ? noff[t] : 0, j1 = has_near ? noff[t + 1] : 0;
   const int nst = (j1 - j0 + PT_KP - 1) / PT_KP;
   const unsigned pair_bytes = (unsigned)(pairc * sizeof(cx<R>));
   // stage st -> slot st % PT_NSTG, issued by lane 0
@@ -634,7 +471,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
     bulk_load(ring + (st % PT_NSTG) * PT_KP * pairc, corr + (int64_t)pj * pairc, np * pair_bytes,
               bars + st % PT_NSTG);
   };
-  if (SENS && nst > 0) {
+  if (nst > 0) {
     if (lane == 0) {
 #pragma unroll
       for (int i = 0; i < PT_NSTG; ++i) mbar_init(bars + i, 1);
@@ -648,15 +485,13 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
   int src_nxt = lane < npair ? nsrc[j0 + lane] : 0, src_cur = 0;
   cx<R> acc[NREC / 2];
   interp_group<R, P>(grids, base, L, dL, t * q + a, med, h, n1, n2, acc);
-  if (SENS && nst > 0) {
+  if (nst > 0) {
     const int set = h ? 2 : med;  // source J of this medium, or M
     // the interior medium sees -M: accumulate -acc + sum, then negate back
     const bool neg = h && med;
     if (neg)
 #pragma unroll
       for (int c = 0; c < NREC / 2; ++c) acc[c] = -acc[c];
-    NearAcc<R> na;
-    na.begin(acc);
     int st = 0;
     bool ok = true;
     for (; st < nst; ++st) {
@@ -677,7 +512,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
           load_group(summ + (3 * sj + set) * 4, sv);
 #pragma unroll
           for (int c = 0; c < NCORR; c += 2) load_pair_smem(rs + k * pairc + c, d + c);
-          na.add(d, sv);
+          near_part(d, sv, acc);
         }
       }
       __syncwarp();
@@ -688,7 +523,6 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
       if (lane == 0) atomicOr(tmo, 1);
     }
     __syncwarp();  // every lane is done with the ring before it holds records
-    na.end(acc);
     if (neg)
 #pragma unroll
       for (int c = 0; c < NREC / 2; ++c) acc[c] = -acc[c];
@@ -699,39 +533,150 @@ __global__ void __launch_bounds__(PT_WARPS * 32, sizeof(R) == 4 ? (P == 4 ? 4 : 
     for (int c = 0; c < NREC / 2; ++c) o[c] = acc[c];
   }
   __syncwarp();
-  if constexpr (SENS) {
-    if (lane < 3 * q) {
-      const int kk = lane / q, pa = lane - kk * q;
-      cx<R> d2, d3;
-      test_point_sigma(recs + pa * 2 * NREC, summ, tri, tp, t, kk, pa, q, ke, ki, ze, zi, d2, d3);
-      const int r2 = valrow[(t * 3 + kk) * 4 + 2], r3 = valrow[(t * 3 + kk) * 4 + 3];
-      cx<R> c = czero<R>();
-      if (r2 >= 0) c += lam[r2] * d2;
-      if (r3 >= 0) c += lam[r3] * d3;
-      part[kk * q + pa] = c;
-    }
-    __syncwarp();
-    if (lane < q) hs[t * q + lane] = R(ETA0) * (part[lane] + part[q + lane] + part[2 * q + lane]);
-    return;
-  }
   if (lane < 3 * q) {
     const int kk = lane / q, pa = lane - kk * q;
-    cx<R> o[4];
-    test_point(recs + pa * 2 * NREC, tri, tp, sig, t, kk, pa, q, ke, ki, ze, zi, o);
-    cx<R>* d = part + (kk * q + pa) * 4;
+    cx<R> d2, d3;
+    test_point_sigma(recs + pa * 2 * NREC, summ, tri, tp, t, kk, pa, q, ke, ki, ze, zi, d2, d3);
+    const int r2 = valrow[(t * 3 + kk) * 4 + 2], r3 = valrow[(t * 3 + kk) * 4 + 3];
+    cx<R> c = czero<R>();
+    if (r2 >= 0) c += lam[r2] * d2;
+    if (r3 >= 0) c += lam[r3] * d3;
+    part[kk * q + pa] = c;
+  }
+  __syncwarp();
+  if (lane < q) hs[t * q + lane] = R(ETA0) * (part[lane] + part[q + lane] + part[2 * q + lane]);
+}
+
+// K6-7: interpolation and testing by the triangle moments (moments.cu), one
+// warp per triangle.  Lane = slot * 4 + group takes entries slot, slot + 8, ...
+// of the triangle's grid points and the four potentials of its (medium, J or
+// M set) group there (32 bytes in complex64): the value sums V = <pot>, S =
+// <rel . pot> - 2/k^2 <charge potential> and the curl sums C = <curl pot>,
+// D = <rel . curl pot>; on triangles with an absorber edge also Z, Y, the
+// sigma-weighted strong-form E sums of its medium (rel -> n x rel in the
+// exterior one, for Eq. 13).  The slots meet by halving exchanges, and lane (kk,
+// type) forms the tested value of local edge kk:
+//   type 0 <X, E_e - E_i>, 1 <X, H_e - H_i> (weak forms), 2 Eq. 13, 3 Eq. 14,
+// with X_kk = cX_kk (rel - rel_kk).
+constexpr int TS_WARPS = 4;
+
+template <typename R>
+__global__ void __launch_bounds__(TS_WARPS * 32)
+    k_test(const cx<R>* __restrict__ grids, const int32_t* __restrict__ toff, const int32_t* __restrict__ tgi,
+           const int32_t* __restrict__ soff, const R* __restrict__ wA, const R* __restrict__ wB,
+           const R* __restrict__ wC, const R* __restrict__ sW, int64_t ns, const R* __restrict__ geo, int64_t nt, R ke,
+           R ki, R ze, R zi, cx<R>* __restrict__ val, int64_t cs_g, int64_t cs_v) {
+  __shared__ cx<R> red[TS_WARPS][48];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * TS_WARPS + warp;
+  if (t >= nt) return;  // whole warp; no CTA-wide barrier below
+  grids += blockIdx.y * cs_g;  // right-hand side blockIdx.y of a batch
+  const int grp = lane & 3, slot = lane >> 2;
+  const bool isM = grp & 1, inner = grp & 2;
+  const int e0 = toff[t], e1 = toff[t + 1], s0 = soff[t];
+  const R k = inner ? ki : ke, ik2 = R(1) / (k * k), kap = R(-2) * ik2;
+  cx<R> v[8], z[4];  // V, S, C, D; Z, Y
 #pragma unroll
-    for (int c = 0; c < 4; ++c) d[c] = o[c];
+  for (int i = 0; i < 8; ++i) v[i] = czero<R>();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) z[i] = czero<R>();
+  const R* sA = sW + 4 * (int64_t)(s0 - e0);
+  // sigma block of this lane: J exterior D, interior B; M exterior E, interior C
+  const R* sB = sA + 4 * ns * (isM ? (inner ? 2 : 4) : (inner ? 1 : 3));
+  const cx<R>* gb = grids + 4 * grp;
+#pragma unroll 2
+  for (int e = e0 + slot; e < e1; e += 8) {
+    cx<R> g[4];
+    R a[4], b[4], c[2];
+    load_group(gb + (int64_t)tgi[e] * NFIELD_OUT, g);
+    load4(wA + 4 * (int64_t)e, a);
+    load4(wB + 4 * (int64_t)e, b);
+    load2(wC + 2 * (int64_t)e, c);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      axpy2(v[i], a[0], g[i]);
+      axpy2(v[3], a[1 + i], g[i]);
+    }
+    axpy2(v[3], kap * a[0], g[3]);
+    axpy2(v[4], b[1], g[2]);
+    axpy2(v[4], -b[2], g[1]);
+    axpy2(v[5], b[2], g[0]);
+    axpy2(v[5], -b[0], g[2]);
+    axpy2(v[6], b[0], g[1]);
+    axpy2(v[6], -b[1], g[0]);
+    axpy2(v[7], b[3], g[0]);
+    axpy2(v[7], c[0], g[1]);
+    axpy2(v[7], c[1], g[2]);
+    if (s0 >= 0) {
+      R p[4], r[4];
+      load4(sA + 4 * (int64_t)e, p);
+      load4(sB + 4 * (int64_t)e, r);
+      if (!isM) {  // A + grad phi / k^2
+        const R f = ik2;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          axpy2(z[i], p[0], g[i]);
+          axpy2(z[i], f * p[1 + i], g[3]);
+          axpy2(z[3], r[i], g[i]);
+        }
+        axpy2(z[3], f * r[3], g[3]);
+      } else {  // curl F
+        axpy2(z[0], p[2], g[2]);
+        axpy2(z[0], -p[3], g[1]);
+        axpy2(z[1], p[3], g[0]);
+        axpy2(z[1], -p[1], g[2]);
+        axpy2(z[2], p[1], g[1]);
+        axpy2(z[2], -p[2], g[0]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) axpy2(z[3], r[i], g[i]);
+      }
+    }
+  }
+  halve(v, 4, lane, 16);
+  halve(v, 2, lane, 8);
+  halve(v, 1, lane, 4);
+  cx<R>* rw = red[warp];
+  rw[grp * 12 + ((lane >> 2) & 4) + ((lane >> 2) & 2) + ((lane >> 2) & 1)] = v[0];
+  if (s0 >= 0) {
+    halve(z, 2, lane, 16);
+    halve(z, 1, lane, 8);
+    z[0] = xadd(z[0], 4);
+    if (!(lane & 4)) rw[grp * 12 + 8 + ((lane >> 3) & 2) + ((lane >> 3) & 1)] = z[0];
   }
   __syncwarp();
   if (lane < 12) {
-    const int kk = lane >> 2, c = lane & 3;
-    const cx<R>* sp = part + kk * q * 4 + c;
-    cx<R> v = czero<R>();
-    for (int pa = 0; pa < q; ++pa) v += sp[pa * 4];
-    val[blockIdx.y * cs_val + t * 12 + lane] = v;
+    const int kk = lane >> 2, ty = lane & 3;
+    R gk[4], nr[4];
+    load4(geo + 16 * t + 4 * kk, gk);
+    load4(geo + 16 * t + 12, nr);
+    const cx<R>*eJ = rw, *eM = rw + 12, *iJ = rw + 24, *iM = rw + 36;
+    cx<R> o = czero<R>();
+    if (ty < 3) {
+      cx<R> f[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        f[c] = ty == 0 ? mulj((zi * ki) * iJ[c] - (ze * ke) * eJ[c]) - eM[4 + c] + iM[4 + c]
+                       : eJ[4 + c] - iJ[4 + c] + mulj((ki / zi) * iM[c] - (ke / ze) * eM[c]);
+      o = gk[0] * (f[3] - (gk[1] * f[0] + gk[2] * f[1] + gk[3] * f[2]));
+    }
+    if (ty >= 2 && s0 >= 0) {
+      const bool in = ty == 3;
+      const R zk = in ? zi * ki : ze * ke;
+      const cx<R>*J = (in ? iJ : eJ) + 8, *M = (in ? iM : eM) + 8;
+      cx<R> f[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) f[c] = -(zk * mulj(J[c])) - M[c];
+      R x[3] = {gk[1], gk[2], gk[3]};
+      if (!in) {  // n x rel_kk
+        x[0] = nr[1] * gk[3] - nr[2] * gk[2];
+        x[1] = nr[2] * gk[1] - nr[0] * gk[3];
+        x[2] = nr[0] * gk[2] - nr[1] * gk[1];
+      }
+      o -= gk[0] * (f[3] - (x[0] * f[0] + x[1] * f[1] + x[2] * f[2]));
+    }
+    val[blockIdx.y * cs_v + t * 12 + lane] = o;
   }
 }
-
 
 // ================================================================ transposed apply
 // x_bar = A^T y_bar: the stages of the apply in reverse order, each the
@@ -1146,11 +1091,6 @@ __global__ void k_x_adj(const cx<R>* __restrict__ stot, const int32_t* __restric
 }
 
 template <typename R>
-using PointsFn = void (*)(const cx<R>*, const int32_t*, const R*, const R*, const cx<R>*, const int32_t*,
-                          const int32_t*, const cx<R>*, const double*, const R*, const R*, int64_t, int, int, int,
-                          int, R, R, R, R, int, const int32_t*, cx<R>*, int*, const cx<R>*, cx<R>*, int64_t, int64_t);
-
-template <typename R>
 PrecData<R>& pdata(scabem_op* op);
 template <>
 PrecData<float>& pdata<float>(scabem_op* op) {
@@ -1163,6 +1103,23 @@ PrecData<double>& pdata<double>(scabem_op* op) {
 
 }  // namespace
 
+// The grid part up to the potentials, for k right-hand sides: summaries,
+// projection, convolution.
+template <typename R>
+int grid_potentials(scabem_op* op, const cx<R>* x, int64_t ldx, int k, cudaStream_t s) {
+  PrecData<R>& pd = pdata<R>(op);
+  const int64_t ng = (int64_t)op->n[0] * op->n[1] * op->n[2];
+  prof_mark(op, s);
+  k_summ<R><<<dim3((unsigned)cdiv(3 * op->nt, 128), k), 128, 0, s>>>(x, op->unk, pd.geo, op->nt, pd.summ, ldx);
+  CK(cudaGetLastError());
+  prof_mark(op, s);
+  k_project<R><<<dim3((unsigned)cdiv(op->ngnz * 32, 256), k), 256, 0, s>>>(
+      pd.summ, op->gpt, op->eoff, op->gtri, pd.gA, op->ngnz, ng, pd.src, col_stride_summ(op), col_stride_grid(op));
+  CK(cudaGetLastError());
+  prof_mark(op, s);
+  return fft_conv<R>(op, pd, s, false, k);
+}
+
 template <typename R>
 int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int k, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
@@ -1170,37 +1127,13 @@ int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
     set_error("apply_batch: batch size outside the workspace capacity");
     return SCABEM_E_ARG;
   }
-  const int64_t nt = op->nt, Q = op->Q;
-  const int n0 = op->n[0], n1 = op->n[1], n2 = op->n[2];
-  const int64_t ng = (int64_t)n0 * n1 * n2;
+  if (int rc = grid_potentials<R>(op, x, ldx, k, s)) return rc;
   prof_mark(op, s);
-  k_sources<R><<<dim3((unsigned)cdiv(Q, 128), k), 128, 0, s>>>(x, op->unk, op->cX, op->tri, op->qp, op->qw, Q,
-                                                               op->q, pd.summ, pd.qsrc, ldx);
+  k_test<R><<<dim3((unsigned)cdiv(op->nt, TS_WARPS), k), TS_WARPS * 32, 0, s>>>(
+      pd.grid, op->toff, op->tgi, op->soff, pd.wA, pd.wB, pd.wC, pd.sW, op->nsent, pd.geo, op->nt, (R)op->ke, (R)op->ki,
+      (R)op->ze, (R)op->zi, pd.val, col_stride_grid(op), col_stride_val(op));
   CK(cudaGetLastError());
-  prof_mark(op, s);
-  if (op->ngnz > 0) {
-    k_gather<R><<<dim3((unsigned)cdiv(op->ngnz * 32, 256), k), 256, 0, s>>>(
-        pd.qsrc, op->gpt, op->goff, op->gent, gather_weights<R>(op), op->ngnz, ng, pd.src, col_stride_qsrc(op),
-        col_stride_grid(op));
-    CK(cudaGetLastError());
-  }
-  prof_mark(op, s);
-  int rc = fft_conv<R>(op, pd, s, false, k);
-  if (rc) return rc;
-  prof_mark(op, s);
-  {
-    const size_t sm = pt_smem_bytes(op->q, sizeof(cx<R>));
-    PointsFn<R> fn = op->q == 6 ? (op->p == 2 ? k_points<R, 2, false, 6> : op->p == 3 ? k_points<R, 3, false, 6>
-                                                                                   : k_points<R, 4, false, 6>)
-                                : (op->p == 2 ? k_points<R, 2> : op->p == 3 ? k_points<R, 3> : k_points<R, 4>);
-    if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
-    fn<<<dim3((unsigned)cdiv(nt, PT_WARPS), k), PT_WARPS * 32, sm, s>>>(
-        pd.grid, op->base, pd.L, pd.dL, pd.near, op->noff, op->nsrc, pd.summ, op->tri, pd.tp, pd.sig, nt, op->q, n0,
-        n1, n2, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi, 0, op->valrow, pd.val, op->tmo_d, nullptr, nullptr,
-        col_stride_grid(op), col_stride_val(op));
-    CK(cudaGetLastError());
-  }
-  if ((rc = near_rows<R>(op, x, ldx, y, ldy, k, s))) return rc;
+  if (int rc = near_rows<R>(op, x, ldx, y, ldy, k, s)) return rc;
   prof_mark(op, s);
   return SCABEM_OK;
 }
@@ -1267,28 +1200,16 @@ int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_
 int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* lam, cx<double>* hs,
                          cudaStream_t s) {
   PrecData<double>& pd = op->d;
-  const int64_t nt = op->nt, Q = op->Q;
-  const int n0 = op->n[0], n1 = op->n[1], n2 = op->n[2];
-  const int64_t ng = (int64_t)n0 * n1 * n2;
-  k_sources<double><<<(int)cdiv(Q, 128), 128, 0, s>>>(x, op->unk, op->cX, op->tri, op->qp, op->qw, Q, op->q,
-                                                      pd.summ, pd.qsrc, op->N);
-  CK(cudaGetLastError());
-  if (op->ngnz > 0) {
-    k_gather<double><<<(int)cdiv(op->ngnz * 32, 256), 256, 0, s>>>(pd.qsrc, op->gpt, op->goff, op->gent, op->gwd,
-                                                                   op->ngnz, ng, pd.src, 0, 0);
-    CK(cudaGetLastError());
-  }
-  int rc = fft_conv<double>(op, pd, s, false);
-  if (rc) return rc;
+  if (int rc = grid_potentials<double>(op, x, op->N, 1, s)) return rc;
+  prof_mark(op, s);
   const size_t sm = pt_smem_bytes(op->q, sizeof(cx<double>));
-  PointsFn<double> fn = op->p == 2 ? k_points<double, 2, true> : op->p == 3 ? k_points<double, 3, true>
-                                                                            : k_points<double, 4, true>;
+  auto fn = op->p == 2 ? k_points_sens<double, 2> : op->p == 3 ? k_points_sens<double, 3> : k_points_sens<double, 4>;
   if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
-  fn<<<(int)cdiv(nt, PT_WARPS), PT_WARPS * 32, sm, s>>>(pd.grid, op->base, pd.L, pd.dL, pd.near, op->noff, op->nsrc,
-                                                        pd.summ, op->tri, pd.tp, pd.sig, nt, op->q, n0, n1, n2, op->ke,
-                                                        op->ki, op->ze, op->zi, op->npairs > 0 ? 1 : 0, op->valrow,
-                                                        nullptr, op->tmo_d, lam, hs, 0, 0);
+  fn<<<(int)cdiv(op->nt, PT_WARPS), PT_WARPS * 32, sm, s>>>(
+      pd.grid, op->base, pd.L, pd.dL, pd.near, op->noff, op->nsrc, pd.summ, op->tri, pd.tp, op->nt, op->q, op->n[1],
+      op->n[2], op->ke, op->ki, op->ze, op->zi, op->npairs > 0 ? 1 : 0, op->valrow, op->tmo_d, lam, hs);
   CK(cudaGetLastError());
+  prof_mark(op, s);
   return SCABEM_OK;
 }
 
@@ -1302,7 +1223,7 @@ int selftest_wait(scabem_op* op, cudaStream_t s) {
 // Current summaries only (used by the field evaluation at probe points).
 template <typename R>
 int compute_summ(scabem_op* op, const cx<R>* x, cx<R>* summ, cudaStream_t s) {
-  k_summ<R><<<(int)cdiv(op->nt, 128), 128, 0, s>>>(x, op->unk, op->cX, op->tri, op->nt, summ);
+  k_summ<R><<<(int)cdiv(3 * op->nt, 128), 128, 0, s>>>(x, op->unk, pdata<R>(op).geo, op->nt, summ, op->N);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }

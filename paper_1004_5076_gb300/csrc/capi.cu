@@ -90,7 +90,6 @@ void free_prec(PrecData<R>& pd) {
   cudaFree(pd.sig);
   cudaFree(pd.tp);
   cudaFree(pd.summ);
-  cudaFree(pd.qsrc);
   cudaFree(pd.src);
   cudaFree(pd.stA);
   cudaFree(pd.stB);
@@ -101,6 +100,12 @@ void free_prec(PrecData<R>& pd) {
   cudaFree(pd.nmv);
   cudaFree(pd.nmt);
   cudaFree(pd.gram);
+  cudaFree(pd.wA);
+  cudaFree(pd.wB);
+  cudaFree(pd.wC);
+  cudaFree(pd.gA);
+  cudaFree(pd.sW);
+  cudaFree(pd.geo);
   cudaFree(pd.sbar);
   cudaFree(pd.xs);
   cudaFree(pd.ys);
@@ -136,7 +141,6 @@ int alloc_prec(scabem_op* op, PrecData<R>& pd, bool workspaces, cudaStream_t s) 
     if ((rc = make_twiddles<R>(pd.tw[a], op->P[a], s))) return rc;
   }
   if ((rc = dalloc(&pd.summ, op->nt * 12))) return rc;
-  if ((rc = dalloc(&pd.qsrc, op->Q * 12))) return rc;
   if ((rc = dalloc(&pd.src, NFIELD_OUT * ng))) return rc;
   // grid points no stencil covers are never written by the projection
   CK(cudaMemsetAsync(pd.src, 0, sizeof(cx<R>) * NFIELD_OUT * ng, s));
@@ -151,8 +155,8 @@ int alloc_prec(scabem_op* op, PrecData<R>& pd, bool workspaces, cudaStream_t s) 
 }  // namespace
 
 // Grow the forward workspaces of one precision to k right-hand sides side by
-// side (column c at c * col_stride_*): the summaries, point sources, source
-// grids, axis-0 intermediates and potential grids.  New source grids and
+// side (column c at c * col_stride_*): the summaries, source grids,
+// axis-0 intermediates, potential grids and tested values.  New source grids and
 // intermediates start at zero (stencils and active columns leave the rest
 // untouched), as at creation.
 template <typename R>
@@ -164,10 +168,10 @@ int ensure_batch(scabem_op* op, int k, cudaStream_t s) {
   }
   if (k <= pd.kcap) return SCABEM_OK;
   CK(cudaStreamSynchronize(s));  // nothing in flight uses the old buffers
-  constexpr int NB = 7;
+  constexpr int NB = 6;
   cx<R>* nb[NB] = {};
-  cx<R>** cur[NB] = {&pd.summ, &pd.qsrc, &pd.src, &pd.stA, &pd.stB, &pd.grid, &pd.val};
-  const int64_t cs[NB] = {col_stride_summ(op), col_stride_qsrc(op), col_stride_grid(op), col_stride_st(op),
+  cx<R>** cur[NB] = {&pd.summ, &pd.src, &pd.stA, &pd.stB, &pd.grid, &pd.val};
+  const int64_t cs[NB] = {col_stride_summ(op), col_stride_grid(op), col_stride_st(op),
                           col_stride_st(op), col_stride_grid(op), col_stride_val(op)};
   for (int i = 0; i < NB; ++i) {
     int rc = dalloc(&nb[i], cs[i] * k);
@@ -662,6 +666,7 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
   TRY(upload(op->eunk, eunk.data(), sizeof(int32_t) * eunk.size()));
   TRY(setup_geometry(op, m, s));
   TRY(setup_gather(op, s));
+  TRY(setup_moments(op, s));
   op->cst = op->tdirect ? op->nac : (int64_t)op->n[1] * op->n[2];
   TRY(alloc_st(op, op->d, s));
   TRY(alloc_st(op, op->f, s));
@@ -822,6 +827,12 @@ void scabem_op_destroy(scabem_op_t op) {
   cudaFree(op->xsrc);
   cudaFree(op->rtk);
   cudaFree(op->tedge);
+  cudaFree(op->toff);
+  cudaFree(op->soff);
+  cudaFree(op->tgi);
+  cudaFree(op->eoff);
+  cudaFree(op->gtri);
+  cudaFree(op->gent2);
   cudaFree(op->nm_off);
   cudaFree(op->nm_nl);
   cudaFree(op->nm_col);

@@ -142,7 +142,6 @@ struct PrecData {
   R* tp = nullptr;                      // Q * 16 testing geometry: rel (3), w, X_k (3 x 3), div X_k (3)
   // workspaces
   cx<R>* summ = nullptr;  // nt * 3 sets * 4
-  cx<R>* qsrc = nullptr;  // Q * 12 weighted point sources
   cx<R>* src = nullptr;   // 16 * n0 n1 n2 (12 sources; 16 in the transposed apply)
   cx<R>* stA = nullptr;   // 16 * P0 * cst (12 fields in the apply, 16 in the transposed apply)
   cx<R>* recb = nullptr;  // Q * 2 * NREC record adjoints (transposed apply)
@@ -153,11 +152,18 @@ struct PrecData {
   cx<R>* val = nullptr;   // nt * 3 * 4 tested values of the grid part
   cx<R>* nmv = nullptr;   // near matrix, row-wise (near.cu)
   cx<R>* nmt = nullptr;   // near matrix, transposed
+  // triangle moments of the stencils (moments.cu), per entry of toff / soff
+  R* wA = nullptr;        // 4: m0, m1
+  R* wB = nullptr;        // 4: n0, c1.x
+  R* wC = nullptr;        // 2: c1.y, c1.z
+  R* gA = nullptr;        // wA in grid-point order
+  R* sW = nullptr;        // five blocks of 4 per entry: conductivity-weighted
+  R* geo = nullptr;       // nt * 16: cX_k, v_k - c (k < 3), normal
   R* gram = nullptr;      // nR * 5: <X_r, X_m> of absorber edges sharing a triangle
   cx<R>* xs = nullptr;    // staging for host x/y: N * nrhs_cap
   cx<R>* ys = nullptr;
   int64_t stage_cap = 0;
-  // right-hand sides the forward workspaces (summ, qsrc, src, stA, stB, grid)
+  // right-hand sides the forward workspaces (summ, src, stA, stB, grid, val)
   // hold side by side, at the column strides below
   int kcap = 1;
 };
@@ -232,6 +238,17 @@ struct scabem_op {
   int64_t npairs = 0;
   int32_t* noff = nullptr;  // nt + 1
   int32_t* nsrc = nullptr;  // npairs
+  // grid points of each triangle's stencils (moments.cu): entries toff[t] ..
+  // toff[t+1] at points tgi; soff[t] = the first of its conductivity-weighted
+  // entries (-1 without an absorber edge); covered point gpt[i] has the
+  // entries gent2[eoff[i] .. eoff[i+1]) of triangles gtri
+  int64_t ntent = 0, nsent = 0;
+  int32_t* toff = nullptr;
+  int32_t* soff = nullptr;
+  int32_t* tgi = nullptr;
+  int32_t* eoff = nullptr;
+  int32_t* gtri = nullptr;
+  int32_t* gent2 = nullptr;
   // near matrix over pairs of edges in class order (near.cu): row r's columns
   // nm_col[nm_off[r] .. nm_off[r+1]), the nm_nl[r] plain ones first; nm_tpos =
   // position of r among the columns of nm_col[i]; values of row r from
@@ -280,7 +297,6 @@ inline int64_t col_stride_st(const scabem_op* op) {  // stA and stB
 }
 inline int64_t col_stride_val(const scabem_op* op) { return op->nt * 12; }
 inline int64_t col_stride_summ(const scabem_op* op) { return op->nt * 12; }
-inline int64_t col_stride_qsrc(const scabem_op* op) { return op->Q * 12; }
 // Right-hand sides the batched apply handles per pass (one CTA of that many
 // warps shares each target triangle's near-record stream).
 constexpr int KBATCH = 8;
@@ -334,6 +350,9 @@ int setup_circulant(scabem_op* op, const scabem_mesh* mesh, const scabem_circula
 int circulant_apply(scabem_op* op, const cx<double>* in, cx<double>* out, int k, int64_t cs_in, int64_t cs_out,
                     cudaStream_t s);
 void circulant_release(scabem_op* op);
+// moments.cu
+int setup_moments(scabem_op* op, cudaStream_t s);
+int moments_update(scabem_op* op, cudaStream_t s);
 // near.cu
 int setup_near_matrix(scabem_op* op, cudaStream_t s);
 int near_matrix_update(scabem_op* op, cudaStream_t s);

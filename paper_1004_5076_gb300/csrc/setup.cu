@@ -1107,6 +1107,7 @@ int setup_sigma_monomial(scabem_op* op, int nseg, const double* seg, cudaStream_
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   if (dseg) cudaFree(dseg);
+  if (int rc = moments_update(op, s)) return rc;
   if (int rc = near_matrix_update(op, s)) return rc;
   return setup_precond(op, s);  // the absorber blocks depend on sigma
 }
@@ -1120,6 +1121,7 @@ int setup_sigma_bspline(scabem_op* op, double x0, double L, int axis, int ncoef,
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   cudaFree(dc);
+  if (int rc = moments_update(op, s)) return rc;
   if (int rc = near_matrix_update(op, s)) return rc;
   return setup_precond(op, s);
 }
@@ -1132,6 +1134,7 @@ int setup_sigma_values(scabem_op* op, const double* per_q_host, cudaStream_t s) 
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   cudaFree(tmp);
+  if (int rc = moments_update(op, s)) return rc;
   if (int rc = near_matrix_update(op, s)) return rc;
   return setup_precond(op, s);
 }
