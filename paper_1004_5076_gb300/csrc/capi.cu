@@ -94,25 +94,17 @@ void free_prec(PrecData<R>& pd) {
   cudaFree(pd.stA);
   cudaFree(pd.stB);
   cudaFree(pd.grid);
-  cudaFree(pd.val);
-  cudaFree(pd.recb);
-  cudaFree(pd.nadj);
   cudaFree(pd.nmv);
   cudaFree(pd.nmt);
   cudaFree(pd.gram);
-  cudaFree(pd.wA);
-  cudaFree(pd.wB);
-  cudaFree(pd.wC);
-  cudaFree(pd.gA);
-  cudaFree(pd.sW);
-  cudaFree(pd.geo);
-  cudaFree(pd.sbar);
+  cudaFree(pd.xw);
+  cudaFree(pd.gq);
   cudaFree(pd.xs);
   cudaFree(pd.ys);
   pd = PrecData<R>();
 }
 
-// The axis-0 intermediates, once the active columns and the (y, z) mode are
+// The axis-0 intermediates, source and potential grids, once the active columns and the (y, z) mode are
 // known: compact (active columns only) for the direct sums, whole planes for
 // the FFT planes; the axis-0 transform writes only the active columns, so
 // the rest of a whole plane stays zero from here.
@@ -124,6 +116,9 @@ int alloc_st(scabem_op* op, PrecData<R>& pd, cudaStream_t s) {
   if ((rc = dalloc(&pd.stA, n)) || (rc = dalloc(&pd.stB, n))) return rc;
   CK(cudaMemsetAsync(pd.stA, 0, sizeof(cx<R>) * n, s));
   CK(cudaMemsetAsync(pd.stB, 0, sizeof(cx<R>) * n, s));
+  // points of active columns that no stencil covers are never written by the projection
+  if ((rc = dalloc(&pd.src, col_stride_src(op))) || (rc = dalloc(&pd.grid, col_stride_pot(op)))) return rc;
+  CK(cudaMemsetAsync(pd.src, 0, sizeof(cx<R>) * col_stride_src(op), s));
   return SCABEM_OK;
 }
 
@@ -135,19 +130,11 @@ int alloc_prec(scabem_op* op, PrecData<R>& pd, bool workspaces, cudaStream_t s) 
   if ((rc = dalloc(&pd.sig, op->Q))) return rc;
   if ((rc = dalloc(&pd.tp, op->Q * 16))) return rc;
   if (!workspaces) return SCABEM_OK;
-  const int64_t ng = (int64_t)op->n[0] * op->n[1] * op->n[2];
   for (int a = 0; a < 3; ++a) {
     if ((rc = dalloc(&pd.tw[a], op->P[a]))) return rc;
     if ((rc = make_twiddles<R>(pd.tw[a], op->P[a], s))) return rc;
   }
   if ((rc = dalloc(&pd.summ, op->nt * 12))) return rc;
-  if ((rc = dalloc(&pd.src, NFIELD_OUT * ng))) return rc;
-  // grid points no stencil covers are never written by the projection
-  CK(cudaMemsetAsync(pd.src, 0, sizeof(cx<R>) * NFIELD_OUT * ng, s));
-  if ((rc = dalloc(&pd.recb, op->Q * 2 * NREC))) return rc;
-  if ((rc = dalloc(&pd.sbar, 2 * op->nt * 12))) return rc;
-  if ((rc = dalloc(&pd.grid, NFIELD_OUT * ng))) return rc;
-  if ((rc = dalloc(&pd.val, op->nt * 12))) return rc;
   pd.built = true;
   return SCABEM_OK;
 }
@@ -155,8 +142,8 @@ int alloc_prec(scabem_op* op, PrecData<R>& pd, bool workspaces, cudaStream_t s) 
 }  // namespace
 
 // Grow the forward workspaces of one precision to k right-hand sides side by
-// side (column c at c * col_stride_*): the summaries, source grids,
-// axis-0 intermediates, potential grids and tested values.  New source grids and
+// side (column c at c * col_stride_*): the source grids,
+// axis-0 intermediates and potential grids.  New source grids and
 // intermediates start at zero (stencils and active columns leave the rest
 // untouched), as at creation.
 template <typename R>
@@ -168,11 +155,10 @@ int ensure_batch(scabem_op* op, int k, cudaStream_t s) {
   }
   if (k <= pd.kcap) return SCABEM_OK;
   CK(cudaStreamSynchronize(s));  // nothing in flight uses the old buffers
-  constexpr int NB = 6;
+  constexpr int NB = 4;
   cx<R>* nb[NB] = {};
-  cx<R>** cur[NB] = {&pd.summ, &pd.src, &pd.stA, &pd.stB, &pd.grid, &pd.val};
-  const int64_t cs[NB] = {col_stride_summ(op), col_stride_grid(op), col_stride_st(op),
-                          col_stride_st(op), col_stride_grid(op), col_stride_val(op)};
+  cx<R>** cur[NB] = {&pd.src, &pd.stA, &pd.stB, &pd.grid};
+  const int64_t cs[NB] = {col_stride_src(op), col_stride_st(op), col_stride_st(op), col_stride_pot(op)};
   for (int i = 0; i < NB; ++i) {
     int rc = dalloc(&nb[i], cs[i] * k);
     if (rc) {
@@ -569,27 +555,6 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
       rowsrc[2 * r3 + 1] = (int32_t)(src[1] + 3);
     }
   }
-  // uses of each unknown in the current expansion (transposed apply)
-  std::vector<int32_t> xsrc(4 * m->N, 0);
-  {
-    std::vector<int> nuse(m->N, 0);
-    for (int64_t t = 0; t < m->nt; ++t)
-      for (int k = 0; k < 3; ++k)
-        for (int set = 0; set < 3; ++set) {
-          const int32_t u = unk[(3 * t + k) * 3 + set];
-          if (u == 0) continue;
-          const int64_t idx = (u > 0 ? u : -u) - 1;
-          const int32_t code = (int32_t)((t * 3 + k) * 3 + set) + 1;
-          if (nuse[idx] < 4) xsrc[4 * idx + nuse[idx]] = u > 0 ? code : -code;
-          ++nuse[idx];
-        }
-    for (int64_t i = 0; i < m->N; ++i)
-      if (nuse[i] > 4) {
-        set_error("internal: an unknown has more than four current uses");
-        scabem_op_destroy(op);
-        return SCABEM_E_MESH;
-      }
-  }
   // row of each (triangle, local edge, type) tested value, -1 if none
   std::vector<int32_t> valrow(12 * m->nt, -1);
   for (int64_t r = 0; r < m->N; ++r) {
@@ -638,7 +603,6 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
   TRY(dalloc(&op->region, op->nt));
   TRY(dalloc(&op->rowsrc, 2 * op->N));
   TRY(dalloc(&op->valrow, 12 * op->nt));
-  TRY(dalloc(&op->xsrc, 4 * op->N));
   TRY(dalloc(&op->qp, 3 * op->Q));
   TRY(dalloc(&op->qw, op->Q));
   TRY(dalloc(&op->base, 3 * op->Q));
@@ -657,7 +621,6 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
   TRY(upload(op->unk, unk.data(), sizeof(int32_t) * unk.size()));
   TRY(upload(op->rowsrc, rowsrc.data(), sizeof(int32_t) * rowsrc.size()));
   TRY(upload(op->valrow, valrow.data(), sizeof(int32_t) * valrow.size()));
-  TRY(upload(op->xsrc, xsrc.data(), sizeof(int32_t) * xsrc.size()));
   TRY(upload(op->region, m->region.data(), sizeof(int32_t) * m->nt));
   TRY(upload(op->etk, etk.data(), sizeof(int32_t) * etk.size()));
   TRY(upload(op->rtk, rtk.data(), sizeof(int32_t) * rtk.size()));
@@ -666,7 +629,7 @@ int scabem_op_create(scabem_mesh_t m, const scabem_media* md, const scabem_grid_
   TRY(upload(op->eunk, eunk.data(), sizeof(int32_t) * eunk.size()));
   TRY(setup_geometry(op, m, s));
   TRY(setup_gather(op, s));
-  TRY(setup_moments(op, s));
+  TRY(setup_stencils(op, s));
   op->cst = op->tdirect ? op->nac : (int64_t)op->n[1] * op->n[2];
   TRY(alloc_st(op, op->d, s));
   TRY(alloc_st(op, op->f, s));
@@ -804,11 +767,6 @@ void scabem_op_destroy(scabem_op_t op) {
   cudaFree(op->qp);
   cudaFree(op->qw);
   cudaFree(op->base);
-  cudaFree(op->goff);
-  cudaFree(op->gent);
-  cudaFree(op->gpt);
-  cudaFree(op->gwd);
-  cudaFree(op->gwf);
   cudaFree(op->sig64);
   cudaFree(op->noff);
   cudaFree(op->nsrc);
@@ -820,19 +778,16 @@ void scabem_op_destroy(scabem_op_t op) {
   cudaFree(op->pinv);
   cudaFree(op->err);
   cudaFree(op->acol);
-  cudaFree(op->gdd);
-  cudaFree(op->gdf);
-  cudaFree(op->roff);
-  cudaFree(op->rpair);
-  cudaFree(op->xsrc);
   cudaFree(op->rtk);
   cudaFree(op->tedge);
-  cudaFree(op->toff);
-  cudaFree(op->soff);
-  cudaFree(op->tgi);
-  cudaFree(op->eoff);
-  cudaFree(op->gtri);
-  cudaFree(op->gent2);
+  cudaFree(op->cmap);
+  cudaFree(op->xoff);
+  cudaFree(op->xpt);
+  cudaFree(op->gp);
+  cudaFree(op->gpoff);
+  cudaFree(op->gpl);
+  cudaFree(op->gpr);
+  cudaFree(op->gpe);
   cudaFree(op->nm_off);
   cudaFree(op->nm_nl);
   cudaFree(op->nm_col);

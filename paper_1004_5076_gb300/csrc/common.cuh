@@ -101,6 +101,7 @@ constexpr int MAXQ = 7;    // quadrature points per triangle
 constexpr int MAXP = 4;    // stencil points per axis
 constexpr int NFIELD_IN = 12;
 constexpr int NFIELD_OUT = 16;
+constexpr int NPOT = 32;  // complex values per grid point that the rows read: 8 groups of 4 (fft.cu)
 constexpr int NREC = 20;   // per point and medium: A(3) phi gphi(3) curlA(3) F(3) psi gpsi(3) curlF(3)
 constexpr int NCORR = 10;  // per point and medium: dP0, dP1(3), dQ(3), dC(3)
 constexpr double ETA0 = 376.730313668;
@@ -142,28 +143,19 @@ struct PrecData {
   R* tp = nullptr;                      // Q * 16 testing geometry: rel (3), w, X_k (3 x 3), div X_k (3)
   // workspaces
   cx<R>* summ = nullptr;  // nt * 3 sets * 4
-  cx<R>* src = nullptr;   // 16 * n0 n1 n2 (12 sources; 16 in the transposed apply)
+  cx<R>* src = nullptr;   // 16 * n0 * nac (12 sources; 16 in the transposed apply), [field][i0][active column]
   cx<R>* stA = nullptr;   // 16 * P0 * cst (12 fields in the apply, 16 in the transposed apply)
-  cx<R>* recb = nullptr;  // Q * 2 * NREC record adjoints (transposed apply)
-  cx<R>* sbar = nullptr;  // 2 * nt * 12: summary adjoints (near + direct, total)
-  cx<R>* nadj = nullptr;  // npairs * 12: per-pair near contributions (transposed apply)
   cx<R>* stB = nullptr;   // 16 * P0 * cst
-  cx<R>* grid = nullptr;  // n0 n1 n2 * 16, point-major: [point][medium][J, M set][A or F (3), phi or psi]
-  cx<R>* val = nullptr;   // nt * 3 * 4 tested values of the grid part
+  cx<R>* grid = nullptr;  // n0 * nac * NPOT potential groups, point-major (fft.cu)
   cx<R>* nmv = nullptr;   // near matrix, row-wise (near.cu)
   cx<R>* nmt = nullptr;   // near matrix, transposed
-  // triangle moments of the stencils (moments.cu), per entry of toff / soff
-  R* wA = nullptr;        // 4: m0, m1
-  R* wB = nullptr;        // 4: n0, c1.x
-  R* wC = nullptr;        // 2: c1.y, c1.z
-  R* gA = nullptr;        // wA in grid-point order
-  R* sW = nullptr;        // five blocks of 4 per entry: conductivity-weighted
-  R* geo = nullptr;       // nt * 16: cX_k, v_k - c (k < 3), normal
+  R* xw = nullptr;        // edge stencils (stencil.cu): 8 or 24 weights per entry
+  R* gq = nullptr;        // their Q0 blocks in grid-point order
   R* gram = nullptr;      // nR * 5: <X_r, X_m> of absorber edges sharing a triangle
   cx<R>* xs = nullptr;    // staging for host x/y: N * nrhs_cap
   cx<R>* ys = nullptr;
   int64_t stage_cap = 0;
-  // right-hand sides the forward workspaces (summ, src, stA, stB, grid, val)
+  // right-hand sides the forward workspaces (src, stA, stB, grid)
   // hold side by side, at the column strides below
   int kcap = 1;
 };
@@ -199,24 +191,14 @@ struct scabem_op {
   double* qp = nullptr;       // Q * 3
   double* qw = nullptr;       // Q
   int32_t* base = nullptr;    // Q * 3
-  // projection as a gather over the ngnz grid points that some stencil
-  // covers: point gpt[i] sums entries goff[i] .. goff[i+1]-1, entry e being
-  // quadrature point gent[e] with stencil weight gwd[e] / gwf[e]; entries
-  // are in (quadrature point, stencil slot) order within a grid point
-  int64_t ngnz = 0;
-  int32_t* gpt = nullptr;   // ngnz
-  int32_t* goff = nullptr;  // ngnz + 1
-  int32_t* gent = nullptr;  // Q * p^3
-  double* gwd = nullptr;    // Q * p^3
-  float* gwf = nullptr;     // Q * p^3
-  double* gdd = nullptr;    // Q * p^3 * 3 derivative weights of the entries (transposed interpolation)
-  float* gdf = nullptr;
+  int64_t ngnz = 0;  // grid points that some stencil covers
   // columns (i1, i2) of the grid that some stencil covers, ascending: the
   // only ones whose sources are non-zero and whose potentials are read, so
   // the axis-0 transforms run on these alone; rowmask bit i1 is set when row
   // i1 holds one of them
   int64_t nac = 0;
   int32_t* acol = nullptr;  // nac
+  int32_t* cmap = nullptr;  // n1 n2: position of a column among the active ones, -1 elsewhere
   uint64_t rowmask = 0;
   // (y, z) convolution: direct sum over the active columns (tdirect) with
   // gt[medium][q0][|d1|][|d2|] = (1/P0) x axis-0 transform of the spatial
@@ -238,17 +220,18 @@ struct scabem_op {
   int64_t npairs = 0;
   int32_t* noff = nullptr;  // nt + 1
   int32_t* nsrc = nullptr;  // npairs
-  // grid points of each triangle's stencils (moments.cu): entries toff[t] ..
-  // toff[t+1] at points tgi; soff[t] = the first of its conductivity-weighted
-  // entries (-1 without an absorber edge); covered point gpt[i] has the
-  // entries gent2[eoff[i] .. eoff[i+1]) of triangles gtri
-  int64_t ntent = 0, nsent = 0;
-  int32_t* toff = nullptr;
-  int32_t* soff = nullptr;
-  int32_t* tgi = nullptr;
-  int32_t* eoff = nullptr;
-  int32_t* gtri = nullptr;
-  int32_t* gent2 = nullptr;
+  // edge stencils (stencil.cu), edges in class order: edge r has the entries
+  // xoff[r] .. xoff[r+1] at compact grid points xpt, the nxl entries of plain
+  // edges first; covered point gp[i] has the entries gpe[gpoff[i] .. gpoff[i+1]) of
+  // edges gpr, gpl[i] of them of plain edges
+  int64_t nx = 0, nxl = 0, ngp = 0;
+  int32_t* xoff = nullptr;
+  int32_t* xpt = nullptr;
+  int32_t* gp = nullptr;
+  int32_t* gpoff = nullptr;
+  int32_t* gpl = nullptr;
+  int32_t* gpr = nullptr;
+  int32_t* gpe = nullptr;
   // near matrix over pairs of edges in class order (near.cu): row r's columns
   // nm_col[nm_off[r] .. nm_off[r+1]), the nm_nl[r] plain ones first; nm_tpos =
   // position of r among the columns of nm_col[i]; values of row r from
@@ -264,12 +247,6 @@ struct scabem_op {
   int64_t* nm_vt = nullptr;
   int32_t* nm_gcol = nullptr;  // nR * 5 columns of gram, -1 past the last
   bool nm_ready = false;       // values formed for all rows
-  // reverse list: pairs rpair[roff[s] .. roff[s+1]) have source triangle s
-  int32_t* roff = nullptr;   // nt + 1
-  int32_t* rpair = nullptr;  // npairs
-  // unknown -> up to 4 (triangle, local edge, set) uses, (code + 1) * sign,
-  // code = (t * 3 + k) * 3 + set; 0 = unused (transposed current expansion)
-  int32_t* xsrc = nullptr;   // N * 4
   cx<double>* gspatial[2] = {nullptr, nullptr};  // padded G tables, set-up only
   // per-edge block-diagonal preconditioner (exact self blocks, inverted)
   int32_t* etk = nullptr;   // ne * 4: T+, k+, T-, k-
@@ -289,14 +266,11 @@ struct scabem_op {
 };
 
 // Column strides of the forward workspaces (complex values per right-hand side).
-inline int64_t col_stride_grid(const scabem_op* op) {  // src and grid
-  return (int64_t)NFIELD_OUT * op->n[0] * op->n[1] * op->n[2];
-}
+inline int64_t col_stride_src(const scabem_op* op) { return (int64_t)NFIELD_OUT * op->n[0] * op->nac; }
+inline int64_t col_stride_pot(const scabem_op* op) { return (int64_t)NPOT * op->n[0] * op->nac; }
 inline int64_t col_stride_st(const scabem_op* op) {  // stA and stB
   return (int64_t)NFIELD_OUT * op->P[0] * op->cst;
 }
-inline int64_t col_stride_val(const scabem_op* op) { return op->nt * 12; }
-inline int64_t col_stride_summ(const scabem_op* op) { return op->nt * 12; }
 // Right-hand sides the batched apply handles per pass (one CTA of that many
 // warps shares each target triangle's near-record stream).
 constexpr int KBATCH = 8;
@@ -350,15 +324,18 @@ int setup_circulant(scabem_op* op, const scabem_mesh* mesh, const scabem_circula
 int circulant_apply(scabem_op* op, const cx<double>* in, cx<double>* out, int k, int64_t cs_in, int64_t cs_out,
                     cudaStream_t s);
 void circulant_release(scabem_op* op);
-// moments.cu
-int setup_moments(scabem_op* op, cudaStream_t s);
-int moments_update(scabem_op* op, cudaStream_t s);
+// stencil.cu
+int setup_stencils(scabem_op* op, cudaStream_t s);
+int stencils_update(scabem_op* op, cudaStream_t s);
 // near.cu
 int setup_near_matrix(scabem_op* op, cudaStream_t s);
 int near_matrix_update(scabem_op* op, cudaStream_t s);
-// y_c = near part of A x_c + row sums of the tested values pd.val (column c), c < kc <= KBATCH
+// y_c = A x_c from the potentials (pd.grid) and the near matrix, c < kc <= KBATCH
 template <typename R>
-int near_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s);
+int rows_apply(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s);
+// x = A^T y from the convolved adjoint fields (pd.grid) and the transposed near matrix
+template <typename R>
+int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s);
 // apply.cu
 template <typename R>
 int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s);

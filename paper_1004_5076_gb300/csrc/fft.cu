@@ -2,23 +2,27 @@
 // multiply (the FFT acceleration of Appendix B, on the uniform grid of the
 // precorrected-FFT method).
 //
-// Layout: physical grids are [field][i0][i1][i2] with n0 x n1 x n2 points; the
-// transform size is P = 2n per axis.  The convolution runs in three kernels:
+// Layout: physical grids are [field][i0][active column] (n0 points along axis 0,
+// the (i1, i2) columns that some stencil covers); the transform size is P = 2n
+// per axis.  The convolution runs in three kernels:
 //   stage A: forward FFT along axis 0 of the 12 source fields, input pruned
 //            to i0 < n0, output [field][k0][i1][i2] (P0 x n1 x n2);
 //   stage B: per k0 plane, forward 2-D FFT over (i1, i2) (input pruned to the
 //            physical n1 x n2 corner), multiply by the Green spectrum of the
 //            medium, inverse 2-D FFT, keep the physical corner: 12 -> 16 fields;
 //   stage C: inverse FFT along axis 0, keep i0 < n0, written point-major
-//            [i0][i1][i2][16] for the interpolation gathers.
+//            [i0][active column][32] for the testing gathers.
 // Every FFT is an in-place shared-memory Stockham transform (radix 8, then 4
 // or 2) with compile-time power-of-two lengths: each pass loads its
 // butterflies into registers, synchronises, and stores them at their sorted
 // positions.  One CTA owns whole lines, so each field makes one HBM round trip
 // per stage.  The 1/(P0 P1 P2) scale is folded into the stored spectra.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -170,15 +174,15 @@ struct Tot {
 };
 
 // ---------------------------------------------------------------- stage A / C
-// Stage A on the active columns acol[0 .. nac) of the [field][i0][c] layout
-// (C columns per i0); one CTA owns CB of them for one field over the whole
-// axis 0 (smem: [P0][CB], lines = columns).  Inputs i0 >= n_in are zero.
+// Stage A on the nac active columns, [field][i0][active column]; one CTA owns
+// CB of them for one field over the whole axis 0 (smem: [P0][CB], lines =
+// columns).  Inputs i0 >= n_in are zero.
 // The output has Cout columns per (field, k0): active column j goes to
 // column j (compact, Cout = nac) or to acol[j] (whole planes, Cout = C).
 template <typename R>
 __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__ in, cx<R>* __restrict__ out,
-                                                       int n_in, int P0, int C, const int32_t* __restrict__ acol,
-                                                       int nac, int CB, const cx<R>* __restrict__ tw,
+                                                       int n_in, int P0, const int32_t* __restrict__ acol, int nac,
+                                                       int CB, const cx<R>* __restrict__ tw,
                                                        int64_t cs_in, int64_t cs_out, int64_t Cout, int compact) {
   extern __shared__ unsigned char smem_raw[];
   cx<R>* tws = reinterpret_cast<cx<R>*>(smem_raw);
@@ -189,11 +193,11 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__
   const int a0 = blockIdx.x * CB;
   const int lcb = ilog2(CB);
   for (int i = threadIdx.x; i < P0; i += FFT_THREADS) tws[i] = tw[i];
-  const int64_t fin = (int64_t)f * n_in * C;
+  const int64_t fin = (int64_t)f * n_in * nac;
   for (int idx = threadIdx.x; idx < P0 * CB; idx += FFT_THREADS) {
     const int i0 = idx >> lcb, l = idx & (CB - 1);
     cx<R> v = czero<R>();
-    if (i0 < n_in && a0 + l < nac) v = in[fin + (int64_t)i0 * C + acol[a0 + l]];
+    if (i0 < n_in && a0 + l < nac) v = in[fin + (int64_t)i0 * nac + a0 + l];
     b0[idx] = v;
   }
   __syncthreads();
@@ -205,17 +209,26 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__
   }
 }
 
-// Stage C with point-major output, on the active columns acol[0 .. nac)
-// only (the potentials are read nowhere else; the input holds Cin columns
-// per (field, k0), compact or whole planes as stage A wrote them): one CTA owns NC of them for one group of 4
-// output fields over axis 0 (line l = field * NC + column) and writes
-// out[(i0 * C + c) * 16 + 4 * grp + f] for i0 < n_out, so the 16 potentials of
-// a grid point are contiguous and each group of 4 fills whole 32-byte sectors.
-template <typename R>
-__global__ void __launch_bounds__(FFT_THREADS) k_axis0_pm(const cx<R>* __restrict__ in, cx<R>* __restrict__ out,
-                                                          int n_out, int P0, int C, const int32_t* __restrict__ acol,
-                                                          int nac, int NC, const cx<R>* __restrict__ tw,
-                                                          int64_t cs_in, int64_t cs_out, int64_t Cin, int compact) {
+// Stage C with point-major output, on the nac active columns only (the
+// potentials are read nowhere else; the input holds Cin columns per (field,
+// k0), compact or whole planes as stage A wrote them): one CTA owns NC of them
+// for one group of 4 fields over axis 0 (line l = field * NC + column) and
+// writes out[(i0 * nac + column) * 32 + 4 * group + f] for i0 < n_out, whole
+// 32-byte sectors in complex64.
+//
+// The groups are what the rows read (near.cu).  Groups 4 .. 7: the four sets'
+// potentials, [A, phi] scaled by j z k and j z / k (the strong-form E of
+// Eqs. 13, 14) and [F, 0], of the exterior and the interior medium.  Groups 0 ..
+// 3: the weak-form differences of the two media, E from [A, phi] and [F], H from
+// [F, psi] and [A], which halve the products of the testing.  The CTAs of the
+// two media exchange their lines through distributed shared memory (a cluster
+// of the four groups).  COMB = false (transposed apply): the fields themselves in
+// groups 4 .. 7.
+template <typename R, bool COMB>
+__global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FFT_THREADS)
+    k_axis0_pm(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, int n_out, int P0,
+               const int32_t* __restrict__ acol, int nac, int NC, const cx<R>* __restrict__ tw, int64_t cs_in,
+               int64_t cs_out, int64_t Cin, int compact, R ke, R ki, R ze, R zi) {
   extern __shared__ unsigned char smem_raw[];
   cx<R>* tws = reinterpret_cast<cx<R>*>(smem_raw);
   cx<R>* b0 = tws + P0;
@@ -235,11 +248,49 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0_pm(const cx<R>* __restric
   }
   __syncthreads();
   fft_lines<R, 1, Tot<R>::L>(b0, ilog2(P0), lcb, 1, CB, tws);
-  for (int idx = threadIdx.x; idx < n_out * CB; idx += FFT_THREADS) {
-    const int k0 = idx >> lcb, l = idx & (CB - 1);
-    const int cl = l >> 2, fl = l & 3;  // field fastest: consecutive threads fill a sector
-    if (a0 + cl < nac)
-      out[((int64_t)k0 * C + acol[a0 + cl]) * NFIELD_OUT + 4 * grp + fl] = b0[(k0 << lcb) + fl * NC + cl];
+  if constexpr (!COMB) {
+    for (int idx = threadIdx.x; idx < n_out * CB; idx += FFT_THREADS) {
+      const int k0 = idx >> lcb, l = idx & (CB - 1);
+      const int cl = l >> 2, fl = l & 3;  // field fastest: consecutive threads fill a sector
+      if (a0 + cl < nac)
+        out[((int64_t)k0 * nac + a0 + cl) * NPOT + 16 + 4 * grp + fl] = b0[(k0 << lcb) + fl * NC + cl];
+    }
+  } else {
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    const cx<R>* rb = cluster.map_shared_rank(b0, grp ^ 2);  // the same set in the other medium
+    const bool isM = grp & 1, inner = grp & 2;
+    const R k = inner ? ki : ke, z = inner ? zi : ze, ko = inner ? ke : ki, zo = inner ? ze : zi;
+    const R sg = inner ? R(-1) : R(1);  // weak-form rows take exterior - interior
+    // group 0 (rank 0): E from A, phi   group 1 (rank 1): E from F
+    // group 2 (rank 3): H from F, psi   group 3 (rank 2): H from A
+    const int og = grp == 0 ? 0 : grp == 1 ? 1 : grp == 3 ? 2 : 3;
+    for (int idx = threadIdx.x; idx < n_out * CB; idx += FFT_THREADS) {
+      const int k0 = idx >> lcb, l = idx & (CB - 1);
+      const int cl = l >> 2, fl = l & 3;
+      if (a0 + cl >= nac) continue;
+      const int at = (k0 << lcb) + fl * NC + cl;
+      const cx<R> v = b0[at], w = rb[at];
+      cx<R> weak, own;
+      if (!isM) {
+        own = mulj((fl < 3 ? z * k : z / k) * v);
+        if (og == 0)
+          weak = fl < 3 ? mulj((zo * ko) * w - (z * k) * v) : mulj((z / k) * v - (zo / ko) * w);
+        else
+          weak = fl < 3 ? w - v : czero<R>();
+      } else {
+        own = fl < 3 ? v : czero<R>();
+        if (og == 1)
+          weak = fl < 3 ? w - v : czero<R>();
+        else
+          weak = fl < 3 ? mulj((k / z) * v - (ko / zo) * w)
+                        : mulj((R(1) / (ko * zo)) * w + (sg / (k * z)) * v);
+      }
+      cx<R>* o = out + ((int64_t)k0 * nac + a0 + cl) * NPOT + fl;
+      o[4 * og] = weak;
+      o[16 + 4 * grp] = own;
+    }
+    cluster.sync();  // no CTA leaves while another still reads its lines
   }
 }
 
@@ -820,18 +871,18 @@ int pruned_lines(int P0) {
   return l < 8 ? l : 8;
 }
 
-// stage C: 16 fields [field][k0][c] -> point-major grid [i0][c][16], active columns
+// stage C: 16 fields [field][k0][c] -> point-major groups, active columns
 template <typename R>
-static int axis0_inverse(scabem_op* op, PrecData<R>& pd, cudaStream_t s, int ncol) {
-  const int n0 = op->n[0], P0 = op->P[0];
-  const int C = op->n[1] * op->n[2];
+static int axis0_inverse(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int ncol) {
+  const int P0 = op->P[0];
   const int lines = op->a0_lines > 0 ? op->a0_lines : pruned_lines<R>(P0);
   const int nc = lines >= 4 ? lines / 4 : 1;  // P0 <= 1024: 4 lines fit
   const size_t sm = (size_t)P0 * (4 * nc + 1) * sizeof(cx<R>);
-  if (int rc_ = set_max_smem(op->device, (const void*)k_axis0_pm<R>, (int)sm)) return rc_;
-  k_axis0_pm<R><<<dim3((unsigned)cdiv(op->nac, nc), NFIELD_OUT / 4, ncol), FFT_THREADS, sm, s>>>(
-      pd.stB, pd.grid, n0, P0, C, op->acol, (int)op->nac, nc, pd.tw[0], col_stride_st(op), col_stride_grid(op),
-      op->cst, op->tdirect ? 1 : 0);
+  auto fn = adjoint ? k_axis0_pm<R, false> : k_axis0_pm<R, true>;
+  if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
+  fn<<<dim3((unsigned)cdiv(op->nac, nc), NFIELD_OUT / 4, ncol), FFT_THREADS, sm, s>>>(
+      pd.stB, pd.grid, op->n[0], P0, op->acol, (int)op->nac, nc, pd.tw[0], col_stride_st(op), col_stride_pot(op), op->cst,
+      op->tdirect ? 1 : 0, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }
@@ -842,7 +893,6 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
   const int nf = adjoint ? NFIELD_OUT : NFIELD_IN;  // fields transformed along axis 0
   const int id = adjoint ? 1 : 0;
   const int P0 = op->P[0], P1 = op->P[1], P2 = op->P[2];
-  const int C = n1 * n2;
   if (op->nac == 0) {
     set_error("grid: no grid point is covered by a stencil");
     return SCABEM_E_ARG;
@@ -852,7 +902,7 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
   // stage A
   if (int rc_ = set_max_smem(op->device, (const void*)k_axis0<R>, (int)sm0)) return rc_;
   k_axis0<R><<<dim3((unsigned)cdiv(op->nac, cb), nf, ncol), FFT_THREADS, sm0, s>>>(
-      pd.src, pd.stA, n0, P0, C, op->acol, (int)op->nac, cb, pd.tw[0], col_stride_grid(op), col_stride_st(op),
+      pd.src, pd.stA, n0, P0, op->acol, (int)op->nac, cb, pd.tw[0], col_stride_src(op), col_stride_st(op),
       op->cst, op->tdirect ? 1 : 0);
   CK(cudaGetLastError());
   prof_mark(op, s);
@@ -865,7 +915,7 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
                                                                  op->R1, op->R2, id, col_stride_st(op), 1);
     CK(cudaGetLastError());
     prof_mark(op, s);
-    return axis0_inverse(op, pd, s, ncol);
+    return axis0_inverse(op, pd, s, adjoint, ncol);
   }
   if (P1 == 64 && P2 == 64) {
     const size_t sm = ((size_t)2 * 32 * 64 + (size_t)(P64_THREADS / 8) * P64_SCR) * sizeof(cx<R>);
@@ -874,7 +924,7 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
                                                               op->rowmask, id, col_stride_st(op));
     CK(cudaGetLastError());
     prof_mark(op, s);
-    return axis0_inverse(op, pd, s, ncol);
+    return axis0_inverse(op, pd, s, adjoint, ncol);
   }
   const size_t sm1 = ((size_t)P1 + P2 + 2 * (size_t)P1 * (P2 + 2)) * sizeof(cx<R>);
   PlanesFn<R> fn = planes_kernel<R>(ilog2(P1), ilog2(P2));
@@ -887,7 +937,7 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
                                                   pd.tw[2], id, col_stride_st(op));
   CK(cudaGetLastError());
   prof_mark(op, s);
-  return axis0_inverse(op, pd, s, ncol);
+  return axis0_inverse(op, pd, s, adjoint, ncol);
 }
 
 template int make_twiddles<float>(cx<float>*, int, cudaStream_t);

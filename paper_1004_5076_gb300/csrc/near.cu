@@ -33,7 +33,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "common.cuh"
+#include "device.cuh"
 
 namespace {
 
@@ -322,72 +322,73 @@ __global__ void k_near_gram(const int32_t* __restrict__ rtk, const int32_t* __re
 }
 
 // ---------------------------------------------------------------- products
-template <typename R>
-__device__ __forceinline__ void cmac(cx<R>& a, cx<R> v, cx<R> x) {
-  cfma(a, v, x);
-}
-template <>
-__device__ __forceinline__ void cmac(cx<float>& a, cx<float> v, cx<float> x) {
-  // two packed FP32x2 FMAs: a + v.re (x.re, x.im) + v.im (-x.im, x.re)
-  float2 r = __ffma2_rn(make_float2(v.re, v.re), make_float2(x.re, x.im), make_float2(a.re, a.im));
-  r = __ffma2_rn(make_float2(v.im, v.im), make_float2(-x.im, x.re), r);
-  a = mk(r.x, r.y);
-}
-template <typename R>
-__device__ __forceinline__ cx<R> ldstream(const cx<R>* p) {
-  return *p;
+// f(m, v) for the columns m = col[j] with values v[e] = val[e n + j], j = lane,
+// lane + LANES, ..: the next column's loads are issued before the current
+// column's dependent gathers of x, so two columns per lane are in flight.
+template <typename R, int W, int LANES, class F>
+__device__ __forceinline__ void near_segment(const int32_t* __restrict__ col, const cx<R>* __restrict__ val, int n,
+                                             int lane, const F& f) {
+  int j = lane, m = 0;
+  cx<R> v[W];
+  if (j < n) {
+    m = col[j];
+#pragma unroll
+    for (int e = 0; e < W; ++e) v[e] = ldstream(val + (int64_t)e * n + j);
+  }
+  while (j < n) {
+    const int jn = j + LANES;
+    int mn = 0;
+    cx<R> vn[W];
+    if (jn < n) {
+      mn = col[jn];
+#pragma unroll
+      for (int e = 0; e < W; ++e) vn[e] = ldstream(val + (int64_t)e * n + jn);
+    }
+    f(m, v);
+    j = jn;
+    m = mn;
+    if (jn < n)
+#pragma unroll
+      for (int e = 0; e < W; ++e) v[e] = vn[e];
+  }
 }
 
 // One row of the matrix (T = false) or of its transpose (T = true) against
 // the kc <= K columns of x: the row's three (two for a plain edge) sums in
-// acc, each lane of the NM_LANES sharing the row taking every NM_LANES-th
-// column.  x holds the unknowns (or, transposed, the rows) of an edge m at m,
-// nL + m (plain) or nL + m, nL + m + nR, nL + m + 2 nR (absorber).
-constexpr int NM_LANES = 16;
+// acc, each of the LANES lanes sharing the row taking every LANES-th column.
+// x holds the unknowns (or, transposed, the rows) of an edge m at m, nL + m
+// (plain) or nL + m, nL + m + nR, nL + m + 2 nR (absorber).
 constexpr int NM_THREADS = 128;
 
-template <typename R, int K, bool T>
+template <typename R, int K, bool T, int LANES>
 __device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, const int32_t* __restrict__ off,
                                          const int32_t* __restrict__ nl, const int32_t* __restrict__ col,
                                          const int64_t* __restrict__ vo, const cx<R>* __restrict__ val,
                                          const cx<R>* __restrict__ x, int64_t ldx, int kc, int lane, cx<R> acc[3][K]) {
-  const bool isR = r >= nL;
   const int c0 = off[r], cl = nl[r], cr = off[r + 1] - c0 - cl;
   const cx<R>* v0 = val + vo[r];
-  if (!isR) {
-    for (int j = lane; j < cl; j += NM_LANES) {
-      const int m = col[c0 + j];
-      const cx<R> U = v0[j], G = v0[cl + j], V = v0[2 * cl + j];
+  const int32_t *colL = col + c0, *colR = colL + cl;
+  if (r < nL) {
+    near_segment<R, 3, LANES>(colL, v0, cl, lane, [&](int m, const cx<R>* v) {
       const cx<R>* xm = x + m;
 #pragma unroll
       for (int c = 0; c < K; ++c)
-        if (c < kc) {
+        if (c < kc) {  // U G V
           const cx<R> a = xm[c * ldx], b = xm[c * ldx + nL];
-          if (!T) {
-            cmac(acc[0][c], U, a);
-            cmac(acc[0][c], -G, b);
-            cmac(acc[1][c], G, a);
-            cmac(acc[1][c], V, b);
-          } else {
-            cmac(acc[0][c], U, a);
-            cmac(acc[0][c], G, b);
-            cmac(acc[1][c], -G, a);
-            cmac(acc[1][c], V, b);
-          }
+          cmac(acc[0][c], v[0], a);
+          cmac(acc[0][c], T ? v[1] : -v[1], b);
+          cmac(acc[1][c], T ? -v[1] : v[1], a);
+          cmac(acc[1][c], v[2], b);
         }
-    }
-    v0 += (int64_t)nm_words(false, false) * cl;
-    for (int j = lane; j < cr; j += NM_LANES) {
-      const int m = col[c0 + cl + j];
-      cx<R> v[6];
-#pragma unroll
-      for (int e = 0; e < (T ? 6 : 5); ++e) v[e] = v0[(int64_t)e * cr + j];
+    });
+    near_segment<R, T ? 6 : 5, LANES>(colR, v0 + (int64_t)nm_words(false, false) * cl, cr, lane,
+                                      [&](int m, const cx<R>* v) {
       const cx<R>* xm = x + nL + m;
 #pragma unroll
       for (int c = 0; c < K; ++c)
         if (c < kc) {
           const cx<R> a = xm[c * ldx], b = xm[c * ldx + nR], d = xm[c * ldx + 2 * nR];
-          if (!T) {  // Ue Ui ge gi V
+          if constexpr (!T) {  // Ue Ui ge gi V
             cmac(acc[0][c], v[0], a);
             cmac(acc[0][c], -v[1], b);
             cmac(acc[0][c], -(v[2] + v[3]), d);
@@ -403,26 +404,22 @@ __device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, cons
             cmac(acc[1][c], v[5], d);
           }
         }
-    }
+    });
   } else {
-    for (int j = lane; j < cl; j += NM_LANES) {
-      const int m = col[c0 + j];
-      cx<R> v[6];
-#pragma unroll
-      for (int e = 0; e < (T ? 5 : 6); ++e) v[e] = v0[(int64_t)e * cl + j];
+    near_segment<R, T ? 5 : 6, LANES>(colL, v0, cl, lane, [&](int m, const cx<R>* v) {
       const cx<R>* xm = x + m;
 #pragma unroll
       for (int c = 0; c < K; ++c)
         if (c < kc) {
           const cx<R> a = xm[c * ldx], b = xm[c * ldx + nL];
-          if (!T) {
+          if constexpr (!T) {  // U G G13 V13 P Q
             cmac(acc[0][c], v[0], a);
             cmac(acc[0][c], -v[1], b);
             cmac(acc[1][c], v[2], a);
             cmac(acc[1][c], v[3], b);
             cmac(acc[2][c], v[4], a);
             cmac(acc[2][c], v[5], b);
-          } else {
+          } else {  // Ue Ui ge gi V
             cmac(acc[0][c], v[0], a);
             cmac(acc[0][c], v[2], b);
             cmac(acc[1][c], -v[1], a);
@@ -431,20 +428,15 @@ __device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, cons
             cmac(acc[2][c], v[4], b);
           }
         }
-    }
-    v0 += (int64_t)(T ? 5 : 6) * cl;
-    for (int j = lane; j < cr; j += NM_LANES) {
-      const int m = col[c0 + cl + j];
-      cx<R> v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = v0[(int64_t)e * cr + j];
+    });
+    near_segment<R, 8, LANES>(colR, v0 + (int64_t)(T ? 5 : 6) * cl, cr, lane, [&](int m, const cx<R>* v) {
       const cx<R>* xm = x + nL + m;
 #pragma unroll
       for (int c = 0; c < K; ++c)
-        if (c < kc) {
+        if (c < kc) {  // Ue Ui e13 i13 G V13 P Q
           const cx<R> a = xm[c * ldx], b = xm[c * ldx + nR], d = xm[c * ldx + 2 * nR];
-          if (!T) {
-            cmac(acc[0][c], v[0], a);
+          cmac(acc[0][c], v[0], a);
+          if constexpr (!T) {
             cmac(acc[0][c], -v[1], b);
             cmac(acc[0][c], -v[4], d);
             cmac(acc[1][c], v[2], a);
@@ -453,7 +445,6 @@ __device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, cons
             cmac(acc[2][c], v[6], b);
             cmac(acc[2][c], v[7], d);
           } else {
-            cmac(acc[0][c], v[0], a);
             cmac(acc[0][c], v[2], b);
             cmac(acc[1][c], -v[1], a);
             cmac(acc[1][c], v[3], b);
@@ -463,42 +454,17 @@ __device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, cons
             cmac(acc[2][c], v[7], d);
           }
         }
-    }
+    });
   }
 }
 
-// y = near part + the tested values of the grid part (val, summed per row
-// over the edge's two triangles): the last launch of an apply.  Every row is
-// written once, from sums in a fixed order.
-template <typename R, int K>
-__global__ void __launch_bounds__(NM_THREADS)
-    k_near_rows(const int32_t* __restrict__ off, const int32_t* __restrict__ nl, const int32_t* __restrict__ col,
-                const int64_t* __restrict__ vo, const cx<R>* __restrict__ nmv, const int32_t* __restrict__ gcol,
-                const R* __restrict__ gval, const int32_t* __restrict__ rtk, int64_t ne, int64_t nL,
-                const cx<R>* __restrict__ val, int64_t cs_val, const cx<R>* __restrict__ x, int64_t ldx,
-                cx<R>* __restrict__ y, int64_t ldy, int kc) {
-  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / NM_LANES;
-  const int lane = threadIdx.x % NM_LANES;
-  const int64_t nR = ne - nL;
-  cx<R> acc[3][K];
+// Sums over the LANES lanes of a row, in every lane (within a warp), or over
+// the CTA's four warps in the first warp's lanes (LANES = NM_THREADS).
+template <typename R, int K, int LANES>
+__device__ __forceinline__ void near_reduce(cx<R> acc[3][K]) {
+  constexpr int W = LANES < 32 ? LANES : 32;
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int c = 0; c < K; ++c) acc[i][c] = czero<R>();
-  if (r < ne) {
-    near_row<R, K, false>(r, nL, nR, off, nl, col, vo, nmv, x, ldx, kc, lane, acc);
-    if (r >= nL && lane < 5) {
-      const int g = gcol[5 * (r - nL) + lane];
-      if (g >= 0) {
-        const R s = gval[5 * (r - nL) + lane];
-#pragma unroll
-        for (int c = 0; c < K; ++c)
-          if (c < kc) axpy(acc[2][c], s, x[c * ldx + nL + g]);
-      }
-    }
-  }
-#pragma unroll
-  for (int o = NM_LANES / 2; o > 0; o >>= 1)
+  for (int o = W / 2; o > 0; o >>= 1)
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -506,10 +472,115 @@ __global__ void __launch_bounds__(NM_THREADS)
         acc[i][c].re += __shfl_xor_sync(0xffffffffu, acc[i][c].re, o);
         acc[i][c].im += __shfl_xor_sync(0xffffffffu, acc[i][c].im, o);
       }
-  if (r >= ne || lane >= kc) return;
+  if constexpr (LANES > 32) {
+    __shared__ cx<R> sm[LANES / 32][3 * K];
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int c = 0; c < K; ++c) sm[w][i * K + c] = acc[i][c];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        cx<R> v = sm[0][i * K + c];
+#pragma unroll
+        for (int u = 1; u < LANES / 32; ++u) v += sm[u][i * K + c];
+        acc[i][c] = v;
+      }
+  }
+}
+
+// Grid part of an edge's rows: sums over the edge's covered grid points (entries
+// x0 .. x0 + n, compact points xpt) of the entry's weight blocks (stencil.cu)
+// and the potential groups there.  Lane = slot * G + group, G = 4 groups of a
+// plain edge, 8 of an absorber edge: each lane sums one group (four complex
+// values, 32 bytes in complex64, against four weights) into ga[c].
+template <typename R, int K, int G, int LANES>
+__device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n, const R* __restrict__ w,
+                                          const cx<R>* __restrict__ pot, int64_t cs_g, int kc, int lane,
+                                          cx<R> ga[K]) {
+  constexpr int STRIDE = G == 4 ? 8 : 24;
+  const int grp = lane % G, slot = lane / G;
+  w += 4 * (grp < 4 ? grp & 1 : grp - 2);
+  pot += 4 * grp;
+#pragma unroll 2
+  for (int j = slot; j < n; j += LANES / G) {
+    R a[4];
+    load4(w + STRIDE * j, a);
+    const cx<R>* pp = pot + (int64_t)xpt[j] * NPOT;
+#pragma unroll
+    for (int c = 0; c < K; ++c)
+      if (c < kc) {
+        cx<R> g[4];
+        load_group(pp + c * cs_g, g);
+#pragma unroll
+        for (int f = 0; f < 4; ++f) axpy2(ga[c], a[f], g[f]);
+      }
+  }
+}
+
+struct RowTables {
+  const int32_t *off, *nl, *col;  // near matrix (rows in class order)
+  const int64_t* vo;
+  const int32_t* gcol;
+  const int32_t *xoff, *xpt;  // edge stencils
+  int64_t ne, nL, nxl;
+};
+
+// K4: y = grid part + near part of every row, the last launch of an apply:
+// LANES lanes per edge.  The testing of the potentials and the near-field
+// matrix of an edge meet in one reduction, and every row is written once,
+// from sums in a fixed order.  Bound by the stream of near values and
+// weights (HBM on large operators) and by load latency: the near values are
+// loaded a column ahead, the weights two entries at a time.
+template <typename R, int K, int LANES>
+__global__ void __launch_bounds__(NM_THREADS)
+    k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
+           const cx<R>* __restrict__ pot, int64_t cs_g, const cx<R>* __restrict__ x, int64_t ldx, cx<R>* __restrict__ y,
+           int64_t ldy, int kc) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
+  const int lane = threadIdx.x % LANES;
+  const int64_t nL = T.nL, nR = T.ne - nL;
+  cx<R> acc[3][K];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int c = 0; c < K; ++c) acc[i][c] = czero<R>();
+  if (r < T.ne) {
+    near_row<R, K, false, LANES>(r, nL, nR, T.off, T.nl, T.col, T.vo, nmv, x, ldx, kc, lane, acc);
+    const int x0 = T.xoff[r], n = T.xoff[r + 1] - x0;
+    cx<R> ga[K];
+#pragma unroll
+    for (int c = 0; c < K; ++c) ga[c] = czero<R>();
+    int i;
+    if (r < nL) {
+      grid_rows<R, K, 4, LANES>(T.xpt + x0, n, xw + 8 * (int64_t)x0, pot, cs_g, kc, lane, ga);
+      i = (lane & 3) >> 1;  // groups 0, 1 -> E row; 2, 3 -> H row
+    } else {
+      grid_rows<R, K, 8, LANES>(T.xpt + x0, n, xw + 8 * T.nxl + 24 * (x0 - T.nxl), pot, cs_g, kc, lane, ga);
+      i = ((lane & 7) + 2) >> 2;  // groups 0, 1 -> Eq. 3; 2 .. 5 -> Eq. 13; 6, 7 -> Eq. 14
+      if (lane < 5) {
+        const int g = T.gcol[5 * (r - nL) + lane];
+        if (g >= 0) {
+          const R s = gval[5 * (r - nL) + lane];
+#pragma unroll
+          for (int c = 0; c < K; ++c)
+            if (c < kc) axpy2(acc[2][c], s, x[c * ldx + nL + g]);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < K; ++c)
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (u == i) acc[u][c] += ga[c];
+  }
+  near_reduce<R, K, LANES>(acc);
+  if (r >= T.ne || lane >= kc) return;
   // lane c finishes column c
-  const int64_t v0 = ((int64_t)rtk[4 * r] * 3 + rtk[4 * r + 1]) * 4, v1 = ((int64_t)rtk[4 * r + 2] * 3 + rtk[4 * r + 3]) * 4;
-  const cx<R>* vc = val + lane * cs_val;
   cx<R>* yc = y + lane * ldy;
   cx<R> s[3];
 #pragma unroll
@@ -518,12 +589,67 @@ __global__ void __launch_bounds__(NM_THREADS)
 #pragma unroll
       for (int i = 0; i < 3; ++i) s[i] = acc[i][c];
   if (r < nL) {
-    yc[r] = s[0] + (vc[v0] + vc[v1]);
-    yc[nL + r] = s[1] + (vc[v0 + 1] + vc[v1 + 1]);
+    yc[r] = s[0];
+    yc[nL + r] = s[1];
   } else {
-    yc[nL + r] = s[0] + (vc[v0] + vc[v1]);
-    yc[nL + r + nR] = s[1] + (vc[v0 + 2] + vc[v1 + 2]);
-    yc[nL + r + 2 * nR] = s[2] + (vc[v0 + 3] + vc[v1 + 3]);
+    yc[nL + r] = s[0];
+    yc[nL + r + nR] = s[1];
+    yc[nL + r + 2 * nR] = s[2];
+  }
+}
+
+// The same for the transposed apply: x = near part (transposed matrix) +
+// projection transposed (the value blocks Q0 against the convolved adjoint
+// fields of J_e, M outside, J_i, M inside: groups 4 .. 7 of pot).
+template <typename R, int LANES>
+__global__ void __launch_bounds__(NM_THREADS)
+    k_rows_adj(RowTables T, const cx<R>* __restrict__ nmt, const R* __restrict__ gval, const R* __restrict__ xw,
+               const cx<R>* __restrict__ pot, const cx<R>* __restrict__ y, cx<R>* __restrict__ x) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
+  const int lane = threadIdx.x % LANES;
+  const int64_t nL = T.nL, nR = T.ne - nL;
+  cx<R> acc[3][1] = {{czero<R>()}, {czero<R>()}, {czero<R>()}};
+  if (r < T.ne) {
+    near_row<R, 1, true, LANES>(r, nL, nR, T.off, T.nl, T.col, T.vo, nmt, y, 0, 1, lane, acc);
+    const int x0 = T.xoff[r], n = T.xoff[r + 1] - x0;
+    const int stride = r < nL ? 8 : 24, grp = lane & 3;
+    const R* w = xw + (r < nL ? 8 * (int64_t)x0 : 8 * T.nxl + 24 * (x0 - T.nxl));
+    cx<R> ga = czero<R>();
+#pragma unroll 2
+    for (int j = lane >> 2; j < n; j += LANES / 4) {
+      R a[4];
+      cx<R> g[4];
+      load4(w + stride * j, a);
+      load_group(pot + (int64_t)T.xpt[x0 + j] * NPOT + 16 + 4 * grp, g);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) axpy2(ga, a[f], g[f]);
+    }
+    // groups J_e, M, J_i, -M; on plain edges J_i = -J_e
+    if (r < nL) {
+      if (grp == 0) acc[0][0] += ga;
+      if (grp == 2) acc[0][0] -= ga;
+      if (grp == 1) acc[1][0] += ga;
+      if (grp == 3) acc[1][0] -= ga;
+    } else {
+      if (grp == 0) acc[0][0] += ga;
+      if (grp == 2) acc[1][0] += ga;
+      if (grp == 1) acc[2][0] += ga;
+      if (grp == 3) acc[2][0] -= ga;
+      if (lane < 5) {
+        const int g = T.gcol[5 * (r - nL) + lane];
+        if (g >= 0) axpy2(acc[0][0], gval[5 * (r - nL) + lane], y[nL + g + 2 * nR]);
+      }
+    }
+  }
+  near_reduce<R, 1, LANES>(acc);
+  if (r >= T.ne || lane != 0) return;
+  if (r < nL) {
+    x[r] = acc[0][0];
+    x[nL + r] = acc[1][0];
+  } else {
+    x[nL + r] = acc[0][0];
+    x[nL + r + nR] = acc[1][0];
+    x[nL + r + 2 * nR] = acc[2][0];
   }
 }
 
@@ -538,21 +664,29 @@ PrecData<double>& pdata<double>(scabem_op* op) {
   return op->d;
 }
 
+RowTables row_tables(const scabem_op* op, const int64_t* vo) {
+  return {op->nm_off, op->nm_nl, op->nm_col, vo, op->nm_gcol, op->xoff, op->xpt, op->ne, op->nL, op->nxl};
+}
+// a warp per row; a whole CTA per row where warps would leave the chip idle
+// and the rows are long (77 columns per row on the 12 um guide)
+bool wide_rows(const scabem_op* op) { return op->ne < 152 * 32 && op->nm_nnz > 64 * op->ne; }
+
 template <typename R, int K>
 int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
-  k_near_rows<R, K><<<(unsigned)cdiv(op->ne * NM_LANES, NM_THREADS), NM_THREADS, 0, s>>>(
-      op->nm_off, op->nm_nl, op->nm_col, op->nm_vo, pd.nmv, op->nm_gcol, pd.gram, op->rtk, op->ne, op->nL, pd.val,
-      op->nt * 12, x, ldx, y, ldy, kc);
+  const bool wide = wide_rows(op);
+  auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
+  fn<<<(unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS), NM_THREADS, 0, s>>>(
+      row_tables(op, op->nm_vo), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }
 
 }  // namespace
 
-// y_c = near part of A x_c + the row sums of pd.val's column c, c < kc <= KBATCH
+// y_c = A x_c from the potentials pd.grid (column c) and the near matrix, c < kc <= KBATCH
 template <typename R>
-int near_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
+int rows_apply(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
   switch (kc) {
     case 1: return launch_rows<R, 1>(op, x, ldx, y, ldy, kc, s);
     case 2: return launch_rows<R, 2>(op, x, ldx, y, ldy, kc, s);
@@ -563,8 +697,22 @@ int near_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy,
     default: return launch_rows<R, 8>(op, x, ldx, y, ldy, kc, s);
   }
 }
-template int near_rows<float>(scabem_op*, const cx<float>*, int64_t, cx<float>*, int64_t, int, cudaStream_t);
-template int near_rows<double>(scabem_op*, const cx<double>*, int64_t, cx<double>*, int64_t, int, cudaStream_t);
+template int rows_apply<float>(scabem_op*, const cx<float>*, int64_t, cx<float>*, int64_t, int, cudaStream_t);
+template int rows_apply<double>(scabem_op*, const cx<double>*, int64_t, cx<double>*, int64_t, int, cudaStream_t);
+
+// x = A^T y from the convolved adjoint fields and the transposed near matrix
+template <typename R>
+int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s) {
+  PrecData<R>& pd = pdata<R>(op);
+  const bool wide = wide_rows(op);
+  auto fn = wide ? k_rows_adj<R, NM_THREADS> : k_rows_adj<R, 32>;
+  fn<<<(unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS), NM_THREADS, 0, s>>>(
+      row_tables(op, op->nm_vt), pd.nmt, pd.gram, pd.xw, pd.grid, y, x);
+  CK(cudaGetLastError());
+  return SCABEM_OK;
+}
+template int rows_adjoint<float>(scabem_op*, const cx<float>*, cx<float>*, cudaStream_t);
+template int rows_adjoint<double>(scabem_op*, const cx<double>*, cx<double>*, cudaStream_t);
 
 // Pattern and storage of the matrix (after the near list); its values follow
 // with the first conductivity.

@@ -521,33 +521,6 @@ __global__ void k_sigma_copy(const double* __restrict__ in, int64_t Q, double* _
   if (sf) sf[i] = (float)sig;
 }
 
-// Stencil weight W_slot(point) = Lx[i] Ly[j] Lz[k] of every projection entry
-// and its derivative weights (dLx Ly Lz, Lx dLy Lz, Lx Ly dLz: the
-// transposed interpolation of gradients and curls); the entry code
-// (point * p^3 + slot) is then replaced by the point index.
-__global__ void k_gather_weights(int32_t* __restrict__ gent, const double* __restrict__ L,
-                                 const double* __restrict__ dL, int64_t ne, int p, double* __restrict__ wd,
-                                 float* __restrict__ wf, double* __restrict__ gdd, float* __restrict__ gdf) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= ne) return;
-  const int p2 = p * p, p3 = p2 * p;
-  const int code = gent[e];
-  const int64_t Qi = code / p3;
-  const int sl = code - (int)Qi * p3;
-  const int i = sl / p2, j = (sl - i * p2) / p, k = sl - i * p2 - j * p;
-  const double lx = L[(3 * Qi + 0) * p + i], ly = L[(3 * Qi + 1) * p + j], lz = L[(3 * Qi + 2) * p + k];
-  const double W = lx * ly * lz;
-  wd[e] = W;
-  wf[e] = (float)W;
-  const double D[3] = {dL[(3 * Qi + 0) * p + i] * ly * lz, lx * dL[(3 * Qi + 1) * p + j] * lz,
-                       lx * ly * dL[(3 * Qi + 2) * p + k]};
-  for (int c = 0; c < 3; ++c) {
-    gdd[3 * e + c] = D[c];
-    gdf[3 * e + c] = (float)D[c];
-  }
-  gent[e] = (int32_t)Qi;
-}
-
 // ---------------------------------------------------------------- block-diagonal preconditioner
 using cd = cx<double>;
 
@@ -800,9 +773,8 @@ __global__ void k_precond_apply(const cd* __restrict__ pinv, const int32_t* __re
 
 }  // namespace
 
-// Inverse of the projection stencil map: for every grid point, the list of
-// (quadrature point, stencil slot) pairs whose stencil covers it, in point
-// order (a counting sort on the host over the device-computed stencil bases).
+// The grid points that some projection stencil covers (their number), and the
+// active columns and rows of the (i1, i2) cross-section.
 int setup_gather(scabem_op* op, cudaStream_t s) {
   const int p = op->p, p3 = p * p * p;
   const int64_t Q = op->Q;
@@ -815,39 +787,32 @@ int setup_gather(scabem_op* op, cudaStream_t s) {
   CK(cudaMemcpyAsync(base.data(), op->base, sizeof(int32_t) * 3 * Q, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   const int n1 = op->n[1], n2 = op->n[2];
-  std::vector<int32_t> off(ng + 1, 0), ent(Q * p3);
-  auto grid_index = [&](int64_t qi, int sl) {
-    const int i = sl / (p * p), j = (sl / p) % p, k = sl % p;
-    return ((int64_t)(base[3 * qi] + i) * n1 + (base[3 * qi + 1] + j)) * n2 + (base[3 * qi + 2] + k);
-  };
-  for (int64_t qi = 0; qi < Q; ++qi)
-    for (int sl = 0; sl < p3; ++sl) ++off[grid_index(qi, sl) + 1];
-  for (int64_t g = 0; g < ng; ++g) off[g + 1] += off[g];
-  std::vector<int32_t> cur(off.begin(), off.end() - 1);
-  for (int64_t qi = 0; qi < Q; ++qi)
-    for (int sl = 0; sl < p3; ++sl) ent[cur[grid_index(qi, sl)]++] = (int32_t)(qi * p3 + sl);
-  // compact to the grid points that some stencil covers
-  std::vector<int32_t> pts, coff;
-  coff.push_back(0);
-  for (int64_t g = 0; g < ng; ++g)
-    if (off[g + 1] > off[g]) {
-      pts.push_back((int32_t)g);
-      coff.push_back(off[g + 1]);
-    }
-  op->ngnz = (int64_t)pts.size();
-  // active columns and rows of the (i1, i2) cross-section
   const int64_t C = (int64_t)n1 * n2;
-  std::vector<char> colact(C, 0);
-  for (int32_t g : pts) colact[g % C] = 1;
-  std::vector<int32_t> acol;
+  std::vector<char> cov(ng, 0), colact(C, 0);
+  for (int64_t qi = 0; qi < Q; ++qi)
+    for (int i = 0; i < p; ++i)
+      for (int j = 0; j < p; ++j) {
+        const int64_t g = ((int64_t)(base[3 * qi] + i) * n1 + (base[3 * qi + 1] + j)) * n2 + base[3 * qi + 2];
+        for (int k = 0; k < p; ++k) cov[g + k] = 1;
+      }
+  op->ngnz = 0;
+  for (int64_t g = 0; g < ng; ++g)
+    if (cov[g]) {
+      ++op->ngnz;
+      colact[g % C] = 1;
+    }
+  std::vector<int32_t> acol, cmap(C, -1);
   op->rowmask = 0;
   for (int64_t c = 0; c < C; ++c)
     if (colact[c]) {
+      cmap[c] = (int32_t)acol.size();
       acol.push_back((int32_t)c);
       if (c / n2 < 64) op->rowmask |= 1ull << (c / n2);  // read only by the 64 x 64 plane kernel
     }
   op->nac = (int64_t)acol.size();
   if (op->nac > 0) {
+    CK(cudaMalloc(&op->cmap, sizeof(int32_t) * C));
+    CK(cudaMemcpyAsync(op->cmap, cmap.data(), sizeof(int32_t) * C, cudaMemcpyHostToDevice, s));
     CK(cudaMalloc(&op->acol, sizeof(int32_t) * op->nac));
     CK(cudaMemcpyAsync(op->acol, acol.data(), sizeof(int32_t) * op->nac, cudaMemcpyHostToDevice, s));
     // bounding box of the active columns and their coordinates in it
@@ -884,20 +849,6 @@ int setup_gather(scabem_op* op, cudaStream_t s) {
       return SCABEM_E_ARG;
     }
   }
-  const int64_t ne = Q * p3;
-  CK(cudaMalloc(&op->gpt, sizeof(int32_t) * (pts.size() + 1)));
-  CK(cudaMalloc(&op->goff, sizeof(int32_t) * coff.size()));
-  CK(cudaMalloc(&op->gent, sizeof(int32_t) * ne));
-  CK(cudaMalloc(&op->gwd, sizeof(double) * ne));
-  CK(cudaMalloc(&op->gwf, sizeof(float) * ne));
-  CK(cudaMalloc(&op->gdd, sizeof(double) * 3 * ne));
-  CK(cudaMalloc(&op->gdf, sizeof(float) * 3 * ne));
-  CK(cudaMemcpyAsync(op->gpt, pts.data(), sizeof(int32_t) * pts.size(), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(op->goff, coff.data(), sizeof(int32_t) * coff.size(), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(op->gent, ent.data(), sizeof(int32_t) * ne, cudaMemcpyHostToDevice, s));
-  k_gather_weights<<<(int)cdiv(ne, 256), 256, 0, s>>>(op->gent, op->d.L, op->d.dL, ne, p, op->gwd, op->gwf,
-                                                      op->gdd, op->gdf);
-  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return SCABEM_OK;
 }
@@ -1057,16 +1008,13 @@ int setup_near(scabem_op* op, cudaStream_t s) {
       return SCABEM_E_NOMEM;
     }
   }
-  if (op->prec_mask & 1) {
+  if (!(op->prec_mask & 2)) {  // the FP64 records serve both precisions
     cudaError_t e = cudaMalloc(&op->f.near, sizeof(cx<float>) * (nrec > 0 ? nrec : 1));
     if (e != cudaSuccess) {
       set_error("out of device memory for the near-field data");
       return SCABEM_E_NOMEM;
     }
   }
-  // per-pair buffer of the transposed near field
-  if (acc > 0 && op->f.built) CK(cudaMalloc(&op->f.nadj, sizeof(cx<float>) * acc * 12));
-  if (acc > 0 && op->d.built) CK(cudaMalloc(&op->d.nadj, sizeof(cx<double>) * acc * 12));
   const int64_t work = acc * op->q;
   if (work > 0) {
     k_near_corr<double><<<(int)cdiv(work, 128), 128, 0, s>>>(
@@ -1079,20 +1027,6 @@ int setup_near(scabem_op* op, cudaStream_t s) {
   for (int med = 0; med < 2; ++med) {
     cudaFree(op->gspatial[med]);
     op->gspatial[med] = nullptr;
-  }
-  // reverse list for the transposed near field: the pairs of each source
-  // triangle, ascending pair index
-  if (acc > 0) {
-    std::vector<int32_t> hs(acc), rc(nt + 1, 0), rp(acc);
-    CK(cudaMemcpy(hs.data(), op->nsrc, sizeof(int32_t) * acc, cudaMemcpyDeviceToHost));
-    for (int64_t j = 0; j < acc; ++j) ++rc[hs[j] + 1];
-    for (int64_t t = 0; t < nt; ++t) rc[t + 1] += rc[t];
-    std::vector<int32_t> cur(rc.begin(), rc.end() - 1);
-    for (int64_t j = 0; j < acc; ++j) rp[cur[hs[j]]++] = (int32_t)j;
-    CK(cudaMalloc(&op->roff, sizeof(int32_t) * (nt + 1)));
-    CK(cudaMalloc(&op->rpair, sizeof(int32_t) * acc));
-    CK(cudaMemcpy(op->roff, rc.data(), sizeof(int32_t) * (nt + 1), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(op->rpair, rp.data(), sizeof(int32_t) * acc, cudaMemcpyHostToDevice));
   }
   return SCABEM_OK;
 }
@@ -1107,7 +1041,7 @@ int setup_sigma_monomial(scabem_op* op, int nseg, const double* seg, cudaStream_
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   if (dseg) cudaFree(dseg);
-  if (int rc = moments_update(op, s)) return rc;
+  if (int rc = stencils_update(op, s)) return rc;
   if (int rc = near_matrix_update(op, s)) return rc;
   return setup_precond(op, s);  // the absorber blocks depend on sigma
 }
@@ -1121,7 +1055,7 @@ int setup_sigma_bspline(scabem_op* op, double x0, double L, int axis, int ncoef,
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   cudaFree(dc);
-  if (int rc = moments_update(op, s)) return rc;
+  if (int rc = stencils_update(op, s)) return rc;
   if (int rc = near_matrix_update(op, s)) return rc;
   return setup_precond(op, s);
 }
@@ -1134,7 +1068,7 @@ int setup_sigma_values(scabem_op* op, const double* per_q_host, cudaStream_t s) 
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   cudaFree(tmp);
-  if (int rc = moments_update(op, s)) return rc;
+  if (int rc = stencils_update(op, s)) return rc;
   if (int rc = near_matrix_update(op, s)) return rc;
   return setup_precond(op, s);
 }
