@@ -788,6 +788,8 @@ void scabem_op_destroy(scabem_op_t op) {
   cudaFree(op->gpl);
   cudaFree(op->gpr);
   cudaFree(op->gpe);
+  cudaFree(op->rdesc);
+  cudaFree(op->rdesc_t);
   cudaFree(op->nm_off);
   cudaFree(op->nm_nl);
   cudaFree(op->nm_col);
@@ -1145,8 +1147,8 @@ int autotune_prec(scabem_op* op, int nrhs, cudaStream_t s, double* out) {
       if (direct ? !op->direct_fits : !op->planes_fit) continue;
       if ((rc = set_transverse_mode(op, direct, s))) break;
       for (int L = 1; L <= 16 && !rc; L *= 2) {
-        const int cbC = L >= 4 ? L : 4;
-        if ((1 << lp) * L > (1 << totl) || (1 << lp) * cbC > (1 << totl) ||
+        const int cbC = L >= 8 ? L : 8;
+        if ((1 << lp) * L > (1 << totl) || (1 << lp) * cbC > (1 << 13) ||
             (int64_t)op->P[0] * (L + 1) * csz > 227 * 1024 || (int64_t)op->P[0] * (cbC + 1) * csz > 227 * 1024)
           continue;
         op->a0_lines = L;

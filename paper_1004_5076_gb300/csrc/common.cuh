@@ -246,6 +246,9 @@ struct scabem_op {
   int64_t* nm_vo = nullptr;
   int64_t* nm_vt = nullptr;
   int32_t* nm_gcol = nullptr;  // nR * 5 columns of gram, -1 past the last
+  void* rdesc = nullptr;       // ne row descriptors of the rows kernels (near.cu)
+  void* rdesc_t = nullptr;     // the same for the transposed matrix
+  std::vector<int32_t> h_xoff;  // xoff on the host, during set-up
   bool nm_ready = false;       // values formed for all rows
   cx<double>* gspatial[2] = {nullptr, nullptr};  // padded G tables, set-up only
   // per-edge block-diagonal preconditioner (exact self blocks, inverted)

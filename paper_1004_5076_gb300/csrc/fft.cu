@@ -17,12 +17,9 @@
 // butterflies into registers, synchronises, and stores them at their sorted
 // positions.  One CTA owns whole lines, so each field makes one HBM round trip
 // per stage.  The 1/(P0 P1 P2) scale is folded into the stored spectra.
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace {
 
@@ -212,20 +209,19 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__
 // Stage C with point-major output, on the nac active columns only (the
 // potentials are read nowhere else; the input holds Cin columns per (field,
 // k0), compact or whole planes as stage A wrote them): one CTA owns NC of them
-// for one group of 4 fields over axis 0 (line l = field * NC + column) and
-// writes out[(i0 * nac + column) * 32 + 4 * group + f] for i0 < n_out, whole
-// 32-byte sectors in complex64.
+// for the eight fields of one set (J: A, phi of both media; M: F, psi of both)
+// over axis 0, line l = field * NC + column, and writes groups of four complex
+// values, whole 32-byte sectors in complex64, at out[(i0 * nac + column) * 32]
+// for i0 < n_out.
 //
-// The groups are what the rows read (near.cu).  Groups 4 .. 7: the four sets'
-// potentials, [A, phi] scaled by j z k and j z / k (the strong-form E of
-// Eqs. 13, 14) and [F, 0], of the exterior and the interior medium.  Groups 0 ..
-// 3: the weak-form differences of the two media, E from [A, phi] and [F], H from
-// [F, psi] and [A], which halve the products of the testing.  The CTAs of the
-// two media exchange their lines through distributed shared memory (a cluster
-// of the four groups).  COMB = false (transposed apply): the fields themselves in
-// groups 4 .. 7.
-template <typename R, bool COMB>
-__global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FFT_THREADS)
+// The groups are what the rows read (near.cu).  Groups 4 .. 7 (exterior J, M,
+// interior J, M): [A, phi] scaled by j z k and j z / k (the strong-form E of
+// Eqs. 13, 14) and [F, 0].  Groups 0 .. 3: the weak-form differences of the two
+// media, E from [A, phi] and from [F], H from [F, psi] and from [A], which
+// halve the products of the testing; a set's two media meet in its CTA.
+// COMB = false (transposed apply): the fields themselves in groups 4 .. 7.
+template <typename R, bool COMB, int TOTL>
+__global__ void __launch_bounds__(FFT_THREADS)
     k_axis0_pm(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, int n_out, int P0,
                const int32_t* __restrict__ acol, int nac, int NC, const cx<R>* __restrict__ tw, int64_t cs_in,
                int64_t cs_out, int64_t Cin, int compact, R ke, R ki, R ze, R zi) {
@@ -234,63 +230,42 @@ __global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FFT_THREADS)
   cx<R>* b0 = tws + P0;
   in += blockIdx.z * cs_in;  // right-hand side blockIdx.z
   out += blockIdx.z * cs_out;
-  const int grp = blockIdx.y;
+  const int set = blockIdx.y;
   const int a0 = blockIdx.x * NC;
-  const int CB = 4 * NC;
+  const int CB = 8 * NC;
   const int lcb = ilog2(CB), lnc = ilog2(NC);
   for (int i = threadIdx.x; i < P0; i += FFT_THREADS) tws[i] = tw[i];
   for (int idx = threadIdx.x; idx < P0 * CB; idx += FFT_THREADS) {
     const int i0 = idx >> lcb, l = idx & (CB - 1);
     const int fl = l >> lnc, cl = l & (NC - 1);
+    const int field = (fl & 3) + 4 * set + 2 * (fl & 4);
     cx<R> v = czero<R>();
-    if (a0 + cl < nac) v = in[((int64_t)(4 * grp + fl) * P0 + i0) * Cin + (compact ? a0 + cl : acol[a0 + cl])];
+    if (a0 + cl < nac) v = in[((int64_t)field * P0 + i0) * Cin + (compact ? a0 + cl : acol[a0 + cl])];
     b0[idx] = v;
   }
   __syncthreads();
-  fft_lines<R, 1, Tot<R>::L>(b0, ilog2(P0), lcb, 1, CB, tws);
-  if constexpr (!COMB) {
-    for (int idx = threadIdx.x; idx < n_out * CB; idx += FFT_THREADS) {
-      const int k0 = idx >> lcb, l = idx & (CB - 1);
-      const int cl = l >> 2, fl = l & 3;  // field fastest: consecutive threads fill a sector
-      if (a0 + cl < nac)
-        out[((int64_t)k0 * nac + a0 + cl) * NPOT + 16 + 4 * grp + fl] = b0[(k0 << lcb) + fl * NC + cl];
+  fft_lines<R, 1, TOTL>(b0, ilog2(P0), lcb, 1, CB, tws);
+  const R wE = ze * ke, wI = zi * ki, pE = ze / ke, pI = zi / ki, yE = ke / ze, yI = ki / zi;
+  const R qE = R(1) / (ke * ze), qI = R(1) / (ki * zi);
+  for (int idx = threadIdx.x; idx < 4 * n_out * NC; idx += FFT_THREADS) {
+    const int fl = idx & 3, cl = (idx >> 2) & (NC - 1), k0 = idx >> (2 + lnc);  // component fastest: whole sectors
+    if (a0 + cl >= nac) continue;
+    const cx<R> e = b0[(k0 << lcb) + fl * NC + cl], i = b0[(k0 << lcb) + (fl + 4) * NC + cl];
+    cx<R>* o = out + ((int64_t)k0 * nac + a0 + cl) * NPOT + fl;
+    if (!COMB) {
+      o[16 + 4 * set] = e;
+      o[24 + 4 * set] = i;
+    } else if (set == 0) {  // A, phi
+      o[0] = fl < 3 ? mulj(wI * i - wE * e) : mulj(pE * e - pI * i);
+      o[12] = fl < 3 ? e - i : czero<R>();
+      o[16] = mulj((fl < 3 ? wE : pE) * e);
+      o[24] = mulj((fl < 3 ? wI : pI) * i);
+    } else {  // F, psi (the interior M set carries its sign)
+      o[4] = fl < 3 ? i - e : czero<R>();
+      o[8] = fl < 3 ? mulj(yI * i - yE * e) : mulj(qE * e - qI * i);
+      o[20] = fl < 3 ? e : czero<R>();
+      o[28] = fl < 3 ? i : czero<R>();
     }
-  } else {
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();
-    const cx<R>* rb = cluster.map_shared_rank(b0, grp ^ 2);  // the same set in the other medium
-    const bool isM = grp & 1, inner = grp & 2;
-    const R k = inner ? ki : ke, z = inner ? zi : ze, ko = inner ? ke : ki, zo = inner ? ze : zi;
-    const R sg = inner ? R(-1) : R(1);  // weak-form rows take exterior - interior
-    // group 0 (rank 0): E from A, phi   group 1 (rank 1): E from F
-    // group 2 (rank 3): H from F, psi   group 3 (rank 2): H from A
-    const int og = grp == 0 ? 0 : grp == 1 ? 1 : grp == 3 ? 2 : 3;
-    for (int idx = threadIdx.x; idx < n_out * CB; idx += FFT_THREADS) {
-      const int k0 = idx >> lcb, l = idx & (CB - 1);
-      const int cl = l >> 2, fl = l & 3;
-      if (a0 + cl >= nac) continue;
-      const int at = (k0 << lcb) + fl * NC + cl;
-      const cx<R> v = b0[at], w = rb[at];
-      cx<R> weak, own;
-      if (!isM) {
-        own = mulj((fl < 3 ? z * k : z / k) * v);
-        if (og == 0)
-          weak = fl < 3 ? mulj((zo * ko) * w - (z * k) * v) : mulj((z / k) * v - (zo / ko) * w);
-        else
-          weak = fl < 3 ? w - v : czero<R>();
-      } else {
-        own = fl < 3 ? v : czero<R>();
-        if (og == 1)
-          weak = fl < 3 ? w - v : czero<R>();
-        else
-          weak = fl < 3 ? mulj((k / z) * v - (ko / zo) * w)
-                        : mulj((R(1) / (ko * zo)) * w + (sg / (k * z)) * v);
-      }
-      cx<R>* o = out + ((int64_t)k0 * nac + a0 + cl) * NPOT + fl;
-      o[4 * og] = weak;
-      o[16 + 4 * grp] = own;
-    }
-    cluster.sync();  // no CTA leaves while another still reads its lines
   }
 }
 
@@ -863,24 +838,31 @@ int fft3d_full(scabem_op* op, cx<R>* data, const cx<R>* const tw[3], int dir, cu
   return SCABEM_OK;
 }
 
-// Lines per CTA of the pruned axis-0 stages: at most 8, so that the few
-// active columns still spread over the SMs.
+// Lines per CTA of the pruned axis-0 stages for `units` lines (field, column):
+// 8, so that the few active columns of a long guide still spread over the
+// SMs; more for short transforms, up to the eight elements per thread that
+// the radix-8 passes take, while a CTA per SM remains (a 64-point transform
+// of 8 lines keeps 64 of 512 threads busy).
 template <typename R>
-int pruned_lines(int P0) {
-  const int l = lines_per_cta<R>(P0);
-  return l < 8 ? l : 8;
+int pruned_lines(int P0, int64_t units) {
+  int l = lines_per_cta<R>(P0);
+  l = l < 8 ? l : 8;
+  while (P0 * l < 8 * FFT_THREADS && units / (2 * l) >= 152) l *= 2;
+  return l;
 }
 
 // stage C: 16 fields [field][k0][c] -> point-major groups, active columns
 template <typename R>
 static int axis0_inverse(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int ncol) {
   const int P0 = op->P[0];
-  const int lines = op->a0_lines > 0 ? op->a0_lines : pruned_lines<R>(P0);
-  const int nc = lines >= 4 ? lines / 4 : 1;  // P0 <= 1024: 4 lines fit
-  const size_t sm = (size_t)P0 * (4 * nc + 1) * sizeof(cx<R>);
-  auto fn = adjoint ? k_axis0_pm<R, false> : k_axis0_pm<R, true>;
+  const int lines = op->a0_lines > 0 ? op->a0_lines : pruned_lines<R>(P0, 16 * op->nac * ncol);
+  const int nc = lines >= 8 ? lines / 8 : 1;  // eight lines of P0 <= 1024 always fit
+  const size_t sm = (size_t)P0 * (8 * nc + 1) * sizeof(cx<R>);
+  const bool big = P0 * 8 * nc > (1 << Tot<R>::L);
+  auto fn = big ? (adjoint ? k_axis0_pm<R, false, 13> : k_axis0_pm<R, true, 13>)
+                : (adjoint ? k_axis0_pm<R, false, Tot<R>::L> : k_axis0_pm<R, true, Tot<R>::L>);
   if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
-  fn<<<dim3((unsigned)cdiv(op->nac, nc), NFIELD_OUT / 4, ncol), FFT_THREADS, sm, s>>>(
+  fn<<<dim3((unsigned)cdiv(op->nac, nc), 2, ncol), FFT_THREADS, sm, s>>>(
       pd.stB, pd.grid, op->n[0], P0, op->acol, (int)op->nac, nc, pd.tw[0], col_stride_st(op), col_stride_pot(op), op->cst,
       op->tdirect ? 1 : 0, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi);
   CK(cudaGetLastError());
@@ -897,7 +879,7 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
     set_error("grid: no grid point is covered by a stencil");
     return SCABEM_E_ARG;
   }
-  const int cb = op->a0_lines > 0 ? op->a0_lines : pruned_lines<R>(P0);
+  const int cb = op->a0_lines > 0 ? op->a0_lines : pruned_lines<R>(P0, nf * op->nac * ncol);
   const size_t sm0 = (size_t)P0 * (cb + 1) * sizeof(cx<R>);
   // stage A
   if (int rc_ = set_max_smem(op->device, (const void*)k_axis0<R>, (int)sm0)) return rc_;

@@ -113,6 +113,27 @@ __global__ void __launch_bounds__(128) k_near_pattern(const int32_t* __restrict_
   }
 }
 
+// Sorts each class segment of a row's columns by edge number, one warp per row
+// (rank by counting): neighbouring lanes of the products then gather from
+// neighbouring unknowns.  Segments longer than NM_SORT stay as they are.
+constexpr int NM_SORT = 1024;
+__global__ void __launch_bounds__(128) k_near_sort(const int32_t* __restrict__ off, const int32_t* __restrict__ nl,
+                                                   int64_t ne, const int32_t* __restrict__ in,
+                                                   int32_t* __restrict__ out) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (r >= ne) return;
+  for (int seg = 0; seg < 2; ++seg) {
+    const int b = off[r] + (seg ? nl[r] : 0), n = (seg ? off[r + 1] : off[r] + nl[r]) - b;
+    for (int j = threadIdx.x & 31; j < n; j += 32) {
+      const int m = in[b + j];
+      int rank = n > NM_SORT ? j : 0;
+      if (n <= NM_SORT)
+        for (int k = 0; k < n; ++k) rank += in[b + k] < m;
+      out[b + rank] = m;
+    }
+  }
+}
+
 // tpos[i] = position of row r among the columns of row m = col[i] (the
 // pattern is symmetric), one warp per row r
 __global__ void __launch_bounds__(128) k_near_tpos(const int32_t* __restrict__ off, const int32_t* __restrict__ nl,
@@ -322,34 +343,35 @@ __global__ void k_near_gram(const int32_t* __restrict__ rtk, const int32_t* __re
 }
 
 // ---------------------------------------------------------------- products
-// f(m, v) for the columns m = col[j] with values v[e] = val[e n + j], j = lane,
-// lane + LANES, ..: the next column's loads are issued before the current
-// column's dependent gathers of x, so two columns per lane are in flight.
+// f(m, v) for the columns m = col[j] of one segment of a row, with values v[e]
+// = val[e n + j], j = lane, lane + LANES, ..: the next column's values and the
+// index after it are loaded before the current column's gathers of x.
 template <typename R, int W, int LANES, class F>
 __device__ __forceinline__ void near_segment(const int32_t* __restrict__ col, const cx<R>* __restrict__ val, int n,
                                              int lane, const F& f) {
-  int j = lane, m = 0;
+  int j = lane;
+  if (j >= n) return;
+  int m = col[j], mn = j + LANES < n ? col[j + LANES] : 0;
   cx<R> v[W];
-  if (j < n) {
-    m = col[j];
 #pragma unroll
-    for (int e = 0; e < W; ++e) v[e] = ldstream(val + (int64_t)e * n + j);
-  }
-  while (j < n) {
+  for (int e = 0; e < W; ++e) v[e] = ldstream(val + (int64_t)e * n + j);
+  while (true) {
     const int jn = j + LANES;
-    int mn = 0;
+    const bool more = jn < n;
     cx<R> vn[W];
-    if (jn < n) {
-      mn = col[jn];
+    int m2 = 0;
+    if (more) {
+      if (jn + LANES < n) m2 = col[jn + LANES];
 #pragma unroll
       for (int e = 0; e < W; ++e) vn[e] = ldstream(val + (int64_t)e * n + jn);
     }
     f(m, v);
+    if (!more) break;
     j = jn;
     m = mn;
-    if (jn < n)
+    mn = m2;
 #pragma unroll
-      for (int e = 0; e < W; ++e) v[e] = vn[e];
+    for (int e = 0; e < W; ++e) v[e] = vn[e];
   }
 }
 
@@ -360,102 +382,87 @@ __device__ __forceinline__ void near_segment(const int32_t* __restrict__ col, co
 // (plain) or nL + m, nL + m + nR, nL + m + 2 nR (absorber).
 constexpr int NM_THREADS = 128;
 
+// Where a row's data lie: near columns off .. off + cnt (nl plain ones), near
+// values from vo, stencil entries xoff .. xoff + nx.
+struct __align__(16) RowDesc {
+  int32_t off, nl, cnt, xoff;
+  int64_t vo;
+  int32_t nx, pad;
+};
+__device__ __forceinline__ RowDesc load_desc(const RowDesc* p) {
+  const int4 a = __ldg(reinterpret_cast<const int4*>(p)), b = __ldg(reinterpret_cast<const int4*>(p) + 1);
+  RowDesc d;
+  d.off = a.x;
+  d.nl = a.y;
+  d.cnt = a.z;
+  d.xoff = a.w;
+  d.vo = (int64_t)(((uint64_t)(uint32_t)b.y << 32) | (uint32_t)b.x);
+  d.nx = b.z;
+  d.pad = 0;
+  return d;
+}
+
 template <typename R, int K, bool T, int LANES>
-__device__ __forceinline__ void near_row(int64_t r, int64_t nL, int64_t nR, const int32_t* __restrict__ off,
-                                         const int32_t* __restrict__ nl, const int32_t* __restrict__ col,
-                                         const int64_t* __restrict__ vo, const cx<R>* __restrict__ val,
+__device__ __forceinline__ void near_row(const RowDesc& D, bool isR, int64_t nL, int64_t nR,
+                                         const int32_t* __restrict__ col, const cx<R>* __restrict__ val,
                                          const cx<R>* __restrict__ x, int64_t ldx, int kc, int lane, cx<R> acc[3][K]) {
-  const int c0 = off[r], cl = nl[r], cr = off[r + 1] - c0 - cl;
-  const cx<R>* v0 = val + vo[r];
-  const int32_t *colL = col + c0, *colR = colL + cl;
-  if (r < nL) {
+  const int cl = D.nl, cr = D.cnt - cl;
+  const cx<R>* v0 = val + D.vo;
+  const int32_t *colL = col + D.off, *colR = colL + cl;
+  const cx<R>* xR = x + nL;
+  // the entries of x of column m: J, M of a plain edge; J_e, J_i, M of an absorber edge
+#define COLUMNS2(...)                                                 \
+  _Pragma("unroll") for (int c = 0; c < K; ++c) if (c < kc) {         \
+    const cx<R> a = x[c * ldx + m], b = x[c * ldx + m + nL];          \
+    __VA_ARGS__                                                       \
+  }
+#define COLUMNS3(...)                                                                                       \
+  _Pragma("unroll") for (int c = 0; c < K; ++c) if (c < kc) {                                               \
+    const cx<R> a = xR[c * ldx + m], b = xR[c * ldx + m + nR], d = xR[c * ldx + m + 2 * nR];                \
+    __VA_ARGS__                                                                                             \
+  }
+  if (!isR) {
     near_segment<R, 3, LANES>(colL, v0, cl, lane, [&](int m, const cx<R>* v) {
-      const cx<R>* xm = x + m;
-#pragma unroll
-      for (int c = 0; c < K; ++c)
-        if (c < kc) {  // U G V
-          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nL];
-          cmac(acc[0][c], v[0], a);
-          cmac(acc[0][c], T ? v[1] : -v[1], b);
-          cmac(acc[1][c], T ? -v[1] : v[1], a);
-          cmac(acc[1][c], v[2], b);
-        }
+      COLUMNS2(  // U G V
+          cmac(acc[0][c], v[0], a); cmac(acc[0][c], T ? v[1] : -v[1], b); cmac(acc[1][c], T ? -v[1] : v[1], a);
+          cmac(acc[1][c], v[2], b);)
     });
     near_segment<R, T ? 6 : 5, LANES>(colR, v0 + (int64_t)nm_words(false, false) * cl, cr, lane,
-                                      [&](int m, const cx<R>* v) {
-      const cx<R>* xm = x + nL + m;
-#pragma unroll
-      for (int c = 0; c < K; ++c)
-        if (c < kc) {
-          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nR], d = xm[c * ldx + 2 * nR];
-          if constexpr (!T) {  // Ue Ui ge gi V
-            cmac(acc[0][c], v[0], a);
-            cmac(acc[0][c], -v[1], b);
-            cmac(acc[0][c], -(v[2] + v[3]), d);
-            cmac(acc[1][c], v[2], a);
-            cmac(acc[1][c], -v[3], b);
-            cmac(acc[1][c], v[4], d);
-          } else {  // U G G13 V13 P Q against the rows of Eqs. 3, 13, 14
-            cmac(acc[0][c], v[0], a);
-            cmac(acc[0][c], v[2], b);
-            cmac(acc[0][c], v[4], d);
-            cmac(acc[1][c], -v[1], a);
-            cmac(acc[1][c], v[3], b);
-            cmac(acc[1][c], v[5], d);
-          }
-        }
+                                            [&](int m, const cx<R>* v) {
+      if constexpr (!T) {  // Ue Ui ge gi V
+        COLUMNS3(cmac(acc[0][c], v[0], a); cmac(acc[0][c], -v[1], b); cmac(acc[0][c], -(v[2] + v[3]), d);
+                 cmac(acc[1][c], v[2], a); cmac(acc[1][c], -v[3], b); cmac(acc[1][c], v[4], d);)
+      } else {  // U G G13 V13 P Q against the rows of Eqs. 3, 13, 14
+        COLUMNS3(cmac(acc[0][c], v[0], a); cmac(acc[0][c], v[2], b); cmac(acc[0][c], v[4], d);
+                 cmac(acc[1][c], -v[1], a); cmac(acc[1][c], v[3], b); cmac(acc[1][c], v[5], d);)
+      }
     });
   } else {
-    near_segment<R, T ? 5 : 6, LANES>(colL, v0, cl, lane, [&](int m, const cx<R>* v) {
-      const cx<R>* xm = x + m;
-#pragma unroll
-      for (int c = 0; c < K; ++c)
-        if (c < kc) {
-          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nL];
-          if constexpr (!T) {  // U G G13 V13 P Q
-            cmac(acc[0][c], v[0], a);
-            cmac(acc[0][c], -v[1], b);
-            cmac(acc[1][c], v[2], a);
-            cmac(acc[1][c], v[3], b);
-            cmac(acc[2][c], v[4], a);
-            cmac(acc[2][c], v[5], b);
-          } else {  // Ue Ui ge gi V
-            cmac(acc[0][c], v[0], a);
-            cmac(acc[0][c], v[2], b);
-            cmac(acc[1][c], -v[1], a);
-            cmac(acc[1][c], -v[3], b);
-            cmac(acc[2][c], -(v[2] + v[3]), a);
-            cmac(acc[2][c], v[4], b);
-          }
-        }
+    near_segment<R, T ? 5 : 6, LANES>(colL, v0, cl, lane,
+                                            [&](int m, const cx<R>* v) {
+      if constexpr (!T) {  // U G G13 V13 P Q
+        COLUMNS2(cmac(acc[0][c], v[0], a); cmac(acc[0][c], -v[1], b); cmac(acc[1][c], v[2], a);
+                cmac(acc[1][c], v[3], b); cmac(acc[2][c], v[4], a); cmac(acc[2][c], v[5], b);)
+      } else {  // Ue Ui ge gi V
+        COLUMNS2(cmac(acc[0][c], v[0], a); cmac(acc[0][c], v[2], b); cmac(acc[1][c], -v[1], a);
+                cmac(acc[1][c], -v[3], b); cmac(acc[2][c], -(v[2] + v[3]), a); cmac(acc[2][c], v[4], b);)
+      }
     });
-    near_segment<R, 8, LANES>(colR, v0 + (int64_t)(T ? 5 : 6) * cl, cr, lane, [&](int m, const cx<R>* v) {
-      const cx<R>* xm = x + nL + m;
-#pragma unroll
-      for (int c = 0; c < K; ++c)
-        if (c < kc) {  // Ue Ui e13 i13 G V13 P Q
-          const cx<R> a = xm[c * ldx], b = xm[c * ldx + nR], d = xm[c * ldx + 2 * nR];
-          cmac(acc[0][c], v[0], a);
-          if constexpr (!T) {
-            cmac(acc[0][c], -v[1], b);
-            cmac(acc[0][c], -v[4], d);
-            cmac(acc[1][c], v[2], a);
-            cmac(acc[1][c], v[3], b);
-            cmac(acc[1][c], v[5], d);
-            cmac(acc[2][c], v[6], b);
-            cmac(acc[2][c], v[7], d);
-          } else {
-            cmac(acc[0][c], v[2], b);
-            cmac(acc[1][c], -v[1], a);
-            cmac(acc[1][c], v[3], b);
-            cmac(acc[1][c], v[6], d);
-            cmac(acc[2][c], -v[4], a);
-            cmac(acc[2][c], v[5], b);
-            cmac(acc[2][c], v[7], d);
-          }
-        }
+    near_segment<R, 8, LANES>(colR, v0 + (int64_t)(T ? 5 : 6) * cl, cr, lane,
+                                    [&](int m, const cx<R>* v) {
+      if constexpr (!T) {  // Ue Ui e13 i13 G V13 P Q
+        COLUMNS3(cmac(acc[0][c], v[0], a); cmac(acc[0][c], -v[1], b); cmac(acc[0][c], -v[4], d);
+                 cmac(acc[1][c], v[2], a); cmac(acc[1][c], v[3], b); cmac(acc[1][c], v[5], d);
+                 cmac(acc[2][c], v[6], b); cmac(acc[2][c], v[7], d);)
+      } else {
+        COLUMNS3(cmac(acc[0][c], v[0], a); cmac(acc[0][c], v[2], b); cmac(acc[1][c], -v[1], a);
+                 cmac(acc[1][c], v[3], b); cmac(acc[1][c], v[6], d); cmac(acc[2][c], -v[4], a);
+                 cmac(acc[2][c], v[5], b); cmac(acc[2][c], v[7], d);)
+      }
     });
   }
+#undef COLUMNS3
+#undef COLUMNS2
 }
 
 // Sums over the LANES lanes of a row, in every lane (within a warp), or over
@@ -493,40 +500,84 @@ __device__ __forceinline__ void near_reduce(cx<R> acc[3][K]) {
   }
 }
 
-// Grid part of an edge's rows: sums over the edge's covered grid points (entries
-// x0 .. x0 + n, compact points xpt) of the entry's weight blocks (stencil.cu)
-// and the potential groups there.  Lane = slot * G + group, G = 4 groups of a
-// plain edge, 8 of an absorber edge: each lane sums one group (four complex
-// values, 32 bytes in complex64, against four weights) into ga[c].
-template <typename R, int K, int G, int LANES>
+// Grid part of an edge's rows: sums over the edge's n covered grid points
+// (compact points xpt) of the entry's weight blocks (stencil.cu) and the
+// potential groups there.  Lane = slot * H + half group, H = 8 half groups of
+// a plain edge, 16 of an absorber edge: each lane sums two complex values of
+// a point against two weights into ga[c], so that a warp's loads are
+// contiguous (the 128 or 256 bytes of a point in complex64).  Entries go in
+// blocks of GR_IF slots: a block's point indices are loaded by the lanes one
+// block ahead and handed out by shuffles, and all of its weights and (one
+// right-hand side) potentials are loaded before the first is used.
+constexpr int GR_IF = 4;
+
+__device__ __forceinline__ void load_two(const float* p, float* v) {
+  const float2 u = __ldg(reinterpret_cast<const float2*>(p));
+  v[0] = u.x;
+  v[1] = u.y;
+}
+__device__ __forceinline__ void load_two(const double* p, double* v) {
+  const double2 u = __ldg(reinterpret_cast<const double2*>(p));
+  v[0] = u.x;
+  v[1] = u.y;
+}
+__device__ __forceinline__ void load_two(const cx<float>* p, cx<float>* v) {
+  const float4 u = __ldg(reinterpret_cast<const float4*>(p));
+  v[0] = mk(u.x, u.y);
+  v[1] = mk(u.z, u.w);
+}
+__device__ __forceinline__ void load_two(const cx<double>* p, cx<double>* v) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  v[0] = mk(a.x, a.y);
+  v[1] = mk(b.x, b.y);
+}
+
+template <typename R, int K, int H, int STRIDE, int LANES>
 __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n, const R* __restrict__ w,
                                           const cx<R>* __restrict__ pot, int64_t cs_g, int kc, int lane,
                                           cx<R> ga[K]) {
-  constexpr int STRIDE = G == 4 ? 8 : 24;
-  const int grp = lane % G, slot = lane / G;
-  w += 4 * (grp < 4 ? grp & 1 : grp - 2);
-  pot += 4 * grp;
-#pragma unroll 2
-  for (int j = slot; j < n; j += LANES / G) {
-    R a[4];
-    load4(w + STRIDE * j, a);
-    const cx<R>* pp = pot + (int64_t)xpt[j] * NPOT;
+  constexpr int S = 32 / H, BLK = GR_IF * S, STEP = BLK * (LANES / 32);
+  const int wl = lane & 31, slot = wl / H;
+  int b = BLK * (lane >> 5);  // the warps of a wide row take the blocks in turn
+  int id = wl < BLK && b + wl < n ? xpt[b + wl] : 0;
+  for (; b < n; b += STEP) {
+    const int cur = id;
+    if (b + STEP + wl < n && wl < BLK) id = xpt[b + STEP + wl];
+    R a[GR_IF][2];
+    cx<R> g[GR_IF][2];
+    const cx<R>* pp[GR_IF];
 #pragma unroll
-    for (int c = 0; c < K; ++c)
-      if (c < kc) {
-        cx<R> g[4];
-        load_group(pp + c * cs_g, g);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) axpy2(ga[c], a[f], g[f]);
+    for (int u = 0; u < GR_IF; ++u) {
+      const int j = b + u * S + slot;
+      pp[u] = pot + (int64_t)__shfl_sync(0xffffffffu, cur, u * S + slot) * NPOT;
+      a[u][0] = a[u][1] = R(0);
+      g[u][0] = g[u][1] = czero<R>();
+      if (j < n) {
+        load_two(w + (int64_t)STRIDE * j, a[u]);
+        if constexpr (K == 1) load_two(pp[u], g[u]);
       }
+    }
+#pragma unroll
+    for (int u = 0; u < GR_IF; ++u) {
+      if constexpr (K == 1) {
+        axpy2(ga[0], a[u][0], g[u][0]);
+        axpy2(ga[0], a[u][1], g[u][1]);
+      } else if (b + u * S + slot < n) {
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+          if (c < kc) {
+            load_two(pp[u] + c * cs_g, g[u]);
+            axpy2(ga[c], a[u][0], g[u][0]);
+            axpy2(ga[c], a[u][1], g[u][1]);
+          }
+      }
+    }
   }
 }
 
 struct RowTables {
-  const int32_t *off, *nl, *col;  // near matrix (rows in class order)
-  const int64_t* vo;
-  const int32_t* gcol;
-  const int32_t *xoff, *xpt;  // edge stencils
+  const RowDesc* desc;
+  const int32_t *col, *gcol, *xpt;
   int64_t ne, nL, nxl;
 };
 
@@ -537,7 +588,7 @@ struct RowTables {
 // weights (HBM on large operators) and by load latency: the near values are
 // loaded a column ahead, the weights two entries at a time.
 template <typename R, int K, int LANES>
-__global__ void __launch_bounds__(NM_THREADS)
+__global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 && K == 1 ? 8 : 1)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
            const cx<R>* __restrict__ pot, int64_t cs_g, const cx<R>* __restrict__ x, int64_t ldx, cx<R>* __restrict__ y,
            int64_t ldy, int kc) {
@@ -550,18 +601,23 @@ __global__ void __launch_bounds__(NM_THREADS)
 #pragma unroll
     for (int c = 0; c < K; ++c) acc[i][c] = czero<R>();
   if (r < T.ne) {
-    near_row<R, K, false, LANES>(r, nL, nR, T.off, T.nl, T.col, T.vo, nmv, x, ldx, kc, lane, acc);
-    const int x0 = T.xoff[r], n = T.xoff[r + 1] - x0;
+    const RowDesc D = load_desc(T.desc + r);
+    const int64_t x0 = D.xoff;
+    near_row<R, K, false, LANES>(D, r >= nL, nL, nR, T.col, nmv, x, ldx, kc, lane, acc);
     cx<R> ga[K];
 #pragma unroll
     for (int c = 0; c < K; ++c) ga[c] = czero<R>();
     int i;
     if (r < nL) {
-      grid_rows<R, K, 4, LANES>(T.xpt + x0, n, xw + 8 * (int64_t)x0, pot, cs_g, kc, lane, ga);
-      i = (lane & 3) >> 1;  // groups 0, 1 -> E row; 2, 3 -> H row
+      const int h = lane & 7;
+      grid_rows<R, K, 8, 8, LANES>(T.xpt + x0, D.nx, xw + 8 * x0 + 2 * (h & 3), pot + 2 * h, cs_g, kc, lane, ga);
+      i = h >> 2;  // groups 0, 1 -> E row; 2, 3 -> H row
     } else {
-      grid_rows<R, K, 8, LANES>(T.xpt + x0, n, xw + 8 * T.nxl + 24 * (x0 - T.nxl), pot, cs_g, kc, lane, ga);
-      i = ((lane & 7) + 2) >> 2;  // groups 0, 1 -> Eq. 3; 2 .. 5 -> Eq. 13; 6, 7 -> Eq. 14
+      const int h = lane & 15, g = h >> 1;
+      grid_rows<R, K, 16, 24, LANES>(T.xpt + x0, D.nx,
+                                     xw + 8 * T.nxl + 24 * (x0 - T.nxl) + 2 * (g < 4 ? h & 3 : h - 4), pot + 2 * h, cs_g,
+                                     kc, lane, ga);
+      i = (g + 2) >> 2;  // groups 0, 1 -> Eq. 3; 2 .. 5 -> Eq. 13; 6, 7 -> Eq. 14
       if (lane < 5) {
         const int g = T.gcol[5 * (r - nL) + lane];
         if (g >= 0) {
@@ -602,7 +658,7 @@ __global__ void __launch_bounds__(NM_THREADS)
 // projection transposed (the value blocks Q0 against the convolved adjoint
 // fields of J_e, M outside, J_i, M inside: groups 4 .. 7 of pot).
 template <typename R, int LANES>
-__global__ void __launch_bounds__(NM_THREADS)
+__global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
     k_rows_adj(RowTables T, const cx<R>* __restrict__ nmt, const R* __restrict__ gval, const R* __restrict__ xw,
                const cx<R>* __restrict__ pot, const cx<R>* __restrict__ y, cx<R>* __restrict__ x) {
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
@@ -610,20 +666,17 @@ __global__ void __launch_bounds__(NM_THREADS)
   const int64_t nL = T.nL, nR = T.ne - nL;
   cx<R> acc[3][1] = {{czero<R>()}, {czero<R>()}, {czero<R>()}};
   if (r < T.ne) {
-    near_row<R, 1, true, LANES>(r, nL, nR, T.off, T.nl, T.col, T.vo, nmt, y, 0, 1, lane, acc);
-    const int x0 = T.xoff[r], n = T.xoff[r + 1] - x0;
-    const int stride = r < nL ? 8 : 24, grp = lane & 3;
-    const R* w = xw + (r < nL ? 8 * (int64_t)x0 : 8 * T.nxl + 24 * (x0 - T.nxl));
-    cx<R> ga = czero<R>();
-#pragma unroll 2
-    for (int j = lane >> 2; j < n; j += LANES / 4) {
-      R a[4];
-      cx<R> g[4];
-      load4(w + stride * j, a);
-      load_group(pot + (int64_t)T.xpt[x0 + j] * NPOT + 16 + 4 * grp, g);
-#pragma unroll
-      for (int f = 0; f < 4; ++f) axpy2(ga, a[f], g[f]);
-    }
+    const RowDesc D = load_desc(T.desc + r);
+    const int64_t x0 = D.xoff;
+    near_row<R, 1, true, LANES>(D, r >= nL, nL, nR, T.col, nmt, y, 0, 1, lane, acc);
+    const int h = lane & 7, grp = h >> 1;
+    cx<R> gs[1] = {czero<R>()};
+    if (r < nL)
+      grid_rows<R, 1, 8, 8, LANES>(T.xpt + x0, D.nx, xw + 8 * x0 + 2 * (h & 1), pot + 16 + 2 * h, 0, 1, lane, gs);
+    else
+      grid_rows<R, 1, 8, 24, LANES>(T.xpt + x0, D.nx, xw + 8 * T.nxl + 24 * (x0 - T.nxl) + 2 * (h & 1), pot + 16 + 2 * h,
+                                    0, 1, lane, gs);
+    const cx<R> ga = gs[0];
     // groups J_e, M, J_i, -M; on plain edges J_i = -J_e
     if (r < nL) {
       if (grp == 0) acc[0][0] += ga;
@@ -664,8 +717,8 @@ PrecData<double>& pdata<double>(scabem_op* op) {
   return op->d;
 }
 
-RowTables row_tables(const scabem_op* op, const int64_t* vo) {
-  return {op->nm_off, op->nm_nl, op->nm_col, vo, op->nm_gcol, op->xoff, op->xpt, op->ne, op->nL, op->nxl};
+RowTables row_tables(const scabem_op* op, const void* desc) {
+  return {(const RowDesc*)desc, op->nm_col, op->nm_gcol, op->xpt, op->ne, op->nL, op->nxl};
 }
 // a warp per row; a whole CTA per row where warps would leave the chip idle
 // and the rows are long (77 columns per row on the 12 um guide)
@@ -677,7 +730,7 @@ int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
   const bool wide = wide_rows(op);
   auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
   fn<<<(unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS), NM_THREADS, 0, s>>>(
-      row_tables(op, op->nm_vo), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc);
+      row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }
@@ -707,7 +760,7 @@ int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s) {
   const bool wide = wide_rows(op);
   auto fn = wide ? k_rows_adj<R, NM_THREADS> : k_rows_adj<R, 32>;
   fn<<<(unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS), NM_THREADS, 0, s>>>(
-      row_tables(op, op->nm_vt), pd.nmt, pd.gram, pd.xw, pd.grid, y, x);
+      row_tables(op, op->rdesc_t), pd.nmt, pd.gram, pd.xw, pd.grid, y, x);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }
@@ -753,11 +806,26 @@ int setup_near_matrix(scabem_op* op, cudaStream_t s) {
   CK(cudaMemcpyAsync(op->nm_off, hc.data(), sizeof(int32_t) * (ne + 1), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(op->nm_vo, vo.data(), sizeof(int64_t) * (ne + 1), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(op->nm_vt, vt.data(), sizeof(int64_t) * (ne + 1), cudaMemcpyHostToDevice, s));
+  std::vector<RowDesc> rd(ne), rt(ne);
+  for (int64_t r = 0; r < ne; ++r) {
+    rd[r] = {hc[r], hl[r], hc[r + 1] - hc[r], op->h_xoff[r], vo[r], op->h_xoff[r + 1] - op->h_xoff[r], 0};
+    rt[r] = rd[r];
+    rt[r].vo = vt[r];
+  }
+  std::vector<int32_t>().swap(op->h_xoff);
+  CK(cudaMalloc(&op->rdesc, sizeof(RowDesc) * ne));
+  CK(cudaMalloc(&op->rdesc_t, sizeof(RowDesc) * ne));
+  CK(cudaMemcpyAsync(op->rdesc, rd.data(), sizeof(RowDesc) * ne, cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(op->rdesc_t, rt.data(), sizeof(RowDesc) * ne, cudaMemcpyHostToDevice, s));
   CK(cudaMalloc(&op->nm_col, sizeof(int32_t) * acc));
   CK(cudaMalloc(&op->nm_tpos, sizeof(int32_t) * acc));
   k_near_pattern<<<gw, 128, 0, s>>>(op->rtk, op->tedge, op->noff, op->nsrc, ne, nL, nullptr, op->nm_nl, op->nm_off,
                                     op->nm_col);
   CK(cudaGetLastError());
+  // sorted through the position table's storage
+  k_near_sort<<<gw, 128, 0, s>>>(op->nm_off, op->nm_nl, ne, op->nm_col, op->nm_tpos);
+  CK(cudaGetLastError());
+  std::swap(op->nm_col, op->nm_tpos);
   k_near_tpos<<<gw, 128, 0, s>>>(op->nm_off, op->nm_nl, op->nm_col, ne, nL, op->nm_tpos);
   CK(cudaGetLastError());
   if (op->f.built) {

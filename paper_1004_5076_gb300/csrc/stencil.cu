@@ -216,6 +216,7 @@ int setup_stencils(scabem_op* op, cudaStream_t s) {
   k_grid_order<<<(unsigned)cdiv(acc, 256), 256, 0, s>>>(op->gpe, acc, op->nxl, op->d.xw, op->f.xw, op->d.gq, op->f.gq);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
+  op->h_xoff = std::move(off);
   return SCABEM_OK;
 }
 
