@@ -134,7 +134,7 @@ template <typename R>
 struct PrecData {
   bool built = false;
   cx<R>* ghat[2] = {nullptr, nullptr};  // octant spectra [q0][q2][q1], scaled by 1/(P0 P1 P2)
-  cx<R>* gt[2] = {nullptr, nullptr};    // transverse tables [q0][|d1|][|d2|] (direct mode)
+  cx<R>* gt[2] = {nullptr, nullptr};    // tables of the direct (y, z) sums: [q0][|d1|][|d2|], or by parity
   cx<R>* near = nullptr;                // [npairs][NCORR][q][2]
   cx<R>* tw[3] = {nullptr, nullptr, nullptr};  // forward twiddles per axis length
   R* L = nullptr;                       // Q * 3 * p stencil weights
@@ -213,6 +213,7 @@ struct scabem_op {
   // for the FFT planes
   int64_t cst = 0;
   bool tdirect = false;
+  bool parity = false;  // the direct sums run block-diagonalised by parity (gt: its tables)
   int R1 = 0, R2 = 0;
   int32_t* acoord = nullptr;  // nac
   double* sig64 = nullptr;    // Q normalised (master copy)
@@ -273,6 +274,11 @@ inline int64_t col_stride_src(const scabem_op* op) { return (int64_t)NFIELD_OUT 
 inline int64_t col_stride_pot(const scabem_op* op) { return (int64_t)NPOT * op->n[0] * op->nac; }
 inline int64_t col_stride_st(const scabem_op* op) {  // stA and stB
   return (int64_t)NFIELD_OUT * op->P[0] * op->cst;
+}
+// table values per (medium, axis-0 frequency) of the parity form of the direct sums
+inline int64_t parity_words(const scabem_op* op) {
+  const int64_t E1 = (op->R1 + 1) / 2, O1 = op->R1 - E1, E2 = (op->R2 + 1) / 2, O2 = op->R2 - E2;
+  return (E1 * E1 + O1 * O1) * (E2 * E2 + O2 * O2);
 }
 // Right-hand sides the batched apply handles per pass (one CTA of that many
 // warps shares each target triangle's near-record stream).
@@ -357,6 +363,7 @@ int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* l
 template <typename R>
 int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_t s);
 // fft.cu
+void choose_parity(scabem_op* op);
 // adjoint = false: 12 sources -> 16 potentials (the apply); true: 16 -> 16,
 // each field convolved with its medium's Green function (the transposed apply)
 // ncol right-hand sides at once: column c of each workspace starts at

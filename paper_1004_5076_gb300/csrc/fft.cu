@@ -740,6 +740,191 @@ __global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __res
   }
 }
 
+// ---------------------------------------------------------------- stage B, direct, by parity
+// The direct sum over the box R1 x R2 of the active columns, block
+// diagonalised by its reflection symmetry: gt depends on |i1 - j1| and |i2 - j2|
+// only, so sums and differences of mirrored columns along either axis do not
+// mix.  The four parity blocks need a quarter of the products of the whole box
+// (guide: 3,136 per field against 104^2 = 10,816 over the active columns).
+// Positions keep their place: e = x_i + x_(n-1-i) lies at i (the middle one as
+// it is), o = x_i - x_(n-1-i) at n - 1 - i.  The tables hold, per axis-0
+// frequency and block, M[j][i] = (1/4) sum of gt over the direct and mirrored
+// offsets with the block's signs (setup.cu: k_parity_tables), so that the
+// same butterflies lead back.
+//
+// One CTA per (q0, medium): the planes k0 = q0 and P0 - q0 share the table.
+// One thread per (plane, position), 8 fields each; a table value serves 8
+// fields, the sources are shared-memory broadcasts.  In complex64 the products
+// take a few microseconds, so the rest is kept short: the table is copied to
+// shared memory while the sources arrive (STAGE), the sources of all rows are in
+// flight at once, and the two axes' butterflies are one pass.  The CTA takes
+// the right-hand sides of a batch in turn.
+constexpr int PS_THREADS = 256;
+constexpr int PS_W = 10;  // words per position: 8 fields, padded so that a row's stores spread over the banks
+
+// butterflies of both axes over the planes s [plane][i1][i2][PS_W], in place
+template <typename R>
+__device__ __forceinline__ void parity_pass(cx<R>* s, int R1, int R2, int npl) {
+  const int E1 = (R1 + 1) / 2, E2 = (R2 + 1) / 2;
+  for (int u = threadIdx.x; u < npl * E1 * E2 * 8; u += PS_THREADS) {
+    const int v = u & 7, w = u >> 3, q = w / E2, i2 = w - q * E2, pl = q >= E1, i1 = q - pl * E1;
+    const int m1 = R1 - 1 - i1, m2 = R2 - 1 - i2;
+    cx<R>* b = s + (int64_t)pl * R1 * R2 * PS_W + v;
+    cx<R>*p00 = b + (i1 * R2 + i2) * PS_W, *p10 = b + (m1 * R2 + i2) * PS_W, *p01 = b + (i1 * R2 + m2) * PS_W,
+         *p11 = b + (m1 * R2 + m2) * PS_W;
+    cx<R> x00 = *p00, x10 = *p10, x01 = *p01, x11 = *p11;
+    if (m1 != i1) {
+      const cx<R> a = x00 - x10, c = x01 - x11;
+      x00 = x00 + x10;
+      x01 = x01 + x11;
+      x10 = a;
+      x11 = c;
+    }
+    if (m2 != i2) {
+      const cx<R> a = x00 - x01, c = x10 - x11;
+      x00 = x00 + x01;
+      x10 = x10 + x11;
+      x01 = a;
+      x11 = c;
+    }
+    *p00 = x00;
+    if (m1 != i1) *p10 = x10;
+    if (m2 != i2) *p01 = x01;
+    if (m1 != i1 && m2 != i2) *p11 = x11;
+  }
+}
+
+__device__ __forceinline__ cx<float> ldg_cx(const cx<float>* p) {
+  const float2 u = __ldg(reinterpret_cast<const float2*>(p));
+  return mk(u.x, u.y);
+}
+__device__ __forceinline__ cx<double> ldg_cx(const cx<double>* p) {
+  const double2 u = __ldg(reinterpret_cast<const double2*>(p));
+  return mk(u.x, u.y);
+}
+
+template <typename R, bool STAGE>
+__global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
+    k_planes_parity(const cx<R>* __restrict__ A, cx<R>* __restrict__ B, const cx<R>* __restrict__ mE,
+                    const cx<R>* __restrict__ mI, int P0, const int32_t* __restrict__ acoord, int nac, int R1, int R2,
+                    int words, int ident, int64_t cs, int ncol) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int q0 = blockIdx.x, med = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nb = R1 * R2, npl = (q0 == 0 || 2 * q0 == P0) ? 1 : 2, tot = npl * nb;
+  const bool onepass = 2 * nb <= PS_THREADS;  // every result waits in its thread's registers
+  cx<R>* src = reinterpret_cast<cx<R>*>(smem_raw);  // [plane][i1][i2][PS_W]
+  cx<R>* res = onepass ? src : src + 2 * nb * PS_W;
+  cx<R>* Ms = res + 2 * nb * PS_W;
+  int32_t* crd = reinterpret_cast<int32_t*>(Ms + (STAGE ? words + (words & 1) : 0));
+  const cx<R>* Mg = (med ? mI : mE) + (int64_t)q0 * words;
+  if (STAGE) {  // 8 bytes per copy in complex64 (a table may start on an odd value), 16 in complex128
+    for (int i = threadIdx.x; i < words; i += PS_THREADS)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(Ms + i)),
+                   "l"(Mg + i), "n"((int)sizeof(cx<R>))
+                   : "memory");
+  }
+  const cx<R>* M0 = STAGE ? Ms : Mg;
+  const int E1 = (R1 + 1) / 2, E2 = (R2 + 1) / 2, O1 = R1 - E1, O2 = R2 - E2;
+  for (int i = threadIdx.x; i < nac; i += PS_THREADS) {
+    const int c = acoord[i];
+    crd[i] = (c >> 16) * R2 + (c & 0xffff);
+  }
+  // rows (plane, field) warp and warp + 8; four columns per lane in flight
+  int in0[2], out0[2];
+  bool neg[2];
+  const cx<R>* rp[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int v = warp, pl = h, k0 = pl ? P0 - q0 : q0;
+    const int f = ident ? 8 * med + v : (v < 4 ? (med ? 4 + v : v) : 8 + (v - 4));
+    const int fo = ident ? 8 * med + v : (med ? (v < 4 ? 8 + v : 12 + (v - 4)) : v);
+    in0[h] = f * P0 + k0;
+    out0[h] = fo * P0 + k0;
+    neg[h] = !ident && med && v >= 4;
+    rp[h] = A + (int64_t)in0[h] * nac;
+  }
+  for (int col = 0; col < ncol; ++col) {
+    for (int i = threadIdx.x; i < 2 * nb * PS_W; i += PS_THREADS) src[i] = czero<R>();
+    __syncthreads();
+    for (int jb = 0; jb < nac; jb += 128) {
+      cx<R> x[2][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = jb + 32 * u + lane;
+          if (h < npl && j < nac) x[h][u] = ldg_cx(rp[h] + col * cs + j);
+        }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = jb + 32 * u + lane;
+          if (h < npl && j < nac) src[(h * nb + crd[j]) * PS_W + warp] = x[h][u];
+        }
+    }
+    __syncthreads();
+    parity_pass<R>(src, R1, R2, npl);
+    if (STAGE && col == 0) asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    for (int u = threadIdx.x; u < (onepass ? PS_THREADS : tot); u += PS_THREADS) {
+      Acc8<R> acc;
+      acc.zero();
+      int at = 0;
+      if (u < tot) {
+        // block (odd along axis 1, odd along axis 2) and index in it; blocks in
+        // the order (even, even), (even, odd), (odd, even), (odd, odd)
+        const int pl = u >= nb;
+        int a = u - pl * nb;
+        const bool s1 = a >= E1 * R2;
+        a -= s1 ? E1 * R2 : 0;
+        const int n1 = s1 ? O1 : E1;
+        const bool s2 = a >= n1 * E2;
+        a -= s2 ? n1 * E2 : 0;
+        const int n2 = s2 ? O2 : E2, n = n1 * n2, a1 = a / n2, a2 = a - a1 * n2;
+        at = pl * nb + (s1 ? R1 - 1 - a1 : a1) * R2 + (s2 ? R2 - 1 - a2 : a2);
+        const cx<R>* M = M0 + (s1 ? E1 * E1 * (E2 * E2 + O2 * O2) : 0) + (s2 ? n1 * n1 * E2 * E2 : 0) + a;
+        const cx<R>* sp = src + (pl * nb + (s1 ? (R1 - 1) * R2 : 0) + (s2 ? R2 - 1 : 0)) * PS_W;
+        const int st1 = (s1 ? -R2 : R2) * PS_W, st2 = s2 ? -PS_W : PS_W;
+        for (int j1 = 0; j1 < n1; ++j1) {
+          const cx<R>* sj = sp + j1 * st1;
+#pragma unroll 4
+          for (int j2 = 0; j2 < n2; ++j2) {
+            acc.mac(STAGE ? *M : ldg_cx(M), sj);
+            M += n;
+            sj += st2;
+          }
+        }
+      }
+      if (onepass) __syncthreads();  // the sources are read before the results replace them
+      if (u < tot)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) res[(int64_t)at * PS_W + v] = acc.get(v);
+    }
+    __syncthreads();
+    parity_pass<R>(res, R1, R2, npl);
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (h < npl) {
+        cx<R>* o = B + col * cs + (int64_t)out0[h] * nac;
+        for (int j = lane; j < nac; j += 32) {
+          const cx<R> val = res[(h * nb + crd[j]) * PS_W + warp];
+          o[j] = neg[h] ? -val : val;
+        }
+      }
+    __syncthreads();
+  }
+}
+
+// Shared memory of the parity form: the two planes, a second pair for the
+// results when the positions outnumber the threads, the table when staged, the
+// columns' positions.
+size_t parity_smem(int nb, int64_t nac, int64_t staged, size_t csz) {
+  return (size_t)2 * nb * PS_W * csz * (2 * nb <= PS_THREADS ? 1 : 2) + (size_t)(staged + (staged & 1)) * csz +
+         sizeof(int32_t) * nac;
+}
+
 // Compiled plane sizes: (2^l1) x (2^l2) with 3 <= l1, l2 <= 7 and l1 + l2 <= 12.
 template <typename R>
 PlanesFn<R> planes_kernel(int l1, int l2) {
@@ -889,6 +1074,18 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
   CK(cudaGetLastError());
   prof_mark(op, s);
   // stage B
+  if (op->tdirect && op->parity) {
+    const int words = (int)parity_words(op), nb = op->R1 * op->R2;
+    const bool stage = parity_smem(nb, op->nac, words, sizeof(cx<R>)) <= 100 * 1024;  // two CTAs per SM and more
+    const size_t sm = parity_smem(nb, op->nac, stage ? words : 0, sizeof(cx<R>));
+    auto fn = stage ? k_planes_parity<R, true> : k_planes_parity<R, false>;
+    if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
+    fn<<<dim3(P0 / 2 + 1, 2), PS_THREADS, sm, s>>>(pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0, op->acoord, (int)op->nac,
+                                                   op->R1, op->R2, words, id, col_stride_st(op), ncol);
+    CK(cudaGetLastError());
+    prof_mark(op, s);
+    return axis0_inverse(op, pd, s, adjoint, ncol);
+  }
   if (op->tdirect) {
     const size_t sm = ((size_t)op->nac * 8 + (size_t)op->R1 * op->R2) * sizeof(cx<R>) + sizeof(int32_t) * op->nac;
     if (int rc_ = set_max_smem(op->device, (const void*)k_planes_direct<R>, (int)sm)) return rc_;
@@ -920,6 +1117,18 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
   CK(cudaGetLastError());
   prof_mark(op, s);
   return axis0_inverse(op, pd, s, adjoint, ncol);
+}
+
+// The parity form where its products, (E1^2 + O1^2)(E2^2 + O2^2) per field and
+// frequency against nac^2, are fewer (they are not when the box holds few
+// active columns: two guides far apart), its planes fit in shared memory and
+// its tables stay below 1 GiB.
+void choose_parity(scabem_op* op) {
+  const int64_t nb = (int64_t)op->R1 * op->R2;
+  const size_t csz = (op->prec_mask & 2) ? sizeof(cx<double>) : sizeof(cx<float>);
+  const int64_t w = parity_words(op);
+  op->parity = w < op->nac * op->nac && w <= INT32_MAX && nb < (1 << 16) && parity_smem((int)nb, op->nac, 0, csz) <= 227 * 1024 &&
+               2 * w * (op->P[0] / 2 + 1) * (int64_t)csz <= (1ll << 30);
 }
 
 template int make_twiddles<float>(cx<float>*, int, cudaStream_t);

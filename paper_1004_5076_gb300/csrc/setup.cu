@@ -207,6 +207,33 @@ __global__ void k_transverse(const cx<double>* __restrict__ F, int P0, int P1, i
   if (of) of[idx] = mk((float)v.re, (float)v.im);
 }
 
+// Parity tables of the same (fft.cu: k_planes_parity): for frequency q0, block
+// (odd along axis 1, odd along axis 2), column j and row i of the block,
+//   (1/4)(1/P0) (F(d1, d2) + s1 F(h1, d2) + s2 F(d1, h2) + s1 s2 F(h1, h2)),
+// d = |i - j|, h = R - 1 - i - j, s = -1 for an odd axis.
+__global__ void k_parity_tables(const cx<double>* __restrict__ F, int P0, int P1, int P2, int R1, int R2, int64_t words,
+                                cx<double>* __restrict__ od, cx<float>* __restrict__ of) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (idx >= (P0 / 2 + 1) * words) return;
+  const int q0 = (int)(idx / words);
+  int64_t w = idx - q0 * words;
+  const int64_t E1 = (R1 + 1) / 2, O1 = R1 - E1, E2 = (R2 + 1) / 2, O2 = R2 - E2, m2 = E2 * E2 + O2 * O2;
+  const bool s1 = w >= E1 * E1 * m2;
+  if (s1) w -= E1 * E1 * m2;
+  const int64_t n1 = s1 ? O1 : E1;
+  const bool s2 = w >= n1 * n1 * E2 * E2;
+  if (s2) w -= n1 * n1 * E2 * E2;
+  const int64_t n2 = s2 ? O2 : E2, n = n1 * n2;
+  const int j = (int)(w / n), i = (int)(w - (int64_t)j * n);
+  const int j1 = j / (int)n2, j2 = j - j1 * (int)n2, i1 = i / (int)n2, i2 = i - i1 * (int)n2;
+  const int d1 = abs(i1 - j1), h1 = R1 - 1 - i1 - j1, d2 = abs(i2 - j2), h2 = R2 - 1 - i2 - j2;
+  const double g1 = s1 ? -1.0 : 1.0, g2 = s2 ? -1.0 : 1.0;
+  auto f = [&](int a, int b) { return F[((int64_t)q0 * P1 + a) * P2 + b]; };
+  const cx<double> v = (0.25 / P0) * ((f(d1, d2) + g1 * f(h1, d2)) + g2 * (f(d1, h2) + g1 * f(h1, h2)));
+  if (od) od[idx] = v;
+  if (of) of[idx] = mk((float)v.re, (float)v.im);
+}
+
 // ---------------------------------------------------------------- near list
 __global__ void k_near_count(const double* __restrict__ tri, int64_t nt, double r2, int32_t* __restrict__ cnt) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -844,6 +871,7 @@ int setup_gather(scabem_op* op, cudaStream_t s) {
                 std::to_string(sm) + " bytes of shared memory)");
       return SCABEM_E_ARG;
     }
+    choose_parity(op);
     if (op->transverse == 2 && !op->direct_fits) {
       set_error("grid: the direct (y, z) sums were asked for, but their columns do not fit in shared memory");
       return SCABEM_E_ARG;
@@ -952,11 +980,16 @@ int setup_green(scabem_op* op, cudaStream_t s) {
     int rc = fft_axis_full<double>(op, F, 0, twd[0], -1, s);
     if (rc) return rc;
     if (op->direct_fits) {
-      const int64_t nt_ = (int64_t)(op->P[0] / 2 + 1) * op->R1 * op->R2;
+      const int64_t words = op->parity ? parity_words(op) : (int64_t)op->R1 * op->R2;
+      const int64_t nt_ = (int64_t)(op->P[0] / 2 + 1) * words;
       if (op->prec_mask & 2) CK(cudaMalloc(&op->d.gt[med], sizeof(cx<double>) * nt_));
       if (op->prec_mask & 1) CK(cudaMalloc(&op->f.gt[med], sizeof(cx<float>) * nt_));
-      k_transverse<<<(int)cdiv(nt_, 256), 256, 0, s>>>(F, op->P[0], op->P[1], op->P[2], op->R1, op->R2,
-                                                       op->d.gt[med], op->f.gt[med]);
+      if (op->parity)
+        k_parity_tables<<<(int)cdiv(nt_, 256), 256, 0, s>>>(F, op->P[0], op->P[1], op->P[2], op->R1, op->R2, words,
+                                                            op->d.gt[med], op->f.gt[med]);
+      else
+        k_transverse<<<(int)cdiv(nt_, 256), 256, 0, s>>>(F, op->P[0], op->P[1], op->P[2], op->R1, op->R2,
+                                                         op->d.gt[med], op->f.gt[med]);
       CK(cudaGetLastError());
     }
     if (!op->planes_fit) continue;
