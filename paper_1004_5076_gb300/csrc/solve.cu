@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -241,91 +242,171 @@ __global__ void k_rows_out(const cd* __restrict__ val, const int32_t* __restrict
 
 // E and H of one current set at points (Eqs. 15-16 evaluated off the
 // surface, Eq. 8): side 0 = the interior set (J_i, -M) radiating in the
-// interior medium, plus the interior incident field when has_inc; side 1 =
+// interior medium, plus the interior incident field when asked; side 1 =
 // the exterior set (J_e, M) in the exterior medium.  With A, phi of J and F,
 // psi of M (point-source quadrature over every source point):
 //   E = -z (jk A + (j/k) grad phi) - curl F,   H = curl A - (jk F + (j/k) grad psi) / z.
-// One block per point; the 18 complex sums are reduced by warp shuffles and
-// shared memory.
-__global__ void __launch_bounds__(256) k_fields_eh(const cd* __restrict__ summ, const double* __restrict__ tri,
-                                                   const double* __restrict__ qp, const double* __restrict__ qw,
-                                                   int64_t Q, int q, const double* __restrict__ pts, double k,
-                                                   double z, int side, scabem_source inc, int has_inc,
-                                                   cd* __restrict__ E, cd* __restrict__ H) {
-  const int pi = blockIdx.x;
-  const double r[3] = {pts[3 * pi], pts[3 * pi + 1], pts[3 * pi + 2]};
-  const double msign = side ? 1.0 : -1.0;
-  cd acc[18];  // A_J, grad phi_J, curl A_J, F_M, grad psi_M, curl F_M
+//
+// k_point_currents forms each source point's weighted currents once:
+// pc[b] = { position (3), J w / 4 pi (3), M w / 4 pi (3), r1, r2, 0 } with r1 = -(z j / k) div J
+// and r2 = -(j / (k z)) div M (weighted alike), 20 doubles.  k_point_fields then
+// sums, with G = exp(-jkR) / R and grad G = g D (D = r - r', g = -(1/R + jk) G / R),
+//   E += -jzk G J + g (r1 D - D x M),   H += -(jk/z) G M + g (D x J + r2 D)
+// over a slice of the sources for FP_PTS points per CTA.  It is bound by the
+// FP64 units (about 180 operations per point and source, a third of them the
+// sincos), so the sources are split over enough CTAs to fill the chip
+// (one CTA per point left 63 points on 63 of 152 SMs: 7.6 ms against 1.8 ms
+// on the 12 um guide); the slices' partial sums are added in order.
+__global__ void k_point_currents(const cd* __restrict__ summ, const double* __restrict__ tri,
+                                 const double* __restrict__ qp, const double* __restrict__ qw, int64_t Q, int q,
+                                 double k, double z, int side, double* __restrict__ pc) {
+  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (b >= Q) return;
+  const int64_t t = b / q;
+  const double* g = tri + 16 * t;
+  const cd* sj = summ + (3 * t + (side ? 0 : 1)) * 4;
+  const cd* sm = summ + (3 * t + 2) * 4;
+  const double w = qw[b] / (4.0 * M_PI), wm = side ? w : -w;
+  double o[20];
+  for (int c = 0; c < 3; ++c) {
+    const double rel = qp[3 * b + c] - g[9 + c];
+    const cd J = w * (rel * sj[0] - sj[1 + c]), M = wm * (rel * sm[0] - sm[1 + c]);
+    o[c] = qp[3 * b + c];
+    o[3 + 2 * c] = J.re;
+    o[4 + 2 * c] = J.im;
+    o[9 + 2 * c] = M.re;
+    o[10 + 2 * c] = M.im;
+  }
+  const cd r1 = (-2.0 * w * z / k) * mulj(sj[0]), r2 = (-2.0 * wm / (k * z)) * mulj(sm[0]);
+  o[15] = r1.re;
+  o[16] = r1.im;
+  o[17] = r2.re;
+  o[18] = r2.im;
+  o[19] = 0.0;
+  for (int c = 0; c < 20; c += 2) reinterpret_cast<double2*>(pc + 20 * b)[c / 2] = make_double2(o[c], o[c + 1]);
+}
+
+constexpr int FP_PTS = 2;
+constexpr int FP_THREADS = 256;
+
+// part[(slice * npts + point) * 12 + {E (3 complex), H (3 complex)}]
+template <bool WITH_H>
+__global__ void __launch_bounds__(FP_THREADS) k_point_fields(const double* __restrict__ pc, int64_t Q,
+                                                             const double* __restrict__ pts, int npts, double k,
+                                                             double z, double* __restrict__ part) {
+  constexpr int NV = WITH_H ? 12 : 6;
+  const int p0 = blockIdx.x * FP_PTS;
+  double r[FP_PTS][3], acc[FP_PTS][NV];
 #pragma unroll
-  for (int v = 0; v < 18; ++v) acc[v] = mk(0.0, 0.0);
-  for (int64_t b = threadIdx.x; b < Q; b += blockDim.x) {
-    const int64_t t = b / q;
-    const double* g = tri + 16 * t;
-    const double rel[3] = {qp[3 * b] - g[9], qp[3 * b + 1] - g[10], qp[3 * b + 2] - g[11]};
-    const cd* sj = summ + (3 * t + (side ? 0 : 1)) * 4;
-    const cd* sm = summ + (3 * t + 2) * 4;
-    const double D[3] = {r[0] - qp[3 * b], r[1] - qp[3 * b + 1], r[2] - qp[3 * b + 2]};
-    const double R = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
-    double sn, cs;
-    sincos(k * R, &sn, &cs);
-    const double w = qw[b] / (4.0 * M_PI * R);
-    const cd G = mk(w * cs, -w * sn);
-    const cd dG = -(mk(1.0 / R, k) * G) * (1.0 / R);  // grad G = dG D
-    const cd gG[3] = {D[0] * dG, D[1] * dG, D[2] * dG};
-    cd J[3], M[3];
+  for (int u = 0; u < FP_PTS; ++u) {
+    const int p = min(p0 + u, npts - 1);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      J[c] = rel[c] * sj[0] - sj[1 + c];
-      M[c] = msign * (rel[c] * sm[0] - sm[1 + c]);
+    for (int c = 0; c < 3; ++c) r[u][c] = pts[3 * p + c];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[u][v] = 0.0;
+  }
+  const double zk = -z * k, kz = -k / z;
+  for (int64_t b = blockIdx.y * (int64_t)FP_THREADS + threadIdx.x; b < Q; b += (int64_t)gridDim.y * FP_THREADS) {
+    double s[20];
+#pragma unroll
+    for (int c = 0; c < 10; ++c) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(pc + 20 * b) + c);
+      s[2 * c] = v.x;
+      s[2 * c + 1] = v.y;
     }
-    const cd rJ = 2.0 * sj[0], rM = (2.0 * msign) * sm[0];
+    const cd J[3] = {mk(s[3], s[4]), mk(s[5], s[6]), mk(s[7], s[8])};
+    const cd M[3] = {mk(s[9], s[10]), mk(s[11], s[12]), mk(s[13], s[14])};
+    const cd r1 = mk(s[15], s[16]), r2 = mk(s[17], s[18]);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
-      acc[c] += G * J[c];
-      acc[3 + c] += gG[c] * rJ;
-      acc[6 + c] += gG[c1] * J[c2] - gG[c2] * J[c1];
-      acc[9 + c] += G * M[c];
-      acc[12 + c] += gG[c] * rM;
-      acc[15 + c] += gG[c1] * M[c2] - gG[c2] * M[c1];
+    for (int u = 0; u < FP_PTS; ++u) {
+      const double D[3] = {r[u][0] - s[0], r[u][1] - s[1], r[u][2] - s[2]};
+      const double d2 = D[0] * D[0] + D[1] * D[1] + D[2] * D[2];
+      const double iR = rsqrt(d2), R = d2 * iR;
+      double sn, cs;
+      sincos(k * R, &sn, &cs);
+      const cd G = mk(iR * cs, -iR * sn);
+      const cd g = (-iR) * (mk(iR, k) * G);
+      const cd jG = mulj(G), GE = zk * jG, GH = kz * jG;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+        cd T = D[c] * r1;
+        axpy(T, -D[c1], M[c2]);
+        axpy(T, D[c2], M[c1]);
+        cd a = mk(acc[u][2 * c], acc[u][2 * c + 1]);
+        cfma(a, GE, J[c]);
+        cfma(a, g, T);
+        acc[u][2 * c] = a.re;
+        acc[u][2 * c + 1] = a.im;
+        if constexpr (WITH_H) {
+          cd U = D[c] * r2;
+          axpy(U, D[c1], J[c2]);
+          axpy(U, -D[c2], J[c1]);
+          cd h = mk(acc[u][6 + 2 * c], acc[u][7 + 2 * c]);
+          cfma(h, GH, M[c]);
+          cfma(h, g, U);
+          acc[u][6 + 2 * c] = h.re;
+          acc[u][7 + 2 * c] = h.im;
+        }
+      }
     }
   }
-  __shared__ double red[8][36];
+  __shared__ double red[FP_THREADS / 32][FP_PTS * NV];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
-  for (int v = 0; v < 18; ++v)
+  for (int u = 0; u < FP_PTS; ++u)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      acc[v].re += __shfl_xor_sync(0xffffffffu, acc[v].re, o);
-      acc[v].im += __shfl_xor_sync(0xffffffffu, acc[v].im, o);
-    }
-  if (lane == 0)
+    for (int v = 0; v < NV; ++v) {
 #pragma unroll
-    for (int v = 0; v < 18; ++v) {
-      red[wp][2 * v] = acc[v].re;
-      red[wp][2 * v + 1] = acc[v].im;
+      for (int o = 16; o > 0; o >>= 1) acc[u][v] += __shfl_xor_sync(0xffffffffu, acc[u][v], o);
+      if (lane == 0) red[wp][u * NV + v] = acc[u][v];
     }
   __syncthreads();
-  __shared__ double tot[36];
-  if (threadIdx.x < 36) {
-    double v = 0.0;
-    for (int k2 = 0; k2 < (int)(blockDim.x >> 5); ++k2) v += red[k2][threadIdx.x];
-    tot[threadIdx.x] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    cd Ei[3], Hi[3];
-    for (int c = 0; c < 3; ++c) Ei[c] = Hi[c] = mk(0.0, 0.0);
-    if (has_inc && side == 0) incident(inc, k, z, r, Ei, Hi);
-    for (int c = 0; c < 3; ++c) {
-      const cd AJ = mk(tot[2 * c], tot[2 * c + 1]), gJ = mk(tot[6 + 2 * c], tot[7 + 2 * c]);
-      const cd cJ = mk(tot[12 + 2 * c], tot[13 + 2 * c]), AM = mk(tot[18 + 2 * c], tot[19 + 2 * c]);
-      const cd gM = mk(tot[24 + 2 * c], tot[25 + 2 * c]), cM = mk(tot[30 + 2 * c], tot[31 + 2 * c]);
-      E[3 * pi + c] = Ei[c] - z * (k * mulj(AJ) + (1.0 / k) * mulj(gJ)) - cM;
-      H[3 * pi + c] = Hi[c] + cJ - (1.0 / z) * (k * mulj(AM) + (1.0 / k) * mulj(gM));
-    }
+  for (int i = threadIdx.x; i < FP_PTS * NV; i += FP_THREADS) {
+    const int u = i / NV, v = i - u * NV;
+    if (p0 + u >= npts) continue;
+    double t = 0.0;
+    for (int w = 0; w < FP_THREADS / 32; ++w) t += red[w][i];
+    part[((int64_t)blockIdx.y * npts + p0 + u) * 12 + v] = t;
   }
 }
+
+// the slices' sums in order, plus the incident field; H may be null
+__global__ void k_point_finish(const double* __restrict__ part, int nsl, const double* __restrict__ pts, int npts,
+                               double k, double z, scabem_source inc, int has_inc, cd* __restrict__ E,
+                               cd* __restrict__ H) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= npts) return;
+  cd Ei[3], Hi[3];
+  for (int c = 0; c < 3; ++c) Ei[c] = Hi[c] = mk(0.0, 0.0);
+  if (has_inc) incident(inc, k, z, pts + 3 * p, Ei, Hi);
+  double v[12];
+  for (int c = 0; c < 12; ++c) v[c] = 0.0;
+  for (int s = 0; s < nsl; ++s)
+    for (int c = 0; c < (H ? 12 : 6); ++c) v[c] += part[((int64_t)s * npts + p) * 12 + c];
+  for (int c = 0; c < 3; ++c) {
+    E[3 * p + c] = Ei[c] + mk(v[2 * c], v[2 * c + 1]);
+    if (H) H[3 * p + c] = Hi[c] + mk(v[6 + 2 * c], v[7 + 2 * c]);
+  }
+}
+
+// Device scratch of the field evaluation at npts points
+struct FieldScratch {
+  double *pc = nullptr, *part = nullptr;
+  int nsl = 1;
+  ~FieldScratch() {
+    cudaFree(pc);
+    cudaFree(part);
+  }
+  int init(const scabem_op* op, int npts) {
+    // four CTAs per SM, at least 512 source points each
+    const int64_t tiles = cdiv(npts, FP_PTS);
+    nsl = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(4 * 152, tiles), cdiv(op->Q, 2 * FP_THREADS)));
+    CK(cudaMalloc(&pc, sizeof(double) * 20 * op->Q));
+    CK(cudaMalloc(&part, sizeof(double) * 12 * npts * nsl));
+    return SCABEM_OK;
+  }
+};
 
 // Perimeter loss of a band of the surface (Sec. III-B): part[b] = sum over the
 // quadrature points of block b with |x_axis - xc| < slab of sigma eta0 w |M|^2
@@ -1227,148 +1308,44 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
   return SCABEM_OK;
 }
 
-// ---------------------------------------------------------------- fields at points
-// One block per (point, rhs): sum over all source quadrature points of the
-// interior set: E = -z_i (jk A + (j/k) grad phi) - curl F_i, M_i = -M.
-__global__ void k_fields(const cd* __restrict__ summ, const double* __restrict__ tri, const double* __restrict__ qp,
-                         const double* __restrict__ qw, int64_t Q, int q, const double* __restrict__ pts, double k,
-                         double z, scabem_source inc, int has_inc, cd* __restrict__ E) {
-  const int pi = blockIdx.x;
-  const double r[3] = {pts[3 * pi], pts[3 * pi + 1], pts[3 * pi + 2]};
-  cd A[3], gp[3], cF[3];
-  for (int c = 0; c < 3; ++c) A[c] = gp[c] = cF[c] = mk(0.0, 0.0);
-  for (int64_t b = threadIdx.x; b < Q; b += blockDim.x) {
-    const int64_t t = b / q;
-    const double* g = tri + 16 * t;
-    const double rel[3] = {qp[3 * b] - g[9], qp[3 * b + 1] - g[10], qp[3 * b + 2] - g[11]};
-    const cd* si = summ + (3 * t + 1) * 4;
-    const cd* sm = summ + (3 * t + 2) * 4;
-    const double D[3] = {r[0] - qp[3 * b], r[1] - qp[3 * b + 1], r[2] - qp[3 * b + 2]};
-    const double R = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
-    double sn, cs;
-    sincos(k * R, &sn, &cs);
-    const double w = qw[b] / (4.0 * M_PI * R);
-    const cd G = mk(w * cs, -w * sn);
-    const cd dG = -(mk(1.0 / R, k) * G) * (1.0 / R);  // times D gives grad G
-    const cd rho = 2.0 * si[0];
-    cd J[3], M[3];
-    for (int c = 0; c < 3; ++c) {
-      J[c] = rel[c] * si[0] - si[1 + c];
-      M[c] = -(rel[c] * sm[0] - sm[1 + c]);
-    }
-    for (int c = 0; c < 3; ++c) {
-      A[c] += G * J[c];
-      gp[c] += (D[c] * dG) * rho;
-    }
-    const cd gx = D[0] * dG, gy = D[1] * dG, gz = D[2] * dG;
-    cF[0] += gy * M[2] - gz * M[1];
-    cF[1] += gz * M[0] - gx * M[2];
-    cF[2] += gx * M[1] - gy * M[0];
-  }
-  __shared__ double red[256][2];
-  cd* accs[9] = {&A[0], &A[1], &A[2], &gp[0], &gp[1], &gp[2], &cF[0], &cF[1], &cF[2]};
-  cd tot[9];
-  for (int v = 0; v < 9; ++v) {
-    red[threadIdx.x][0] = accs[v]->re;
-    red[threadIdx.x][1] = accs[v]->im;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-      if (threadIdx.x < st) {
-        red[threadIdx.x][0] += red[threadIdx.x + st][0];
-        red[threadIdx.x][1] += red[threadIdx.x + st][1];
-      }
-      __syncthreads();
-    }
-    tot[v] = mk(red[0][0], red[0][1]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    cd Ei[3], Hi[3];
-    for (int c = 0; c < 3; ++c) Ei[c] = mk(0.0, 0.0);
-    if (has_inc) incident(inc, k, z, r, Ei, Hi);
-    for (int c = 0; c < 3; ++c) {
-      const cd jA = mk(-tot[c].im, tot[c].re), jg = mk(-tot[3 + c].im, tot[3 + c].re);
-      E[3 * pi + c] = Ei[c] - z * (k * jA + (1.0 / k) * jg) - tot[6 + c];
-    }
-  }
+// ---------------------------------------------------------------- fits
+// The scans of both fits: one warp per candidate, lanes over the samples, with
+// the explicit residual of each candidate's least-squares amplitudes.  Each CTA
+// keeps its best candidate (ties to the lowest index); the finishing kernel
+// takes the best of the CTAs and forms the results.  (One CTA with a thread
+// per candidate took 0.8 ms for 601 candidates of 48 samples.)
+constexpr int FIT_WARPS = 8;
+constexpr int FIT_BLOCKS = 4 * 152;
+
+__device__ __forceinline__ double wsum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ cd wsum(cd v) { return mk(wsum(v.re), wsum(v.im)); }
+__device__ __forceinline__ bool better(double r, int i, double rb, int ib) {
+  return i >= 0 && (r < rb || (r == rb && i < ib));
 }
 
-// Least-squares split E(t) = a exp(-j beta t) + c exp(j beta t); one block,
-// threads over beta candidates.  out: {Re r, Im r, beta, residual, SWR, r_swr}.
-__global__ void k_fit(const cd* __restrict__ E, const double* __restrict__ tt, int npts, double blo, double bhi,
-                      int nbeta, double* __restrict__ out) {
-  __shared__ double best_res[256];
-  __shared__ int best_i[256];
-  double enorm = 0.0;
-  for (int i = 0; i < npts; ++i) enorm += E[i].re * E[i].re + E[i].im * E[i].im;
-  double bres = 1e300;
-  int bi = -1;
-  for (int ib = threadIdx.x; ib < nbeta; ib += blockDim.x) {
-    const double beta = nbeta > 1 ? blo + (bhi - blo) * ib / (nbeta - 1) : blo;
-    cd a12 = mk(0.0, 0.0), r1 = a12, r2 = a12;
-    for (int i = 0; i < npts; ++i) {
-      double sn, cs;
-      sincos(beta * tt[i], &sn, &cs);
-      const cd ep = mk(cs, sn);    // exp(+j beta t)
-      const cd em = mk(cs, -sn);   // exp(-j beta t)
-      a12 += ep * ep;              // conj(em) * ep
-      r1 += ep * E[i];             // conj(em) * E
-      r2 += em * E[i];             // conj(ep) * E
-    }
-    const double n = npts;
-    const double det = n * n - (a12.re * a12.re + a12.im * a12.im);
-    const cd a = (1.0 / det) * (n * r1 - a12 * r2);
-    const cd c = (1.0 / det) * (n * r2 - conj(a12) * r1);
-    double res = 0.0;
-    for (int i = 0; i < npts; ++i) {
-      double sn, cs;
-      sincos(beta * tt[i], &sn, &cs);
-      const cd f = a * mk(cs, -sn) + c * mk(cs, sn) - E[i];
-      res += f.re * f.re + f.im * f.im;
-    }
-    if (res < bres) {
-      bres = res;
-      bi = ib;
-    }
+// E(t) = a exp(-j beta t) + c exp(j beta t): the amplitudes for one beta (a warp)
+__device__ void two_wave(const cd* __restrict__ E, const double* __restrict__ tt, int npts, double beta, int lane, cd& a,
+                         cd& c) {
+  cd a12 = mk(0.0, 0.0), r1 = a12, r2 = a12;
+  for (int i = lane; i < npts; i += 32) {
+    double sn, cs;
+    sincos(beta * tt[i], &sn, &cs);
+    const cd ep = mk(cs, sn), em = mk(cs, -sn);
+    a12 += ep * ep;   // conj(em) * ep
+    r1 += ep * E[i];  // conj(em) * E
+    r2 += em * E[i];  // conj(ep) * E
   }
-  best_res[threadIdx.x] = bres;
-  best_i[threadIdx.x] = bi;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int b = -1;
-    double r = 1e300;
-    for (int i = 0; i < blockDim.x; ++i)
-      if (best_i[i] >= 0 && (best_res[i] < r || (best_res[i] == r && best_i[i] < b))) {
-        r = best_res[i];
-        b = best_i[i];
-      }
-    const double beta = nbeta > 1 ? blo + (bhi - blo) * b / (nbeta - 1) : blo;
-    cd a12 = mk(0.0, 0.0), r1 = a12, r2 = a12;
-    double emax = 0.0, emin = 1e300;
-    for (int i = 0; i < npts; ++i) {
-      double sn, cs;
-      sincos(beta * tt[i], &sn, &cs);
-      const cd ep = mk(cs, sn), em = mk(cs, -sn);
-      a12 += ep * ep;
-      r1 += ep * E[i];
-      r2 += em * E[i];
-      const double m = sqrt(E[i].re * E[i].re + E[i].im * E[i].im);
-      emax = fmax(emax, m);
-      emin = fmin(emin, m);
-    }
-    const double n = npts;
-    const double det = n * n - (a12.re * a12.re + a12.im * a12.im);
-    const cd a = (1.0 / det) * (n * r1 - a12 * r2);
-    const cd c = (1.0 / det) * (n * r2 - conj(a12) * r1);
-    const cd rr = cdivd(c, a);
-    const double swr = emax / emin;
-    out[0] = rr.re;
-    out[1] = rr.im;
-    out[2] = beta;
-    out[3] = sqrt(r / enorm);
-    out[4] = swr;
-    out[5] = (swr - 1.0) / (swr + 1.0);
-  }
+  a12 = wsum(a12);
+  r1 = wsum(r1);
+  r2 = wsum(r2);
+  const double n = npts;
+  const double det = n * n - (a12.re * a12.re + a12.im * a12.im);
+  a = (1.0 / det) * (n * r1 - a12 * r2);
+  c = (1.0 / det) * (n * r2 - conj(a12) * r1);
 }
 
 // Decay-rate fit (Sec. III): least squares for E(t) = a exp(-g tau) +
@@ -1378,13 +1355,11 @@ __global__ void k_fit(const cd* __restrict__ E, const double* __restrict__ tt, i
 //   [g11 g12; conj(g12) g22] [a; c] = [r1; r2],
 //   g11 = sum exp(-2 alpha tau), g22 = sum exp(2 alpha tau),
 //   g12 = sum exp(2 j beta tau), r1 = sum conj(phi1) E, r2 = sum conj(phi2) E.
-// One block scans the nalpha x nbeta candidates (alpha-major), each with its
-// explicit residual; the smallest wins, ties to the lowest index.
 __device__ void decay_amplitudes(const cd* __restrict__ E, const double* __restrict__ tt, int npts, double tm,
-                                 double al, double be, cd& a, cd& c) {
+                                 double al, double be, int lane, cd& a, cd& c) {
   double g11 = 0.0, g22 = 0.0;
   cd g12 = mk(0.0, 0.0), r1 = g12, r2 = g12;
-  for (int i = 0; i < npts; ++i) {
+  for (int i = lane; i < npts; i += 32) {
     const double tau = tt[i] - tm;
     const double em = exp(-al * tau), ep = exp(al * tau);
     double sn, cs;
@@ -1395,69 +1370,154 @@ __device__ void decay_amplitudes(const cd* __restrict__ E, const double* __restr
     r1 += mk(em * cs, em * sn) * E[i];   // conj(phi1) = exp(-alpha tau) exp(+j beta tau)
     r2 += mk(ep * cs, -ep * sn) * E[i];  // conj(phi2) = exp(alpha tau) exp(-j beta tau)
   }
+  g11 = wsum(g11);
+  g22 = wsum(g22);
+  g12 = wsum(g12);
+  r1 = wsum(r1);
+  r2 = wsum(r2);
   const double det = g11 * g22 - (g12.re * g12.re + g12.im * g12.im);
   a = (1.0 / det) * (g22 * r1 - g12 * r2);
   c = (1.0 / det) * (g11 * r2 - conj(g12) * r1);
 }
-__device__ double decay_residual(const cd* __restrict__ E, const double* __restrict__ tt, int npts, double tm,
-                                 double al, double be, cd a, cd c) {
-  double res = 0.0;
-  for (int i = 0; i < npts; ++i) {
-    const double tau = tt[i] - tm;
-    const double em = exp(-al * tau), ep = exp(al * tau);
-    double sn, cs;
-    sincos(be * tau, &sn, &cs);
-    const cd f = a * mk(em * cs, -em * sn) + c * mk(ep * cs, ep * sn) - E[i];
-    res += f.re * f.re + f.im * f.im;
+
+struct FitGrid {  // candidates alpha-major: index = ia * nb + ib; na = 0: the two-wave fit
+  double alo, ahi;
+  int na;
+  double blo, bhi;
+  int nb;
+  __device__ double alpha(int i) const { return na > 1 ? alo + (ahi - alo) * (i / nb) / (na - 1) : alo; }
+  __device__ double beta(int i) const {
+    const int ib = na > 0 ? i - (i / nb) * nb : i;
+    return nb > 1 ? blo + (bhi - blo) * ib / (nb - 1) : blo;
   }
-  return res;
-}
-__global__ void k_fit_decay(const cd* __restrict__ E, const double* __restrict__ tt, int npts, double alo,
-                            double ahi, int na, double blo, double bhi, int nb, double* __restrict__ out) {
-  __shared__ double best_res[256];
-  __shared__ int best_i[256];
+};
+
+__global__ void __launch_bounds__(FIT_WARPS * 32) k_fit_scan(const cd* __restrict__ E, const double* __restrict__ tt,
+                                                             int npts, FitGrid F, double* __restrict__ bres,
+                                                             int* __restrict__ bidx) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int ncand = F.na > 0 ? F.na * F.nb : F.nb;
   const double tm = 0.5 * (tt[0] + tt[npts - 1]);
-  double enorm = 0.0;
-  for (int i = 0; i < npts; ++i) enorm += E[i].re * E[i].re + E[i].im * E[i].im;
-  const int ncand = na * nb;
-  double bres = 1e300;
+  double best = 1e300;
   int bi = -1;
-  for (int ic = threadIdx.x; ic < ncand; ic += blockDim.x) {
-    const int ia = ic / nb, ib = ic - (ic / nb) * nb;
-    const double al = na > 1 ? alo + (ahi - alo) * ia / (na - 1) : alo;
-    const double be = nb > 1 ? blo + (bhi - blo) * ib / (nb - 1) : blo;
+  for (int ic = blockIdx.x * FIT_WARPS + wp; ic < ncand; ic += gridDim.x * FIT_WARPS) {
+    const double be = F.beta(ic);
     cd a, c;
-    decay_amplitudes(E, tt, npts, tm, al, be, a, c);
-    const double res = decay_residual(E, tt, npts, tm, al, be, a, c);
-    if (res < bres) {
-      bres = res;
+    double res = 0.0;
+    if (F.na > 0) {
+      const double al = F.alpha(ic);
+      decay_amplitudes(E, tt, npts, tm, al, be, lane, a, c);
+      for (int i = lane; i < npts; i += 32) {
+        const double tau = tt[i] - tm, em = exp(-al * tau), ep = exp(al * tau);
+        double sn, cs;
+        sincos(be * tau, &sn, &cs);
+        const cd f = a * mk(em * cs, -em * sn) + c * mk(ep * cs, ep * sn) - E[i];
+        res += f.re * f.re + f.im * f.im;
+      }
+    } else {
+      two_wave(E, tt, npts, be, lane, a, c);
+      for (int i = lane; i < npts; i += 32) {
+        double sn, cs;
+        sincos(be * tt[i], &sn, &cs);
+        const cd f = a * mk(cs, -sn) + c * mk(cs, sn) - E[i];
+        res += f.re * f.re + f.im * f.im;
+      }
+    }
+    res = wsum(res);
+    if (res < best) {
+      best = res;
       bi = ic;
     }
   }
-  best_res[threadIdx.x] = bres;
-  best_i[threadIdx.x] = bi;
+  __shared__ double sr[FIT_WARPS];
+  __shared__ int si[FIT_WARPS];
+  if (lane == 0) {
+    sr[wp] = best;
+    si[wp] = bi;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int b = -1;
-    double r = 1e300;
-    for (int i = 0; i < blockDim.x; ++i)
-      if (best_i[i] >= 0 && (best_res[i] < r || (best_res[i] == r && best_i[i] < b))) {
-        r = best_res[i];
-        b = best_i[i];
+    for (int w = 1; w < FIT_WARPS; ++w)
+      if (better(sr[w], si[w], best, bi < 0 ? INT_MAX : bi)) {
+        best = sr[w];
+        bi = si[w];
       }
-    const int ia = b / nb, ib = b - (b / nb) * nb;
-    const double al = na > 1 ? alo + (ahi - alo) * ia / (na - 1) : alo;
-    const double be = nb > 1 ? blo + (bhi - blo) * ib / (nb - 1) : blo;
-    cd a, c;
-    decay_amplitudes(E, tt, npts, tm, al, be, a, c);
-    const cd rr = cdivd(c, a);
-    out[0] = al;
+    bres[blockIdx.x] = best;
+    bidx[blockIdx.x] = bi;
+  }
+}
+
+// out: {Re r, Im r, beta, residual, SWR, r_swr} (two-wave fit) or {alpha, beta,
+// residual, Re c/a, Im c/a, |a|} (decay fit); one warp
+__global__ void k_fit_finish(const cd* __restrict__ E, const double* __restrict__ tt, int npts, FitGrid F,
+                             const double* __restrict__ bres, const int* __restrict__ bidx, int nblk,
+                             double* __restrict__ out) {
+  const int lane = threadIdx.x;
+  double r = 1e300;
+  int b = -1;
+  for (int i = lane; i < nblk; i += 32)
+    if (better(bres[i], bidx[i], r, b < 0 ? INT_MAX : b)) {
+      r = bres[i];
+      b = bidx[i];
+    }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double r2 = __shfl_xor_sync(0xffffffffu, r, o);
+    const int b2 = __shfl_xor_sync(0xffffffffu, b, o);
+    if (better(r2, b2, r, b < 0 ? INT_MAX : b)) {
+      r = r2;
+      b = b2;
+    }
+  }
+  double en = 0.0, emax = 0.0, emin = 1e300;
+  for (int i = lane; i < npts; i += 32) {
+    const double m2 = E[i].re * E[i].re + E[i].im * E[i].im, m = sqrt(m2);
+    en += m2;
+    emax = fmax(emax, m);
+    emin = fmin(emin, m);
+  }
+  en = wsum(en);
+  for (int o = 16; o > 0; o >>= 1) {
+    emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    emin = fmin(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+  }
+  const double be = F.beta(b);
+  cd a, c;
+  if (F.na > 0)
+    decay_amplitudes(E, tt, npts, 0.5 * (tt[0] + tt[npts - 1]), F.alpha(b), be, lane, a, c);
+  else
+    two_wave(E, tt, npts, be, lane, a, c);
+  if (lane != 0) return;
+  const cd rr = cdivd(c, a);
+  if (F.na > 0) {
+    out[0] = F.alpha(b);
     out[1] = be;
-    out[2] = sqrt(r / enorm);
+    out[2] = sqrt(r / en);
     out[3] = rr.re;
     out[4] = rr.im;
     out[5] = sqrt(a.re * a.re + a.im * a.im);
+  } else {
+    const double swr = emax / emin;
+    out[0] = rr.re;
+    out[1] = rr.im;
+    out[2] = be;
+    out[3] = sqrt(r / en);
+    out[4] = swr;
+    out[5] = (swr - 1.0) / (swr + 1.0);
   }
+}
+
+// scan and finish on device samples; scratch: FIT_BLOCKS doubles, then FIT_BLOCKS ints
+constexpr size_t FIT_SCRATCH = FIT_BLOCKS * (sizeof(double) + sizeof(int));
+int fit_dev(const cd* E, const double* tt, int npts, const FitGrid& F, void* scratch, double* out, cudaStream_t s) {
+  const int64_t ncand = F.na > 0 ? (int64_t)F.na * F.nb : F.nb;
+  const int nblk = (int)std::min<int64_t>(FIT_BLOCKS, cdiv(ncand, FIT_WARPS));
+  double* bres = (double*)scratch;
+  int* bidx = (int*)(bres + FIT_BLOCKS);
+  k_fit_scan<<<nblk, FIT_WARPS * 32, 0, s>>>(E, tt, npts, F, bres, bidx);
+  CK(cudaGetLastError());
+  k_fit_finish<<<1, 32, 0, s>>>(E, tt, npts, F, bres, bidx, nblk, out);
+  CK(cudaGetLastError());
+  return SCABEM_OK;
 }
 
 }  // namespace
@@ -1620,14 +1680,23 @@ int solve_impl(scabem_op* op, const void* bv, void* xv, int nrhs, int64_t ld, co
   return status;
 }
 
-static int fields_dev(scabem_op* op, const cd* x, const double* dpts, int npts, const scabem_source* inc, cd* dE,
-                      cudaStream_t s) {
-  int rc = compute_summ<double>(op, x, op->d.summ, s);
-  if (rc) return rc;
+// E (and H unless null) of one current set of x at device points
+static int fields_dev(scabem_op* op, const cd* x, const double* dpts, int npts, int side, const scabem_source* inc,
+                      FieldScratch& W, cd* dE, cd* dH, cudaStream_t s) {
+  if (int rc = compute_summ<double>(op, x, op->d.summ, s)) return rc;
+  const double k = side ? op->ke : op->ki, z = side ? op->ze : op->zi;
+  k_point_currents<<<(int)cdiv(op->Q, 128), 128, 0, s>>>(op->d.summ, op->tri, op->qp, op->qw, op->Q, op->q, k, z, side,
+                                                         W.pc);
+  CK(cudaGetLastError());
+  const dim3 g((unsigned)cdiv(npts, FP_PTS), W.nsl);
+  if (dH)
+    k_point_fields<true><<<g, FP_THREADS, 0, s>>>(W.pc, op->Q, dpts, npts, k, z, W.part);
+  else
+    k_point_fields<false><<<g, FP_THREADS, 0, s>>>(W.pc, op->Q, dpts, npts, k, z, W.part);
+  CK(cudaGetLastError());
   scabem_source S{};
   if (inc) S = *inc;
-  k_fields<<<npts, 256, 0, s>>>(op->d.summ, op->tri, op->qp, op->qw, op->Q, op->q, dpts, op->ki, op->zi, S,
-                                inc ? 1 : 0, dE);
+  k_point_finish<<<(int)cdiv(npts, 64), 64, 0, s>>>(W.part, W.nsl, dpts, npts, k, z, S, inc && side == 0 ? 1 : 0, dE, dH);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }
@@ -1636,11 +1705,13 @@ int fields_impl(scabem_op* op, const void* x, int nrhs, int64_t ld, const double
                 const scabem_source* inc, double* E, cudaStream_t s) {
   double* dpts = nullptr;
   cd* dE = nullptr;
+  FieldScratch W;
+  if (int rc = W.init(op, npts)) return rc;
   CK(cudaMalloc(&dpts, sizeof(double) * 3 * npts));
   CK(cudaMalloc(&dE, sizeof(cd) * 3 * npts));
   CK(cudaMemcpyAsync(dpts, pts, sizeof(double) * 3 * npts, cudaMemcpyHostToDevice, s));
   for (int col = 0; col < nrhs; ++col) {
-    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, inc, dE, s);
+    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, 0, inc, W, dE, nullptr, s);
     if (rc) return rc;
     CK(cudaMemcpyAsync(E + (int64_t)col * 6 * npts, dE, sizeof(cd) * 3 * npts, cudaMemcpyDeviceToHost, s));
   }
@@ -1650,23 +1721,19 @@ int fields_impl(scabem_op* op, const void* x, int nrhs, int64_t ld, const double
   return SCABEM_OK;
 }
 
-// E and H of one current set at host points (see k_fields_eh), per right-hand side.
+// E and H of one current set at host points, per right-hand side.
 int fields_eh_impl(scabem_op* op, const void* x, int nrhs, int64_t ld, const double* pts, int npts, int side,
                    const scabem_source* inc, double* E, double* H, cudaStream_t s) {
   double* dpts = nullptr;
   cd* dE = nullptr;
+  FieldScratch W;
+  if (int rc = W.init(op, npts)) return rc;
   CK(cudaMalloc(&dpts, sizeof(double) * 3 * npts));
   CK(cudaMalloc(&dE, sizeof(cd) * 6 * npts));
   CK(cudaMemcpyAsync(dpts, pts, sizeof(double) * 3 * npts, cudaMemcpyHostToDevice, s));
-  scabem_source S{};
-  if (inc) S = *inc;
-  const double k = side ? op->ke : op->ki, z = side ? op->ze : op->zi;
   for (int col = 0; col < nrhs; ++col) {
-    int rc = compute_summ<double>(op, (const cd*)x + (int64_t)col * ld, op->d.summ, s);
+    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, side, inc, W, dE, dE + 3 * npts, s);
     if (rc) return rc;
-    k_fields_eh<<<npts, 256, 0, s>>>(op->d.summ, op->tri, op->qp, op->qw, op->Q, op->q, dpts, k, z, side, S,
-                                     inc ? 1 : 0, dE, dE + 3 * npts);
-    CK(cudaGetLastError());
     CK(cudaMemcpyAsync(E + (int64_t)col * 6 * npts, dE, sizeof(cd) * 3 * npts, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(H + (int64_t)col * 6 * npts, dE + 3 * npts, sizeof(cd) * 3 * npts, cudaMemcpyDeviceToHost, s));
   }
@@ -1819,16 +1886,18 @@ int reflection_impl(scabem_op* op, const void* x, int nrhs, int64_t ld, const sc
   CK(cudaMalloc(&dtt, sizeof(double) * npts));
   CK(cudaMalloc(&dE, sizeof(cd) * 3 * npts));
   CK(cudaMalloc(&dc, sizeof(cd) * npts));
-  CK(cudaMalloc(&dout, sizeof(double) * 6));
+  CK(cudaMalloc(&dout, sizeof(double) * 6 + FIT_SCRATCH));
+  FieldScratch W;
+  if (int rc = W.init(op, npts)) return rc;
   CK(cudaMemcpyAsync(dpts, pts.data(), sizeof(double) * 3 * npts, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(dtt, tt.data(), sizeof(double) * npts, cudaMemcpyHostToDevice, s));
   for (int col = 0; col < nrhs; ++col) {
-    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, inc, dE, s);
+    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, 0, inc, W, dE, nullptr, s);
     if (rc) return rc;
     CK(cudaMemcpy2DAsync(dc, sizeof(cd), (const char*)dE + sizeof(cd) * pr->comp, 3 * sizeof(cd), sizeof(cd), npts,
                          cudaMemcpyDeviceToDevice, s));
-    k_fit<<<1, 256, 0, s>>>(dc, dtt, npts, pr->beta_lo, pr->beta_hi, pr->nbeta, dout);
-    CK(cudaGetLastError());
+    const FitGrid F{0.0, 0.0, 0, pr->beta_lo, pr->beta_hi, pr->nbeta};
+    if ((rc = fit_dev(dc, dtt, npts, F, dout + 6, dout, s))) return rc;
     CK(cudaMemcpyAsync(out + 6 * col, dout, sizeof(double) * 6, cudaMemcpyDeviceToHost, s));
   }
   CK(cudaStreamSynchronize(s));
@@ -1847,11 +1916,10 @@ int decay_fit_impl(const double* t, const double* E, int npts, double alo, doubl
   cd* dE = nullptr;
   CK(cudaMalloc(&dt, sizeof(double) * npts));
   CK(cudaMalloc(&dE, sizeof(cd) * npts));
-  CK(cudaMalloc(&dout, sizeof(double) * 6));
+  CK(cudaMalloc(&dout, sizeof(double) * 6 + FIT_SCRATCH));
   CK(cudaMemcpyAsync(dt, t, sizeof(double) * npts, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(dE, E, sizeof(cd) * npts, cudaMemcpyHostToDevice, s));
-  k_fit_decay<<<1, 256, 0, s>>>(dE, dt, npts, alo, ahi, na, blo, bhi, nb, dout);
-  CK(cudaGetLastError());
+  if (int rc = fit_dev(dE, dt, npts, FitGrid{alo, ahi, na, blo, bhi, nb}, dout + 6, dout, s)) return rc;
   CK(cudaMemcpyAsync(out, dout, sizeof(double) * 6, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   cudaFree(dt);
@@ -1877,16 +1945,18 @@ int decay_rate_impl(scabem_op* op, const void* x, int nrhs, int64_t ld, const sc
   CK(cudaMalloc(&dtt, sizeof(double) * npts));
   CK(cudaMalloc(&dE, sizeof(cd) * 3 * npts));
   CK(cudaMalloc(&dc, sizeof(cd) * npts));
-  CK(cudaMalloc(&dout, sizeof(double) * 6));
+  CK(cudaMalloc(&dout, sizeof(double) * 6 + FIT_SCRATCH));
+  FieldScratch W;
+  if (int rc = W.init(op, npts)) return rc;
   CK(cudaMemcpyAsync(dpts, pts.data(), sizeof(double) * 3 * npts, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(dtt, tt.data(), sizeof(double) * npts, cudaMemcpyHostToDevice, s));
   for (int col = 0; col < nrhs; ++col) {
-    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, inc, dE, s);
+    int rc = fields_dev(op, (const cd*)x + (int64_t)col * ld, dpts, npts, 0, inc, W, dE, nullptr, s);
     if (rc) return rc;
     CK(cudaMemcpy2DAsync(dc, sizeof(cd), (const char*)dE + sizeof(cd) * pr->comp, 3 * sizeof(cd), sizeof(cd), npts,
                          cudaMemcpyDeviceToDevice, s));
-    k_fit_decay<<<1, 256, 0, s>>>(dc, dtt, npts, alo, ahi, na, pr->beta_lo, pr->beta_hi, pr->nbeta, dout);
-    CK(cudaGetLastError());
+    const FitGrid F{alo, ahi, na, pr->beta_lo, pr->beta_hi, pr->nbeta};
+    if ((rc = fit_dev(dc, dtt, npts, F, dout + 6, dout, s))) return rc;
     CK(cudaMemcpyAsync(out + 6 * col, dout, sizeof(double) * 6, cudaMemcpyDeviceToHost, s));
   }
   CK(cudaStreamSynchronize(s));
