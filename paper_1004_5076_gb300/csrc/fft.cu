@@ -19,6 +19,8 @@
 // per stage.  The 1/(P0 P1 P2) scale is folded into the stored spectra.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace {
@@ -758,7 +760,7 @@ __global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __res
 // take a few microseconds, so the rest is kept short: the table is copied to
 // shared memory while the sources arrive (STAGE), the sources of all rows are in
 // flight at once, and the two axes' butterflies are one pass.  The CTA takes
-// the right-hand sides of a batch in turn.
+// every gridDim.z-th right-hand side of a batch in turn.
 constexpr int PS_THREADS = 256;
 constexpr int PS_W = 10;  // words per position: 8 fields, padded so that a row's stores spread over the banks
 
@@ -843,7 +845,8 @@ __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
     neg[h] = !ident && med && v >= 4;
     rp[h] = A + (int64_t)in0[h] * nac;
   }
-  for (int col = 0; col < ncol; ++col) {
+  bool first = true;
+  for (int col = blockIdx.z; col < ncol; col += gridDim.z, first = false) {
     for (int i = threadIdx.x; i < 2 * nb * PS_W; i += PS_THREADS) src[i] = czero<R>();
     __syncthreads();
     for (int jb = 0; jb < nac; jb += 128) {
@@ -865,7 +868,7 @@ __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
     }
     __syncthreads();
     parity_pass<R>(src, R1, R2, npl);
-    if (STAGE && col == 0) asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (STAGE && first) asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
     for (int u = threadIdx.x; u < (onepass ? PS_THREADS : tot); u += PS_THREADS) {
       Acc8<R> acc;
@@ -1080,7 +1083,9 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
     const size_t sm = parity_smem(nb, op->nac, stage ? words : 0, sizeof(cx<R>));
     auto fn = stage ? k_planes_parity<R, true> : k_planes_parity<R, false>;
     if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
-    fn<<<dim3(P0 / 2 + 1, 2), PS_THREADS, sm, s>>>(pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0, op->acoord, (int)op->nac,
+    // two CTAs per SM from the columns of a batch where the frequencies are few
+    const unsigned zs = (unsigned)std::min<int64_t>(ncol, cdiv(2 * 152, P0 + 2));
+    fn<<<dim3(P0 / 2 + 1, 2, zs), PS_THREADS, sm, s>>>(pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0, op->acoord, (int)op->nac,
                                                    op->R1, op->R2, words, id, col_stride_st(op), ncol);
     CK(cudaGetLastError());
     prof_mark(op, s);

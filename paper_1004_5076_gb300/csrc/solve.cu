@@ -508,17 +508,35 @@ __device__ __forceinline__ cdf ld_df(const cx<float>* p) {
 __device__ __forceinline__ cdf ld_df(const cx<double>* p) { return df_split(*p); }
 __device__ __forceinline__ cdf ld_df(const cdf* p) { return *p; }
 
+// Counts this block at *done; true in the last of n blocks, which sees the
+// others' writes (and resets the counter for the next launch).
+__device__ __forceinline__ bool last_block(int* done, int n) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(done, 1) == n - 1;
+    if (s_last) *done = 0;
+  }
+  __syncthreads();
+  if (s_last) __threadfence();
+  return s_last;
+}
+
 // part[(c * rb + b) * ldp + col] = sum over row block b of conj(V_c[:, col]) . w_c,
 // col in the tile blockIdx.y; with self_col, column nv is w_c itself (its
 // squared norm); skipped for columns with need[c] == 0.  The basis is held
 // as FP32 (hi, lo) pairs and w is read in its own precision WT (the
 // complex64 operator's output in the first pass, exact as a hi part); every
 // product is formed on the FP32 units with its rounding error and summed
-// with compensation, so that the sums keep about 48 bits.
+// with compensation, so that the sums keep about 48 bits.  The last row block
+// of a tile adds the parts into hout[c * ldh + col] (a separate reduction launch
+// cost 3.3 us of every Arnoldi step).
 template <typename WT>
 __global__ void __launch_bounds__(BG_THREADS) k_bdots(const cdf* __restrict__ V, int64_t csV, int nv,
                                                       const WT* __restrict__ w, int64_t N, cd* __restrict__ part,
-                                                      int ldp, const int* __restrict__ need, int self_col) {
+                                                      int ldp, const int* __restrict__ need, int self_col,
+                                                      cd* __restrict__ hout, int ldh, int* __restrict__ done) {
   constexpr bool WLO = !std::is_same<WT, cx<float>>::value;  // w has lo parts
   const int c = blockIdx.z;
   if (need && !need[c]) return;  // the whole block
@@ -603,31 +621,21 @@ __global__ void __launch_bounds__(BG_THREADS) k_bdots(const cdf* __restrict__ V,
     double* o = reinterpret_cast<double*>(part + ((int64_t)c * gridDim.x + blockIdx.x) * ldp + c0);
     o[threadIdx.x] = df_d(t);
   }
-}
-
-// h[c * ldh + col] = sum over the rb row blocks (grid: nv x K)
-__global__ void k_breduce(const cd* __restrict__ part, int rb, int ldp, cd* __restrict__ h, int ldh,
-                          const int* __restrict__ need) {
-  const int col = blockIdx.x, c = blockIdx.y;
-  if (need && !need[c]) return;
-  __shared__ double sre[BG_THREADS], sim[BG_THREADS];
-  double ar = 0.0, ai = 0.0;
-  for (int b = threadIdx.x; b < rb; b += blockDim.x) {
-    const cd v = part[((int64_t)c * rb + b) * ldp + col];
-    ar += v.re;
-    ai += v.im;
-  }
-  sre[threadIdx.x] = ar;
-  sim[threadIdx.x] = ai;
+  if (!last_block(done + c * gridDim.y + blockIdx.y, gridDim.x)) return;
+  // the tile's last block adds the row blocks' parts, in a fixed order
+  __shared__ double sr[BG_THREADS];
+  const int v2 = threadIdx.x % (2 * BG_TC), g = threadIdx.x / (2 * BG_TC);
+  double t = 0.0;
+  if (v2 < 2 * nc)
+    for (int b = g; b < gridDim.x; b += BG_THREADS / (2 * BG_TC))
+      t += __ldcg(reinterpret_cast<const double*>(part + ((int64_t)c * gridDim.x + b) * ldp + c0) + v2);
+  sr[threadIdx.x] = t;
   __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) {
-      sre[threadIdx.x] += sre[threadIdx.x + st];
-      sim[threadIdx.x] += sim[threadIdx.x + st];
-    }
+  for (int st = BG_THREADS / 2; st >= 2 * BG_TC; st >>= 1) {
+    if (threadIdx.x < st) sr[threadIdx.x] += sr[threadIdx.x + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) h[(int64_t)c * ldh + col] = mk(sre[0], sim[0]);
+  if (threadIdx.x < 2 * nc) reinterpret_cast<double*>(hout + (int64_t)c * ldh + c0)[threadIdx.x] = sr[threadIdx.x];
 }
 
 // Squared norm of each column of an FP64 vector per row block (grid:
@@ -672,7 +680,8 @@ template <typename WT>
 __global__ void __launch_bounds__(BG_THREADS) k_bvsub_norm(const cdf* __restrict__ V, int64_t csV, int nv,
                                                            const cd* __restrict__ h, int ldh, const WT* win,
                                                            cdf* wout, int64_t N, double* __restrict__ nparts,
-                                                           const int* __restrict__ need) {
+                                                           const int* __restrict__ need, double* __restrict__ nrm,
+                                                           int* __restrict__ set_need, int* __restrict__ done) {
   const int c = blockIdx.y;
   if (need && !need[c]) return;
   V += c * csV;
@@ -749,18 +758,32 @@ __global__ void __launch_bounds__(BG_THREADS) k_bvsub_norm(const cdf* __restrict
     for (int k = 1; k < BG_THREADS / 32; ++k) v = df_add(v, sm[k]);
     nparts[(int64_t)c * gridDim.x + blockIdx.x] = df_d(v);
   }
+  if (!last_block(done + c, gridDim.x)) return;
+  // the column's last block: |w| after the pass into nrm[4c] (pass 1: with |w|
+  // before it, from the self column of the dot products, and the DGKS test)
+  __shared__ double sr[BG_THREADS];
+  double v = 0.0;
+  for (int b = threadIdx.x; b < gridDim.x; b += BG_THREADS) v += __ldcg(nparts + (int64_t)c * gridDim.x + b);
+  sr[threadIdx.x] = v;
+  __syncthreads();
+  for (int st = BG_THREADS / 2; st > 0; st >>= 1) {
+    if (threadIdx.x < st) sr[threadIdx.x] += sr[threadIdx.x + st];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    const double n = sqrt(fmax(sr[0], 0.0));
+    nrm[4 * c] = n;
+    if (set_need) {
+      const double before = sqrt(fmax(h[nv].re, 0.0));
+      nrm[4 * c - 1] = before;
+      set_need[c] = !(n >= 0.70710678118654752 * before);
+    }
+  }
 }
 
-// out[c * ostride] = sqrt(sum of column c's row-block parts) (grid: K).  With
-// set_need, also need[c] = (out < |w| before the pass / sqrt 2), |w| before
-// read from out[c * ostride - 1] (the DGKS test after the first pass).
-__global__ void k_bnorm_fin(const double* __restrict__ nparts, int nb, double* __restrict__ out, int ostride,
-                            const int* __restrict__ need, int* __restrict__ set_need, const cd* __restrict__ selfdot,
-                            int ldh) {
+// out[c * ostride] = sqrt(sum of column c's row-block parts) (grid: K)
+__global__ void k_bnorm_fin(const double* __restrict__ nparts, int nb, double* __restrict__ out, int ostride) {
   const int c = blockIdx.x;
-  if (need && !need[c]) return;
-  // |w| before the pass, from the self column of the first pass's dot products
-  if (selfdot && threadIdx.x == 0) out[(int64_t)c * ostride - 1] = sqrt(fmax(selfdot[(int64_t)c * ldh].re, 0.0));
   __shared__ double sm[BG_THREADS];
   double v = 0.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) v += nparts[(int64_t)c * nb + b];
@@ -770,11 +793,7 @@ __global__ void k_bnorm_fin(const double* __restrict__ nparts, int nb, double* _
     if (threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    const double n = sqrt(fmax(sm[0], 0.0));
-    out[(int64_t)c * ostride] = n;
-    if (set_need) set_need[c] = !(n >= 0.70710678118654752 * out[(int64_t)c * ostride - 1]);
-  }
+  if (threadIdx.x == 0) out[(int64_t)c * ostride] = sqrt(fmax(sm[0], 0.0));
 }
 
 // Per-column state of the lockstep solver, on the device.
@@ -892,41 +911,77 @@ __global__ void __launch_bounds__(KBATCH * 32) k_givens(BState S, int j, int m, 
   if (threadIdx.x == 0) word[0] = n;
 }
 
-// v_c,j+1 = w_c / |w_c| (|w| after the last pass; zero when it vanishes), in
-// (hi, lo) pairs: 1 / |w| is split once per block and each product is
-// formed with its rounding error
+// x / |w| in (hi, lo) pairs, 1 / |w| = sh + sl: each product with its rounding error
+__device__ __forceinline__ cdf df_scale(cdf x, float sh, float sl) {
+  dfa r = {0.f, 0.f}, m = {0.f, 0.f};
+  df_mac(r, x.rh, sh);
+  df_small(r, x.rh, sl);
+  df_small(r, x.rl, sh);
+  df_mac(m, x.ih, sh);
+  df_small(m, x.ih, sl);
+  df_small(m, x.il, sh);
+  r = df_renorm(r);
+  m = df_renorm(m);
+  cdf o;
+  o.rh = r.h;
+  o.ih = m.h;
+  o.rl = r.l;
+  o.il = m.l;
+  return o;
+}
+// 1 / |w| of slot c (|w| after the last pass; zero when it vanishes) as (hi, lo)
+__device__ __forceinline__ void inv_norm(const double* nrm, const int* need, int c, float& sh, float& sl) {
+  const double n = need[c] ? nrm[4 * c + 2] : nrm[4 * c + 1];
+  const double sd = n > 1e-300 ? 1.0 / n : 0.0;
+  sh = __double2float_rn(sd);
+  sl = __double2float_rn(sd - (double)sh);
+}
+
+// v_c,j+1 = w_c / |w_c|
 __global__ void k_bscale(const cdf* __restrict__ w, cdf* __restrict__ V, int64_t csV, int j1,
                          const double* __restrict__ nrm, const int* __restrict__ need, int64_t N) {
   const int c = blockIdx.y;
-  __shared__ float s_s[2];
-  if (threadIdx.x == 0) {
-    const double n = need[c] ? nrm[4 * c + 2] : nrm[4 * c + 1];
-    const double sd = n > 1e-300 ? 1.0 / n : 0.0;
-    s_s[0] = __double2float_rn(sd);
-    s_s[1] = __double2float_rn(sd - (double)s_s[0]);
-  }
-  __syncthreads();
-  const float sh = s_s[0], sl = s_s[1];
+  float sh, sl;
+  inv_norm(nrm, need, c, sh, sl);
   w += c * N;
   V += c * csV + (int64_t)j1 * N;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const cdf x = w[i];
-    dfa r = {0.f, 0.f}, m = {0.f, 0.f};
-    df_mac(r, x.rh, sh);
-    df_small(r, x.rh, sl);
-    df_small(r, x.rl, sh);
-    df_mac(m, x.ih, sh);
-    df_small(m, x.ih, sl);
-    df_small(m, x.il, sh);
-    r = df_renorm(r);
-    m = df_renorm(m);
-    cdf o;
-    o.rh = r.h;
-    o.ih = m.h;
-    o.rl = r.l;
-    o.il = m.l;
-    V[i] = o;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+    V[i] = df_scale(w[i], sh, sl);
+}
+
+// The same and z_c = P^-1 v_c,j+1 in one launch, for the block-diagonal
+// preconditioner: one thread per (edge, row) scales the edge's entries, keeps
+// its own and forms its row of the block (P^-T when transposed), written in the
+// operator's precision.  One launch instead of two (4.4 + 9.3 us).
+template <typename TO>
+__global__ void __launch_bounds__(128) k_bscale_precond(const cdf* __restrict__ w, cdf* __restrict__ V, int64_t csV,
+                                                        int j1, const double* __restrict__ nrm,
+                                                        const int* __restrict__ need, int64_t N,
+                                                        const cd* __restrict__ pinv, const int32_t* __restrict__ eunk,
+                                                        int64_t ne, int transposed, cx<TO>* __restrict__ z) {
+  const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (u >= 3 * ne) return;
+  const int c = blockIdx.y;
+  const int64_t e = u / 3;
+  const int i = (int)(u - 3 * e);
+  int id[3];
+  for (int l = 0; l < 3; ++l) id[l] = eunk[3 * e + l];
+  const int nb = id[2] < 0 ? 2 : 3;
+  if (i >= nb) return;
+  cd P[3];
+  for (int l = 0; l < nb; ++l) P[l] = pinv[9 * e + (transposed ? 3 * l + i : 3 * i + l)];
+  w += c * N;
+  V += c * csV + (int64_t)j1 * N;
+  z += c * N;
+  float sh, sl;
+  inv_norm(nrm, need, c, sh, sl);
+  cd acc = mk(0.0, 0.0);
+  for (int l = 0; l < nb; ++l) {
+    const cdf v = df_scale(w[id[l]], sh, sl);
+    if (l == i) V[id[l]] = v;
+    acc += P[l] * df_join(v);
   }
+  z[id[i]] = cvt<TO>(acc);
 }
 
 // start of a cycle in slot c (the slot's right-hand side is column col[c]
@@ -1024,7 +1079,7 @@ __global__ void k_from_f(const cx<float>* __restrict__ a, cd* __restrict__ o, in
 constexpr int EW_BLOCKS = 4 * 152;  // element-wise kernels: 4 blocks of 256 threads per SM
 
 struct BWork {
-  int K = 0, m = 0;
+  int K = 0, Kcap = 0, m = 0;
   int64_t N = 0;
   bool tr = false;
   cdf* V = nullptr;          // K (m + 1) N basis, (hi, lo) pairs
@@ -1038,9 +1093,17 @@ struct BWork {
   cd* part = nullptr;        // K BG_BLOCKS (m + 1)
   double* nparts = nullptr;  // K BG_BLOCKS
   BState S;
+  // the Givens step of a column reads the step's h1, h2, norms and DGKS flags on
+  // a stream of its own, beside the next operator apply, so these alternate
+  // between two copies (BState points at the first)
+  cd *h1[2] = {nullptr, nullptr}, *h2[2] = {nullptr, nullptr};
+  double* nrm[2] = {nullptr, nullptr};
+  int* need[2] = {nullptr, nullptr};
+  int* done = nullptr;       // last-block counters of the Gram-Schmidt kernels
   int* word_h = nullptr;     // host-mapped {active columns, flags}
   int* word_d = nullptr;
-  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev[2] = {nullptr, nullptr}, gs[2] = {nullptr, nullptr};
   std::vector<void*> owned;
   template <typename T>
   int get(T** p, int64_t count) {
@@ -1050,13 +1113,19 @@ struct BWork {
     return SCABEM_OK;
   }
   ~BWork() {
+    if (side) {
+      cudaStreamSynchronize(side);
+      cudaStreamDestroy(side);
+    }
+    for (auto& e : gs)
+      if (e) cudaEventDestroy(e);
     for (void* p : owned) cudaFree(p);
     if (word_h) cudaFreeHost(word_h);
     for (auto& e : ev)
       if (e) cudaEventDestroy(e);
   }
   int init(int k, int mm, int64_t n, bool c64) {
-    K = k;
+    K = Kcap = k;
     m = mm;
     N = n;
     int rc;
@@ -1064,10 +1133,21 @@ struct BWork {
         (rc = get(&u, K * N)) || (rc = get(&t, K * N)) || (rc = get(&part, (int64_t)K * BG_BLOCKS * (m + 1))) ||
         (rc = get(&nparts, (int64_t)K * BG_BLOCKS)) || (rc = get(&S.H, (int64_t)K * m * (m + 1))) ||
         (rc = get(&S.cs, K * m)) || (rc = get(&S.sn, K * m)) || (rc = get(&S.g, K * (m + 1))) ||
-        (rc = get(&S.y, K * m)) || (rc = get(&S.h1, K * (m + 1))) || (rc = get(&S.h2, K * (m + 1))) ||
-        (rc = get(&S.nrm, 4 * K)) || (rc = get(&S.rn0, K)) || (rc = get(&S.est, K)) || (rc = get(&S.need, K)) ||
-        (rc = get(&S.act, K)) || (rc = get(&S.jc, K)) || (rc = get(&S.iters, K)) || (rc = get(&S.col, K)))
+        (rc = get(&S.y, K * m)) || (rc = get(&S.rn0, K)) || (rc = get(&S.est, K)) || (rc = get(&S.act, K)) || (rc = get(&S.jc, K)) || (rc = get(&S.iters, K)) || (rc = get(&S.col, K)))
       return rc;
+    for (int b = 0; b < 2; ++b)
+      if ((rc = get(&h1[b], K * (m + 1))) || (rc = get(&h2[b], K * (m + 1))) || (rc = get(&nrm[b], 4 * K)) ||
+          (rc = get(&need[b], K)))
+        return rc;
+    S.h1 = h1[0];
+    S.h2 = h2[0];
+    S.nrm = nrm[0];
+    S.need = need[0];
+    const int64_t nd = K * (cdiv(m + 1, BG_TC) + 2);
+    if ((rc = get(&done, nd))) return rc;
+    CK(cudaMemset(done, 0, sizeof(int) * nd));
+    CK(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+    for (auto& e : gs) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if (c64 && ((rc = get(&zf, K * N)) || (rc = get(&wf, K * N)))) return rc;
     CK(cudaHostAlloc(reinterpret_cast<void**>(&word_h), 2 * sizeof(int), cudaHostAllocMapped));
     CK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&word_d), word_h, 0));
@@ -1080,7 +1160,7 @@ struct BWork {
 int bnorms(const cd* x, BWork& W, double* out, int ostride, cudaStream_t s) {
   k_bnorm_parts<<<dim3(BG_BLOCKS, W.K), BG_THREADS, 0, s>>>(x, W.N, W.nparts);
   CK(cudaGetLastError());
-  k_bnorm_fin<<<W.K, BG_THREADS, 0, s>>>(W.nparts, BG_BLOCKS, out, ostride, nullptr, nullptr, nullptr, 0);
+  k_bnorm_fin<<<W.K, BG_THREADS, 0, s>>>(W.nparts, BG_BLOCKS, out, ostride);
   CK(cudaGetLastError());
   return SCABEM_OK;
 }
@@ -1188,59 +1268,75 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
       const cdf* vj = W.V + (int64_t)j * N;
       const bool bd = precond_is_block_diagonal(op, W.tr);
       const bool f32 = prec == SCABEM_C64 && bd;
-      if (f32) {
-        if (int rc = precond_apply_df(op, vj, W.zf, nullptr, s, W.tr, Ka, csV, N)) return rc;
-        if (int rc = bapply_f32(op, W, s)) return rc;
+      const int cur = j & 1;
+      if (bd) {  // steps after the first: the previous step's last launch left P^-1 v_j
+        if (j == 0)
+          if (int rc = precond_apply_df(op, vj, f32 ? W.zf : nullptr, f32 ? nullptr : W.z, s, W.tr, Ka, csV, N))
+            return rc;
       } else {
-        if (bd) {
-          if (int rc = precond_apply_df(op, vj, nullptr, W.z, s, W.tr, Ka, csV, N)) return rc;
-        } else {
-          k_bjoin<<<dim3(EW_BLOCKS / 4, Ka), 256, 0, s>>>(vj, csV, W.t, N);
-          CK(cudaGetLastError());
-          if (int rc = precond_apply(op, W.t, W.z, s, W.tr, Ka, N, N)) return rc;
-        }
-        if (int rc = bapply(op, W.z, W.w, prec, W, s)) return rc;
+        k_bjoin<<<dim3(EW_BLOCKS / 4, Ka), 256, 0, s>>>(vj, csV, W.t, N);
+        CK(cudaGetLastError());
+        if (int rc = precond_apply(op, W.t, W.z, s, W.tr, Ka, N, N)) return rc;
       }
+      if (int rc = f32 ? bapply_f32(op, W, s) : bapply(op, W.z, W.w, prec, W, s)) return rc;
       // first pass h1 = V^H w with |w|^2 in its column j + 1, w -= V h1, |w|; the
       // DGKS test; the second pass only where it asks
       const int tiles = (int)cdiv(j + 2, BG_TC);
       const int rb = std::max(8, BG_WAVE / tiles);
+      if (j >= 2) CK(cudaStreamWaitEvent(s, W.ev[cur], 0));  // the Givens step that read this copy
       for (int pass = 0; pass < 2; ++pass) {
-        const int* need = pass ? S.need : nullptr;
-        cd* h = pass ? S.h2 : S.h1;
+        const int* need = pass ? W.need[cur] : nullptr;
+        cd* h = pass ? W.h2[cur] : W.h1[cur];
         const int tl = pass ? (int)cdiv(j + 1, BG_TC) : tiles;
         const int rbp = pass ? std::max(8, BG_WAVE / tl) : rb;
         const dim3 gd(rbp, tl, Ka), gv(bv_blocks(N), Ka);
+        int* nd = W.done + (int64_t)W.Kcap * cdiv(m + 1, BG_TC);  // counters of the updates
         if (pass == 0 && f32)
-          k_bdots<cx<float>><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.wf, N, W.part, m + 1, need, 1);
+          k_bdots<cx<float>><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.wf, N, W.part, m + 1, need, 1, h, m + 1,
+                                                       W.done);
         else if (pass == 0)
-          k_bdots<cx<double>><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.w, N, W.part, m + 1, need, 1);
+          k_bdots<cx<double>><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.w, N, W.part, m + 1, need, 1, h, m + 1,
+                                                        W.done);
         else
-          k_bdots<cdf><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.wdf, N, W.part, m + 1, need, 0);
+          k_bdots<cdf><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.wdf, N, W.part, m + 1, need, 0, h, m + 1, W.done);
         CK(cudaGetLastError());
-        k_breduce<<<dim3(j + 1 + (pass ? 0 : 1), Ka), BG_THREADS, 0, s>>>(W.part, rbp, m + 1, h, m + 1, need);
-        CK(cudaGetLastError());
+        double* nr = W.nrm[cur] + 1 + pass;
+        int* sn = pass ? nullptr : W.need[cur];
         if (pass == 0 && f32)
           k_bvsub_norm<cx<float>><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.wf, W.wdf, N, W.nparts,
-                                                            need);
+                                                            need, nr, sn, nd);
         else if (pass == 0)
           k_bvsub_norm<cx<double>><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.w, W.wdf, N, W.nparts,
-                                                             need);
+                                                             need, nr, sn, nd);
         else
-          k_bvsub_norm<cdf><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.wdf, W.wdf, N, W.nparts, need);
-        CK(cudaGetLastError());
-        k_bnorm_fin<<<Ka, BG_THREADS, 0, s>>>(W.nparts, (int)gv.x, S.nrm + 1 + pass, 4, need,
-                                              pass ? nullptr : S.need, pass ? nullptr : S.h1 + (j + 1), m + 1);
+          k_bvsub_norm<cdf><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.wdf, W.wdf, N, W.nparts, need, nr,
+                                                      sn, nd);
         CK(cudaGetLastError());
       }
-      k_givens<<<1, KBATCH * 32, 0, s>>>(S, j, m, Ka, tol, W.word_d);
+      // the Givens step on its own stream (10 us of one CTA), beside the next apply
+      BState St = S;
+      St.h1 = W.h1[cur];
+      St.h2 = W.h2[cur];
+      St.nrm = W.nrm[cur];
+      St.need = W.need[cur];
+      CK(cudaEventRecord(W.gs[cur], s));
+      CK(cudaStreamWaitEvent(W.side, W.gs[cur], 0));
+      k_givens<<<1, KBATCH * 32, 0, W.side>>>(St, j, m, Ka, tol, W.word_d);
       CK(cudaGetLastError());
       if (j + 1 < m) {
-        k_bscale<<<dim3(EW_BLOCKS / 4, Ka), 256, 0, s>>>(W.wdf, W.V, csV, j + 1, S.nrm, S.need, N);
+        const dim3 gp((unsigned)cdiv(3 * op->ne, 128), Ka);
+        if (f32)
+          k_bscale_precond<float><<<gp, 128, 0, s>>>(W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N, op->pinv,
+                                                     op->eunk, op->ne, W.tr ? 1 : 0, W.zf);
+        else if (bd)
+          k_bscale_precond<double><<<gp, 128, 0, s>>>(W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N, op->pinv,
+                                                      op->eunk, op->ne, W.tr ? 1 : 0, W.z);
+        else
+          k_bscale<<<dim3(EW_BLOCKS / 4, Ka), 256, 0, s>>>(W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N);
         CK(cudaGetLastError());
       }
       // the host stays one step ahead: wait for the previous step, read its word
-      CK(cudaEventRecord(W.ev[j & 1], s));
+      CK(cudaEventRecord(W.ev[cur], W.side));
       if (j > 0) {
         CK(cudaEventSynchronize(W.ev[(j - 1) & 1]));
         const int flags = reinterpret_cast<volatile int*>(W.word_h)[1];
@@ -1258,6 +1354,9 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
         }
       }
     }
+    // the cycle's Givens steps are complete, on this stream too
+    CK(cudaStreamWaitEvent(s, W.ev[0], 0));
+    CK(cudaStreamWaitEvent(s, W.ev[1], 0));
     // least squares of the cycle into u (at each slot's column), then d = P^-1 u for all columns
     k_backsub<<<1, KBATCH * 32, sizeof(cd) * KBATCH * m, s>>>(S, m, Ka);
     CK(cudaGetLastError());
