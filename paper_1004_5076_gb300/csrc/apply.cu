@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(256) k_project(const cx<R>* __restrict__ x, in
   if (i >= ngp) return;  // whole warp
   const int lane = threadIdx.x & 31, comp = lane & 3, slot = lane >> 2;
   const int e0 = gpoff[i], el = e0 + gpl[i], e1 = gpoff[i + 1];
+  pdl_wait();
   cx<R> v[4];  // plain J, absorber J_e, absorber J_i, M
 #pragma unroll
   for (int c = 0; c < 4; ++c) v[c] = czero<R>();
@@ -473,6 +474,7 @@ __global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, c
   if (i >= ngp) return;  // whole warp; no CTA-wide barrier below
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   const int e0 = gpoff[i], el = e0 + gpl[i], e1 = gpoff[i + 1];
+  pdl_wait();
   cx<R> v[4], u[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) v[c] = u[c] = czero<R>();
@@ -553,10 +555,8 @@ int grid_potentials(scabem_op* op, const cx<R>* x, int64_t ldx, int k, cudaStrea
   PrecData<R>& pd = pdata<R>(op);
   prof_mark(op, s);
   prof_mark(op, s);  // (the summaries stage is part of the projection)
-  k_project<R><<<dim3((unsigned)cdiv(op->ngp * 32, 256), k), 256, 0, s>>>(
-      x, ldx, op->gp, op->gpoff, op->gpl, op->gpr, pd.gq, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, pd.src,
-      col_stride_src(op));
-  CK(cudaGetLastError());
+  CK(launch_pdl(k_project<R>, dim3((unsigned)cdiv(op->ngp * 32, 256), k), 256, 0, s, x, ldx, op->gp, op->gpoff, op->gpl,
+                op->gpr, pd.gq, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, pd.src, col_stride_src(op)));
   prof_mark(op, s);
   return fft_conv<R>(op, pd, s, false, k);
 }
@@ -584,10 +584,9 @@ int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s) {
 template <typename R>
 int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
-  k_grid_adj<R><<<(int)cdiv(op->ngp * 32, 256), 256, 0, s>>>(
-      ybar, op->gp, op->gpoff, op->gpl, op->gpr, op->gpe, pd.xw, op->nxl, op->ngp, (int64_t)op->n[0] * op->nac, op->nL,
-      op->nR, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi, pd.src);
-  CK(cudaGetLastError());
+  CK(launch_pdl(k_grid_adj<R>, dim3((unsigned)cdiv(op->ngp * 32, 256)), 256, 0, s, ybar, op->gp, op->gpoff, op->gpl,
+                op->gpr, op->gpe, pd.xw, op->nxl, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, (R)op->ke,
+                (R)op->ki, (R)op->ze, (R)op->zi, pd.src));
   if (int rc = fft_conv<R>(op, pd, s, true)) return rc;
   return rows_adjoint<R>(op, ybar, xbar, s);
 }

@@ -80,3 +80,29 @@ template <typename R>
 __device__ __forceinline__ cx<R> xadd(cx<R> v, int o) {
   return v + shfl_xor_cx(v, o);
 }
+
+// Programmatic dependent launch: a kernel of the product starts while its
+// predecessor in the stream still runs, sets itself up from data that no kernel
+// of the stream writes, and waits here for the predecessor's completion.  Only
+// then does it let its own successor start, so a kernel that is running knows
+// that everything before its direct predecessor has completed.  Every kernel
+// launched with launch_pdl comes through pdl_wait before it reads or writes
+// what the stream's kernels share.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+template <typename... KA, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<KA>(args)...);
+}

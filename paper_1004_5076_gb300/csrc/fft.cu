@@ -21,7 +21,7 @@
 
 #include <algorithm>
 
-#include "common.cuh"
+#include "device.cuh"
 
 namespace {
 
@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__
   const int a0 = blockIdx.x * CB;
   const int lcb = ilog2(CB);
   for (int i = threadIdx.x; i < P0; i += FFT_THREADS) tws[i] = tw[i];
+  pdl_wait();
   const int64_t fin = (int64_t)f * n_in * nac;
   for (int idx = threadIdx.x; idx < P0 * CB; idx += FFT_THREADS) {
     const int i0 = idx >> lcb, l = idx & (CB - 1);
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(FFT_THREADS)
   const int CB = 8 * NC;
   const int lcb = ilog2(CB), lnc = ilog2(NC);
   for (int i = threadIdx.x; i < P0; i += FFT_THREADS) tws[i] = tw[i];
+  pdl_wait();
   for (int idx = threadIdx.x; idx < P0 * CB; idx += FFT_THREADS) {
     const int i0 = idx >> lcb, l = idx & (CB - 1);
     const int fl = l >> lnc, cl = l & (NC - 1);
@@ -381,6 +383,7 @@ __global__ void __launch_bounds__(PLANE_THREADS) k_planes(const cx<R>* __restric
   const int f = blockIdx.y;
   for (int i = threadIdx.x; i < P1; i += PLANE_THREADS) t1[i] = tw1[i];
   for (int i = threadIdx.x; i < P2; i += PLANE_THREADS) t2[i] = tw2[i];
+  pdl_wait();
   __syncthreads();
   const int64_t C = (int64_t)n1 * n2;
   const cx<R>* src = A + ((int64_t)f * P0 + k0) * C;
@@ -569,6 +572,7 @@ __global__ void __launch_bounds__(P64_THREADS, sizeof(R) == 4 ? 3 : 1)
   w[0] = mk(R(1), R(0));
 #pragma unroll
   for (int k = 1; k < 8; ++k) w[k] = tw64[t * k];
+  pdl_wait();
   const int k0 = blockIdx.x, f = blockIdx.y;
   const int i1 = warp * 4 + sub;  // the row this lane works on in the row passes
   // rows no stencil covers are zero in and unused out; the test is per warp
@@ -715,6 +719,7 @@ __global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __res
   const int q0 = min(k0, P0 - k0);
   const cx<R>* gt = (med ? gtI : gtE) + (int64_t)q0 * R1 * R2;
   for (int i = threadIdx.x; i < R1 * R2; i += PD_THREADS) T[i] = gt[i];
+  pdl_wait();
   for (int idx = threadIdx.x; idx < nac * 8; idx += PD_THREADS) {
     const int v = idx / nac, j = idx - v * nac;  // consecutive threads: consecutive columns of one field
     const int f = ident ? 8 * med + v : (v < 4 ? (med ? 4 + v : v) : 8 + (v - 4));
@@ -845,6 +850,7 @@ __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
     neg[h] = !ident && med && v >= 4;
     rp[h] = A + (int64_t)in0[h] * nac;
   }
+  pdl_wait();
   bool first = true;
   for (int col = blockIdx.z; col < ncol; col += gridDim.z, first = false) {
     for (int i = threadIdx.x; i < 2 * nb * PS_W; i += PS_THREADS) src[i] = czero<R>();
@@ -1050,10 +1056,9 @@ static int axis0_inverse(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool ad
   auto fn = big ? (adjoint ? k_axis0_pm<R, false, 13> : k_axis0_pm<R, true, 13>)
                 : (adjoint ? k_axis0_pm<R, false, Tot<R>::L> : k_axis0_pm<R, true, Tot<R>::L>);
   if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
-  fn<<<dim3((unsigned)cdiv(op->nac, nc), 2, ncol), FFT_THREADS, sm, s>>>(
-      pd.stB, pd.grid, op->n[0], P0, op->acol, (int)op->nac, nc, pd.tw[0], col_stride_st(op), col_stride_pot(op), op->cst,
-      op->tdirect ? 1 : 0, (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi);
-  CK(cudaGetLastError());
+  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->nac, nc), 2, ncol), FFT_THREADS, sm, s, pd.stB, pd.grid, op->n[0], P0,
+      op->acol, (int)op->nac, nc, pd.tw[0], col_stride_st(op), col_stride_pot(op), op->cst, op->tdirect ? 1 : 0,
+      (R)op->ke, (R)op->ki, (R)op->ze, (R)op->zi));
   return SCABEM_OK;
 }
 
@@ -1071,10 +1076,9 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
   const size_t sm0 = (size_t)P0 * (cb + 1) * sizeof(cx<R>);
   // stage A
   if (int rc_ = set_max_smem(op->device, (const void*)k_axis0<R>, (int)sm0)) return rc_;
-  k_axis0<R><<<dim3((unsigned)cdiv(op->nac, cb), nf, ncol), FFT_THREADS, sm0, s>>>(
-      pd.src, pd.stA, n0, P0, op->acol, (int)op->nac, cb, pd.tw[0], col_stride_src(op), col_stride_st(op),
-      op->cst, op->tdirect ? 1 : 0);
-  CK(cudaGetLastError());
+  CK(launch_pdl(k_axis0<R>, dim3((unsigned)cdiv(op->nac, cb), nf, ncol), FFT_THREADS, sm0, s, pd.src, pd.stA, n0,
+      P0, op->acol, (int)op->nac, cb, pd.tw[0], col_stride_src(op), col_stride_st(op), op->cst, op->tdirect ? 1 :
+      0));
   prof_mark(op, s);
   // stage B
   if (op->tdirect && op->parity) {
@@ -1085,28 +1089,24 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
     if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm)) return rc_;
     // two CTAs per SM from the columns of a batch where the frequencies are few
     const unsigned zs = (unsigned)std::min<int64_t>(ncol, cdiv(2 * 152, P0 + 2));
-    fn<<<dim3(P0 / 2 + 1, 2, zs), PS_THREADS, sm, s>>>(pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0, op->acoord, (int)op->nac,
-                                                   op->R1, op->R2, words, id, col_stride_st(op), ncol);
-    CK(cudaGetLastError());
+    CK(launch_pdl(fn, dim3(P0 / 2 + 1, 2, zs), PS_THREADS, sm, s, pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0, op->acoord,
+      (int)op->nac, op->R1, op->R2, words, id, col_stride_st(op), ncol));
     prof_mark(op, s);
     return axis0_inverse(op, pd, s, adjoint, ncol);
   }
   if (op->tdirect) {
     const size_t sm = ((size_t)op->nac * 8 + (size_t)op->R1 * op->R2) * sizeof(cx<R>) + sizeof(int32_t) * op->nac;
     if (int rc_ = set_max_smem(op->device, (const void*)k_planes_direct<R>, (int)sm)) return rc_;
-    k_planes_direct<R><<<dim3(P0, 2, ncol), PD_THREADS, sm, s>>>(pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0,
-                                                                 (int)op->cst, op->acol, op->acoord, (int)op->nac,
-                                                                 op->R1, op->R2, id, col_stride_st(op), 1);
-    CK(cudaGetLastError());
+    CK(launch_pdl(k_planes_direct<R>, dim3(P0, 2, ncol), PD_THREADS, sm, s, pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0,
+      (int)op->cst, op->acol, op->acoord, (int)op->nac, op->R1, op->R2, id, col_stride_st(op), 1));
     prof_mark(op, s);
     return axis0_inverse(op, pd, s, adjoint, ncol);
   }
   if (P1 == 64 && P2 == 64) {
     const size_t sm = ((size_t)2 * 32 * 64 + (size_t)(P64_THREADS / 8) * P64_SCR) * sizeof(cx<R>);
     if (int rc_ = set_max_smem(op->device, (const void*)k_planes64<R>, (int)sm)) return rc_;
-    k_planes64<R><<<dim3(P0, nf, ncol), P64_THREADS, sm, s>>>(pd.stA, pd.stB, pd.ghat[0], pd.ghat[1], P0, pd.tw[1],
-                                                              op->rowmask, id, col_stride_st(op));
-    CK(cudaGetLastError());
+    CK(launch_pdl(k_planes64<R>, dim3(P0, nf, ncol), P64_THREADS, sm, s, pd.stA, pd.stB, pd.ghat[0], pd.ghat[1], P0,
+      pd.tw[1], op->rowmask, id, col_stride_st(op)));
     prof_mark(op, s);
     return axis0_inverse(op, pd, s, adjoint, ncol);
   }
@@ -1117,9 +1117,8 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
     return SCABEM_E_ARG;
   }
   if (int rc_ = set_max_smem(op->device, (const void*)fn, (int)sm1)) return rc_;
-  fn<<<dim3(P0, nf, ncol), PLANE_THREADS, sm1, s>>>(pd.stA, pd.stB, pd.ghat[0], pd.ghat[1], P0, n1, n2, pd.tw[1],
-                                                  pd.tw[2], id, col_stride_st(op));
-  CK(cudaGetLastError());
+  CK(launch_pdl(fn, dim3(P0, nf, ncol), PLANE_THREADS, sm1, s, pd.stA, pd.stB, pd.ghat[0], pd.ghat[1], P0, n1, n2,
+      pd.tw[1], pd.tw[2], id, col_stride_st(op)));
   prof_mark(op, s);
   return axis0_inverse(op, pd, s, adjoint, ncol);
 }

@@ -604,6 +604,9 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 && K == 1 ? 8 : 1)
     const RowDesc D = load_desc(T.desc + r);
     const int64_t x0 = D.xoff;
     near_row<R, K, false, LANES>(D, r >= nL, nL, nR, T.col, nmv, x, ldx, kc, lane, acc);
+    // the near part needs x only, which was complete before the predecessor
+    // (the last stage of the convolution) started: it runs beside that stage
+    pdl_wait();
     cx<R> ga[K];
 #pragma unroll
     for (int c = 0; c < K; ++c) ga[c] = czero<R>();
@@ -669,6 +672,7 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
     const RowDesc D = load_desc(T.desc + r);
     const int64_t x0 = D.xoff;
     near_row<R, 1, true, LANES>(D, r >= nL, nL, nR, T.col, nmt, y, 0, 1, lane, acc);
+    pdl_wait();  // as in k_rows
     const int h = lane & 7, grp = h >> 1;
     cx<R> gs[1] = {czero<R>()};
     if (r < nL)
@@ -729,9 +733,8 @@ int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
   PrecData<R>& pd = pdata<R>(op);
   const bool wide = wide_rows(op);
   auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
-  fn<<<(unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS), NM_THREADS, 0, s>>>(
-      row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc);
-  CK(cudaGetLastError());
+  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
+                row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc));
   return SCABEM_OK;
 }
 
@@ -759,9 +762,8 @@ int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
   const bool wide = wide_rows(op);
   auto fn = wide ? k_rows_adj<R, NM_THREADS> : k_rows_adj<R, 32>;
-  fn<<<(unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS), NM_THREADS, 0, s>>>(
-      row_tables(op, op->rdesc_t), pd.nmt, pd.gram, pd.xw, pd.grid, y, x);
-  CK(cudaGetLastError());
+  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
+                row_tables(op, op->rdesc_t), pd.nmt, pd.gram, pd.xw, pd.grid, y, x));
   return SCABEM_OK;
 }
 template int rows_adjoint<float>(scabem_op*, const cx<float>*, cx<float>*, cudaStream_t);

@@ -26,7 +26,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "common.cuh"
+#include "device.cuh"
 
 template <typename R>
 int compute_summ(scabem_op* op, const cx<R>* x, cx<R>* summ, cudaStream_t s);
@@ -539,6 +539,7 @@ __global__ void __launch_bounds__(BG_THREADS) k_bdots(const cdf* __restrict__ V,
                                                       cd* __restrict__ hout, int ldh, int* __restrict__ done) {
   constexpr bool WLO = !std::is_same<WT, cx<float>>::value;  // w has lo parts
   const int c = blockIdx.z;
+  pdl_wait();
   if (need && !need[c]) return;  // the whole block
   V += c * csV;
   w += c * N;
@@ -672,17 +673,22 @@ __global__ void __launch_bounds__(BG_THREADS) k_bnorm_parts(const cd* __restrict
 // per block; every product is formed with its rounding error and summed
 // with compensation.
 constexpr int GM_MAXM = 200;  // largest restart length (checked by the C ABI)
-constexpr int BV_KS = 4;
+// Short vectors take 16 lanes per row, so that the chip fills and the chains
+// shorten; long ones are bound by the basis stream and take 4.
+constexpr int BV_KS_LONG = 4, BV_KS_SHORT = 16;
+inline bool bv_short(int64_t N) { return N * BV_KS_LONG < (int64_t)BG_BLOCKS * BG_THREADS / 2; }
 inline unsigned bv_blocks(int64_t N) {
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(BG_BLOCKS, cdiv(N * BV_KS, BG_THREADS)));
+  const int ks = bv_short(N) ? BV_KS_SHORT : BV_KS_LONG;
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(BG_BLOCKS, cdiv(N * ks, BG_THREADS)));
 }
-template <typename WT>
+template <typename WT, int BV_KS>
 __global__ void __launch_bounds__(BG_THREADS) k_bvsub_norm(const cdf* __restrict__ V, int64_t csV, int nv,
                                                            const cd* __restrict__ h, int ldh, const WT* win,
                                                            cdf* wout, int64_t N, double* __restrict__ nparts,
                                                            const int* __restrict__ need, double* __restrict__ nrm,
                                                            int* __restrict__ set_need, int* __restrict__ done) {
   const int c = blockIdx.y;
+  pdl_wait();
   if (need && !need[c]) return;
   V += c * csV;
   win += c * N;
@@ -970,6 +976,7 @@ __global__ void __launch_bounds__(128) k_bscale_precond(const cdf* __restrict__ 
   if (i >= nb) return;
   cd P[3];
   for (int l = 0; l < nb; ++l) P[l] = pinv[9 * e + (transposed ? 3 * l + i : 3 * i + l)];
+  pdl_wait();
   w += c * N;
   V += c * csV + (int64_t)j1 * N;
   z += c * N;
@@ -1282,36 +1289,34 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
       // first pass h1 = V^H w with |w|^2 in its column j + 1, w -= V h1, |w|; the
       // DGKS test; the second pass only where it asks
       const int tiles = (int)cdiv(j + 2, BG_TC);
-      const int rb = std::max(8, BG_WAVE / tiles);
+      // row blocks of the dot products: one wave over all columns, two rows per thread at least
+      const int64_t rmax = cdiv(N, 2 * BG_THREADS);
+      auto row_blocks = [&](int t) { return (int)std::max<int64_t>(1, std::min<int64_t>(rmax, BG_WAVE / (t * Ka))); };
       if (j >= 2) CK(cudaStreamWaitEvent(s, W.ev[cur], 0));  // the Givens step that read this copy
       for (int pass = 0; pass < 2; ++pass) {
         const int* need = pass ? W.need[cur] : nullptr;
         cd* h = pass ? W.h2[cur] : W.h1[cur];
         const int tl = pass ? (int)cdiv(j + 1, BG_TC) : tiles;
-        const int rbp = pass ? std::max(8, BG_WAVE / tl) : rb;
-        const dim3 gd(rbp, tl, Ka), gv(bv_blocks(N), Ka);
+        const dim3 gd(row_blocks(tl), tl, Ka), gv(bv_blocks(N), Ka);
         int* nd = W.done + (int64_t)W.Kcap * cdiv(m + 1, BG_TC);  // counters of the updates
         if (pass == 0 && f32)
-          k_bdots<cx<float>><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.wf, N, W.part, m + 1, need, 1, h, m + 1,
-                                                       W.done);
+          CK(launch_pdl(k_bdots<cx<float>>, gd, BG_THREADS, 0, s, W.V, csV, j + 1, W.wf, N, W.part, m + 1, need, 1, h,
+                        m + 1, W.done));
         else if (pass == 0)
-          k_bdots<cx<double>><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.w, N, W.part, m + 1, need, 1, h, m + 1,
-                                                        W.done);
+          CK(launch_pdl(k_bdots<cx<double>>, gd, BG_THREADS, 0, s, W.V, csV, j + 1, W.w, N, W.part, m + 1, need, 1, h,
+                        m + 1, W.done));
         else
-          k_bdots<cdf><<<gd, BG_THREADS, 0, s>>>(W.V, csV, j + 1, W.wdf, N, W.part, m + 1, need, 0, h, m + 1, W.done);
-        CK(cudaGetLastError());
+          CK(launch_pdl(k_bdots<cdf>, gd, BG_THREADS, 0, s, W.V, csV, j + 1, W.wdf, N, W.part, m + 1, need, 0, h, m + 1,
+                        W.done));
         double* nr = W.nrm[cur] + 1 + pass;
         int* sn = pass ? nullptr : W.need[cur];
-        if (pass == 0 && f32)
-          k_bvsub_norm<cx<float>><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.wf, W.wdf, N, W.nparts,
-                                                            need, nr, sn, nd);
-        else if (pass == 0)
-          k_bvsub_norm<cx<double>><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.w, W.wdf, N, W.nparts,
-                                                             need, nr, sn, nd);
-        else
-          k_bvsub_norm<cdf><<<gv, BG_THREADS, 0, s>>>(W.V, csV, j + 1, h, m + 1, W.wdf, W.wdf, N, W.nparts, need, nr,
-                                                      sn, nd);
-        CK(cudaGetLastError());
+        auto update = [&](auto* in) {
+          using WT = std::remove_const_t<std::remove_pointer_t<decltype(in)>>;
+          auto fn = bv_short(N) ? k_bvsub_norm<WT, BV_KS_SHORT> : k_bvsub_norm<WT, BV_KS_LONG>;
+          return launch_pdl(fn, gv, BG_THREADS, 0, s, W.V, csV, j + 1, h, m + 1, in, W.wdf, N, W.nparts, need, nr, sn,
+                            nd);
+        };
+        CK(pass ? update(W.wdf) : f32 ? update(W.wf) : update(W.w));
       }
       // the Givens step on its own stream (10 us of one CTA), beside the next apply
       BState St = S;
@@ -1326,11 +1331,11 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
       if (j + 1 < m) {
         const dim3 gp((unsigned)cdiv(3 * op->ne, 128), Ka);
         if (f32)
-          k_bscale_precond<float><<<gp, 128, 0, s>>>(W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N, op->pinv,
-                                                     op->eunk, op->ne, W.tr ? 1 : 0, W.zf);
+          CK(launch_pdl(k_bscale_precond<float>, gp, 128, 0, s, W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N,
+                        op->pinv, op->eunk, op->ne, W.tr ? 1 : 0, W.zf));
         else if (bd)
-          k_bscale_precond<double><<<gp, 128, 0, s>>>(W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N, op->pinv,
-                                                      op->eunk, op->ne, W.tr ? 1 : 0, W.z);
+          CK(launch_pdl(k_bscale_precond<double>, gp, 128, 0, s, W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N,
+                        op->pinv, op->eunk, op->ne, W.tr ? 1 : 0, W.z));
         else
           k_bscale<<<dim3(EW_BLOCKS / 4, Ka), 256, 0, s>>>(W.wdf, W.V, csV, j + 1, W.nrm[cur], W.need[cur], N);
         CK(cudaGetLastError());
