@@ -58,46 +58,63 @@ __global__ void k_summ(const cx<R>* __restrict__ x, const int32_t* __restrict__ 
 // covers stay zero from set-up.  The sum order is fixed, so the result does not
 // depend on thread timing.  Bound by the latency of the (edge -> unknown)
 // loads out of L2; the unrolled loop keeps four entries per lane in flight.
-template <typename R>
+// A warp takes K right-hand sides, which share the entries' weights and indices.
+template <typename R, int K>
 __global__ void __launch_bounds__(256) k_project(const cx<R>* __restrict__ x, int64_t ldx,
                                                  const int32_t* __restrict__ gp, const int32_t* __restrict__ gpoff,
                                                  const int32_t* __restrict__ gpl, const int32_t* __restrict__ gpr,
                                                  const R* __restrict__ gq, int64_t ngp, int64_t npt, int64_t nL,
-                                                 int64_t nR, cx<R>* __restrict__ src, int64_t cs) {
-  x += blockIdx.y * ldx;  // right-hand side blockIdx.y of a batch
-  src += blockIdx.y * cs;
+                                                 int64_t nR, cx<R>* __restrict__ src, int64_t cs, int kc) {
+  const int c0 = blockIdx.y * K;  // right-hand sides c0 .. of a batch of kc
+  x += c0 * ldx;
+  src += c0 * cs;
+  kc = min(K, kc - c0);
   const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (i >= ngp) return;  // whole warp
   const int lane = threadIdx.x & 31, comp = lane & 3, slot = lane >> 2;
   const int e0 = gpoff[i], el = e0 + gpl[i], e1 = gpoff[i + 1];
   pdl_wait();
-  cx<R> v[4];  // plain J, absorber J_e, absorber J_i, M
+  cx<R> v[K][4];  // plain J, absorber J_e, absorber J_i, M
 #pragma unroll
-  for (int c = 0; c < 4; ++c) v[c] = czero<R>();
-#pragma unroll 4
+  for (int k = 0; k < K; ++k)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[k][c] = czero<R>();
+  constexpr int UN = K == 1 ? 4 : K < 4 ? 2 : 1;
+#pragma unroll UN
   for (int e = e0 + slot; e < el; e += 8) {
     const cx<R>* xm = x + gpr[e];
     const R w = gq[4 * (int64_t)e + comp];
-    axpy2(v[0], w, xm[0]);
-    axpy2(v[3], w, xm[nL]);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k < kc) {
+        axpy2(v[k][0], w, xm[k * ldx]);
+        axpy2(v[k][3], w, xm[k * ldx + nL]);
+      }
   }
-#pragma unroll 4
+#pragma unroll UN
   for (int e = el + slot; e < e1; e += 8) {
     const cx<R>* xm = x + nL + gpr[e];
     const R w = gq[4 * (int64_t)e + comp];
-    axpy2(v[1], w, xm[0]);
-    axpy2(v[2], w, xm[nR]);
-    axpy2(v[3], w, xm[2 * nR]);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k < kc) {
+        axpy2(v[k][1], w, xm[k * ldx]);
+        axpy2(v[k][2], w, xm[k * ldx + nR]);
+        axpy2(v[k][3], w, xm[k * ldx + 2 * nR]);
+      }
   }
-  halve(v, 2, lane, 16);
-  halve(v, 1, lane, 8);
-  v[0] = xadd(v[0], 4);
-  // lane bits (4, 3) hold plain J, J_e, J_i, M: add the plain part to J_e and -J_i
-  const cx<R> pe = shfl_xor_cx(v[0], 8), pi = shfl_xor_cx(v[0], 16);
   const int set = (lane >> 3) - 1;
-  if (set < 0 || (lane & 4)) return;
-  const cx<R> o = set == 0 ? v[0] + pe : set == 1 ? v[0] - pi : v[0];
-  src[(int64_t)(4 * set + comp) * npt + gp[i]] = o;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    halve(v[k], 2, lane, 16);
+    halve(v[k], 1, lane, 8);
+    v[k][0] = xadd(v[k][0], 4);
+    // lane bits (4, 3) hold plain J, J_e, J_i, M: add the plain part to J_e and -J_i
+    const cx<R> pe = shfl_xor_cx(v[k][0], 8), pi = shfl_xor_cx(v[k][0], 16);
+    if (set < 0 || (lane & 4) || k >= kc) continue;
+    const cx<R> o = set == 0 ? v[k][0] + pe : set == 1 ? v[k][0] - pi : v[k][0];
+    src[k * cs + (int64_t)(4 * set + comp) * npt + gp[i]] = o;
+  }
 }
 
 // Two consecutive complex values of shared memory on a 16-byte boundary.
@@ -555,8 +572,11 @@ int grid_potentials(scabem_op* op, const cx<R>* x, int64_t ldx, int k, cudaStrea
   PrecData<R>& pd = pdata<R>(op);
   prof_mark(op, s);
   prof_mark(op, s);  // (the summaries stage is part of the projection)
-  CK(launch_pdl(k_project<R>, dim3((unsigned)cdiv(op->ngp * 32, 256), k), 256, 0, s, x, ldx, op->gp, op->gpoff, op->gpl,
-                op->gpr, pd.gq, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, pd.src, col_stride_src(op)));
+  const int kw = k == 1 ? 1 : k == 2 || k == 3 ? k : 4;
+  auto fn = kw == 1 ? k_project<R, 1> : kw == 2 ? k_project<R, 2> : kw == 3 ? k_project<R, 3> : k_project<R, 4>;
+  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ngp * 32, 256), (unsigned)cdiv(k, kw)), 256, 0, s, x, ldx, op->gp, op->gpoff,
+                op->gpl, op->gpr, pd.gq, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, pd.src,
+                col_stride_src(op), k));
   prof_mark(op, s);
   return fft_conv<R>(op, pd, s, false, k);
 }

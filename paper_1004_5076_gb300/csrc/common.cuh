@@ -208,9 +208,9 @@ struct scabem_op {
   bool planes_fit = true;   // the (y, z) plane fits the 2-D FFT plane kernels
   bool direct_fits = true;  // the active columns fit one CTA of the direct (y, z) sums
   int a0_lines = 0;         // lines per CTA of the axis-0 transforms (0: the default rule)
-  // columns per (field, k0) of the axis-0 intermediates stA, stB: the nac
-  // active columns in order (compact) for the direct (y, z) sums, all n1 n2
-  // for the FFT planes
+  // columns per (field, k0) of the axis-0 intermediates: the nac active columns
+  // in order (compact; stB with the 16 fields of a column together) for the
+  // direct (y, z) sums, all n1 n2 for the FFT planes
   int64_t cst = 0;
   bool tdirect = false;
   bool parity = false;  // the direct sums run block-diagonalised by parity (gt: its tables)

@@ -210,8 +210,9 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__
 }
 
 // Stage C with point-major output, on the nac active columns only (the
-// potentials are read nowhere else; the input holds Cin columns per (field,
-// k0), compact or whole planes as stage A wrote them): one CTA owns NC of them
+// potentials are read nowhere else; the input is [k0][active column][16 fields]
+// from the direct sums (compact), [field][k0][Cin columns] from the FFT planes):
+// one CTA owns NC of them
 // for the eight fields of one set (J: A, phi of both media; M: F, psi of both)
 // over axis 0, line l = field * NC + column, and writes groups of four complex
 // values, whole 32-byte sectors in complex64, at out[(i0 * nac + column) * 32]
@@ -241,11 +242,13 @@ __global__ void __launch_bounds__(FFT_THREADS)
   pdl_wait();
   for (int idx = threadIdx.x; idx < P0 * CB; idx += FFT_THREADS) {
     const int i0 = idx >> lcb, l = idx & (CB - 1);
-    const int fl = l >> lnc, cl = l & (NC - 1);
+    const int fl = compact ? l & 7 : l >> lnc, cl = compact ? l >> 3 : l & (NC - 1);  // in the input's order
     const int field = (fl & 3) + 4 * set + 2 * (fl & 4);
     cx<R> v = czero<R>();
-    if (a0 + cl < nac) v = in[((int64_t)field * P0 + i0) * Cin + (compact ? a0 + cl : acol[a0 + cl])];
-    b0[idx] = v;
+    if (a0 + cl < nac)
+      v = compact ? in[((int64_t)i0 * nac + a0 + cl) * NFIELD_OUT + field]
+                  : in[((int64_t)field * P0 + i0) * Cin + acol[a0 + cl]];
+    b0[(i0 << lcb) + fl * NC + cl] = v;
   }
   __syncthreads();
   fft_lines<R, 1, TOTL>(b0, ilog2(P0), lcb, 1, CB, tws);
@@ -705,10 +708,9 @@ struct Acc8<double> {
 template <typename R>
 __global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __restrict__ A, cx<R>* __restrict__ B,
                                                               const cx<R>* __restrict__ gtE,
-                                                              const cx<R>* __restrict__ gtI, int P0, int C,
-                                                              const int32_t* __restrict__ acol,
+                                                              const cx<R>* __restrict__ gtI, int P0,
                                                               const int32_t* __restrict__ acoord, int nac, int R1,
-                                                              int R2, int ident, int64_t cs, int compact) {
+                                                              int R2, int ident, int64_t cs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   A += blockIdx.z * cs;  // right-hand side blockIdx.z
   B += blockIdx.z * cs;
@@ -723,7 +725,7 @@ __global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __res
   for (int idx = threadIdx.x; idx < nac * 8; idx += PD_THREADS) {
     const int v = idx / nac, j = idx - v * nac;  // consecutive threads: consecutive columns of one field
     const int f = ident ? 8 * med + v : (v < 4 ? (med ? 4 + v : v) : 8 + (v - 4));
-    src[j * 8 + v] = A[((int64_t)f * P0 + k0) * C + (compact ? j : acol[j])];
+    src[j * 8 + v] = A[((int64_t)f * P0 + k0) * nac + j];
   }
   for (int i = threadIdx.x; i < nac; i += PD_THREADS) crd[i] = acoord[i];
   __syncthreads();
@@ -737,12 +739,10 @@ __global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __res
       const int d1 = abs(i1 - (cj >> 16)), d2 = abs(i2 - (cj & 0xffff));
       acc.mac(T[d1 * R2 + d2], src + j * 8);
     }
-    const int64_t c = compact ? i : acol[i];
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
-      const int fo = ident ? 8 * med + v : (med ? (v < 4 ? 8 + v : 12 + (v - 4)) : v);
       const cx<R> val = acc.get(v);
-      B[((int64_t)fo * P0 + k0) * C + c] = (!ident && med && v >= 4) ? -val : val;
+      B[((int64_t)k0 * nac + i) * NFIELD_OUT + 8 * med + v] = (!ident && med && v >= 4) ? -val : val;
     }
   }
 }
@@ -837,18 +837,12 @@ __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
     crd[i] = (c >> 16) * R2 + (c & 0xffff);
   }
   // rows (plane, field) warp and warp + 8; four columns per lane in flight
-  int in0[2], out0[2];
-  bool neg[2];
   const cx<R>* rp[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int v = warp, pl = h, k0 = pl ? P0 - q0 : q0;
     const int f = ident ? 8 * med + v : (v < 4 ? (med ? 4 + v : v) : 8 + (v - 4));
-    const int fo = ident ? 8 * med + v : (med ? (v < 4 ? 8 + v : 12 + (v - 4)) : v);
-    in0[h] = f * P0 + k0;
-    out0[h] = fo * P0 + k0;
-    neg[h] = !ident && med && v >= 4;
-    rp[h] = A + (int64_t)in0[h] * nac;
+    rp[h] = A + (int64_t)(f * P0 + k0) * nac;
   }
   pdl_wait();
   bool first = true;
@@ -913,15 +907,12 @@ __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
     __syncthreads();
     parity_pass<R>(res, R1, R2, npl);
     __syncthreads();
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (h < npl) {
-        cx<R>* o = B + col * cs + (int64_t)out0[h] * nac;
-        for (int j = lane; j < nac; j += 32) {
-          const cx<R> val = res[(h * nb + crd[j]) * PS_W + warp];
-          o[j] = neg[h] ? -val : val;
-        }
-      }
+    for (int u = threadIdx.x; u < npl * nac * 8; u += PS_THREADS) {  // fields fastest: 64 bytes in complex64
+      const int v = u & 7, w = u >> 3, h = w >= nac, j = w - h * nac;
+      const cx<R> val = res[(h * nb + crd[j]) * PS_W + v];
+      B[col * cs + ((int64_t)(h ? P0 - q0 : q0) * nac + j) * NFIELD_OUT + 8 * med + v] =
+          (!ident && med && v >= 4) ? -val : val;
+    }
     __syncthreads();
   }
 }
@@ -1098,7 +1089,7 @@ int fft_conv(scabem_op* op, PrecData<R>& pd, cudaStream_t s, bool adjoint, int n
     const size_t sm = ((size_t)op->nac * 8 + (size_t)op->R1 * op->R2) * sizeof(cx<R>) + sizeof(int32_t) * op->nac;
     if (int rc_ = set_max_smem(op->device, (const void*)k_planes_direct<R>, (int)sm)) return rc_;
     CK(launch_pdl(k_planes_direct<R>, dim3(P0, 2, ncol), PD_THREADS, sm, s, pd.stA, pd.stB, pd.gt[0], pd.gt[1], P0,
-      (int)op->cst, op->acol, op->acoord, (int)op->nac, op->R1, op->R2, id, col_stride_st(op), 1));
+                  op->acoord, (int)op->nac, op->R1, op->R2, id, col_stride_st(op)));
     prof_mark(op, s);
     return axis0_inverse(op, pd, s, adjoint, ncol);
   }

@@ -588,12 +588,20 @@ struct RowTables {
 // weights (HBM on large operators) and by load latency: the near values are
 // loaded a column ahead, the weights two entries at a time.
 template <typename R, int K, int LANES>
-__global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 && K == 1 ? 8 : 1)
+__global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : K == 2 ? 7 : 6)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
            const cx<R>* __restrict__ pot, int64_t cs_g, const cx<R>* __restrict__ x, int64_t ldx, cx<R>* __restrict__ y,
            int64_t ldy, int kc) {
-  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
-  const int lane = threadIdx.x % LANES;
+  // unit = (row, group of K right-hand sides): a row's groups sit in
+  // neighbouring warps and share its values and weights through L1
+  const int64_t unit = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
+  const int ng = (kc + K - 1) / K;
+  const int64_t r = K == 1 ? unit : unit / ng;
+  const int lane = threadIdx.x % LANES, c0 = K == 1 ? 0 : (int)(unit - r * ng) * K;
+  x += c0 * ldx;
+  y += c0 * ldy;
+  pot += c0 * cs_g;
+  kc = min(K, kc - c0);
   const int64_t nL = T.nL, nR = T.ne - nL;
   cx<R> acc[3][K];
 #pragma unroll
@@ -733,7 +741,8 @@ int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
   PrecData<R>& pd = pdata<R>(op);
   const bool wide = wide_rows(op);
   auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
-  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
+  const int64_t units = op->ne * cdiv(kc, K);
+  CK(launch_pdl(fn, dim3((unsigned)cdiv(units * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
                 row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc));
   return SCABEM_OK;
 }
@@ -743,15 +752,12 @@ int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
 // y_c = A x_c from the potentials pd.grid (column c) and the near matrix, c < kc <= KBATCH
 template <typename R>
 int rows_apply(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
-  switch (kc) {
-    case 1: return launch_rows<R, 1>(op, x, ldx, y, ldy, kc, s);
-    case 2: return launch_rows<R, 2>(op, x, ldx, y, ldy, kc, s);
-    case 3: return launch_rows<R, 3>(op, x, ldx, y, ldy, kc, s);
-    case 4: return launch_rows<R, 4>(op, x, ldx, y, ldy, kc, s);
-    case 5:
-    case 6: return launch_rows<R, 6>(op, x, ldx, y, ldy, kc, s);
-    default: return launch_rows<R, 8>(op, x, ldx, y, ldy, kc, s);
-  }
+  // at most four right-hand sides per warp: eight hold 126 registers and half
+  // the warps (325 us for 8 columns of the 12 um guide)
+  if (kc == 1) return launch_rows<R, 1>(op, x, ldx, y, ldy, kc, s);
+  if (kc == 2 || kc == 4) return launch_rows<R, 2>(op, x, ldx, y, ldy, kc, s);
+  if (kc == 3 || kc == 5 || kc == 6) return launch_rows<R, 3>(op, x, ldx, y, ldy, kc, s);
+  return launch_rows<R, 4>(op, x, ldx, y, ldy, kc, s);
 }
 template int rows_apply<float>(scabem_op*, const cx<float>*, int64_t, cx<float>*, int64_t, int, cudaStream_t);
 template int rows_apply<double>(scabem_op*, const cx<double>*, int64_t, cx<double>*, int64_t, int, cudaStream_t);
