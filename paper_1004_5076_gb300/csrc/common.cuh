@@ -258,6 +258,8 @@ struct scabem_op {
   int32_t* eunk = nullptr;  // ne * 3: unknown (= row) indices of the edge, -1 unused
   cx<double>* pinv = nullptr;  // ne * 9
   int precond_singular = 0;
+  int precond_bad[2] = {0, 0};  // singular blocks per edge class
+  bool precond_plain = false;   // the plain edges' blocks are formed
   Circulant circ;
   PrecData<float> f;
   PrecData<double> d;

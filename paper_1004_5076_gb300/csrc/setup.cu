@@ -7,7 +7,7 @@
 #include <cmath>
 #include <vector>
 
-#include "common.cuh"
+#include "device.cuh"
 
 namespace {
 
@@ -235,28 +235,30 @@ __global__ void k_parity_tables(const cx<double>* __restrict__ F, int P0, int P1
 }
 
 // ---------------------------------------------------------------- near list
-__global__ void k_near_count(const double* __restrict__ tri, int64_t nt, double r2, int32_t* __restrict__ cnt) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// Triangles whose centroids lie within r_near of each target's, in ascending
+// order: one warp per target, 32 sources at a time (one thread per target left
+// 56 CTAs for 7100 triangles and took 2.2 ms per pass, 0.67 ms now, FP64).  src null: counts only.
+__global__ void __launch_bounds__(128) k_near_list(const double* __restrict__ tri, int64_t nt, double r2,
+                                                   const int32_t* __restrict__ off, int32_t* __restrict__ cnt,
+                                                   int32_t* __restrict__ src) {
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (t >= nt) return;
+  const int lane = threadIdx.x & 31;
   const double cx0 = tri[16 * t + 9], cy0 = tri[16 * t + 10], cz0 = tri[16 * t + 11];
-  int c = 0;
-  for (int64_t s = 0; s < nt; ++s) {
-    const double dx = cx0 - tri[16 * s + 9], dy = cy0 - tri[16 * s + 10], dz = cz0 - tri[16 * s + 11];
-    if (dx * dx + dy * dy + dz * dz < r2) ++c;
+  int64_t n = src ? off[t] : 0;
+#pragma unroll 2
+  for (int64_t s0 = 0; s0 < nt; s0 += 32) {
+    const int64_t s = s0 + lane;
+    bool in = false;
+    if (s < nt) {
+      const double dx = cx0 - tri[16 * s + 9], dy = cy0 - tri[16 * s + 10], dz = cz0 - tri[16 * s + 11];
+      in = dx * dx + dy * dy + dz * dz < r2;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (in && src) src[n + __popc(m & ((1u << lane) - 1))] = (int32_t)s;
+    n += __popc(m);
   }
-  cnt[t] = c;
-}
-
-__global__ void k_near_fill(const double* __restrict__ tri, int64_t nt, double r2, const int32_t* __restrict__ off,
-                            int32_t* __restrict__ src) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= nt) return;
-  const double cx0 = tri[16 * t + 9], cy0 = tri[16 * t + 10], cz0 = tri[16 * t + 11];
-  int64_t o = off[t];
-  for (int64_t s = 0; s < nt; ++s) {
-    const double dx = cx0 - tri[16 * s + 9], dy = cy0 - tri[16 * s + 10], dz = cz0 - tri[16 * s + 11];
-    if (dx * dx + dy * dy + dz * dz < r2) src[o++] = (int32_t)s;
-  }
+  if (cnt && lane == 0) cnt[t] = (int32_t)n;
 }
 
 // ---------------------------------------------------------------- panel integrals
@@ -301,18 +303,37 @@ __device__ void static_tri(const double* r, const double* v, const double* nrm, 
   for (int c = 0; c < 3; ++c) gI[c] -= sg * om * nrm[c];
 }
 
+// Smooth remainder (exp(-jkR) - 1)/R and its radial derivative over R, for
+// iR = 1/R.  1 - cos(kR) without cancellation: sin^2/(1 + cos) near the origin.
+__device__ __forceinline__ void smooth_kernel(double k, double R, double iR, cx<double>& gv, cx<double>& gd) {
+  const double kr = k * R, iR3 = iR * iR * iR;
+  double sn, cn;
+  sincos(kr, &sn, &cn);
+  const double c1 = cn > 0.0 ? sn * sn / (1.0 + cn) : 1.0 - cn;
+  gv = mk(-c1 * iR, -sn * iR);
+  gd = mk((c1 - kr * sn) * iR3, (sn - kr * cn) * iR3);
+}
+
 // Near-field precorrection: one thread per (near pair, target point).  For
 // both media, exact potential moments (P0, P1, Q, C) of the source panel at
 // the target point minus the grid's version of the same interaction.
 // corr layout: [pair][target point][medium][NCORR component], so that the ten
-// values one (point, medium) lane of the point kernel reads are contiguous.
-template <typename RG>
-__global__ void k_near_corr(const double* __restrict__ tri, const double* __restrict__ qp, const double* __restrict__ qw,
-                            const int32_t* __restrict__ base, const double* __restrict__ Ld,
-                            const double* __restrict__ dLd, const int32_t* __restrict__ noff,
-                            const int32_t* __restrict__ nsrc, int64_t nt, int64_t npairs, int q, int p, double ke,
-                            double ki, const cx<RG>* __restrict__ Ge, const cx<RG>* __restrict__ Gi, int P0, int P1,
-                            int P2, cx<double>* __restrict__ outd, cx<float>* __restrict__ outf) {
+// values one (point, medium) lane of a reader needs are contiguous.
+//
+// Bound by the FP64 pipe: per source point and medium the grid interaction is
+// a sum over (2P - 1)^3 offsets of the Green table, for the value and the three
+// derivatives.  Contracting z, then y, then x keeps two, three and four partial
+// sums instead of forming four weights per offset: 690 FMAs at P = 3 against
+// 1600 (89 -> 42 ms for the 0.38 M pairs of a 5 um guide).  The smooth exact part
+// goes into the same sums, with one sincos per medium and one reciprocal.
+template <int P>
+__global__ void __launch_bounds__(128)
+    k_near_corr(const double* __restrict__ tri, const double* __restrict__ qp, const double* __restrict__ qw,
+                const int32_t* __restrict__ base, const double* __restrict__ Ld, const double* __restrict__ dLd,
+                const int32_t* __restrict__ noff, const int32_t* __restrict__ nsrc, int64_t nt, int64_t npairs, int q,
+                double ke, double ki, const cx<double>* __restrict__ Ge, const cx<double>* __restrict__ Gi, int P0,
+                int P1, int P2, cx<double>* __restrict__ outd, cx<float>* __restrict__ outf) {
+  constexpr int ND = 2 * P - 1;
   int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gid >= npairs * q) return;
   const int64_t j = gid / q;
@@ -331,128 +352,124 @@ __global__ void k_near_corr(const double* __restrict__ tri, const double* __rest
   const double* ts = tri + 16 * s;
   const double cs[3] = {ts[9], ts[10], ts[11]};
   const bool self = (s == t);
-  double I, Irho[3], gI[3], rho[3];
-  static_tri(r, ts, ts + 12, self, I, Irho, gI, rho);
   const double inv4pi = 1.0 / (4.0 * M_PI);
   // target stencil weights
   const int ba[3] = {base[3 * Qa], base[3 * Qa + 1], base[3 * Qa + 2]};
-  double La[3][MAXP], dLa[3][MAXP];
+  double La[3][P], dLa[3][P];
+#pragma unroll
   for (int ax = 0; ax < 3; ++ax)
-    for (int i = 0; i < p; ++i) {
-      La[ax][i] = Ld[(3 * Qa + ax) * p + i];
-      dLa[ax][i] = dLd[(3 * Qa + ax) * p + i];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      La[ax][i] = Ld[(3 * Qa + ax) * P + i];
+      dLa[ax][i] = dLd[(3 * Qa + ax) * P + i];
     }
-  const int nd = 2 * p - 1;
-  for (int med = 0; med < 2; ++med) {
-    const double k = med == 0 ? ke : ki;
-    const cx<RG>* G = med == 0 ? Ge : Gi;
-    cx<double> P0s = mk(0.0, 0.0), P1s[3], Qs[3];
-    cx<double> P0g = mk(0.0, 0.0), P1g[3], Qg[3], Cg[3];
-    for (int c = 0; c < 3; ++c) P1s[c] = Qs[c] = P1g[c] = Qg[c] = Cg[c] = mk(0.0, 0.0);
-    for (int b = 0; b < q; ++b) {
-      const int64_t Qb = s * q + b;
-      const double rb[3] = {qp[3 * Qb], qp[3 * Qb + 1], qp[3 * Qb + 2]};
-      const double wb = qw[Qb];
-      const double rel[3] = {rb[0] - cs[0], rb[1] - cs[1], rb[2] - cs[2]};
-      const double D[3] = {r[0] - rb[0], r[1] - rb[1], r[2] - rb[2]};
-      // smooth remainder (exp(-jkR) - 1)/R and its radial derivative
-      cx<double> gv, gd;
-      if (self && b == a) {
-        gv = mk(0.0, -k);
-        gd = mk(0.0, 0.0);
-      } else {
-        const double R = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
-        const double kr = k * R;
-        double sn, cn, sh, ch;
-        sincos(kr, &sn, &cn);
-        sincos(0.5 * kr, &sh, &ch);
-        gv = mk(-2.0 * sh * sh / R, -sn / R);
-        gd = mk((2.0 * sh * sh - kr * sn) / (R * R * R), (sn - kr * cn) / (R * R * R));
-      }
-      P0s += wb * gv;
-      for (int c = 0; c < 3; ++c) {
-        P1s[c] += (wb * rel[c]) * gv;
-        Qs[c] += (wb * D[c]) * gd;
-      }
-      // grid interaction Gh(a,b) and grad_a Gh(a,b), separable over axes
-      const int bb[3] = {base[3 * Qb], base[3 * Qb + 1], base[3 * Qb + 2]};
-      double K[3][2 * MAXP - 1], dK[3][2 * MAXP - 1];
-      for (int ax = 0; ax < 3; ++ax) {
-        double Lb[MAXP];
-        for (int i = 0; i < p; ++i) Lb[i] = Ld[(3 * Qb + ax) * p + i];
-        for (int dd = 0; dd < nd; ++dd) {
-          const int delta = dd - (p - 1);
-          double sv = 0.0, sd = 0.0;
-          for (int i = 0; i < p; ++i) {
-            const int ip = i - delta;
-            if (ip < 0 || ip >= p) continue;
-            sv += La[ax][i] * Lb[ip];
-            sd += dLa[ax][i] * Lb[ip];
-          }
-          K[ax][dd] = sv;
-          dK[ax][dd] = sd;
+  cx<double> acc[2][NCORR];
+#pragma unroll
+  for (int med = 0; med < 2; ++med)
+#pragma unroll
+    for (int c = 0; c < NCORR; ++c) acc[med][c] = mk(0.0, 0.0);
+  for (int b = 0; b < q; ++b) {
+    const int64_t Qb = s * q + b;
+    const double rb[3] = {qp[3 * Qb], qp[3 * Qb + 1], qp[3 * Qb + 2]};
+    const double wb = qw[Qb];
+    const double rel[3] = {rb[0] - cs[0], rb[1] - cs[1], rb[2] - cs[2]};
+    const double D[3] = {r[0] - rb[0], r[1] - rb[1], r[2] - rb[2]};
+    const bool same = self && b == a;
+    const double R = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]), iR = same ? 0.0 : 1.0 / R;
+    // grid interaction Gh(a,b) and grad_a Gh(a,b): weights per offset, separable over axes
+    double K[3][ND], dK[3][ND];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      double Lb[P];
+#pragma unroll
+      for (int i = 0; i < P; ++i) Lb[i] = Ld[(3 * Qb + ax) * P + i];
+#pragma unroll
+      for (int dd = 0; dd < ND; ++dd) {
+        double sv = 0.0, sd = 0.0;
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+          const int ip = i - (dd - (P - 1));
+          if (ip < 0 || ip >= P) continue;
+          sv += La[ax][i] * Lb[ip];
+          sd += dLa[ax][i] * Lb[ip];
         }
+        K[ax][dd] = sv;
+        dK[ax][dd] = sd;
       }
-      const int Dg[3] = {ba[0] - bb[0], ba[1] - bb[1], ba[2] - bb[2]};
+    }
+    const int D0 = ba[0] - base[3 * Qb] - (P - 1), D1 = ba[1] - base[3 * Qb + 1] - (P - 1),
+              D2 = ba[2] - base[3 * Qb + 2] - (P - 1);
+    int o2[ND];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) o2[d] = D2 + d < 0 ? D2 + d + P2 : D2 + d;
+#pragma unroll
+    for (int med = 0; med < 2; ++med) {
+      const cx<double>* G = med == 0 ? Ge : Gi;
       cx<double> gh = mk(0.0, 0.0), gx = gh, gy = gh, gz = gh;
-      for (int dx = 0; dx < nd; ++dx) {
-        int o0 = Dg[0] + dx - (p - 1);
-        o0 = o0 < 0 ? o0 + P0 : o0;
-        for (int dy = 0; dy < nd; ++dy) {
-          int o1 = Dg[1] + dy - (p - 1);
-          o1 = o1 < 0 ? o1 + P1 : o1;
-          const double kxy = K[0][dx] * K[1][dy];
-          const double dxy = dK[0][dx] * K[1][dy];
-          const double xdy = K[0][dx] * dK[1][dy];
-          const cx<RG>* row = G + ((int64_t)o0 * P1 + o1) * P2;
-          for (int dz = 0; dz < nd; ++dz) {
-            int o2 = Dg[2] + dz - (p - 1);
-            o2 = o2 < 0 ? o2 + P2 : o2;
-            const cx<RG> gg = row[o2];
-            const cx<double> g = mk((double)gg.re, (double)gg.im);
-            axpy(gh, kxy * K[2][dz], g);
-            axpy(gx, dxy * K[2][dz], g);
-            axpy(gy, xdy * K[2][dz], g);
-            axpy(gz, kxy * dK[2][dz], g);
+#pragma unroll
+      for (int dx = 0; dx < ND; ++dx) {
+        const int o0 = D0 + dx < 0 ? D0 + dx + P0 : D0 + dx;
+        cx<double> h = mk(0.0, 0.0), hy = h, hz = h;
+#pragma unroll
+        for (int dy = 0; dy < ND; ++dy) {
+          const int o1 = D1 + dy < 0 ? D1 + dy + P1 : D1 + dy;
+          const cx<double>* row = G + ((int64_t)o0 * P1 + o1) * P2;
+          cx<double> u = mk(0.0, 0.0), v = u;
+#pragma unroll
+          for (int dz = 0; dz < ND; ++dz) {
+            const cx<double> g = row[o2[dz]];
+            axpy(u, K[2][dz], g);
+            axpy(v, dK[2][dz], g);
           }
+          axpy(h, K[1][dy], u);
+          axpy(hy, dK[1][dy], u);
+          axpy(hz, K[1][dy], v);
         }
+        axpy(gh, K[0][dx], h);
+        axpy(gx, dK[0][dx], h);
+        axpy(gy, K[0][dx], hy);
+        axpy(gz, K[0][dx], hz);
       }
-      P0g += wb * gh;
-      const cx<double> gg3[3] = {gx, gy, gz};
+      cx<double> gv = mk(0.0, med == 0 ? -ke : -ki), gd = mk(0.0, 0.0);
+      if (!same) smooth_kernel(med == 0 ? ke : ki, R, iR, gv, gd);
+      // exact minus grid: value v, gradient Q, and Q x rel for the curl
+      const cx<double> v = wb * (inv4pi * gv - gh);
+      const cx<double> f = inv4pi * gd;
+      const cx<double> Q[3] = {wb * (D[0] * f - gx), wb * (D[1] * f - gy), wb * (D[2] * f - gz)};
+      acc[med][0] += v;
+#pragma unroll
       for (int c = 0; c < 3; ++c) {
-        P1g[c] += (wb * rel[c]) * gh;
-        Qg[c] += wb * gg3[c];
+        const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+        axpy(acc[med][1 + c], rel[c], v);
+        acc[med][4 + c] += Q[c];
+        axpy(acc[med][7 + c], rel[c2], Q[c1]);
+        axpy(acc[med][7 + c], -rel[c1], Q[c2]);
       }
-      // Cg += wb * grad Gh x rel
-      Cg[0] += wb * (rel[2] * gg3[1] - rel[1] * gg3[2]);
-      Cg[1] += wb * (rel[0] * gg3[2] - rel[2] * gg3[0]);
-      Cg[2] += wb * (rel[1] * gg3[0] - rel[0] * gg3[1]);
-    }
-    // exact moments
-    cx<double> P0e = inv4pi * (mk(I, 0.0) + P0s);
-    cx<double> P1e[3], Qe[3], Ce[3];
-    for (int c = 0; c < 3; ++c) {
-      P1e[c] = inv4pi * (mk(Irho[c] + (rho[c] - cs[c]) * I, 0.0) + P1s[c]);
-      Qe[c] = inv4pi * (mk(gI[c], 0.0) + Qs[c]);
-    }
-    const double rc[3] = {r[0] - cs[0], r[1] - cs[1], r[2] - cs[2]};
-    Ce[0] = rc[2] * Qe[1] - rc[1] * Qe[2];
-    Ce[1] = rc[0] * Qe[2] - rc[2] * Qe[0];
-    Ce[2] = rc[1] * Qe[0] - rc[0] * Qe[1];
-    cx<double> o[NCORR];
-    o[0] = P0e - P0g;
-    for (int c = 0; c < 3; ++c) {
-      o[1 + c] = P1e[c] - P1g[c];
-      o[4 + c] = Qe[c] - Qg[c];
-      o[7 + c] = Ce[c] - Cg[c];
-    }
-    // [pair][point][medium][component]
-    for (int c = 0; c < NCORR; ++c) {
-      const int64_t dst = ((j * q + a) * 2 + med) * NCORR + c;
-      if (outd) outd[dst] = o[c];
-      if (outf) outf[dst] = mk((float)o[c].re, (float)o[c].im);
     }
   }
+  // the static integrals, the same for both media
+  double I, Irho[3], gI[3], rho[3];
+  static_tri(r, ts, ts + 12, self, I, Irho, gI, rho);
+  const double rc[3] = {r[0] - cs[0], r[1] - cs[1], r[2] - cs[2]};
+  double st[NCORR];
+  st[0] = inv4pi * I;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+    st[1 + c] = inv4pi * (Irho[c] + (rho[c] - cs[c]) * I);
+    st[4 + c] = inv4pi * gI[c];
+    st[7 + c] = inv4pi * (rc[c2] * gI[c1] - rc[c1] * gI[c2]);
+  }
+  // [pair][point][medium][component]
+#pragma unroll
+  for (int med = 0; med < 2; ++med)
+#pragma unroll
+    for (int c = 0; c < NCORR; ++c) {
+      const cx<double> o = acc[med][c] + mk(st[c], 0.0);
+      const int64_t dst = (gid * 2 + med) * NCORR + c;
+      if (outd) outd[dst] = o;
+      if (outf) outf[dst] = mk((float)o.re, (float)o.im);
+    }
 }
 
 // Testing geometry per quadrature point Qi (point a of triangle t), formed in
@@ -552,46 +569,45 @@ __global__ void k_sigma_copy(const double* __restrict__ in, int64_t Q, double* _
 using cd = cx<double>;
 
 // Exact moments P0, P1 (about the source centroid), Q, C = Q x (r - c) of
-// source triangle s at point r for wavenumber k, given the static integrals.
+// source triangle s at point r for both wavenumbers, given the static integrals.
 __device__ void exact_moments(const double* r, const double* ts, const double* __restrict__ qp,
-                              const double* __restrict__ qw, int64_t s, int q, bool self, int aself, double k,
-                              double I, const double* Irho, const double* gI, const double* rho, cd* o) {
+                              const double* __restrict__ qw, int64_t s, int q, bool self, int aself, const double* k,
+                              double I, const double* Irho, const double* gI, const double* rho, cd (*o)[10]) {
   const double cs[3] = {ts[9], ts[10], ts[11]};
-  cd P0s = mk(0.0, 0.0), P1s[3], Qs[3];
-  for (int c = 0; c < 3; ++c) P1s[c] = Qs[c] = mk(0.0, 0.0);
+  cd P0s[2], P1s[2][3], Qs[2][3];
+  for (int m = 0; m < 2; ++m) {
+    P0s[m] = mk(0.0, 0.0);
+    for (int c = 0; c < 3; ++c) P1s[m][c] = Qs[m][c] = mk(0.0, 0.0);
+  }
   for (int b = 0; b < q; ++b) {
     const int64_t Qb = s * q + b;
     const double D[3] = {r[0] - qp[3 * Qb], r[1] - qp[3 * Qb + 1], r[2] - qp[3 * Qb + 2]};
     const double wb = qw[Qb];
-    cd gv, gd;
-    if (self && b == aself) {
-      gv = mk(0.0, -k);
-      gd = mk(0.0, 0.0);
-    } else {
-      const double R = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
-      const double kr = k * R;
-      double sn, cn, sh, ch;
-      sincos(kr, &sn, &cn);
-      sincos(0.5 * kr, &sh, &ch);
-      gv = mk(-2.0 * sh * sh / R, -sn / R);
-      gd = mk((2.0 * sh * sh - kr * sn) / (R * R * R), (sn - kr * cn) / (R * R * R));
-    }
-    P0s += wb * gv;
-    for (int c = 0; c < 3; ++c) {
-      P1s[c] += (wb * (qp[3 * Qb + c] - cs[c])) * gv;
-      Qs[c] += (wb * D[c]) * gd;
+    const bool same = self && b == aself;
+    const double R = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]), iR = same ? 0.0 : 1.0 / R;
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      cd gv = mk(0.0, -k[m]), gd = mk(0.0, 0.0);
+      if (!same) smooth_kernel(k[m], R, iR, gv, gd);
+      P0s[m] += wb * gv;
+      for (int c = 0; c < 3; ++c) {
+        P1s[m][c] += (wb * (qp[3 * Qb + c] - cs[c])) * gv;
+        Qs[m][c] += (wb * D[c]) * gd;
+      }
     }
   }
   const double f = 1.0 / (4.0 * M_PI);
-  o[0] = f * (mk(I, 0.0) + P0s);
-  for (int c = 0; c < 3; ++c) {
-    o[1 + c] = f * (mk(Irho[c] + (rho[c] - cs[c]) * I, 0.0) + P1s[c]);
-    o[4 + c] = f * (mk(gI[c], 0.0) + Qs[c]);
-  }
   const double rc[3] = {r[0] - cs[0], r[1] - cs[1], r[2] - cs[2]};
-  o[7] = rc[2] * o[5] - rc[1] * o[6];
-  o[8] = rc[0] * o[6] - rc[2] * o[4];
-  o[9] = rc[1] * o[4] - rc[0] * o[5];
+  for (int m = 0; m < 2; ++m) {
+    o[m][0] = f * (mk(I, 0.0) + P0s[m]);
+    for (int c = 0; c < 3; ++c) {
+      o[m][1 + c] = f * (mk(Irho[c] + (rho[c] - cs[c]) * I, 0.0) + P1s[m][c]);
+      o[m][4 + c] = f * (mk(gI[c], 0.0) + Qs[m][c]);
+    }
+    o[m][7] = rc[2] * o[m][5] - rc[1] * o[m][6];
+    o[m][8] = rc[0] * o[m][6] - rc[2] * o[m][4];
+    o[m][9] = rc[1] * o[m][4] - rc[0] * o[m][5];
+  }
 }
 
 // Potentials A, phi, grad phi, curl A of the summary (alpha, beta) from moments.
@@ -690,64 +706,71 @@ __device__ bool cinv(cd* A, int n) {
   return true;
 }
 
-// One thread per edge: the edge's own block of the operator (its two
-// triangles as targets and sources, exact panel interactions), inverted.
+// One warp per edge of class cls: the edge's own block of the operator (its two
+// triangles as targets and sources, exact panel interactions), inverted.  A
+// lane takes one (target triangle, source triangle, target point): 4 q of them
+// for q at most 7 (one thread per edge: 2.5 ms for 10600 edges; 1.2 ms now, FP64 pipe).
 // Columns: plain edge (J^L, M^L), absorber edge (J_e^R, J_i^R, M^R); rows:
 // plain (Eq. 1, Eq. 2), absorber (Eq. 3, Eq. 13, Eq. 14).
 __global__ void k_precond(const double* __restrict__ tri, const double* __restrict__ cX, const double* __restrict__ qp,
                           const double* __restrict__ qw, const double* __restrict__ sig,
-                          const int32_t* __restrict__ etk, const int32_t* __restrict__ ecls, int64_t ne, int q,
-                          double ke, double ki, double ze, double zi, cd* __restrict__ pinv, int* __restrict__ bad) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= ne) return;
+                          const int32_t* __restrict__ etk, const int32_t* __restrict__ ecls, int cls, int64_t ne,
+                          int q, double ke, double ki, double ze, double zi, cd* __restrict__ pinv,
+                          int* __restrict__ bad) {
+  const int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (e >= ne || ecls[e] != cls) return;  // whole warp
+  const int lane = threadIdx.x & 31;
+  const double kk[2] = {ke, ki};
   // B[col type (Je, Ji, M)][row type 0..3]
   cd B[3][4];
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 4; ++j) B[i][j] = mk(0.0, 0.0);
   const cd zero10[10] = {};
-  for (int it = 0; it < 2; ++it) {
+  for (int u = lane; u < 4 * q; u += 32) {
+    const int it = u / (2 * q), is = u / q & 1, a = u % q;
     const int64_t t = etk[4 * e + 2 * it];
     const int kt = etk[4 * e + 2 * it + 1];
     const double* gt = tri + 16 * t;
     const double cxt = cX[3 * t + kt];
     const double* n = gt + 12;
-    for (int is = 0; is < 2; ++is) {
-      const int64_t s = etk[4 * e + 2 * is];
-      const int ks = etk[4 * e + 2 * is + 1];
-      const double* gs = tri + 16 * s;
-      const double al = cX[3 * s + ks];
-      const double be[3] = {al * (gs[3 * ks] - gs[9]), al * (gs[3 * ks + 1] - gs[10]), al * (gs[3 * ks + 2] - gs[11])};
-      const bool self = (s == t);
-      for (int a = 0; a < q; ++a) {
-        const int64_t Qa = t * q + a;
-        const double r[3] = {qp[3 * Qa], qp[3 * Qa + 1], qp[3 * Qa + 2]};
-        double I, Irho[3], gI[3], rho[3];
-        static_tri(r, gs, gs + 12, self, I, Irho, gI, rho);
-        cd me[10], mi[10], Ue[10], Ui[10], nUi[10];
-        exact_moments(r, gs, qp, qw, s, q, self, a, ke, I, Irho, gI, rho, me);
-        exact_moments(r, gs, qp, qw, s, q, self, a, ki, I, Irho, gI, rho, mi);
-        unit_pot(me, al, be, Ue);
-        unit_pot(mi, al, be, Ui);
-        for (int c = 0; c < 10; ++c) nUi[c] = -Ui[c];
-        double X[3], nX[3], Xe[3] = {0, 0, 0};
-        for (int c = 0; c < 3; ++c) X[c] = cxt * (r[c] - gt[3 * kt + c]);
-        nX[0] = n[1] * X[2] - n[2] * X[1];
-        nX[1] = n[2] * X[0] - n[0] * X[2];
-        nX[2] = n[0] * X[1] - n[1] * X[0];
-        if (self)
-          for (int c = 0; c < 3; ++c) Xe[c] = al * (r[c] - gs[3 * ks + c]);  // the basis itself at the point
-        const double zero3[3] = {0, 0, 0};
-        const double w = qw[Qa], sg = sig[Qa];
-        cd o[4];
-        test_point(Ue, zero10, zero10, zero10, ke, ki, ze, zi, X, nX, 2.0 * cxt, n, sg, Xe, zero3, o);
-        for (int j = 0; j < 4; ++j) B[0][j] += w * o[j];
-        test_point(zero10, zero10, Ui, zero10, ke, ki, ze, zi, X, nX, 2.0 * cxt, n, sg, Xe, zero3, o);
-        for (int j = 0; j < 4; ++j) B[1][j] += w * o[j];
-        test_point(zero10, Ue, zero10, nUi, ke, ki, ze, zi, X, nX, 2.0 * cxt, n, sg, zero3, Xe, o);
-        for (int j = 0; j < 4; ++j) B[2][j] += w * o[j];
-      }
-    }
+    const int64_t s = etk[4 * e + 2 * is];
+    const int ks = etk[4 * e + 2 * is + 1];
+    const double* gs = tri + 16 * s;
+    const double al = cX[3 * s + ks];
+    const double be[3] = {al * (gs[3 * ks] - gs[9]), al * (gs[3 * ks + 1] - gs[10]), al * (gs[3 * ks + 2] - gs[11])};
+    const bool self = (s == t);
+    const int64_t Qa = t * q + a;
+    const double r[3] = {qp[3 * Qa], qp[3 * Qa + 1], qp[3 * Qa + 2]};
+    double I, Irho[3], gI[3], rho[3];
+    static_tri(r, gs, gs + 12, self, I, Irho, gI, rho);
+    cd mom[2][10], Ue[10], Ui[10], nUi[10];
+    exact_moments(r, gs, qp, qw, s, q, self, a, kk, I, Irho, gI, rho, mom);
+    unit_pot(mom[0], al, be, Ue);
+    unit_pot(mom[1], al, be, Ui);
+    for (int c = 0; c < 10; ++c) nUi[c] = -Ui[c];
+    double X[3], nX[3], Xe[3] = {0, 0, 0};
+    for (int c = 0; c < 3; ++c) X[c] = cxt * (r[c] - gt[3 * kt + c]);
+    nX[0] = n[1] * X[2] - n[2] * X[1];
+    nX[1] = n[2] * X[0] - n[0] * X[2];
+    nX[2] = n[0] * X[1] - n[1] * X[0];
+    if (self)
+      for (int c = 0; c < 3; ++c) Xe[c] = al * (r[c] - gs[3 * ks + c]);  // the basis itself at the point
+    const double zero3[3] = {0, 0, 0};
+    const double w = qw[Qa], sg = sig[Qa];
+    cd o[4];
+    test_point(Ue, zero10, zero10, zero10, ke, ki, ze, zi, X, nX, 2.0 * cxt, n, sg, Xe, zero3, o);
+    for (int j = 0; j < 4; ++j) B[0][j] += w * o[j];
+    test_point(zero10, zero10, Ui, zero10, ke, ki, ze, zi, X, nX, 2.0 * cxt, n, sg, Xe, zero3, o);
+    for (int j = 0; j < 4; ++j) B[1][j] += w * o[j];
+    test_point(zero10, Ue, zero10, nUi, ke, ki, ze, zi, X, nX, 2.0 * cxt, n, sg, zero3, Xe, o);
+    for (int j = 0; j < 4; ++j) B[2][j] += w * o[j];
   }
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      for (int d = 16; d > 0; d >>= 1) B[i][j] = xadd(B[i][j], d);
+  if (lane) return;
   cd A[9];
   for (int i = 0; i < 9; ++i) A[i] = mk(0.0, 0.0);
   int nb;
@@ -881,15 +904,20 @@ int setup_gather(scabem_op* op, cudaStream_t s) {
   return SCABEM_OK;
 }
 
+// The blocks of the plain edges do not depend on sigma: they are formed once,
+// those of the absorber edges whenever sigma is set.
 int setup_precond(scabem_op* op, cudaStream_t s) {
-  CK(cudaMemsetAsync(op->err, 0, sizeof(int), s));
-  k_precond<<<(int)cdiv(op->ne, 64), 64, 0, s>>>(op->tri, op->cX, op->qp, op->qw, op->sig64, op->etk, op->ecls,
-                                                  op->ne, op->q, op->ke, op->ki, op->ze, op->zi, op->pinv, op->err);
-  CK(cudaGetLastError());
-  int bad = 0;
-  CK(cudaMemcpyAsync(&bad, op->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  op->precond_singular = bad;
+  for (int cls = op->precond_plain ? 1 : 0; cls < 2; ++cls) {
+    CK(cudaMemsetAsync(op->err, 0, sizeof(int), s));
+    k_precond<<<(unsigned)cdiv(op->ne, 2), 64, 0, s>>>(op->tri, op->cX, op->qp, op->qw, op->sig64, op->etk, op->ecls,
+                                                       cls, op->ne, op->q, op->ke, op->ki, op->ze, op->zi, op->pinv,
+                                                       op->err);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(&op->precond_bad[cls], op->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    op->precond_plain = true;
+  }
+  op->precond_singular = op->precond_bad[0] + op->precond_bad[1];
   return SCABEM_OK;
 }
 
@@ -1011,7 +1039,7 @@ int setup_near(scabem_op* op, cudaStream_t s) {
   int32_t* cnt = nullptr;
   CK(cudaMalloc(&cnt, sizeof(int32_t) * nt));
   const double r2 = op->r_near * op->r_near;
-  k_near_count<<<(int)cdiv(nt, 128), 128, 0, s>>>(op->tri, nt, r2, cnt);
+  k_near_list<<<(unsigned)cdiv(nt, 4), 128, 0, s>>>(op->tri, nt, r2, nullptr, cnt, nullptr);
   CK(cudaGetLastError());
   std::vector<int32_t> hc(nt), ho(nt + 1);
   CK(cudaMemcpyAsync(hc.data(), cnt, sizeof(int32_t) * nt, cudaMemcpyDeviceToHost, s));
@@ -1031,7 +1059,7 @@ int setup_near(scabem_op* op, cudaStream_t s) {
   CK(cudaMalloc(&op->noff, sizeof(int32_t) * (nt + 1)));
   CK(cudaMalloc(&op->nsrc, sizeof(int32_t) * (acc > 0 ? acc : 1)));
   CK(cudaMemcpyAsync(op->noff, ho.data(), sizeof(int32_t) * (nt + 1), cudaMemcpyHostToDevice, s));
-  k_near_fill<<<(int)cdiv(nt, 128), 128, 0, s>>>(op->tri, nt, r2, op->noff, op->nsrc);
+  k_near_list<<<(unsigned)cdiv(nt, 4), 128, 0, s>>>(op->tri, nt, r2, op->noff, nullptr, op->nsrc);
   CK(cudaGetLastError());
   const int64_t nrec = acc * op->q * 2 * NCORR;
   if (op->prec_mask & 2) {
@@ -1050,9 +1078,11 @@ int setup_near(scabem_op* op, cudaStream_t s) {
   }
   const int64_t work = acc * op->q;
   if (work > 0) {
-    k_near_corr<double><<<(int)cdiv(work, 128), 128, 0, s>>>(
-        op->tri, op->qp, op->qw, op->base, op->d.L, op->d.dL, op->noff, op->nsrc, nt, acc, op->q, op->p, op->ke,
-        op->ki, op->gspatial[0], op->gspatial[1], op->P[0], op->P[1], op->P[2], op->d.near, op->f.near);
+    auto corr = op->p == 2 ? k_near_corr<2> : op->p == 3 ? k_near_corr<3> : k_near_corr<4>;
+    corr<<<(unsigned)cdiv(work, 128), 128, 0, s>>>(op->tri, op->qp, op->qw, op->base, op->d.L, op->d.dL, op->noff,
+                                                   op->nsrc, nt, acc, op->q, op->ke, op->ki, op->gspatial[0],
+                                                   op->gspatial[1], op->P[0], op->P[1], op->P[2], op->d.near,
+                                                   op->f.near);
     CK(cudaGetLastError());
   }
   CK(cudaStreamSynchronize(s));
