@@ -57,21 +57,28 @@ __global__ void k_summ(const cx<R>* __restrict__ x, const int32_t* __restrict__ 
 // -J_e with one sum.  The slots meet by halving exchanges.  Points no stencil
 // covers stay zero from set-up.  The sum order is fixed, so the result does not
 // depend on thread timing.  Bound by the latency of the (edge -> unknown)
-// loads out of L2; the unrolled loop keeps four entries per lane in flight.
+// loads out of L2.
 // A warp takes K right-hand sides, which share the entries' weights and indices.
-template <typename R, int K>
-__global__ void __launch_bounds__(256) k_project(const cx<R>* __restrict__ x, int64_t ldx,
-                                                 const int32_t* __restrict__ gp, const int32_t* __restrict__ gpoff,
-                                                 const int32_t* __restrict__ gpl, const int32_t* __restrict__ gpr,
-                                                 const R* __restrict__ gq, int64_t ngp, int64_t npt, int64_t nL,
-                                                 int64_t nR, cx<R>* __restrict__ src, int64_t cs, int kc) {
-  const int c0 = blockIdx.y * K;  // right-hand sides c0 .. of a batch of kc
-  x += c0 * ldx;
-  src += c0 * cs;
-  kc = min(K, kc - c0);
-  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (i >= ngp) return;  // whole warp
-  const int lane = threadIdx.x & 31, comp = lane & 3, slot = lane >> 2;
+// LANES = 128 puts four warps on a point, for operators with few points
+// (project_wide).
+constexpr int PJ_THREADS = 128;
+
+template <typename R, int K, int LANES>
+__global__ void __launch_bounds__(PJ_THREADS) k_project(const cx<R>* __restrict__ x, int xst,
+                                                        const int32_t* __restrict__ gp,
+                                                        const int32_t* __restrict__ gpoff,
+                                                        const int32_t* __restrict__ gpl,
+                                                        const int32_t* __restrict__ gpr, const R* __restrict__ gq,
+                                                        int64_t ngp, int64_t npt, int64_t nL, int64_t nR,
+                                                        cx<R>* __restrict__ src, int64_t cs, int kc) {
+  constexpr int ST = LANES / 4;  // slots
+  const int64_t st = K == 1 ? 1 : xst;
+  x += blockIdx.y * group_pad(K);  // group blockIdx.y of a batch of kc
+  src += blockIdx.y * K * cs;
+  kc = min(K, kc - (int)blockIdx.y * K);
+  const int64_t i = (blockIdx.x * (int64_t)PJ_THREADS + threadIdx.x) / LANES;
+  if (i >= ngp) return;  // whole warp; LANES = 128: no CTA
+  const int lane = threadIdx.x & 31, comp = lane & 3, slot = (threadIdx.x % LANES) >> 2;
   const int e0 = gpoff[i], el = e0 + gpl[i], e1 = gpoff[i + 1];
   pdl_wait();
   cx<R> v[K][4];  // plain J, absorber J_e, absorber J_i, M
@@ -79,42 +86,122 @@ __global__ void __launch_bounds__(256) k_project(const cx<R>* __restrict__ x, in
   for (int k = 0; k < K; ++k)
 #pragma unroll
     for (int c = 0; c < 4; ++c) v[k][c] = czero<R>();
-  constexpr int UN = K == 1 ? 4 : K < 4 ? 2 : 1;
-#pragma unroll UN
-  for (int e = e0 + slot; e < el; e += 8) {
-    const cx<R>* xm = x + gpr[e];
-    const R w = gq[4 * (int64_t)e + comp];
+  auto plain = [&](R w, const cx<R>* a, const cx<R>* b) {
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (k < kc) {
-        axpy2(v[k][0], w, xm[k * ldx]);
-        axpy2(v[k][3], w, xm[k * ldx + nL]);
-      }
-  }
-#pragma unroll UN
-  for (int e = el + slot; e < e1; e += 8) {
-    const cx<R>* xm = x + nL + gpr[e];
-    const R w = gq[4 * (int64_t)e + comp];
+    for (int k = 0; k < K; ++k) {
+      axpy2(v[k][0], w, a[k]);
+      axpy2(v[k][3], w, b[k]);
+    }
+  };
+  auto absorber = [&](R w, const cx<R>* a, const cx<R>* b, const cx<R>* d) {
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (k < kc) {
-        axpy2(v[k][1], w, xm[k * ldx]);
-        axpy2(v[k][2], w, xm[k * ldx + nR]);
-        axpy2(v[k][3], w, xm[k * ldx + 2 * nR]);
+    for (int k = 0; k < K; ++k) {
+      axpy2(v[k][1], w, a[k]);
+      axpy2(v[k][2], w, b[k]);
+      axpy2(v[k][3], w, d[k]);
+    }
+  };
+  if constexpr (LANES == 32) {  // many warps: few registers
+    constexpr int UN = K == 1 ? 4 : K < 4 ? 2 : 1;
+#pragma unroll UN
+    for (int e = e0 + slot; e < el; e += ST) {
+      const int64_t m = gpr[e];
+      const R w = gq[4 * (int64_t)e + comp];
+      cx<R> a[K], b[K];
+      load_cols<R, K>(x + m * st, a);
+      load_cols<R, K>(x + (m + nL) * st, b);
+      plain(w, a, b);
+    }
+#pragma unroll UN
+    for (int e = el + slot; e < e1; e += ST) {
+      const int64_t m = nL + gpr[e];
+      const R w = gq[4 * (int64_t)e + comp];
+      cx<R> a[K], b[K], d[K];
+      load_cols<R, K>(x + m * st, a);
+      load_cols<R, K>(x + (m + nR) * st, b);
+      load_cols<R, K>(x + (m + 2 * nR) * st, d);
+      absorber(w, a, b, d);
+    }
+  } else {  // few entries per lane: all of a block's loads before the first use
+    constexpr int IF = K == 1 ? 4 : 2;
+    for (int e = e0 + slot; e < el; e += IF * ST) {
+      cx<R> a[IF][K], b[IF][K];
+      R w[IF];
+#pragma unroll
+      for (int u = 0; u < IF; ++u) {
+        w[u] = R(0);
+#pragma unroll
+        for (int k = 0; k < K; ++k) a[u][k] = b[u][k] = czero<R>();
+        if (e + u * ST < el) {
+          const int64_t m = gpr[e + u * ST];
+          w[u] = gq[4 * (int64_t)(e + u * ST) + comp];
+          load_cols<R, K>(x + m * st, a[u]);
+          load_cols<R, K>(x + (m + nL) * st, b[u]);
+        }
       }
+#pragma unroll
+      for (int u = 0; u < IF; ++u) plain(w[u], a[u], b[u]);
+    }
+    for (int e = el + slot; e < e1; e += IF * ST) {
+      cx<R> a[IF][K], b[IF][K], d[IF][K];
+      R w[IF];
+#pragma unroll
+      for (int u = 0; u < IF; ++u) {
+        w[u] = R(0);
+#pragma unroll
+        for (int k = 0; k < K; ++k) a[u][k] = b[u][k] = d[u][k] = czero<R>();
+        if (e + u * ST < e1) {
+          const int64_t m = nL + gpr[e + u * ST];
+          w[u] = gq[4 * (int64_t)(e + u * ST) + comp];
+          load_cols<R, K>(x + m * st, a[u]);
+          load_cols<R, K>(x + (m + nR) * st, b[u]);
+          load_cols<R, K>(x + (m + 2 * nR) * st, d[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < IF; ++u) absorber(w[u], a[u], b[u], d[u]);
+    }
   }
-  const int set = (lane >> 3) - 1;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     halve(v[k], 2, lane, 16);
     halve(v[k], 1, lane, 8);
     v[k][0] = xadd(v[k][0], 4);
+  }
+  if constexpr (LANES > 32) {
+    __shared__ cx<R> sm[3][K][32];
+    const int wp = threadIdx.x >> 5;
+    if (wp > 0)
+#pragma unroll
+      for (int k = 0; k < K; ++k) sm[wp - 1][k][lane] = v[k][0];
+    __syncthreads();
+    if (wp > 0) return;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int u = 0; u < 3; ++u) v[k][0] += sm[u][k][lane];
+  }
+  const int set = (lane >> 3) - 1;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
     // lane bits (4, 3) hold plain J, J_e, J_i, M: add the plain part to J_e and -J_i
     const cx<R> pe = shfl_xor_cx(v[k][0], 8), pi = shfl_xor_cx(v[k][0], 16);
     if (set < 0 || (lane & 4) || k >= kc) continue;
     const cx<R> o = set == 0 ? v[k][0] + pe : set == 1 ? v[k][0] - pi : v[k][0];
     src[k * cs + (int64_t)(4 * set + comp) * npt + gp[i]] = o;
   }
+}
+
+// x of a batch of k in the layout of load_cols: out[u][group][column], st = batch_stride(k)
+template <typename R>
+__global__ void __launch_bounds__(256) k_interleave(const cx<R>* __restrict__ x, int64_t ldx, int64_t N, int k, int K,
+                                                    int st, cx<R>* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();
+  if (i >= N * st) return;
+  const int64_t u = i / st;
+  const int l = (int)(i - u * st), kp = group_pad(K), c = l / kp * K + l % kp;
+  out[i] = l % kp < K && c < k ? x[c * ldx + u] : czero<R>();
 }
 
 // Two consecutive complex values of shared memory on a 16-byte boundary.
@@ -472,14 +559,15 @@ __global__ void __launch_bounds__(PT_WARPS * 32, 3) k_points_sens(
 //   T3 k_rows_adj  (near.cu) projection transposed, plus the transposed near
 //                  matrix -> unknowns
 
-// T1: one warp per covered grid point, a gather over its (edge, entry) pairs:
+// T1: one warp (WPP = 8: a CTA, for operators with few points, project_wide) per
+// covered grid point, a gather over its (edge, entry) pairs:
 // lane = slot * 8 + group takes the group's weight block (four reals) of an
 // entry against the edge's row that reads the group (groups 0, 1: E rows; 2, 3:
 // H rows and Eq. 13; 4, 5: Eq. 13; 6, 7: Eq. 14); entries of plain edges have
 // the first four groups only and use the spare lane bit as a slot.  The
 // groups' adjoints are then combined into the 16 fields, as the transpose of
 // the combination that stage C of the convolution forms.
-template <typename R>
+template <typename R, int WPP>
 __global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, const int32_t* __restrict__ gp,
                                                   const int32_t* __restrict__ gpoff, const int32_t* __restrict__ gpl,
                                                   const int32_t* __restrict__ gpr, const int32_t* __restrict__ gpe,
@@ -487,9 +575,9 @@ __global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, c
                                                   int64_t nL, int64_t nR, R ke, R ki, R ze, R zi,
                                                   cx<R>* __restrict__ src) {
   __shared__ cx<R> red[8][32];  // [warp in CTA][group * 4 + component]
-  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (i >= ngp) return;  // whole warp; no CTA-wide barrier below
-  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / (32 * WPP);
+  if (i >= ngp) return;  // whole warp; WPP = 8: no CTA
+  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5, wp = wl % WPP;
   const int e0 = gpoff[i], el = e0 + gpl[i], e1 = gpoff[i + 1];
   pdl_wait();
   cx<R> v[4], u[4];
@@ -499,7 +587,7 @@ __global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, c
     const R* w = xw + 4 * (lane & 1);
     const cx<R>* yr = y + ((lane & 2) ? nL : 0);
 #pragma unroll 2
-    for (int e = e0 + (lane >> 2); e < el; e += 8) {
+    for (int e = e0 + (lane >> 2) + 8 * wp; e < el; e += 8 * WPP) {
       R a[4];
       load4(w + 8 * (int64_t)gpe[e], a);
       const cx<R> b = yr[gpr[e]];
@@ -512,7 +600,7 @@ __global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, c
     const R* w = xw + 8 * nxl + 4 * (g < 4 ? g & 1 : g - 2);
     const cx<R>* yr = y + nL + nR * ((g + 2) >> 2);
 #pragma unroll 2
-    for (int e = el + (lane >> 3); e < e1; e += 4) {
+    for (int e = el + (lane >> 3) + 4 * wp; e < e1; e += 4 * WPP) {
       R a[4];
       load4(w + 24 * (int64_t)(gpe[e] - nxl), a);
       const cx<R> b = yr[gpr[e]];
@@ -529,6 +617,14 @@ __global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, c
   halve(v, 1, lane, 8);
   cx<R>* rw = red[wl];
   rw[(lane & 7) * 4 + ((lane >> 3) & 2) + ((lane >> 3) & 1)] = v[0];
+  if constexpr (WPP > 1) {
+    __syncthreads();
+    if (wl > 0) return;
+    cx<R> t = rw[lane];
+#pragma unroll
+    for (int w = 1; w < WPP; ++w) t += red[w][lane];
+    rw[lane] = t;
+  }
   __syncwarp();
   if (lane < 16) {
     const int f = lane >> 2, c = lane & 3;  // field group (medium, set), component
@@ -565,18 +661,26 @@ PrecData<double>& pdata<double>(scabem_op* op) {
 
 }  // namespace
 
+// Four warps per grid point where one per point and group leaves less than 32
+// per SM (2 um guide, 1800 points: 13.3 -> 8.0 us)
+static bool project_wide(const scabem_op* op, int groups) { return op->ngp * groups < (int64_t)152 * 32; }
+
 // The grid part up to the potentials, for k right-hand sides: projection and
-// convolution.
+// convolution.  x in the layout of load_cols (k = 1: as it is).
 template <typename R>
-int grid_potentials(scabem_op* op, const cx<R>* x, int64_t ldx, int k, cudaStream_t s) {
+int grid_potentials(scabem_op* op, const cx<R>* x, int k, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
   prof_mark(op, s);
   prof_mark(op, s);  // (the summaries stage is part of the projection)
-  const int kw = k == 1 ? 1 : k == 2 || k == 3 ? k : 4;
-  auto fn = kw == 1 ? k_project<R, 1> : kw == 2 ? k_project<R, 2> : kw == 3 ? k_project<R, 3> : k_project<R, 4>;
-  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ngp * 32, 256), (unsigned)cdiv(k, kw)), 256, 0, s, x, ldx, op->gp, op->gpoff,
-                op->gpl, op->gpr, pd.gq, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, pd.src,
-                col_stride_src(op), k));
+  const int K = batch_group(k), groups = (int)cdiv(k, K);
+  const bool wide = project_wide(op, groups);
+  auto fn = K == 1   ? (wide ? k_project<R, 1, 128> : k_project<R, 1, 32>)
+            : K == 2 ? (wide ? k_project<R, 2, 128> : k_project<R, 2, 32>)
+            : K == 3 ? (wide ? k_project<R, 3, 128> : k_project<R, 3, 32>)
+                     : (wide ? k_project<R, 4, 128> : k_project<R, 4, 32>);
+  CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ngp * (wide ? 128 : 32), PJ_THREADS), groups), PJ_THREADS, 0, s, x,
+                batch_stride(k), op->gp, op->gpoff, op->gpl, op->gpr, pd.gq, op->ngp, (int64_t)op->n[0] * op->nac,
+                op->nL, op->nR, pd.src, col_stride_src(op), k));
   prof_mark(op, s);
   return fft_conv<R>(op, pd, s, false, k);
 }
@@ -588,9 +692,15 @@ int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
     set_error("apply_batch: batch size outside the workspace capacity");
     return SCABEM_E_ARG;
   }
-  if (int rc = grid_potentials<R>(op, x, ldx, k, s)) return rc;
+  if (k > 1) {
+    const int st = batch_stride(k);
+    CK(launch_pdl(k_interleave<R>, dim3((unsigned)cdiv(op->N * st, 256)), 256, 0, s, x, ldx, op->N, k, batch_group(k),
+                  st, pd.xi));
+    x = pd.xi;
+  }
+  if (int rc = grid_potentials<R>(op, x, k, s)) return rc;
   prof_mark(op, s);
-  if (int rc = rows_apply<R>(op, x, ldx, y, ldy, k, s)) return rc;
+  if (int rc = rows_apply<R>(op, x, y, ldy, k, s)) return rc;
   prof_mark(op, s);
   return SCABEM_OK;
 }
@@ -604,7 +714,8 @@ int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s) {
 template <typename R>
 int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
-  CK(launch_pdl(k_grid_adj<R>, dim3((unsigned)cdiv(op->ngp * 32, 256)), 256, 0, s, ybar, op->gp, op->gpoff, op->gpl,
+  const bool wide = project_wide(op, 1);
+  CK(launch_pdl(wide ? k_grid_adj<R, 8> : k_grid_adj<R, 1>, dim3((unsigned)cdiv(op->ngp * (wide ? 256 : 32), 256)), 256, 0, s, ybar, op->gp, op->gpoff, op->gpl,
                 op->gpr, op->gpe, pd.xw, op->nxl, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, (R)op->ke,
                 (R)op->ki, (R)op->ze, (R)op->zi, pd.src));
   if (int rc = fft_conv<R>(op, pd, s, true)) return rc;
@@ -626,7 +737,7 @@ int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* l
                          cudaStream_t s) {
   PrecData<double>& pd = op->d;
   if (int rc = compute_summ<double>(op, x, pd.summ, s)) return rc;
-  if (int rc = grid_potentials<double>(op, x, op->N, 1, s)) return rc;
+  if (int rc = grid_potentials<double>(op, x, 1, s)) return rc;
   prof_mark(op, s);
   const size_t sm = pt_smem_bytes(op->q, sizeof(cx<double>));
   auto fn = op->p == 2 ? k_points_sens<double, 2> : op->p == 3 ? k_points_sens<double, 3> : k_points_sens<double, 4>;

@@ -13,7 +13,7 @@
 #include <unordered_map>
 #include <vector>
 
-#include "common.cuh"
+#include "device.cuh"
 
 static thread_local std::string g_last_error;
 
@@ -99,6 +99,7 @@ void free_prec(PrecData<R>& pd) {
   cudaFree(pd.gram);
   cudaFree(pd.xw);
   cudaFree(pd.gq);
+  cudaFree(pd.xi);
   cudaFree(pd.xs);
   cudaFree(pd.ys);
   pd = PrecData<R>();
@@ -156,11 +157,11 @@ int ensure_batch(scabem_op* op, int k, cudaStream_t s) {
   if (k <= pd.kcap) return SCABEM_OK;
   CK(cudaStreamSynchronize(s));  // nothing in flight uses the old buffers
   constexpr int NB = 4;
-  cx<R>* nb[NB] = {};
-  cx<R>** cur[NB] = {&pd.src, &pd.stA, &pd.stB, &pd.grid};
+  cx<R>* nb[NB + 1] = {};
+  cx<R>** cur[NB + 1] = {&pd.src, &pd.stA, &pd.stB, &pd.grid, &pd.xi};
   const int64_t cs[NB] = {col_stride_src(op), col_stride_st(op), col_stride_st(op), col_stride_pot(op)};
-  for (int i = 0; i < NB; ++i) {
-    int rc = dalloc(&nb[i], cs[i] * k);
+  for (int i = 0; i < NB + 1; ++i) {
+    int rc = dalloc(&nb[i], i < NB ? cs[i] * k : op->N * batch_stride(k));
     if (rc) {
       for (int j = 0; j < i; ++j) cudaFree(nb[j]);
       return rc;
@@ -172,7 +173,7 @@ int ensure_batch(scabem_op* op, int k, cudaStream_t s) {
     CK(cudaMemsetAsync(nb[i] + cs[i], 0, sizeof(cx<R>) * cs[i] * (k - 1), s));
   }
   CK(cudaStreamSynchronize(s));
-  for (int i = 0; i < NB; ++i) {
+  for (int i = 0; i < NB + 1; ++i) {
     cudaFree(*cur[i]);
     *cur[i] = nb[i];
   }

@@ -152,6 +152,7 @@ struct PrecData {
   R* xw = nullptr;        // edge stencils (stencil.cu): 8 or 24 weights per entry
   R* gq = nullptr;        // their Q0 blocks in grid-point order
   R* gram = nullptr;      // nR * 5: <X_r, X_m> of absorber edges sharing a triangle
+  cx<R>* xi = nullptr;    // x of a batch, [unknown][right-hand side]: N * batch_stride(kcap), kcap > 1
   cx<R>* xs = nullptr;    // staging for host x/y: N * nrhs_cap
   cx<R>* ys = nullptr;
   int64_t stage_cap = 0;
@@ -343,7 +344,7 @@ int setup_near_matrix(scabem_op* op, cudaStream_t s);
 int near_matrix_update(scabem_op* op, cudaStream_t s);
 // y_c = A x_c from the potentials (pd.grid) and the near matrix, c < kc <= KBATCH
 template <typename R>
-int rows_apply(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s);
+int rows_apply(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cudaStream_t s);
 // x = A^T y from the convolved adjoint fields (pd.grid) and the transposed near matrix
 template <typename R>
 int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s);

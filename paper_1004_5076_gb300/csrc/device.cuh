@@ -60,6 +60,34 @@ __device__ __forceinline__ cx<double> ldstream(const cx<double>* p) {
   return mk(u.x, u.y);
 }
 
+// Right-hand sides of a batch of k go in groups of K, what one warp takes; the
+// kernels that gather x read it as [unknown][group][column of the group], the
+// columns padded to a power of two with zeros, so that an unknown's entries
+// come with one or two 16-byte loads (k_interleave, apply.cu).
+inline int batch_group(int k) { return k <= 3 ? k : k == 5 || k == 6 ? 3 : 4; }
+__host__ __device__ constexpr int group_pad(int K) { return K == 3 ? 4 : K; }
+inline int batch_stride(int k) { return (int)cdiv(k, batch_group(k)) * group_pad(batch_group(k)); }
+
+template <typename R, int K>
+__device__ __forceinline__ void load_cols(const cx<R>* p, cx<R>* v) {
+  if constexpr (K == 1) {
+    v[0] = *p;
+  } else if constexpr (sizeof(R) == 8) {
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+      const double2 u = *(reinterpret_cast<const double2*>(p) + c);
+      v[c] = mk((R)u.x, (R)u.y);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < K; c += 2) {
+      const float4 u = *reinterpret_cast<const float4*>(p + c);
+      v[c] = mk((R)u.x, (R)u.y);
+      if (c + 1 < K) v[c + 1] = mk((R)u.z, (R)u.w);
+    }
+  }
+}
+
 template <typename R>
 __device__ __forceinline__ cx<R> shfl_xor_cx(cx<R> v, int o) {
   return mk(__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o));

@@ -405,30 +405,36 @@ __device__ __forceinline__ RowDesc load_desc(const RowDesc* p) {
 template <typename R, int K, bool T, int LANES>
 __device__ __forceinline__ void near_row(const RowDesc& D, bool isR, int64_t nL, int64_t nR,
                                          const int32_t* __restrict__ col, const cx<R>* __restrict__ val,
-                                         const cx<R>* __restrict__ x, int64_t ldx, int kc, int lane, cx<R> acc[3][K]) {
+                                         const cx<R>* __restrict__ x, int64_t xst, int lane, cx<R> acc[3][K]) {
   const int cl = D.nl, cr = D.cnt - cl;
   const cx<R>* v0 = val + D.vo;
   const int32_t *colL = col + D.off, *colR = colL + cl;
-  const cx<R>* xR = x + nL;
   // the entries of x of column m: J, M of a plain edge; J_e, J_i, M of an absorber edge
-#define COLUMNS2(...)                                                 \
-  _Pragma("unroll") for (int c = 0; c < K; ++c) if (c < kc) {         \
-    const cx<R> a = x[c * ldx + m], b = x[c * ldx + m + nL];          \
-    __VA_ARGS__                                                       \
+#define COLUMNS2(...)                                       \
+  cx<R> xa[K], xb[K];                                       \
+  load_cols<R, K>(x + m * xst, xa);                \
+  load_cols<R, K>(x + (m + nL) * xst, xb);                  \
+  _Pragma("unroll") for (int c = 0; c < K; ++c) {           \
+    const cx<R> a = xa[c], b = xb[c];                       \
+    __VA_ARGS__                                             \
   }
-#define COLUMNS3(...)                                                                                       \
-  _Pragma("unroll") for (int c = 0; c < K; ++c) if (c < kc) {                                               \
-    const cx<R> a = xR[c * ldx + m], b = xR[c * ldx + m + nR], d = xR[c * ldx + m + 2 * nR];                \
-    __VA_ARGS__                                                                                             \
+#define COLUMNS3(...)                                       \
+  cx<R> xa[K], xb[K], xd[K];                                \
+  load_cols<R, K>(x + (m + nL) * xst, xa);                  \
+  load_cols<R, K>(x + (m + nL + nR) * xst, xb);             \
+  load_cols<R, K>(x + (m + nL + 2 * nR) * xst, xd);         \
+  _Pragma("unroll") for (int c = 0; c < K; ++c) {           \
+    const cx<R> a = xa[c], b = xb[c], d = xd[c];            \
+    __VA_ARGS__                                             \
   }
   if (!isR) {
-    near_segment<R, 3, LANES>(colL, v0, cl, lane, [&](int m, const cx<R>* v) {
+    near_segment<R, 3, LANES>(colL, v0, cl, lane, [&](int64_t m, const cx<R>* v) {
       COLUMNS2(  // U G V
           cmac(acc[0][c], v[0], a); cmac(acc[0][c], T ? v[1] : -v[1], b); cmac(acc[1][c], T ? -v[1] : v[1], a);
           cmac(acc[1][c], v[2], b);)
     });
     near_segment<R, T ? 6 : 5, LANES>(colR, v0 + (int64_t)nm_words(false, false) * cl, cr, lane,
-                                            [&](int m, const cx<R>* v) {
+                                            [&](int64_t m, const cx<R>* v) {
       if constexpr (!T) {  // Ue Ui ge gi V
         COLUMNS3(cmac(acc[0][c], v[0], a); cmac(acc[0][c], -v[1], b); cmac(acc[0][c], -(v[2] + v[3]), d);
                  cmac(acc[1][c], v[2], a); cmac(acc[1][c], -v[3], b); cmac(acc[1][c], v[4], d);)
@@ -439,7 +445,7 @@ __device__ __forceinline__ void near_row(const RowDesc& D, bool isR, int64_t nL,
     });
   } else {
     near_segment<R, T ? 5 : 6, LANES>(colL, v0, cl, lane,
-                                            [&](int m, const cx<R>* v) {
+                                            [&](int64_t m, const cx<R>* v) {
       if constexpr (!T) {  // U G G13 V13 P Q
         COLUMNS2(cmac(acc[0][c], v[0], a); cmac(acc[0][c], -v[1], b); cmac(acc[1][c], v[2], a);
                 cmac(acc[1][c], v[3], b); cmac(acc[2][c], v[4], a); cmac(acc[2][c], v[5], b);)
@@ -449,7 +455,7 @@ __device__ __forceinline__ void near_row(const RowDesc& D, bool isR, int64_t nL,
       }
     });
     near_segment<R, 8, LANES>(colR, v0 + (int64_t)(T ? 5 : 6) * cl, cr, lane,
-                                    [&](int m, const cx<R>* v) {
+                                    [&](int64_t m, const cx<R>* v) {
       if constexpr (!T) {  // Ue Ui e13 i13 G V13 P Q
         COLUMNS3(cmac(acc[0][c], v[0], a); cmac(acc[0][c], -v[1], b); cmac(acc[0][c], -v[4], d);
                  cmac(acc[1][c], v[2], a); cmac(acc[1][c], v[3], b); cmac(acc[1][c], v[5], d);
@@ -590,7 +596,7 @@ struct RowTables {
 template <typename R, int K, int LANES>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : K == 2 ? 7 : 6)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
-           const cx<R>* __restrict__ pot, int64_t cs_g, const cx<R>* __restrict__ x, int64_t ldx, cx<R>* __restrict__ y,
+           const cx<R>* __restrict__ pot, int64_t cs_g, const cx<R>* __restrict__ x, int xst, cx<R>* __restrict__ y,
            int64_t ldy, int kc) {
   // unit = (row, group of K right-hand sides): a row's groups sit in
   // neighbouring warps and share its values and weights through L1
@@ -598,7 +604,7 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
   const int ng = (kc + K - 1) / K;
   const int64_t r = K == 1 ? unit : unit / ng;
   const int lane = threadIdx.x % LANES, c0 = K == 1 ? 0 : (int)(unit - r * ng) * K;
-  x += c0 * ldx;
+  x += c0 / K * group_pad(K);
   y += c0 * ldy;
   pot += c0 * cs_g;
   kc = min(K, kc - c0);
@@ -611,7 +617,8 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
   if (r < T.ne) {
     const RowDesc D = load_desc(T.desc + r);
     const int64_t x0 = D.xoff;
-    near_row<R, K, false, LANES>(D, r >= nL, nL, nR, T.col, nmv, x, ldx, kc, lane, acc);
+    const int64_t st = K == 1 ? 1 : xst;
+    near_row<R, K, false, LANES>(D, r >= nL, nL, nR, T.col, nmv, x, st, lane, acc);
     // the near part needs x only, which was complete before the predecessor
     // (the last stage of the convolution) started: it runs beside that stage
     pdl_wait();
@@ -634,8 +641,7 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
         if (g >= 0) {
           const R s = gval[5 * (r - nL) + lane];
 #pragma unroll
-          for (int c = 0; c < K; ++c)
-            if (c < kc) axpy2(acc[2][c], s, x[c * ldx + nL + g]);
+          for (int c = 0; c < K; ++c) axpy2(acc[2][c], s, x[(nL + g) * st + c]);
         }
       }
     }
@@ -679,7 +685,7 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
   if (r < T.ne) {
     const RowDesc D = load_desc(T.desc + r);
     const int64_t x0 = D.xoff;
-    near_row<R, 1, true, LANES>(D, r >= nL, nL, nR, T.col, nmt, y, 0, 1, lane, acc);
+    near_row<R, 1, true, LANES>(D, r >= nL, nL, nR, T.col, nmt, y, 1, lane, acc);
     pdl_wait();  // as in k_rows
     const int h = lane & 7, grp = h >> 1;
     cx<R> gs[1] = {czero<R>()};
@@ -737,30 +743,34 @@ RowTables row_tables(const scabem_op* op, const void* desc) {
 bool wide_rows(const scabem_op* op) { return op->ne < 152 * 32 && op->nm_nnz > 64 * op->ne; }
 
 template <typename R, int K>
-int launch_rows(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
+int launch_rows(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
   const bool wide = wide_rows(op);
   auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
   const int64_t units = op->ne * cdiv(kc, K);
   CK(launch_pdl(fn, dim3((unsigned)cdiv(units * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
-                row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, ldx, y, ldy, kc));
+                row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, batch_stride(kc),
+                y, ldy, kc));
   return SCABEM_OK;
 }
 
 }  // namespace
 
-// y_c = A x_c from the potentials pd.grid (column c) and the near matrix, c < kc <= KBATCH
+// y_c = A x_c from the potentials pd.grid (column c) and the near matrix, c <
+// kc <= KBATCH, x in the layout of load_cols.  At most four right-hand sides
+// per warp: eight hold 126 registers and half the warps (325 us for 8 columns
+// of the 12 um guide; 300 us with four; 274 us with x interleaved).
 template <typename R>
-int rows_apply(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
-  // at most four right-hand sides per warp: eight hold 126 registers and half
-  // the warps (325 us for 8 columns of the 12 um guide)
-  if (kc == 1) return launch_rows<R, 1>(op, x, ldx, y, ldy, kc, s);
-  if (kc == 2 || kc == 4) return launch_rows<R, 2>(op, x, ldx, y, ldy, kc, s);
-  if (kc == 3 || kc == 5 || kc == 6) return launch_rows<R, 3>(op, x, ldx, y, ldy, kc, s);
-  return launch_rows<R, 4>(op, x, ldx, y, ldy, kc, s);
+int rows_apply(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
+  switch (batch_group(kc)) {
+    case 1: return launch_rows<R, 1>(op, x, y, ldy, kc, s);
+    case 2: return launch_rows<R, 2>(op, x, y, ldy, kc, s);
+    case 3: return launch_rows<R, 3>(op, x, y, ldy, kc, s);
+    default: return launch_rows<R, 4>(op, x, y, ldy, kc, s);
+  }
 }
-template int rows_apply<float>(scabem_op*, const cx<float>*, int64_t, cx<float>*, int64_t, int, cudaStream_t);
-template int rows_apply<double>(scabem_op*, const cx<double>*, int64_t, cx<double>*, int64_t, int, cudaStream_t);
+template int rows_apply<float>(scabem_op*, const cx<float>*, cx<float>*, int64_t, int, cudaStream_t);
+template int rows_apply<double>(scabem_op*, const cx<double>*, cx<double>*, int64_t, int, cudaStream_t);
 
 // x = A^T y from the convolved adjoint fields and the transposed near matrix
 template <typename R>
