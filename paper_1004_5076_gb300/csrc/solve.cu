@@ -673,12 +673,13 @@ __global__ void __launch_bounds__(BG_THREADS) k_bnorm_parts(const cd* __restrict
 // per block; every product is formed with its rounding error and summed
 // with compensation.
 constexpr int GM_MAXM = 200;  // largest restart length (checked by the C ABI)
-// Short vectors take 16 lanes per row, so that the chip fills and the chains
-// shorten; long ones are bound by the basis stream and take 4.
+// Short vectors (all K right-hand sides together) take 16 lanes per row, so that
+// the chip fills and the chains shorten; long ones are bound by the basis stream
+// and take 4 (8 x 5500 unknowns: 23 us with 16, 13.5 us with 4).
 constexpr int BV_KS_LONG = 4, BV_KS_SHORT = 16;
-inline bool bv_short(int64_t N) { return N * BV_KS_LONG < (int64_t)BG_BLOCKS * BG_THREADS / 2; }
-inline unsigned bv_blocks(int64_t N) {
-  const int ks = bv_short(N) ? BV_KS_SHORT : BV_KS_LONG;
+inline bool bv_short(int64_t NK) { return NK * BV_KS_LONG < (int64_t)BG_BLOCKS * BG_THREADS / 2; }
+inline unsigned bv_blocks(int64_t N, int K) {
+  const int ks = bv_short(N * K) ? BV_KS_SHORT : BV_KS_LONG;
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(BG_BLOCKS, cdiv(N * ks, BG_THREADS)));
 }
 template <typename WT, int BV_KS>
@@ -1297,7 +1298,7 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
         const int* need = pass ? W.need[cur] : nullptr;
         cd* h = pass ? W.h2[cur] : W.h1[cur];
         const int tl = pass ? (int)cdiv(j + 1, BG_TC) : tiles;
-        const dim3 gd(row_blocks(tl), tl, Ka), gv(bv_blocks(N), Ka);
+        const dim3 gd(row_blocks(tl), tl, Ka), gv(bv_blocks(N, Ka), Ka);
         int* nd = W.done + (int64_t)W.Kcap * cdiv(m + 1, BG_TC);  // counters of the updates
         if (pass == 0 && f32)
           CK(launch_pdl(k_bdots<cx<float>>, gd, BG_THREADS, 0, s, W.V, csV, j + 1, W.wf, N, W.part, m + 1, need, 1, h,
@@ -1312,7 +1313,7 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
         int* sn = pass ? nullptr : W.need[cur];
         auto update = [&](auto* in) {
           using WT = std::remove_const_t<std::remove_pointer_t<decltype(in)>>;
-          auto fn = bv_short(N) ? k_bvsub_norm<WT, BV_KS_SHORT> : k_bvsub_norm<WT, BV_KS_LONG>;
+          auto fn = bv_short(N * Ka) ? k_bvsub_norm<WT, BV_KS_SHORT> : k_bvsub_norm<WT, BV_KS_LONG>;
           return launch_pdl(fn, gv, BG_THREADS, 0, s, W.V, csV, j + 1, h, m + 1, in, W.wdf, N, W.nparts, need, nr, sn,
                             nd);
         };
