@@ -1019,51 +1019,74 @@ __global__ void k_bjoin(const cdf* __restrict__ V, int64_t csV, cd* __restrict__
     out[i] = df_join(V[i]);
 }
 
-// least squares of the cycle: y_c = R^-1 g_c over its jc[c] columns (warp c
-// for right-hand side c: the lanes split each row's sum over the solved
-// entries, which stay in shared memory)
-__global__ void __launch_bounds__(KBATCH * 32) k_backsub(BState S, int m, int K) {
-  extern __shared__ cd s_y[];  // KBATCH x m
-  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (c >= K) return;  // warp-uniform; no block barrier below
-  const int j = S.jc[c];
+// least squares of the cycle: y_c = R^-1 g_c over its jc[c] columns, block c for
+// right-hand side c.  Thread k holds row k's remaining right-hand side and takes
+// each solved entry out of it as it becomes known: one barrier and a short FP64
+// chain per entry (the pivots' reciprocals are formed before), and the columns
+// of R, contiguous over the rows, are loaded a block of entries ahead.  A warp
+// per column with a sum per entry took 350 us for 120 entries; 56 us now.
+constexpr int BS_THREADS = 256, BS_IF = 4;
+__global__ void __launch_bounds__(BS_THREADS) k_backsub(BState S, int m) {
+  __shared__ cd ys[2];  // alternating: a thread is at most one entry ahead
+  const int c = blockIdx.x, k = threadIdx.x, j = S.jc[c];
   const cd* H = S.H + (int64_t)c * m * (m + 1);
-  const cd* g = S.g + (int64_t)c * (m + 1);
-  cd* y = S.y + (int64_t)c * m;
-  cd* ys = s_y + (int64_t)c * m;
-  for (int i = j - 1; i >= 0; --i) {
-    cd acc = mk(0.0, 0.0);
-    for (int l = i + 1 + lane; l < j; l += 32) acc += H[(int64_t)l * (m + 1) + i] * ys[l];
+  cd r = mk(0.0, 0.0), inv = r, h[BS_IF];
+  if (k < j) {
+    r = S.g[(int64_t)c * (m + 1) + k];
+    const cd hd = H[(int64_t)k * (m + 1) + k];
+    const double dd = hd.re * hd.re + hd.im * hd.im;
+    inv = mk(hd.re / dd, -hd.im / dd);
+  }
+  auto fetch = [&](int i0) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
-      acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
+    for (int u = 0; u < BS_IF; ++u) h[u] = k < i0 - u ? H[(int64_t)(i0 - u) * (m + 1) + k] : mk(0.0, 0.0);
+  };
+  fetch(j - 1);
+  for (int i0 = j - 1; i0 >= 0; i0 -= BS_IF) {
+    cd a[BS_IF];
+#pragma unroll
+    for (int u = 0; u < BS_IF; ++u) a[u] = h[u];
+    fetch(i0 - BS_IF);
+#pragma unroll
+    for (int u = 0; u < BS_IF; ++u) {
+      const int i = i0 - u;
+      if (i < 0) break;  // the whole block
+      if (k == i) {
+        const cd y = r * inv;
+        ys[i & 1] = y;
+        S.y[(int64_t)c * m + i] = y;
+      }
+      __syncthreads();
+      const cd y = ys[i & 1];
+      cfma(r, -a[u], y);
     }
-    if (lane == 0) {
-      acc = g[i] - acc;
-      const cd hd = H[(int64_t)i * (m + 1) + i];
-      const double dd = hd.re * hd.re + hd.im * hd.im;
-      const cd yi = mk((acc.re * hd.re + acc.im * hd.im) / dd, (acc.im * hd.re - acc.re * hd.im) / dd);
-      ys[i] = yi;
-      y[i] = yi;
-    }
-    __syncwarp();
   }
 }
+static_assert(BS_THREADS >= GM_MAXM, "a thread per row");
 
-// u (column col[c]) += V_c y_c over slot c's jc[c] basis vectors
-__global__ void k_bupdate(const cdf* __restrict__ V, int64_t csV, BState S, int m, const int* __restrict__ col,
-                          cd* __restrict__ u, int64_t N) {
+// u (column col[c]) += V_c y_c over slot c's jc[c] basis vectors; eight lanes
+// share a row, so that short vectors fill the chip (one thread per row took
+// 81 us for 1572 rows and 120 vectors; 17 us now)
+constexpr int BU_ROWS = 4;  // rows per warp: 64 contiguous bytes of a basis vector
+__global__ void __launch_bounds__(256) k_bupdate(const cdf* __restrict__ V, int64_t csV, BState S, int m,
+                                                 const int* __restrict__ col, cd* __restrict__ u, int64_t N) {
   const int c = blockIdx.y;
   const int j = S.jc[c];
   if (j == 0) return;
   V += c * csV;
   u += col[c] * N;
   const cd* y = S.y + (int64_t)c * m;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    cd acc = u[i];
-    for (int l = 0; l < j; ++l) cfma(acc, df_join(V[(int64_t)l * N + i]), y[l]);
-    u[i] = acc;
+  const int lane = threadIdx.x & 31, sub = lane / BU_ROWS;
+  const int64_t step = (int64_t)gridDim.x * 8 * BU_ROWS;
+  for (int64_t i0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * BU_ROWS; i0 < N; i0 += step) {  // per warp
+    const int64_t i = i0 + lane % BU_ROWS;
+    cd acc = mk(0.0, 0.0);
+    if (i < N)
+#pragma unroll 4
+      for (int l = sub; l < j; l += 32 / BU_ROWS) cfma(acc, df_join(V[(int64_t)l * N + i]), y[l]);
+#pragma unroll
+    for (int o = BU_ROWS; o < 32; o <<= 1) acc = xadd(acc, o);
+    if (i < N && sub == 0) u[i] += acc;
   }
 }
 
@@ -1364,9 +1387,9 @@ int gmres_batch(scabem_op* op, const cd* r, cd* d, const std::vector<char>& use,
     CK(cudaStreamWaitEvent(s, W.ev[0], 0));
     CK(cudaStreamWaitEvent(s, W.ev[1], 0));
     // least squares of the cycle into u (at each slot's column), then d = P^-1 u for all columns
-    k_backsub<<<1, KBATCH * 32, sizeof(cd) * KBATCH * m, s>>>(S, m, Ka);
+    k_backsub<<<Ka, BS_THREADS, 0, s>>>(S, m);
     CK(cudaGetLastError());
-    k_bupdate<<<dim3(EW_BLOCKS / 4, Ka), 256, 0, s>>>(W.V, csV, S, m, S.col, W.u, N);
+    k_bupdate<<<dim3((unsigned)std::min<int64_t>(EW_BLOCKS, cdiv(N, 8 * BU_ROWS)), Ka), 256, 0, s>>>(W.V, csV, S, m, S.col, W.u, N);
     CK(cudaGetLastError());
     W.K = K;
     if (int rc = precond_apply(op, W.u, d, s, W.tr, K, N, N)) return rc;
