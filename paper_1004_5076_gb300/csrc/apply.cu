@@ -732,7 +732,7 @@ int compute_summ(scabem_op* op, const cx<R>* x, cx<R>* summ, cudaStream_t s) {
 
 // hs[p] = d(lam^T A x)/d sigma_p [per S] at every quadrature point
 // (complex128): the apply's stages up to the records, then the derivative
-// of the sigma-weighted testing (k_points in its sensitivity mode).
+// of the sigma-weighted testing (k_points_sens).
 int sigma_sensitivity_op(scabem_op* op, const cx<double>* x, const cx<double>* lam, cx<double>* hs,
                          cudaStream_t s) {
   PrecData<double>& pd = op->d;

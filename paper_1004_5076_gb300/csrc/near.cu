@@ -581,6 +581,26 @@ __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n
   }
 }
 
+// Requests the lines of n bytes at p into L2, shared between the LANES lanes of a row
+template <int LANES>
+__device__ __forceinline__ void prefetch_l2(const void* p, int64_t n, int lane) {
+  for (int64_t o = 128 * (int64_t)lane; o < n; o += 128 * LANES)
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(static_cast<const char*>(p) + o));
+}
+// The whole row at its start: near values, weights and points, so
+// that the passes over them, which follow one another, wait for L2 and not HBM
+// (apply on the 12 um guide 122 -> 115 us: the requests run under the
+// predecessor's tail).  Operators with few rows hold all of it in L2 (sphere of
+// 320 triangles 20.4 -> 20.6 us), complex128 is bound by the FP64 pipe (771 ->
+// 775 us), and a batch's groups would request it twice: they go without.
+template <typename R, int LANES>
+__device__ __forceinline__ void prefetch_row(const RowDesc& D, int wl, int wr, const cx<R>* val,
+                                             const int32_t* xpt, const R* w, int wn, int lane) {
+  prefetch_l2<LANES>(val + D.vo, (int64_t)(wl * D.nl + wr * (D.cnt - D.nl)) * sizeof(cx<R>), lane);
+  prefetch_l2<LANES>(w, (int64_t)wn * D.nx * sizeof(R), lane);
+  prefetch_l2<LANES>(xpt, (int64_t)D.nx * sizeof(int32_t), lane);
+}
+
 struct RowTables {
   const RowDesc* desc;
   const int32_t *col, *gcol, *xpt;
@@ -592,7 +612,7 @@ struct RowTables {
 // matrix of an edge meet in one reduction, and every row is written once,
 // from sums in a fixed order.  Bound by the stream of near values and
 // weights (HBM on large operators) and by load latency: the near values are
-// loaded a column ahead, the weights two entries at a time.
+// loaded a column ahead, the weights a block of entries ahead of their use.
 template <typename R, int K, int LANES>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : K == 2 ? 7 : 6)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
@@ -618,6 +638,9 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
     const RowDesc D = load_desc(T.desc + r);
     const int64_t x0 = D.xoff;
     const int64_t st = K == 1 ? 1 : xst;
+    if constexpr (K == 1 && LANES == 32 && sizeof(R) == 4)
+      prefetch_row<R, LANES>(D, r < nL ? 3 : 6, r < nL ? 5 : 8, nmv, T.xpt + x0,
+                             r < nL ? xw + 8 * x0 : xw + 8 * T.nxl + 24 * (x0 - T.nxl), r < nL ? 8 : 24, lane);
     near_row<R, K, false, LANES>(D, r >= nL, nL, nR, T.col, nmv, x, st, lane, acc);
     // the near part needs x only, which was complete before the predecessor
     // (the last stage of the convolution) started: it runs beside that stage
@@ -685,6 +708,9 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
   if (r < T.ne) {
     const RowDesc D = load_desc(T.desc + r);
     const int64_t x0 = D.xoff;
+    if constexpr (LANES == 32 && sizeof(R) == 4)
+      prefetch_row<R, LANES>(D, r < nL ? 3 : 5, r < nL ? 6 : 8, nmt, T.xpt + x0,
+                             r < nL ? xw + 8 * x0 : xw + 8 * T.nxl + 24 * (x0 - T.nxl), r < nL ? 8 : 24, lane);
     near_row<R, 1, true, LANES>(D, r >= nL, nL, nR, T.col, nmt, y, 1, lane, acc);
     pdl_wait();  // as in k_rows
     const int h = lane & 7, grp = h >> 1;
