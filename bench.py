@@ -309,33 +309,72 @@ def barrier(ws):
 
 
 # ------------------------------------------------------------------ byte models
-def stage_bytes(info, ginfo, case, N, b, k=1):
+def operator_counts(case, sample=1):
+    """What the sparse parts of the operator hold, counted on the host from the mesh and the grid:
+    edge pairs of the near matrix by the classes of (row, column) edge, entries (edge, covered grid
+    point) of the plain and the absorber edges' stencils, and the box of active (y, z) columns.
+    sample > 1 counts every sample-th edge and scales."""
+    import numpy as np
+    import scipy.sparse as sp
+    from scipy.spatial import cKDTree
+
+    from oracle import mesh, pfft
+
+    g = mesh.build(case.mesh.V, case.mesh.T, case.mesh.region, q=case.q)
+    nt, rows = case.mesh.nt, np.arange(0, g.ne, sample)
+    scale = g.ne / len(rows)
+    inc = sp.csr_matrix((np.ones(2 * g.ne, np.int32), (np.repeat(np.arange(g.ne), 2), g.edge_t.reshape(-1))),
+                        shape=(g.ne, nt))
+    near = sp.identity(nt, dtype=np.int32, format="csr")
+    pairs = cKDTree(g.centroid).query_pairs(case.r_near, output_type="ndarray")
+    near += sp.csr_matrix((np.ones(2 * len(pairs), np.int32), (pairs.reshape(-1), pairs[:, ::-1].reshape(-1))),
+                          shape=(nt, nt))
+    e = (inc[rows] @ near @ inc.T).tocoo()
+    cls = 2 * g.edge_class[rows][e.row] + g.edge_class[e.col]
+    n_pairs = np.bincount(cls, minlength=4) * scale
+    base, _, _ = pfft.stencils(case.grid, g.qpts.reshape(-1, 3))
+    base = base.reshape(nt, case.q, 3)
+    lo, hi = base.min((0, 1))[1:], base.max((0, 1))[1:] + case.grid.p
+    off = pfft._offsets(case.grid.p)
+    n = np.asarray(case.grid.n, np.int64)
+    keys = []
+    for t in (0, 1):
+        i3 = base[g.edge_t[rows, t]][:, :, None, :] + off
+        gi = (i3[..., 0] * n[1] + i3[..., 1]) * n[2] + i3[..., 2]
+        keys.append((np.arange(len(rows))[:, None, None] * int(n.prod()) + gi).reshape(len(rows), -1))
+    k = np.sort(np.concatenate(keys, 1), 1)
+    ents = 1 + np.count_nonzero(np.diff(k, axis=1), axis=1)
+    plain = g.edge_class[rows] == 0
+    return {"pairs": n_pairs, "plain": ents[plain].sum() * scale, "absorber": ents[~plain].sum() * scale,
+            "box": tuple(int(v) for v in hi - lo)}
+
+
+def stage_bytes(cnt, ginfo, case, N, b, k=1):
     """Algorithmic HBM bytes per apply of each stage (one complex word = b
     bytes, one real word = b / 2) for a call of k right-hand sides: the near
-    records, the tables and the geometry are read once per call, everything
-    per right-hand side k times.  Grid stages count only the covered grid
-    points and active columns that the pruned transforms need."""
+    matrix, the stencil weights and the tables are read once per call,
+    everything per right-hand side k times.  Grid stages count only the covered
+    grid points and active columns that the pruned transforms need.  cnt:
+    operator_counts."""
     n0, n1, n2 = case.grid.n
     P0 = 2 * n0
     nac, ngnz = ginfo["active_columns"], ginfo["covered_points"]
-    oct_ = (P0 // 2 + 1) * (n1 + 1) * (n2 + 1)
-    Q, q, p = info["qpoints"], case.q, case.grid.p
-    nt = Q // q
-    npairs = info["near_pairs"]
     r = b // 2
+    (e1, o1), (e2, o2) = (((w + 1) // 2, w // 2) for w in cnt["box"])
+    table = (P0 // 2 + 1) * ((e1 * e1 + o1 * o1) * (e2 * e2 + o2 * o2) if ginfo["transverse_direct"]
+                             else (n1 + 1) * (n2 + 1))
+    ent = cnt["plain"] + cnt["absorber"]
+    ll, lr, rl, rr = cnt["pairs"]
     return {
-        # x in; summaries and point sources out; triangle and point geometry
-        "summaries": k * b * (N + nt * 12 + Q * 12) + 4 * nt * 9 + 8 * (nt * 15 + Q * 4),
-        # point sources in, the gather map (point, weight), 12 fields out
-        "projection": k * b * (Q * 12 + 12 * ngnz) + Q * p**3 * (4 + r) + 8 * ngnz,
+        # x in, per (edge, point) entry its row and four weights, 12 fields out
+        "projection": k * b * (N + 12 * ngnz) + ent * (4 + 4 * r),
         "fft_axis0_fwd": k * b * 12 * nac * (n0 + P0),
-        "fft_planes_green": k * b * (12 * P0 * nac + 16 * P0 * nac) + b * 2 * oct_,
-        "fft_axis0_inv": k * b * 16 * nac * (P0 + n0),
-        # near records, the 16 potentials at covered points, summaries, tested
-        # values out; per point: position, weight, stencil base and weights,
-        # conductivity; per triangle: geometry
-        "points": b * npairs * q * 2 * 10 + k * b * (16 * ngnz + nt * 12 + nt * 12 + N) + 4 * (nt + 1 + npairs)
-        + Q * (24 + 8 + 12 + 2 * 3 * p * r + r) + nt * (16 + 3) * 8 + 4 * 12 * nt,
+        "fft_planes_green": k * b * (12 * P0 * nac + 16 * P0 * nac) + b * 2 * table,
+        "fft_axis0_inv": k * b * (16 * nac * P0 + 32 * nac * n0),
+        # near matrix and its columns, stencil weights and points, the
+        # potential groups at covered points, x in, y out
+        "points": b * (3 * ll + 5 * lr + 6 * rl + 8 * rr) + 4 * (ll + lr + rl + rr) + r * (8 * cnt["plain"]
+        + 24 * cnt["absorber"]) + 4 * ent + k * b * (32 * ngnz + 2 * N),
     }
 
 
@@ -350,17 +389,15 @@ def full_grid_model_bytes(info, case, N, b):
     return b * (2 * 28 * n // 2 + 2 * n // 8) + b * nnz + 2 * Q * (4 + 3 * p * (b // 2)) + Q * 48 + 2 * N * b
 
 
-def points_flops(info, case):
-    """Floating-point operations of one apply's point stage (interpolation of
-    the 16 potentials with value and gradient stencils, near-field
-    corrections, testing), counted as the kernel performs them: each real
-    stencil weight times a complex value is 2 FMAs, each complex multiply-add
-    of the near records 4 FMAs; an FMA is 2 flops."""
-    Q, p, q = info["qpoints"], case.grid.p, case.q
-    interp = Q * 4 * p**3 * 4 * 4 * 2 * 2  # (medium, group) x stencil x 4 values x (v, gx, gy, gz) x 2 FMA x 2
-    near = info["near_pairs"] * q * 4 * 19 * 4 * 2  # (pair, point, medium, group) x 19 complex MACs
-    testing = Q * 3 * 4 * 60  # per (point, edge, row type): about 60 flops
-    return interp + near + testing
+def points_flops(cnt):
+    """Floating-point operations of one apply's rows (near matrix times x and
+    stencil weights against the potential groups), counted as the kernel performs
+    them: a complex multiply-add is 4 FMAs, a real weight times a complex
+    value 2, an FMA is 2 flops."""
+    ll, lr, rl, rr = cnt["pairs"]
+    near = (4 * ll + 6 * lr + 6 * rl + 8 * rr) * 4 * 2
+    grid = (16 * cnt["plain"] + 32 * cnt["absorber"]) * 2 * 2
+    return near + grid
 
 
 def run_gpu(args):
@@ -403,6 +440,7 @@ def run_gpu(args):
 
     mh = sc.scabem_mesh_create(m.V, m.T, m.region)
     op, t_setup = make_op(case.r_near, 1 if args.no_extras else 3)
+    cnt = operator_counts(case)
     info = sc.scabem_op_info(op)
     ginfo = sc.scabem_op_grid_info(op)
     N = sc.scabem_mesh_info(mh)[2]
@@ -456,7 +494,6 @@ def run_gpu(args):
         for _ in range(args.warmup):
             step()
         torch.cuda.synchronize()
-        sc.scabem_profile(op, True, max(args.steps, 1))
         barrier(ws)
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -468,6 +505,11 @@ def run_gpu(args):
         ms = e0.elapsed_time(e1)
     clocks = clk.summary("load, warm-up and timed applies (the timed region alone is too short for samples)")
     barrier(ws)
+    # stage times on applies of their own: the events between the stages keep a
+    # launch from starting under its predecessor's tail, as the timed ones do
+    sc.scabem_profile(op, True, max(args.steps, 1))
+    for _ in range(args.steps):
+        step()
     stages, napp = sc.scabem_profile_read(op)
     sc.scabem_profile(op, False)
     ms_max = max_over_ranks(ms, ws, device=torch.device("cuda", local))
@@ -513,7 +555,7 @@ def run_gpu(args):
         st128, n128 = sc.scabem_profile_read(op)
         sc.scabem_profile(op, False)
         pts128_ms = st128["points"] / max(n128, 1)
-        fl = points_flops(info, case)
+        fl = points_flops(cnt)
         c128 = {"value": 1e3 / ms128, "unit": UNIT, "ms_per_step": ms128, "dtype": "c128",
                 "stages_ms_per_step": {k: v / max(n128, 1) for k, v in st128.items()},
                 "roofline": {"bound": "fp64_fma", "kernel": "points", "achieved": fl / (pts128_ms * 1e-3) / 1e12,
@@ -666,7 +708,7 @@ def run_gpu(args):
     # roofline of the dominant kernel, and of the whole matvec
     _, src_peak = peaks()
     per = {k: v / max(napp, 1) for k, v in stages.items()}
-    bmodel = stage_bytes(info, ginfo, case, N, 8, kb)
+    bmodel = stage_bytes(cnt, ginfo, case, N, 8, kb)
     dom = max(per, key=per.get)
     roof = None
     if dom in bmodel:
@@ -693,12 +735,13 @@ def run_gpu(args):
                        "q": case.q, "r_near_um": case.r_near, "r_near_h": args.near_radius_h,
                        "near_pairs": info["near_pairs"],
                        "covered_grid_points": ginfo["covered_points"], "active_columns": ginfo["active_columns"],
-                       "l2": "working set per step > L2 (near data %.0f MB)" % (info["near_bytes_c64"] / 1e6),
+                       "l2": "working set per step > L2 (near matrix and stencil weights %.0f MB)" % (bmodel["points"] / 1e6),
                        "parallelism": "replicas" if ws > 1 else "single GPU", "setup_s": t_setup,
                        "rhs_per_step": kb},
             "e2e": {"value": ws * kb * args.steps / e2e_s, "unit": UNIT, "h2d_bytes_per_step": int(kb * N * 8),
                     "d2h_bytes_per_step": int(kb * N * 8)},
-            "gpu_launches": 6 * ((kb + 7) // 8) * args.steps,
+            # a batch of up to 8 right-hand sides takes six launches, a single one five
+            "gpu_launches": (6 * (kb // 8) + (0 if kb % 8 == 0 else 5 if kb % 8 == 1 else 6)) * args.steps,
             "stages_ms_per_step": per,
             "roofline": roof,
             "matvec_roofline": mv_roof,
@@ -743,7 +786,7 @@ def run_coupler(sc, torch, stream, timed, rand_x, hbm):
     st, napp = sc.scabem_profile_read(op)
     sc.scabem_profile(op, False)
     pts_ms = st["points"] / max(napp, 1)
-    bmodel = stage_bytes(info, ginfo, case, N, 8)
+    bmodel = stage_bytes(operator_counts(case, 16), ginfo, case, N, 8)
     X = rand_x((8, N), torch.complex64)
     Y = torch.empty_like(X)
     ms8 = timed(lambda: sc.scabem_apply(op, X, Y, nrhs=8, ld=N, prec=sc.SCABEM_C64, stream=stream), 3)

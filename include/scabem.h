@@ -128,8 +128,10 @@ void scabem_mesh_destroy(scabem_mesh_t mesh);
 int scabem_op_create(scabem_mesh_t mesh, const scabem_media* media, const scabem_grid_opts* opts,
                      void* stream, scabem_op_t* out);
 
-/* Sizes of the built operator: near pairs, bytes of near data per matvec in
- * the given precision, quadrature points. */
+/* Sizes of the built operator: near triangle pairs, bytes of their near
+ * records (per target point) in the given precision, quadrature points.  A
+ * matvec reads the near matrix over edge pairs that is formed from the records,
+ * a tenth to a sixth of that; the records stay for set_sigma and the gradient. */
 int scabem_op_info(scabem_op_t op, int64_t* n_near_pairs, int64_t* near_bytes_c64,
                    int64_t* near_bytes_c128, int64_t* n_qpoints);
 
@@ -192,11 +194,10 @@ int scabem_set_sigma(scabem_op_t op, const scabem_sigma* sigma);
  * (host buffers are staged through device copies on `stream`).  prec selects
  * complex64 or complex128 arithmetic; the operator must have been built with
  * that precision.  Stream-ordered: returns after enqueueing (device buffers)
- * or after completion (host buffers).  The near-field stage waits on its
- * own bulk copies with a time limit (about a second); if one expires, that
- * launch's y is not valid and the next scabem_apply or scabem_solve on the
- * operator returns SCABEM_E_TIMEOUT (scabem_solve also reports it for its own
- * launches). */
+ * or after completion (host buffers).  scabem_sigma_gradient waits on its
+ * own bulk copies of near records with a time limit (about a second); if one
+ * expires, that call's result is not valid and the next scabem_apply or
+ * scabem_solve on the operator returns SCABEM_E_TIMEOUT. */
 int scabem_apply(scabem_op_t op, const void* x, void* y, int32_t nrhs, int64_t ld, int32_t prec, void* stream);
 
 /* Circulant preconditioner for the plain-surface block of a straight guide
@@ -460,10 +461,12 @@ int scabem_decay_rate(scabem_op_t op, const void* x, int32_t nrhs, int64_t ld, c
  * boundaries on its own stream, for at most max_applies applies (events are
  * created here, so enable before any stream capture).  scabem_profile_read
  * waits for the recorded events, returns per-stage summed milliseconds in
- * stage_ms[6] = {summaries and point sources, projection, FFT axis-0
- * forward, (y, z) convolution with the Green functions (direct sums or FFT
- * planes), FFT axis-0 inverse, points (interpolation + near field + testing
- * + row sums)} and the number of applies, and starts a new record.
+ * stage_ms[6] = {0 (the current summaries are part of the projection),
+ * projection, FFT axis-0 forward, (y, z) convolution with the Green functions
+ * (direct sums or FFT planes), FFT axis-0 inverse, rows (testing of the
+ * potentials + near matrix)} and the number of applies, and starts a new
+ * record.  The events keep a stage from starting under its predecessor's tail,
+ * so the sum is above an unprofiled apply.
  * enable = 0 releases the events. */
 int scabem_profile(scabem_op_t op, int32_t enable, int32_t max_applies);
 int scabem_profile_read(scabem_op_t op, double* stage_ms, int64_t* n_applies);
