@@ -309,7 +309,7 @@ def barrier(ws):
 
 
 # ------------------------------------------------------------------ byte models
-def operator_counts(case, sample=1):
+def operator_counts(sc, mesh, case, sample=1):
     """What the sparse parts of the operator hold, counted on the host from the mesh and the grid:
     edge pairs of the near matrix by the classes of (row, column) edge, entries (edge, covered grid
     point) of the plain and the absorber edges' stencils, and the box of active (y, z) columns.
@@ -318,35 +318,34 @@ def operator_counts(case, sample=1):
     import scipy.sparse as sp
     from scipy.spatial import cKDTree
 
-    from oracle import mesh, pfft
-
-    g = mesh.build(case.mesh.V, case.mesh.T, case.mesh.region, q=case.q)
-    nt, rows = case.mesh.nt, np.arange(0, g.ne, sample)
-    scale = g.ne / len(rows)
-    inc = sp.csr_matrix((np.ones(2 * g.ne, np.int32), (np.repeat(np.arange(g.ne), 2), g.edge_t.reshape(-1))),
-                        shape=(g.ne, nt))
+    _, edge_t, edge_class = sc.scabem_mesh_edges(mesh)
+    v = case.mesh.V[case.mesh.T]
+    nt, ne = case.mesh.nt, len(edge_t)
+    rows = np.arange(0, ne, sample)
+    scale = ne / len(rows)
+    inc = sp.csr_matrix((np.ones(2 * ne, np.int32), (np.repeat(np.arange(ne), 2), edge_t.reshape(-1))), shape=(ne, nt))
     near = sp.identity(nt, dtype=np.int32, format="csr")
-    pairs = cKDTree(g.centroid).query_pairs(case.r_near, output_type="ndarray")
+    pairs = cKDTree(v.mean(1)).query_pairs(case.r_near, output_type="ndarray")
     near += sp.csr_matrix((np.ones(2 * len(pairs), np.int32), (pairs.reshape(-1), pairs[:, ::-1].reshape(-1))),
                           shape=(nt, nt))
     e = (inc[rows] @ near @ inc.T).tocoo()
-    cls = 2 * g.edge_class[rows][e.row] + g.edge_class[e.col]
-    n_pairs = np.bincount(cls, minlength=4) * scale
-    base, _, _ = pfft.stencils(case.grid, g.qpts.reshape(-1, 3))
-    base = base.reshape(nt, case.q, 3)
-    lo, hi = base.min((0, 1))[1:], base.max((0, 1))[1:] + case.grid.p
-    off = pfft._offsets(case.grid.p)
-    n = np.asarray(case.grid.n, np.int64)
+    n_pairs = np.bincount(2 * edge_class[rows][e.row] + edge_class[e.col], minlength=4) * scale
+    # grid points under an edge's quadrature points (Dunavant's 6-point rule)
+    assert case.q == 6
+    bary = np.array([np.roll((1 - 2 * c, c, c), k) for c in (0.445948490915965, 0.091576213509771) for k in range(3)])
+    p, n = case.grid.p, np.asarray(case.grid.n, np.int64)
+    u = (np.einsum("ak,tkc->tac", bary, v) - np.asarray(case.grid.origin)) / case.grid.h
+    base = np.floor(u - 0.5 * (p - 2)).astype(np.int64)
+    off = np.stack(np.meshgrid(*[np.arange(p)] * 3, indexing="ij"), -1).reshape(-1, 3)
     keys = []
     for t in (0, 1):
-        i3 = base[g.edge_t[rows, t]][:, :, None, :] + off
-        gi = (i3[..., 0] * n[1] + i3[..., 1]) * n[2] + i3[..., 2]
-        keys.append((np.arange(len(rows))[:, None, None] * int(n.prod()) + gi).reshape(len(rows), -1))
+        i3 = base[edge_t[rows, t]][:, :, None, :] + off
+        keys.append(((i3[..., 0] * n[1] + i3[..., 1]) * n[2] + i3[..., 2]).reshape(len(rows), -1))
     k = np.sort(np.concatenate(keys, 1), 1)
     ents = 1 + np.count_nonzero(np.diff(k, axis=1), axis=1)
-    plain = g.edge_class[rows] == 0
+    plain = edge_class[rows] == 0
     return {"pairs": n_pairs, "plain": ents[plain].sum() * scale, "absorber": ents[~plain].sum() * scale,
-            "box": tuple(int(v) for v in hi - lo)}
+            "box": tuple(int(w) for w in (base.max((0, 1)) + p - base.min((0, 1)))[1:])}
 
 
 def stage_bytes(cnt, ginfo, case, N, b, k=1):
@@ -440,7 +439,7 @@ def run_gpu(args):
 
     mh = sc.scabem_mesh_create(m.V, m.T, m.region)
     op, t_setup = make_op(case.r_near, 1 if args.no_extras else 3)
-    cnt = operator_counts(case)
+    cnt = operator_counts(sc, mh, case)
     info = sc.scabem_op_info(op)
     ginfo = sc.scabem_op_grid_info(op)
     N = sc.scabem_mesh_info(mh)[2]
@@ -786,7 +785,7 @@ def run_coupler(sc, torch, stream, timed, rand_x, hbm):
     st, napp = sc.scabem_profile_read(op)
     sc.scabem_profile(op, False)
     pts_ms = st["points"] / max(napp, 1)
-    bmodel = stage_bytes(operator_counts(case, 16), ginfo, case, N, 8)
+    bmodel = stage_bytes(operator_counts(sc, mh, case, 16), ginfo, case, N, 8)
     X = rand_x((8, N), torch.complex64)
     Y = torch.empty_like(X)
     ms8 = timed(lambda: sc.scabem_apply(op, X, Y, nrhs=8, ld=N, prec=sc.SCABEM_C64, stream=stream), 3)
