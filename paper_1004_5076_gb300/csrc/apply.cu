@@ -59,6 +59,8 @@ __global__ void k_summ(const cx<R>* __restrict__ x, const int32_t* __restrict__ 
 // depend on thread timing.  Bound by the latency of the (edge -> unknown)
 // loads out of L2.
 // A warp takes K right-hand sides, which share the entries' weights and indices.
+// 12 um guide: 24 us, 76 for 8 columns (33 and 188 as a gather of point sources
+// behind a kernel that formed them in 13 and 56).
 // LANES = 128 puts four warps on a point, for operators with few points
 // (project_wide).
 constexpr int PJ_THREADS = 128;
@@ -559,7 +561,8 @@ __global__ void __launch_bounds__(PT_WARPS * 32, 3) k_points_sens(
 //   T3 k_rows_adj  (near.cu) projection transposed, plus the transposed near
 //                  matrix -> unknowns
 
-// T1: one warp (WPP = 8: a CTA, for operators with few points, project_wide) per
+// T1 (replaces a 180 us gather of 320-byte point adjoints on the 12 um guide):
+// one warp (WPP = 8: a CTA, for operators with few points, project_wide) per
 // covered grid point, a gather over its (edge, entry) pairs:
 // lane = slot * 8 + group takes the group's weight block (four reals) of an
 // entry against the edge's row that reads the group (groups 0, 1: E rows; 2, 3:

@@ -65,7 +65,8 @@ __global__ void __launch_bounds__(128) k_edge_points(const int32_t* __restrict__
   if (cnt && lane == 0) cnt[r] = n;
 }
 
-// Weights of the entries, one warp per edge, lanes over its entries; sums over
+// Weights of the entries, one warp per edge, lanes over its entries (0.3 ms per call
+// on the 5 um guide, FP64; once per operator and, SIG, per conductivity); sums over
 // the quadrature points in FP64.  SIG: blocks S4 .. S7 of the absorber edges,
 // else Q0, Q1 of all edges.
 template <bool SIG>
