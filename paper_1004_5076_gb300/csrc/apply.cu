@@ -717,6 +717,13 @@ int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s) {
 template <typename R>
 int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
+  // the last kernel still reads y while it writes x: in place, y is copied first
+  const auto a = reinterpret_cast<uintptr_t>(ybar), b = reinterpret_cast<uintptr_t>(xbar);
+  const uintptr_t len = sizeof(cx<R>) * (uintptr_t)op->N;
+  if (a < b + len && b < a + len) {
+    CK(launch_pdl(k_interleave<R>, dim3((unsigned)cdiv(op->N, 256)), 256, 0, s, ybar, op->N, op->N, 1, 1, 1, pd.xi));
+    ybar = pd.xi;
+  }
   const bool wide = project_wide(op, 1);
   CK(launch_pdl(wide ? k_grid_adj<R, 8> : k_grid_adj<R, 1>, dim3((unsigned)cdiv(op->ngp * (wide ? 256 : 32), 256)), 256, 0, s, ybar, op->gp, op->gpoff, op->gpl,
                 op->gpr, op->gpe, pd.xw, op->nxl, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, (R)op->ke,

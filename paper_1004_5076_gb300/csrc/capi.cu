@@ -135,7 +135,7 @@ int alloc_prec(scabem_op* op, PrecData<R>& pd, bool workspaces, cudaStream_t s) 
     if ((rc = dalloc(&pd.tw[a], op->P[a]))) return rc;
     if ((rc = make_twiddles<R>(pd.tw[a], op->P[a], s))) return rc;
   }
-  if ((rc = dalloc(&pd.summ, op->nt * 12))) return rc;
+  if ((rc = dalloc(&pd.summ, op->nt * 12)) || (rc = dalloc(&pd.xi, op->N))) return rc;
   pd.built = true;
   return SCABEM_OK;
 }

@@ -152,7 +152,7 @@ struct PrecData {
   R* xw = nullptr;        // edge stencils (stencil.cu): 8 or 24 weights per entry
   R* gq = nullptr;        // their Q0 blocks in grid-point order
   R* gram = nullptr;      // nR * 5: <X_r, X_m> of absorber edges sharing a triangle
-  cx<R>* xi = nullptr;    // x of a batch, [unknown][right-hand side]: N * batch_stride(kcap), kcap > 1
+  cx<R>* xi = nullptr;    // x of a batch, [unknown][right-hand side]: N * batch_stride(kcap)
   cx<R>* xs = nullptr;    // staging for host x/y: N * nrhs_cap
   cx<R>* ys = nullptr;
   int64_t stage_cap = 0;

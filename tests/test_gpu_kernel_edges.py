@@ -95,6 +95,20 @@ def test_products_of_every_batch_size(mk):
         assert _dot_gap(op, g.N, prec, 50) < (1e-12 if prec == sc.SCABEM_C128 else 1e-5)
 
 
+@pytest.mark.parametrize("mk", [cases.plate_thin, cases.guide_small], ids=lambda f: f.__name__)
+@pytest.mark.parametrize("shift", [0, 3])
+def test_transposed_product_in_place(mk, shift):
+    case = mk()
+    mh, op, g, med, sig = build(case)
+    for dt, prec in ((torch.complex128, sc.SCABEM_C128), (torch.complex64, sc.SCABEM_C64)):
+        v = torch.as_tensor(cases.synth.complex_normal(g.N + shift, seed=90)).to(dt).cuda()
+        ref = torch.empty(g.N, dtype=dt, device="cuda")
+        sc.scabem_apply_adjoint(op, v[:g.N].clone(), ref, prec=prec)
+        sc.scabem_apply_adjoint(op, v[:g.N], v[shift:], prec=prec)  # overlapping by all but `shift` values
+        torch.cuda.synchronize()
+        assert torch.equal(v[shift:], ref)
+
+
 def test_second_conductivity_equals_a_new_operator():
     case = cases.guide_short()
     m, x = case.mesh, None
