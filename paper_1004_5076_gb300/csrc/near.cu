@@ -770,7 +770,9 @@ RowTables row_tables(const scabem_op* op, const void* desc) {
   return {(const RowDesc*)desc, op->nm_col, op->nm_gcol, op->xpt, op->ne, op->nL, op->nxl};
 }
 // a warp per row; a whole CTA per row where warps would leave the chip idle
-// and the rows are long (77 columns per row on the 12 um guide)
+// and the rows are long (77 columns per row on the 12 um guide).  Apply of a 480
+// edge sphere: 23.4 us with warps, 20.4 with CTAs; at 2268 edges the two meet
+// (solve of the 2 um guide 121 and 123 ms), and from 32 rows per SM on warps fill it.
 bool wide_rows(const scabem_op* op) { return op->ne < 152 * 32 && op->nm_nnz > 64 * op->ne; }
 
 template <typename R, int K>
