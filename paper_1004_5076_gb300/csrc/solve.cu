@@ -1157,7 +1157,7 @@ struct BWork {
     for (auto& e : ev)
       if (e) cudaEventDestroy(e);
   }
-  int init(int k, int mm, int64_t n, bool c64) {
+  int init(int k, int mm, int64_t n, bool c64, cudaStream_t s) {
     K = Kcap = k;
     m = mm;
     N = n;
@@ -1178,7 +1178,7 @@ struct BWork {
     S.need = need[0];
     const int64_t nd = K * (cdiv(m + 1, BG_TC) + 2);
     if ((rc = get(&done, nd))) return rc;
-    CK(cudaMemset(done, 0, sizeof(int) * nd));
+    CK(cudaMemsetAsync(done, 0, sizeof(int) * nd, s));  // before the kernels of s that count
     CK(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
     for (auto& e : gs) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if (c64 && ((rc = get(&zf, K * N)) || (rc = get(&wf, K * N)))) return rc;
@@ -1738,7 +1738,7 @@ int solve_impl(scabem_op* op, const void* bv, void* xv, int nrhs, int64_t ld, co
   }
   BWork W;
   W.tr = tr;
-  if (int rc = W.init(KB, m, N, prec == SCABEM_C64)) return rc;
+  if (int rc = W.init(KB, m, N, prec == SCABEM_C64, s)) return rc;
   cd *B = nullptr, *X = nullptr, *R = nullptr, *D = nullptr;
   if (int rc = W.get(&B, KB * N)) return rc;
   if (int rc = W.get(&X, KB * N)) return rc;
