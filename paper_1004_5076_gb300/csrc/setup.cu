@@ -12,17 +12,22 @@
 namespace {
 
 // Symmetric triangle rules (Dunavant 1985): barycentric coordinates and
-// weights summing to one; the point order is part of the interface.
-__constant__ double c_bary[MAXQ][3];
-__constant__ double c_w[MAXQ];
+// weights summing to one; the point order is part of the interface.  A kernel
+// takes the rule as an argument, so that set-ups on several streams or threads
+// share nothing.
+struct Rule {
+  double bary[MAXQ][3];
+  double w[MAXQ];
+};
 
-int load_rule(int q) {
+int make_rule(int q, Rule& rule) {
   const double a6 = 0.445948490915965, b6 = 0.091576213509771;
   const double wa6 = 0.223381589678011, wb6 = 0.109951743655322;
   const double a7 = 0.059715871789770, b7 = 0.470142064105115;
   const double c7 = 0.797426985353087, d7 = 0.101286507323456;
-  double B[MAXQ][3] = {};
-  double W[MAXQ] = {};
+  rule = {};
+  auto& B = rule.bary;
+  auto& W = rule.w;
   if (q == 1) {
     B[0][0] = B[0][1] = B[0][2] = 1.0 / 3.0;
     W[0] = 1.0;
@@ -55,8 +60,6 @@ int load_rule(int q) {
     set_error("q must be 1, 3, 6 or 7");
     return SCABEM_E_ARG;
   }
-  CK(cudaMemcpyToSymbol(c_bary, B, sizeof(B)));
-  CK(cudaMemcpyToSymbol(c_w, W, sizeof(W)));
   return SCABEM_OK;
 }
 
@@ -88,11 +91,11 @@ __device__ void lagrange(double t, int p, double* L, double* dL) {
 // Per triangle: vertices, centroid, unit normal, area, s_k l_k/(2A), and the
 // quadrature points with their stencils.
 __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restrict__ T,
-                           const int32_t* __restrict__ tsign, int64_t nt, int q, int p, double h, double ox,
-                           double oy, double oz, int n0, int n1, int n2, double* __restrict__ tri,
-                           double* __restrict__ cX, double* __restrict__ qp, double* __restrict__ qw,
-                           int32_t* __restrict__ base, double* __restrict__ Ld, double* __restrict__ dLd,
-                           float* __restrict__ Lf, float* __restrict__ dLf, int* err) {
+                           const int32_t* __restrict__ tsign, int64_t nt, int q, const __grid_constant__ Rule rule,
+                           int p, double h, double ox, double oy, double oz, int n0, int n1, int n2,
+                           double* __restrict__ tri, double* __restrict__ cX, double* __restrict__ qp,
+                           double* __restrict__ qw, int32_t* __restrict__ base, double* __restrict__ Ld,
+                           double* __restrict__ dLd, float* __restrict__ Lf, float* __restrict__ dLf, int* err) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double v[3][3];
@@ -126,9 +129,10 @@ __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restri
   for (int a = 0; a < q; ++a) {
     const int64_t Qi = t * q + a;
     double r[3];
-    for (int c = 0; c < 3; ++c) r[c] = c_bary[a][0] * v[0][c] + c_bary[a][1] * v[1][c] + c_bary[a][2] * v[2][c];
+    for (int c = 0; c < 3; ++c)
+      r[c] = rule.bary[a][0] * v[0][c] + rule.bary[a][1] * v[1][c] + rule.bary[a][2] * v[2][c];
     for (int c = 0; c < 3; ++c) qp[3 * Qi + c] = r[c];
-    qw[Qi] = c_w[a] * area;
+    qw[Qi] = rule.w[a] * area;
     for (int ax = 0; ax < 3; ++ax) {
       const double u = (r[ax] - org[ax]) / h;
       const int b = (int)floor(u - 0.5 * (p - 2));
@@ -951,8 +955,8 @@ int precond_apply_df(scabem_op* op, const cdf* in, cx<float>* outf, cx<double>* 
 }
 
 int setup_geometry(scabem_op* op, const scabem_mesh* m, cudaStream_t s) {
-  int rc = load_rule(op->q);
-  if (rc) return rc;
+  Rule rule;
+  if (int rc = make_rule(op->q, rule)) return rc;
   double* dV = nullptr;
   int32_t* dT = nullptr;
   int32_t* dS = nullptr;
@@ -963,7 +967,7 @@ int setup_geometry(scabem_op* op, const scabem_mesh* m, cudaStream_t s) {
   CK(cudaMemcpyAsync(dT, m->T.data(), sizeof(int32_t) * 3 * m->nt, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(dS, m->tri_sign.data(), sizeof(int32_t) * 3 * m->nt, cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(op->err, 0, sizeof(int), s));
-  k_geometry<<<(int)cdiv(op->nt, 128), 128, 0, s>>>(dV, dT, dS, op->nt, op->q, op->p, op->h, op->origin[0],
+  k_geometry<<<(int)cdiv(op->nt, 128), 128, 0, s>>>(dV, dT, dS, op->nt, op->q, rule, op->p, op->h, op->origin[0],
                                                      op->origin[1], op->origin[2], op->n[0], op->n[1], op->n[2],
                                                      op->tri, op->cX, op->qp, op->qw, op->base, op->d.L, op->d.dL,
                                                      op->f.L, op->f.dL, op->err);

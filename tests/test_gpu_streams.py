@@ -40,17 +40,46 @@ def _calls(op, N, nrhs, b, stream):
     return out
 
 
+def _busy():
+    """About 0.1 s of ordinary work on the current stream."""
+    a = torch.full((4096, 4096), 1e-4, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(40):
+        a = a @ a
+
+
 @pytest.mark.parametrize("nrhs", [1, 8])
 def test_calls_on_another_stream(nrhs):
     mh, op, g, med, sig = build(cases.guide_small())
     b = torch.as_tensor(np.stack([cases.synth.complex_normal(g.N, seed=110 + c) for c in range(nrhs)])).cuda()
     ref = _calls(op, g.N, nrhs, b, torch.cuda.current_stream())
-    a = torch.full((4096, 4096), 1e-4, device="cuda")
-    torch.cuda.synchronize()
     own = torch.cuda.Stream()
-    for _ in range(40):  # about 0.1 s of work
-        a = a @ a
+    _busy()
     out = _calls(op, g.N, nrhs, b, own)
     torch.cuda.synchronize()
     for u, v in zip(out, ref):
         assert torch.equal(u, v)
+
+
+def _create(case):
+    m = case.mesh
+    mh = sc.scabem_mesh_create(m.V, m.T, m.region)
+    return sc.scabem_op_create(mh, case.media, case.grid.n, case.grid.h, case.grid.origin, case.grid.p, case.q,
+                               case.r_near, 3), sc.scabem_mesh_info(mh)[2]
+
+
+def test_operator_created_on_another_stream():
+    """After an operator with another quadrature rule, whose points must not be met."""
+    out = []
+    for own in (None, torch.cuda.Stream()):
+        _create(cases.plate_p4_q7())
+        if own is not None:
+            _busy()
+        with torch.cuda.stream(own):
+            op, N = _create(cases.plate_thin())
+        x = torch.as_tensor(cases.synth.complex_normal(N, seed=120)).cuda()
+        torch.cuda.synchronize()
+        out.append(torch.empty_like(x))
+        sc.scabem_apply(op, x, out[-1])
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], out[1])

@@ -1,7 +1,7 @@
 """Order of the library's device work, read from its sources.
 
 A caller's stream need not be ordered with the legacy default stream, so every launch and every
-clear of device memory names its stream.
+copy or clear of device memory names its stream.
 """
 
 import os
@@ -26,3 +26,8 @@ def test_every_launch_and_clear_names_its_stream():
                 depth -= ch in ")]}"
                 commas += ch == "," and depth == 0
             assert commas == 3, (f, args)
+
+
+def test_every_copy_names_its_stream():
+    for f, src in _sources():
+        assert not re.findall(r"\bcudaMemcpy\w*(?<!Async)\s*\(", src), f
