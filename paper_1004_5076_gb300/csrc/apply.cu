@@ -66,7 +66,7 @@ __global__ void k_summ(const cx<R>* __restrict__ x, const int32_t* __restrict__ 
 constexpr int PJ_THREADS = 128;
 
 template <typename R, int K, int LANES>
-__global__ void __launch_bounds__(PJ_THREADS) k_project(const cx<R>* __restrict__ x, int xst,
+__global__ void __launch_bounds__(PJ_THREADS) k_project(const cx<R>* x, int xst,
                                                         const int32_t* __restrict__ gp,
                                                         const int32_t* __restrict__ gpoff,
                                                         const int32_t* __restrict__ gpl,
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(PJ_THREADS) k_project(const cx<R>* __restrict_
 
 // x of a batch of k in the layout of load_cols: out[u][group][column], st = batch_stride(k)
 template <typename R>
-__global__ void __launch_bounds__(256) k_interleave(const cx<R>* __restrict__ x, int64_t ldx, int64_t N, int k, int K,
+__global__ void __launch_bounds__(256) k_interleave(const cx<R>* x, int64_t ldx, int64_t N, int k, int K,
                                                     int st, cx<R>* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   pdl_wait();
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(PT_WARPS * 32, 3) k_points_sens(
 // groups' adjoints are then combined into the 16 fields, as the transpose of
 // the combination that stage C of the convolution forms.
 template <typename R, int WPP>
-__global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* __restrict__ y, const int32_t* __restrict__ gp,
+__global__ void __launch_bounds__(256) k_grid_adj(const cx<R>* y, const int32_t* __restrict__ gp,
                                                   const int32_t* __restrict__ gpoff, const int32_t* __restrict__ gpl,
                                                   const int32_t* __restrict__ gpr, const int32_t* __restrict__ gpe,
                                                   const R* __restrict__ xw, int64_t nxl, int64_t ngp, int64_t npt,

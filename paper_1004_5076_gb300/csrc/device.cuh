@@ -116,6 +116,13 @@ __device__ __forceinline__ cx<R> xadd(cx<R> v, int o) {
 // that everything before its direct predecessor has completed.  Every kernel
 // launched with launch_pdl comes through pdl_wait before it reads or writes
 // what the stream's kernels share.
+//
+// What the direct predecessor writes is therefore written during this kernel's
+// lifetime, and the read-only path (__ldg, or const with __restrict__) is defined
+// only for memory that nobody writes meanwhile.  These kernels read it with plain loads
+// through pointers without __restrict__, which the "memory" clobber keeps below
+// the wait; const __restrict__ is for set-up tables and for vectors that were
+// complete before the predecessor started.
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

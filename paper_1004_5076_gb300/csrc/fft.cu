@@ -179,7 +179,7 @@ struct Tot {
 // The output has Cout columns per (field, k0): active column j goes to
 // column j (compact, Cout = nac) or to acol[j] (whole planes, Cout = C).
 template <typename R>
-__global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__ in, cx<R>* __restrict__ out,
+__global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* in, cx<R>* __restrict__ out,
                                                        int n_in, int P0, const int32_t* __restrict__ acol, int nac,
                                                        int CB, const cx<R>* __restrict__ tw,
                                                        int64_t cs_in, int64_t cs_out, int64_t Cout, int compact) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis0(const cx<R>* __restrict__
 // COMB = false (transposed apply): the fields themselves in groups 4 .. 7.
 template <typename R, bool COMB, int TOTL>
 __global__ void __launch_bounds__(FFT_THREADS)
-    k_axis0_pm(const cx<R>* __restrict__ in, cx<R>* __restrict__ out, int n_out, int P0,
+    k_axis0_pm(const cx<R>* in, cx<R>* __restrict__ out, int n_out, int P0,
                const int32_t* __restrict__ acol, int nac, int NC, const cx<R>* __restrict__ tw, int64_t cs_in,
                int64_t cs_out, int64_t Cin, int compact, R ke, R ki, R ze, R zi) {
   extern __shared__ unsigned char smem_raw[];
@@ -368,7 +368,7 @@ __device__ __forceinline__ void for_warp_lines(int nlines, const F& f) {
 constexpr int PLANE_THREADS = 256;
 
 template <typename R, int L1, int L2>
-__global__ void __launch_bounds__(PLANE_THREADS) k_planes(const cx<R>* __restrict__ A, cx<R>* __restrict__ B,
+__global__ void __launch_bounds__(PLANE_THREADS) k_planes(const cx<R>* A, cx<R>* __restrict__ B,
                                                           const cx<R>* __restrict__ ghE,
                                                           const cx<R>* __restrict__ ghI, int P0, int n1, int n2,
                                                           const cx<R>* __restrict__ tw1,
@@ -560,7 +560,7 @@ __device__ __forceinline__ void line64(cx<R>* v, const cx<R>* w, cx<R>* scr, int
 
 template <typename R>
 __global__ void __launch_bounds__(P64_THREADS, sizeof(R) == 4 ? 3 : 1)
-    k_planes64(const cx<R>* __restrict__ A, cx<R>* __restrict__ B, const cx<R>* __restrict__ ghE,
+    k_planes64(const cx<R>* A, cx<R>* __restrict__ B, const cx<R>* __restrict__ ghE,
                const cx<R>* __restrict__ ghI, int P0, const cx<R>* __restrict__ tw64, uint64_t rowmask, int ident,
                int64_t cs) {
   constexpr int NP = 32, H = 33;
@@ -707,7 +707,7 @@ struct Acc8<double> {
 };
 
 template <typename R>
-__global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* __restrict__ A, cx<R>* __restrict__ B,
+__global__ void __launch_bounds__(PD_THREADS) k_planes_direct(const cx<R>* A, cx<R>* __restrict__ B,
                                                               const cx<R>* __restrict__ gtE,
                                                               const cx<R>* __restrict__ gtI, int P0,
                                                               const int32_t* __restrict__ acoord, int nac, int R1,
@@ -813,7 +813,7 @@ __device__ __forceinline__ cx<double> ldg_cx(const cx<double>* p) {
 
 template <typename R, bool STAGE>
 __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
-    k_planes_parity(const cx<R>* __restrict__ A, cx<R>* __restrict__ B, const cx<R>* __restrict__ mE,
+    k_planes_parity(const cx<R>* A, cx<R>* __restrict__ B, const cx<R>* __restrict__ mE,
                     const cx<R>* __restrict__ mI, int P0, const int32_t* __restrict__ acoord, int nac, int R1, int R2,
                     int words, int ident, int64_t cs, int ncol) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(PS_THREADS, sizeof(R) == 4 ? 3 : 2)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int j = jb + 32 * u + lane;
-          if (h < npl && j < nac) x[h][u] = ldg_cx(rp[h] + col * cs + j);
+          if (h < npl && j < nac) x[h][u] = rp[h][col * cs + j];
         }
 #pragma unroll
       for (int h = 0; h < 2; ++h)

@@ -515,8 +515,9 @@ __device__ __forceinline__ void near_reduce(cx<R> acc[3][K]) {
 // a point against two weights into ga[c], so that a warp's loads are
 // contiguous (the 128 or 256 bytes of a point in complex64).  Entries go in
 // blocks of GR_IF slots: a block's point indices are loaded by the lanes one
-// block ahead and handed out by shuffles, and all of its weights and (one
-// right-hand side) potentials are loaded before the first is used.
+// block ahead and handed out by shuffles, and then all of its weights and (one
+// right-hand side) potentials are loaded before the first is used (shuffles and
+// loads in turn: complex128 product of the 12 um guide 780 us, 755 this way).
 constexpr int GR_IF = 4;
 
 __device__ __forceinline__ void load_two(const float* p, float* v) {
@@ -529,21 +530,21 @@ __device__ __forceinline__ void load_two(const double* p, double* v) {
   v[0] = u.x;
   v[1] = u.y;
 }
-__device__ __forceinline__ void load_two(const cx<float>* p, cx<float>* v) {
-  const float4 u = __ldg(reinterpret_cast<const float4*>(p));
+// two potentials, by plain loads (pdl_wait)
+__device__ __forceinline__ void load_pot(const cx<float>* p, cx<float>* v) {
+  const float4 u = *reinterpret_cast<const float4*>(p);
   v[0] = mk(u.x, u.y);
   v[1] = mk(u.z, u.w);
 }
-__device__ __forceinline__ void load_two(const cx<double>* p, cx<double>* v) {
-  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+__device__ __forceinline__ void load_pot(const cx<double>* p, cx<double>* v) {
+  const double2 a = *reinterpret_cast<const double2*>(p), b = *(reinterpret_cast<const double2*>(p) + 1);
   v[0] = mk(a.x, a.y);
   v[1] = mk(b.x, b.y);
 }
 
 template <typename R, int K, int H, int STRIDE, int LANES>
 __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n, const R* __restrict__ w,
-                                          const cx<R>* __restrict__ pot, int64_t cs_g, int kc, int lane,
-                                          cx<R> ga[K]) {
+                                          const cx<R>* pot, int64_t cs_g, int kc, int lane, cx<R> ga[K]) {
   constexpr int S = 32 / H, BLK = GR_IF * S, STEP = BLK * (LANES / 32);
   const int wl = lane & 31, slot = wl / H;
   int b = BLK * (lane >> 5);  // the warps of a wide row take the blocks in turn
@@ -555,14 +556,15 @@ __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n
     cx<R> g[GR_IF][2];
     const cx<R>* pp[GR_IF];
 #pragma unroll
+    for (int u = 0; u < GR_IF; ++u) pp[u] = pot + (int64_t)__shfl_sync(0xffffffffu, cur, u * S + slot) * NPOT;
+#pragma unroll
     for (int u = 0; u < GR_IF; ++u) {
       const int j = b + u * S + slot;
-      pp[u] = pot + (int64_t)__shfl_sync(0xffffffffu, cur, u * S + slot) * NPOT;
       a[u][0] = a[u][1] = R(0);
       g[u][0] = g[u][1] = czero<R>();
       if (j < n) {
         load_two(w + (int64_t)STRIDE * j, a[u]);
-        if constexpr (K == 1) load_two(pp[u], g[u]);
+        if constexpr (K == 1) load_pot(pp[u], g[u]);
       }
     }
 #pragma unroll
@@ -574,7 +576,7 @@ __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n
 #pragma unroll
         for (int c = 0; c < K; ++c)
           if (c < kc) {
-            load_two(pp[u] + c * cs_g, g[u]);
+            load_pot(pp[u] + c * cs_g, g[u]);
             axpy2(ga[c], a[u][0], g[u][0]);
             axpy2(ga[c], a[u][1], g[u][1]);
           }
@@ -621,8 +623,8 @@ struct RowTables {
 template <typename R, int K, int LANES>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : K == 2 ? 7 : 6)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
-           const cx<R>* __restrict__ pot, int64_t cs_g, const cx<R>* __restrict__ x, int xst, cx<R>* __restrict__ y,
-           int64_t ldy, int kc) {
+           const cx<R>* pot, int64_t cs_g, const cx<R>* __restrict__ x, int xst, cx<R>* __restrict__ y, int64_t ldy,
+           int kc) {
   // unit = (row, group of K right-hand sides): a row's groups sit in
   // neighbouring warps and share its values and weights through L1
   const int64_t unit = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
@@ -705,7 +707,7 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
 template <typename R, int LANES>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
     k_rows_adj(RowTables T, const cx<R>* __restrict__ nmt, const R* __restrict__ gval, const R* __restrict__ xw,
-               const cx<R>* __restrict__ pot, const cx<R>* __restrict__ y, cx<R>* __restrict__ x) {
+               const cx<R>* pot, const cx<R>* __restrict__ y, cx<R>* __restrict__ x) {
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
   const int lane = threadIdx.x % LANES;
   const int64_t nL = T.nL, nR = T.ne - nL;

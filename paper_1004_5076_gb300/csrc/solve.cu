@@ -536,8 +536,8 @@ __device__ __forceinline__ bool last_block(int* done, int n) {
 // cost 3.3 us of every Arnoldi step).
 template <typename WT>
 __global__ void __launch_bounds__(BG_THREADS) k_bdots(const cdf* __restrict__ V, int64_t csV, int nv,
-                                                      const WT* __restrict__ w, int64_t N, cd* __restrict__ part,
-                                                      int ldp, const int* __restrict__ need, int self_col,
+                                                      const WT* w, int64_t N, cd* __restrict__ part, int ldp,
+                                                      const int* need, int self_col,
                                                       cd* __restrict__ hout, int ldh, int* __restrict__ done) {
   constexpr bool WLO = !std::is_same<WT, cx<float>>::value;  // w has lo parts
   const int c = blockIdx.z;
@@ -686,10 +686,10 @@ inline unsigned bv_blocks(int64_t N, int K) {
 }
 template <typename WT, int BV_KS>
 __global__ void __launch_bounds__(BG_THREADS) k_bvsub_norm(const cdf* __restrict__ V, int64_t csV, int nv,
-                                                           const cd* __restrict__ h, int ldh, const WT* win,
-                                                           cdf* wout, int64_t N, double* __restrict__ nparts,
-                                                           const int* __restrict__ need, double* __restrict__ nrm,
-                                                           int* __restrict__ set_need, int* __restrict__ done) {
+                                                           const cd* h, int ldh, const WT* win, cdf* wout, int64_t N,
+                                                           double* __restrict__ nparts, const int* need,
+                                                           double* __restrict__ nrm, int* __restrict__ set_need,
+                                                           int* __restrict__ done) {
   const int c = blockIdx.y;
   pdl_wait();
   if (need && !need[c]) return;
@@ -963,9 +963,8 @@ __global__ void k_bscale(const cdf* __restrict__ w, cdf* __restrict__ V, int64_t
 // its own and forms its row of the block (P^-T when transposed), written in the
 // operator's precision.  One launch instead of two (4.4 + 9.3 us).
 template <typename TO>
-__global__ void __launch_bounds__(128) k_bscale_precond(const cdf* __restrict__ w, cdf* __restrict__ V, int64_t csV,
-                                                        int j1, const double* __restrict__ nrm,
-                                                        const int* __restrict__ need, int64_t N,
+__global__ void __launch_bounds__(128) k_bscale_precond(const cdf* w, cdf* __restrict__ V, int64_t csV, int j1,
+                                                        const double* nrm, const int* need, int64_t N,
                                                         const cd* __restrict__ pinv, const int32_t* __restrict__ eunk,
                                                         int64_t ne, int transposed, cx<TO>* __restrict__ z) {
   const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
