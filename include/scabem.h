@@ -193,8 +193,10 @@ int scabem_set_sigma(scabem_op_t op, const scabem_sigma* sigma);
 /* y = A x for nrhs right-hand sides.  x and y may be device or host memory
  * (host buffers are staged through device copies on `stream`).  prec selects
  * complex64 or complex128 arithmetic; the operator must have been built with
- * that precision.  Stream-ordered: returns after enqueueing (device buffers)
- * or after completion (host buffers).  scabem_sigma_gradient waits on its
+ * that precision.  y may be x (in place); with several right-hand sides, a y
+ * that overlaps x in another way is not supported.  Stream-ordered: returns
+ * after enqueueing (device buffers) or after completion (host buffers).
+ * scabem_sigma_gradient waits on its
  * own bulk copies of near records with a time limit (about a second); if one
  * expires, that call's result is not valid and the next scabem_apply or
  * scabem_solve on the operator returns SCABEM_E_TIMEOUT. */

@@ -688,6 +688,19 @@ int grid_potentials(scabem_op* op, const cx<R>* x, int k, cudaStream_t s) {
   return fft_conv<R>(op, pd, s, false, k);
 }
 
+// The last kernel of a product still reads its input while it writes the result:
+// an input column that overlaps the result is copied first, into pd.xi.
+template <typename R>
+static int apart(scabem_op* op, const cx<R>*& in, const cx<R>* out, cudaStream_t s) {
+  const auto a = reinterpret_cast<uintptr_t>(in), b = reinterpret_cast<uintptr_t>(out);
+  const uintptr_t len = sizeof(cx<R>) * (uintptr_t)op->N;
+  if (a >= b + len || b >= a + len) return SCABEM_OK;
+  cx<R>* xi = pdata<R>(op).xi;
+  CK(launch_pdl(k_interleave<R>, dim3((unsigned)cdiv(op->N, 256)), 256, 0, s, in, op->N, op->N, 1, 1, 1, xi));
+  in = xi;
+  return SCABEM_OK;
+}
+
 template <typename R>
 int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int k, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
@@ -700,6 +713,8 @@ int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ld
     CK(launch_pdl(k_interleave<R>, dim3((unsigned)cdiv(op->N * st, 256)), 256, 0, s, x, ldx, op->N, k, batch_group(k),
                   st, pd.xi));
     x = pd.xi;
+  } else if (int rc = apart<R>(op, x, y, s)) {
+    return rc;
   }
   if (int rc = grid_potentials<R>(op, x, k, s)) return rc;
   prof_mark(op, s);
@@ -717,13 +732,7 @@ int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s) {
 template <typename R>
 int apply_adjoint_one(scabem_op* op, const cx<R>* ybar, cx<R>* xbar, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
-  // the last kernel still reads y while it writes x: in place, y is copied first
-  const auto a = reinterpret_cast<uintptr_t>(ybar), b = reinterpret_cast<uintptr_t>(xbar);
-  const uintptr_t len = sizeof(cx<R>) * (uintptr_t)op->N;
-  if (a < b + len && b < a + len) {
-    CK(launch_pdl(k_interleave<R>, dim3((unsigned)cdiv(op->N, 256)), 256, 0, s, ybar, op->N, op->N, 1, 1, 1, pd.xi));
-    ybar = pd.xi;
-  }
+  if (int rc = apart<R>(op, ybar, xbar, s)) return rc;
   const bool wide = project_wide(op, 1);
   CK(launch_pdl(wide ? k_grid_adj<R, 8> : k_grid_adj<R, 1>, dim3((unsigned)cdiv(op->ngp * (wide ? 256 : 32), 256)), 256, 0, s, ybar, op->gp, op->gpoff, op->gpl,
                 op->gpr, op->gpe, pd.xw, op->nxl, op->ngp, (int64_t)op->n[0] * op->nac, op->nL, op->nR, (R)op->ke,
