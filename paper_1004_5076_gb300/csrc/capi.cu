@@ -87,7 +87,6 @@ void free_prec(PrecData<R>& pd) {
   for (int a = 0; a < 3; ++a) cudaFree(pd.tw[a]);
   cudaFree(pd.L);
   cudaFree(pd.dL);
-  cudaFree(pd.sig);
   cudaFree(pd.tp);
   cudaFree(pd.summ);
   cudaFree(pd.src);
@@ -126,16 +125,18 @@ int alloc_st(scabem_op* op, PrecData<R>& pd, cudaStream_t s) {
 template <typename R>
 int alloc_prec(scabem_op* op, PrecData<R>& pd, bool workspaces, cudaStream_t s) {
   int rc;
-  if ((rc = dalloc(&pd.L, op->Q * 3 * op->p))) return rc;
-  if ((rc = dalloc(&pd.dL, op->Q * 3 * op->p))) return rc;
-  if ((rc = dalloc(&pd.sig, op->Q))) return rc;
-  if ((rc = dalloc(&pd.tp, op->Q * 16))) return rc;
+  if (sizeof(R) == sizeof(double)) {  // set-up reads these for either precision
+    if ((rc = dalloc(&pd.L, op->Q * 3 * op->p))) return rc;
+    if ((rc = dalloc(&pd.dL, op->Q * 3 * op->p))) return rc;
+    if ((rc = dalloc(&pd.tp, op->Q * 16))) return rc;
+    if (workspaces && (rc = dalloc(&pd.summ, op->nt * 12))) return rc;
+  }
   if (!workspaces) return SCABEM_OK;
   for (int a = 0; a < 3; ++a) {
     if ((rc = dalloc(&pd.tw[a], op->P[a]))) return rc;
     if ((rc = make_twiddles<R>(pd.tw[a], op->P[a], s))) return rc;
   }
-  if ((rc = dalloc(&pd.summ, op->nt * 12)) || (rc = dalloc(&pd.xi, op->N))) return rc;
+  if ((rc = dalloc(&pd.xi, op->N))) return rc;
   pd.built = true;
   return SCABEM_OK;
 }
@@ -762,7 +763,6 @@ void scabem_op_destroy(scabem_op_t op) {
   cudaFree(op->cX);
   cudaFree(op->unk);
   cudaFree(op->region);
-  cudaFree(op->trirow);
   cudaFree(op->valrow);
   cudaFree(op->rowsrc);
   cudaFree(op->qp);

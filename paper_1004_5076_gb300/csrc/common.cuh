@@ -137,12 +137,12 @@ struct PrecData {
   cx<R>* gt[2] = {nullptr, nullptr};    // tables of the direct (y, z) sums: [q0][|d1|][|d2|], or by parity
   cx<R>* near = nullptr;                // [npairs][NCORR][q][2]
   cx<R>* tw[3] = {nullptr, nullptr, nullptr};  // forward twiddles per axis length
-  R* L = nullptr;                       // Q * 3 * p stencil weights
-  R* dL = nullptr;                      // Q * 3 * p derivative weights [1/um]
-  R* sig = nullptr;                     // Q normalised conductivity
-  R* tp = nullptr;                      // Q * 16 testing geometry: rel (3), w, X_k (3 x 3), div X_k (3)
-  // workspaces
+  // complex128 data only (set-up, the conductivity gradient, fields at points)
+  R* L = nullptr;         // Q * 3 * p stencil weights
+  R* dL = nullptr;        // Q * 3 * p derivative weights [1/um]
+  R* tp = nullptr;        // Q * 16 testing geometry: rel (3), w, X_k (3 x 3), div X_k (3)
   cx<R>* summ = nullptr;  // nt * 3 sets * 4
+  // workspaces
   cx<R>* src = nullptr;   // 16 * n0 * nac (12 sources; 16 in the transposed apply), [field][i0][active column]
   cx<R>* stA = nullptr;   // 16 * P0 * cst (12 fields in the apply, 16 in the transposed apply)
   cx<R>* stB = nullptr;   // 16 * P0 * cst
@@ -186,7 +186,6 @@ struct scabem_op {
   double* cX = nullptr;     // nt * 3: s_k l_k / (2 A)
   int32_t* unk = nullptr;   // nt * 3 (local k) * 3 (set): (index+1)*sign, 0 = none
   int32_t* region = nullptr;
-  int32_t* trirow = nullptr;  // nt * 3 * 4: 1 if that (t,k,type) row exists
   int32_t* rowsrc = nullptr;  // N * 2 : ((t*3+k)*4+type) of T+ and T-
   int32_t* valrow = nullptr;  // nt * 12: row of each (t, k, type) value, -1 if none
   double* qp = nullptr;       // Q * 3
@@ -217,7 +216,7 @@ struct scabem_op {
   bool parity = false;  // the direct sums run block-diagonalised by parity (gt: its tables)
   int R1 = 0, R2 = 0;
   int32_t* acoord = nullptr;  // nac
-  double* sig64 = nullptr;    // Q normalised (master copy)
+  double* sig64 = nullptr;    // Q normalised conductivity
   // near list
   int64_t npairs = 0;
   int32_t* noff = nullptr;  // nt + 1

@@ -95,7 +95,7 @@ __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restri
                            int p, double h, double ox, double oy, double oz, int n0, int n1, int n2,
                            double* __restrict__ tri, double* __restrict__ cX, double* __restrict__ qp,
                            double* __restrict__ qw, int32_t* __restrict__ base, double* __restrict__ Ld,
-                           double* __restrict__ dLd, float* __restrict__ Lf, float* __restrict__ dLf, int* err) {
+                           double* __restrict__ dLd, int* err) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double v[3][3];
@@ -143,8 +143,6 @@ __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restri
       for (int i = 0; i < p; ++i) {
         Ld[(3 * Qi + ax) * p + i] = L[i];
         dLd[(3 * Qi + ax) * p + i] = dL[i] / h;
-        Lf[(3 * Qi + ax) * p + i] = (float)L[i];
-        dLf[(3 * Qi + ax) * p + i] = (float)(dL[i] / h);
       }
     }
   }
@@ -476,13 +474,12 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-// Testing geometry per quadrature point Qi (point a of triangle t), formed in
-// FP64 and stored in each operator precision: the offset from the centroid
-// (3), the weight, the RWG test functions X_k(r) = cX_k (r - v_k) of the three
+// Testing geometry per quadrature point Qi (point a of triangle t): the offset
+// from the centroid (3), the weight, the RWG test functions X_k(r) = cX_k (r - v_k) of the three
 // local edges (3 x 3) and their divergences 2 cX_k.
 __global__ void k_test_geometry(const double* __restrict__ tri, const double* __restrict__ cX,
                                 const double* __restrict__ qp, const double* __restrict__ qw, int64_t Q, int q,
-                                double* __restrict__ td, float* __restrict__ tf) {
+                                double* __restrict__ td) {
   const int64_t Qi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (Qi >= Q) return;
   const int64_t t = Qi / q;
@@ -494,15 +491,12 @@ __global__ void k_test_geometry(const double* __restrict__ tri, const double* __
     for (int c = 0; c < 3; ++c) v[4 + 3 * k + c] = cX[3 * t + k] * (qp[3 * Qi + c] - g[3 * k + c]);
     v[13 + k] = 2.0 * cX[3 * t + k];
   }
-  for (int c = 0; c < 16; ++c) {
-    if (td) td[16 * Qi + c] = v[c];
-    if (tf) tf[16 * Qi + c] = (float)v[c];
-  }
+  for (int c = 0; c < 16; ++c) td[16 * Qi + c] = v[c];
 }
 
 // ---------------------------------------------------------------- conductivity
 __global__ void k_sigma_monomial(const double* __restrict__ qp, int64_t Q, int nseg, const double* __restrict__ seg,
-                                 double* __restrict__ sd, float* __restrict__ sf, double* __restrict__ s64) {
+                                 double* __restrict__ s64) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= Q) return;
   double sig = 0.0;
@@ -514,10 +508,7 @@ __global__ void k_sigma_monomial(const double* __restrict__ qp, int64_t Q, int n
     const double u = s > 1.0 ? 1.0 : s;
     sig += sgp[2] * pow(u, sgp[3]);
   }
-  sig *= ETA0;
-  s64[i] = sig;
-  if (sd) sd[i] = sig;
-  if (sf) sf[i] = (float)sig;
+  s64[i] = sig * ETA0;
 }
 
 // Cubic B-spline profile sum_k coef[k] N_k(s), s = (x_axis - x0) / L, on the
@@ -525,8 +516,7 @@ __global__ void k_sigma_monomial(const double* __restrict__ qp, int64_t Q, int n
 // j / (ncoef - 3)), zero outside [0, 1]: the knot span of s and de Boor's
 // triangular scheme over the four coefficients that act there.
 __global__ void k_sigma_bspline(const double* __restrict__ qp, int64_t Q, double x0, double L, int axis, int ncoef,
-                                const double* __restrict__ coef, double* __restrict__ sd, float* __restrict__ sf,
-                                double* __restrict__ s64) {
+                                const double* __restrict__ coef, double* __restrict__ s64) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= Q) return;
   const double s = (qp[3 * i + axis] - x0) / L;
@@ -553,20 +543,13 @@ __global__ void k_sigma_bspline(const double* __restrict__ qp, int64_t Q, double
       }
     sig = d[3];
   }
-  sig *= ETA0;
-  s64[i] = sig;
-  if (sd) sd[i] = sig;
-  if (sf) sf[i] = (float)sig;
+  s64[i] = sig * ETA0;
 }
 
-__global__ void k_sigma_copy(const double* __restrict__ in, int64_t Q, double* __restrict__ sd, float* __restrict__ sf,
-                             double* __restrict__ s64) {
+__global__ void k_sigma_copy(const double* __restrict__ in, int64_t Q, double* __restrict__ s64) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= Q) return;
-  const double sig = in[i] * ETA0;
-  s64[i] = sig;
-  if (sd) sd[i] = sig;
-  if (sf) sf[i] = (float)sig;
+  s64[i] = in[i] * ETA0;
 }
 
 // ---------------------------------------------------------------- block-diagonal preconditioner
@@ -969,11 +952,9 @@ int setup_geometry(scabem_op* op, const scabem_mesh* m, cudaStream_t s) {
   CK(cudaMemsetAsync(op->err, 0, sizeof(int), s));
   k_geometry<<<(int)cdiv(op->nt, 128), 128, 0, s>>>(dV, dT, dS, op->nt, op->q, rule, op->p, op->h, op->origin[0],
                                                      op->origin[1], op->origin[2], op->n[0], op->n[1], op->n[2],
-                                                     op->tri, op->cX, op->qp, op->qw, op->base, op->d.L, op->d.dL,
-                                                     op->f.L, op->f.dL, op->err);
+                                                     op->tri, op->cX, op->qp, op->qw, op->base, op->d.L, op->d.dL, op->err);
   CK(cudaGetLastError());
-  k_test_geometry<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(op->tri, op->cX, op->qp, op->qw, op->Q, op->q, op->d.tp,
-                                                        op->f.tp);
+  k_test_geometry<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(op->tri, op->cX, op->qp, op->qw, op->Q, op->q, op->d.tp);
   CK(cudaGetLastError());
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, op->err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1104,7 +1085,7 @@ int setup_sigma_monomial(scabem_op* op, int nseg, const double* seg, cudaStream_
     CK(cudaMalloc(&dseg, sizeof(double) * 6 * nseg));
     CK(cudaMemcpyAsync(dseg, seg, sizeof(double) * 6 * nseg, cudaMemcpyHostToDevice, s));
   }
-  k_sigma_monomial<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(op->qp, op->Q, nseg, dseg, op->d.sig, op->f.sig, op->sig64);
+  k_sigma_monomial<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(op->qp, op->Q, nseg, dseg, op->sig64);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   if (dseg) cudaFree(dseg);
@@ -1117,8 +1098,7 @@ int setup_sigma_bspline(scabem_op* op, double x0, double L, int axis, int ncoef,
   double* dc = nullptr;
   CK(cudaMalloc(&dc, sizeof(double) * ncoef));
   CK(cudaMemcpyAsync(dc, coef, sizeof(double) * ncoef, cudaMemcpyHostToDevice, s));
-  k_sigma_bspline<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(op->qp, op->Q, x0, L, axis, ncoef, dc, op->d.sig, op->f.sig,
-                                                        op->sig64);
+  k_sigma_bspline<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(op->qp, op->Q, x0, L, axis, ncoef, dc, op->sig64);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   cudaFree(dc);
@@ -1131,7 +1111,7 @@ int setup_sigma_values(scabem_op* op, const double* per_q_host, cudaStream_t s) 
   double* tmp = nullptr;
   CK(cudaMalloc(&tmp, sizeof(double) * op->Q));
   CK(cudaMemcpyAsync(tmp, per_q_host, sizeof(double) * op->Q, cudaMemcpyHostToDevice, s));
-  k_sigma_copy<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(tmp, op->Q, op->d.sig, op->f.sig, op->sig64);
+  k_sigma_copy<<<(int)cdiv(op->Q, 256), 256, 0, s>>>(tmp, op->Q, op->sig64);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   cudaFree(tmp);
