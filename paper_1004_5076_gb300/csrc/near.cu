@@ -771,16 +771,24 @@ PrecData<double>& pdata<double>(scabem_op* op) {
 RowTables row_tables(const scabem_op* op, const void* desc) {
   return {(const RowDesc*)desc, op->nm_col, op->nm_gcol, op->xpt, op->ne, op->nL, op->nxl};
 }
-// a warp per row; a whole CTA per row where warps would leave the chip idle
-// and the rows are long (77 columns per row on the 12 um guide).  Apply of a 480
-// edge sphere: 23.4 us with warps, 20.4 with CTAs; at 2268 edges the two meet
-// (solve of the 2 um guide 121 and 123 ms), and from 32 rows per SM on warps fill it.
-bool wide_rows(const scabem_op* op) { return op->ne < 152 * 32 && op->nm_nnz > 64 * op->ne; }
+// A warp per row and group of right-hand sides; a whole CTA where these are few
+// and the rows long, so that warps would leave the chip idle.  Products of guides and
+// spheres, warps and CTAs, us, complex64 (rows of 71 to 105 columns): 624 rows
+// 19.9 and 18.4, 1188 rows 20.1 and 18.8, 1992 rows 25.2 and 25.7, 2268 rows 24.0
+// and 25.2, 3900 rows 30.4 and 35.1; eight columns (two groups) of 624 rows 48.7 and
+// 44.4, 1020 rows 53.1 and 53.2, 1188 rows 51.3 and 53.0, 1992 rows 71.9 and 78.2: they
+// meet at 14 rows and groups per SM.  Complex128 keeps the FP64 units busy sooner: 480
+// rows 115.6 and 113.2, 624 rows 87.3 and 89.4, 1020 rows 96.0 and 102.9, 3900 rows
+// 209 and 244: 6 per SM.
+template <typename R>
+bool wide_rows(const scabem_op* op, int groups) {
+  return op->ne * groups < 152 * (sizeof(R) == 4 ? 14 : 6) && op->nm_nnz > 64 * op->ne;
+}
 
 template <typename R, int K>
 int launch_rows(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
-  const bool wide = wide_rows(op);
+  const bool wide = wide_rows<R>(op, (int)cdiv(kc, K));
   auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
   const int64_t units = op->ne * cdiv(kc, K);
   CK(launch_pdl(fn, dim3((unsigned)cdiv(units * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
@@ -811,7 +819,7 @@ template int rows_apply<double>(scabem_op*, const cx<double>*, cx<double>*, int6
 template <typename R>
 int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
-  const bool wide = wide_rows(op);
+  const bool wide = wide_rows<R>(op, 1);
   auto fn = wide ? k_rows_adj<R, NM_THREADS> : k_rows_adj<R, 32>;
   CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
                 row_tables(op, op->rdesc_t), pd.nmt, pd.gram, pd.xw, pd.grid, y, x));
