@@ -173,7 +173,9 @@ void scabem_op_destroy(scabem_op_t op);
  *     finite, >= 0).  A smooth profile for gradient studies with respect to
  *     the coefficients.
  * Conductivity enters only the Eq. 13 / Eq. 14 rows of absorber edges.
- * Fields a kind does not use are ignored. */
+ * Fields a kind does not use are ignored.  scabem_set_sigma runs on the legacy
+ * default stream and returns when it is complete; work of the operator that is
+ * still in flight on a stream not ordered with that one has to end first. */
 typedef enum {
   SCABEM_SIGMA_MONOMIAL = 0,
   SCABEM_SIGMA_PER_QPOINT = 1,
@@ -269,10 +271,9 @@ int scabem_selftest_wait_limit(scabem_op_t op, void* stream);
 /* x = A^T y, the transpose (not the conjugate transpose) of the operator of
  * scabem_apply, for adjoint solves and gradients (reciprocity of the
  * Galerkin system).  The stages of scabem_apply run transposed in reverse
- * order: testing and row sums, near-field precorrection (over the source
- * triangles), interpolation (value and derivative stencils), the grid
- * convolution (each potential field with its medium's Green function),
- * projection and the current expansion.  Same arguments, layouts, host
+ * order: the rows' edge stencils onto the grid, the grid convolution (each
+ * field with its medium's Green function), and the projection's stencils
+ * together with the transposed near matrix.  Same arguments, layouts, host
  * staging and errors as scabem_apply, with y the input and x the output. */
 int scabem_apply_adjoint(scabem_op_t op, const void* y, void* x, int32_t nrhs, int64_t ld, int32_t prec,
                          void* stream);

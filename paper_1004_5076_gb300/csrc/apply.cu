@@ -1,4 +1,5 @@
-// The matvec y = A x of the grid-accelerated operator (one right-hand side).
+// The matvec y = A x of the grid-accelerated operator, for one right-hand side or
+// a batch of up to eight, and its transpose.
 //
 //  K1 k_project  RWG coefficients -> point sources on the grid (12 fields: the
 //                exterior J, interior J and exterior M sets, current reduction
@@ -350,10 +351,10 @@ __device__ __forceinline__ void mbar_init_fence() {
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-// The near records are read once per apply: their copies carry an L2
-// evict-first policy, so that the stream of records does not push the
-// apply's reused data (grids, sources, geometry) and the caller's vectors out
-// of L2.
+// The near records are read once per conductivity gradient, the only reader
+// besides set-up: their copies carry an L2 evict-first policy, so that the
+// stream of records does not push the reused data (potentials, summaries,
+// geometry) and the caller's vectors out of L2.
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(pol));

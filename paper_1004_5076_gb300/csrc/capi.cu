@@ -224,8 +224,8 @@ int apply_prec(scabem_op* op, const void* xv, void* yv, int nrhs, int64_t ld, cu
   const bool xd = is_device_ptr(xv), yd = is_device_ptr(yv);
   const int64_t N = op->N;
   if (!adjoint && nrhs > 1) {
-    // batches of up to KBATCH columns: each stage runs once per batch and the
-    // point kernel reads the near records once per batch
+    // batches of up to KBATCH columns: each stage runs once per batch and the rows
+    // read the near matrix once per group of up to four columns
     const int kb = nrhs < KBATCH ? nrhs : KBATCH;
     int rc = ensure_batch<R>(op, kb, s);
     if (rc) return rc;

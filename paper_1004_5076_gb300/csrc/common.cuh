@@ -107,10 +107,10 @@ constexpr int NCORR = 10;  // per point and medium: dP0, dP1(3), dQ(3), dC(3)
 constexpr double ETA0 = 376.730313668;
 
 // ------------------------------------------------------------------ profiling
-// Stages of one apply: summaries (with the quadrature-point sources),
-// projection, FFT axis 0 forward, (y, z) convolution with the Green
-// function, FFT axis 0 inverse, points (interpolation, near field, testing
-// and the row sums).
+// Stages of one apply: an empty one (the current summaries, which the projection
+// has taken in), projection, FFT axis 0 forward, (y, z) convolution with the
+// Green functions, FFT axis 0 inverse, rows (testing of the potentials and the
+// near matrix).
 constexpr int NSTAGE = 6;
 struct Profiler {
   bool on = false;
@@ -135,7 +135,7 @@ struct PrecData {
   bool built = false;
   cx<R>* ghat[2] = {nullptr, nullptr};  // octant spectra [q0][q2][q1], scaled by 1/(P0 P1 P2)
   cx<R>* gt[2] = {nullptr, nullptr};    // tables of the direct (y, z) sums: [q0][|d1|][|d2|], or by parity
-  cx<R>* near = nullptr;                // [npairs][NCORR][q][2]
+  cx<R>* near = nullptr;                // near records [pair][target point][medium][NCORR]
   cx<R>* tw[3] = {nullptr, nullptr, nullptr};  // forward twiddles per axis length
   // complex128 data only (set-up, the conductivity gradient, fields at points)
   R* L = nullptr;         // Q * 3 * p stencil weights
@@ -282,8 +282,7 @@ inline int64_t parity_words(const scabem_op* op) {
   const int64_t E1 = (op->R1 + 1) / 2, O1 = op->R1 - E1, E2 = (op->R2 + 1) / 2, O2 = op->R2 - E2;
   return (E1 * E1 + O1 * O1) * (E2 * E2 + O2 * O2);
 }
-// Right-hand sides the batched apply handles per pass (one CTA of that many
-// warps shares each target triangle's near-record stream).
+// Right-hand sides that go through the stages of a batched apply together.
 constexpr int KBATCH = 8;
 
 // Record the next stage-boundary event when profiling is on.
@@ -351,8 +350,8 @@ int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s);
 template <typename R>
 int apply_one(scabem_op* op, const cx<R>* x, cx<R>* y, cudaStream_t s);
 // y[:, c] = A x[:, c] for c < k <= pd.kcap (k <= KBATCH), x and y column-major with
-// leading dimensions ldx, ldy; every stage runs once for all k columns and the
-// point kernel reads each near record once for all of them
+// leading dimensions ldx, ldy; every stage runs once for all k columns, and the rows
+// read the near matrix and the weights once per group of up to four columns
 template <typename R>
 int apply_batch(scabem_op* op, const cx<R>* x, int64_t ldx, cx<R>* y, int64_t ldy, int k, cudaStream_t s);
 // grow the forward workspaces of precision R to k right-hand sides

@@ -6,10 +6,11 @@
 // the (i1, i2) columns that some stencil covers); the transform size is P = 2n
 // per axis.  The convolution runs in three kernels:
 //   stage A: forward FFT along axis 0 of the 12 source fields, input pruned
-//            to i0 < n0, output [field][k0][i1][i2] (P0 x n1 x n2);
-//   stage B: per k0 plane, forward 2-D FFT over (i1, i2) (input pruned to the
-//            physical n1 x n2 corner), multiply by the Green spectrum of the
-//            medium, inverse 2-D FFT, keep the physical corner: 12 -> 16 fields;
+//            to i0 < n0, output [field][k0][column];
+//   stage B: per k0, the (y, z) convolution with the Green function of the
+//            medium, 12 -> 16 fields: zero-padded 2-D FFTs over whole planes
+//            (n1 n2 columns), direct sums over the active columns, or those sums
+//            block-diagonalised by parity;
 //   stage C: inverse FFT along axis 0, keep i0 < n0, written point-major
 //            [i0][active column][32] for the testing gathers.
 // Every FFT is an in-place shared-memory Stockham transform (radix 8, then 4

@@ -619,7 +619,7 @@ struct RowTables {
 // loaded a column ahead, the weights a block of entries ahead of their use.  The
 // form before (near records per triangle pair and target point, 706 MB per product
 // instead of 230, tested per triangle) took 145 us in complex64 and 5.0 ms in
-// complex128 on the 12 um guide; this one 67 and 336 us.
+// complex128 on the 12 um guide; this one 62 and 321 us.
 template <typename R, int K, int LANES>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : K == 2 ? 7 : 6)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
@@ -802,7 +802,8 @@ int launch_rows(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cu
 // y_c = A x_c from the potentials pd.grid (column c) and the near matrix, c <
 // kc <= KBATCH, x in the layout of load_cols.  At most four right-hand sides
 // per warp: eight hold 126 registers and half the warps (325 us for 8 columns
-// of the 12 um guide; 300 us with four; 274 us with x interleaved).
+// of the 12 um guide; 300 us with four; 274 us with x interleaved; 249 us with a
+// block's point indices handed out before its loads).
 template <typename R>
 int rows_apply(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
   switch (batch_group(kc)) {

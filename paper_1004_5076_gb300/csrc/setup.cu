@@ -873,6 +873,12 @@ int setup_gather(scabem_op* op, cudaStream_t s) {
     const size_t csz = (op->prec_mask & 2) ? sizeof(cx<double>) : sizeof(cx<float>);
     const size_t sm = ((size_t)op->nac * 8 + (size_t)op->R1 * op->R2) * csz + sizeof(int32_t) * op->nac;
     op->direct_fits = sm <= 227 * 1024;
+    // The line of nac^2 against the planes' size was found for the sums without parity
+    // and holds with it.  Products with planes and with sums, us, complex64:
+    // spheres of 32 x 32 planes (nac 178) 20 and 44, with three columns 37 and 53,
+    // with eight 69 and 67; of 64 x 64 planes (nac 759) 37 and 463; guides of
+    // 32 x 16 planes (nac 60) 24 and 21, 45 and 34, 95 and 66; of 64 x 64 planes
+    // (nac 104) 167 and 102, 401 and 214, 977 and 499.
     const bool want = op->transverse == 2 || !op->planes_fit ||
                       (op->transverse == 0 && op->nac * op->nac <= 16 * (int64_t)op->P[1] * op->P[2]);
     op->tdirect = want && (op->direct_fits || !op->planes_fit);

@@ -441,8 +441,8 @@ __global__ void k_band_loss(const cd* __restrict__ summ, const double* __restric
 
 // ---------------------------------------------------------------- batched GMRES (FP64 Krylov work)
 // K <= KBATCH right-hand sides run in lockstep.  One batched operator apply
-// per Arnoldi step serves all K (the point kernel reads the near records
-// once for them); everything else in the step stays on the device: the
+// per Arnoldi step serves all K (the rows read the near matrix once per group of
+// up to four); everything else in the step stays on the device: the
 // norms, classical Gram-Schmidt whose second pass runs per column only when
 // the first one cancels most of w (|w'| < |w| / sqrt 2, the Daniel-Gragg-
 // Kaufman-Stewart test), the Givens update of the Hessenberg least squares
