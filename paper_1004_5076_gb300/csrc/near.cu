@@ -515,9 +515,10 @@ __device__ __forceinline__ void near_reduce(cx<R> acc[3][K]) {
 // a point against two weights into ga[c], so that a warp's loads are
 // contiguous (the 128 or 256 bytes of a point in complex64).  Entries go in
 // blocks of GR_IF slots: a block's point indices are loaded by the lanes one
-// block ahead and handed out by shuffles, and then all of its weights and (one
-// right-hand side) potentials are loaded before the first is used (shuffles and
-// loads in turn: complex128 product of the 12 um guide 780 us, 755 this way).
+// block ahead and handed out by shuffles, and all of its weights and (one
+// right-hand side) potentials are loaded before the first is used.  AHEAD hands
+// out the whole block's indices before its loads (a plain load does not move across
+// a shuffle); rows_ahead says where not.
 constexpr int GR_IF = 4;
 
 __device__ __forceinline__ void load_two(const float* p, float* v) {
@@ -542,7 +543,7 @@ __device__ __forceinline__ void load_pot(const cx<double>* p, cx<double>* v) {
   v[1] = mk(b.x, b.y);
 }
 
-template <typename R, int K, int H, int STRIDE, int LANES>
+template <typename R, int K, int H, int STRIDE, int LANES, bool AHEAD>
 __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n, const R* __restrict__ w,
                                           const cx<R>* pot, int64_t cs_g, int kc, int lane, cx<R> ga[K]) {
   constexpr int S = 32 / H, BLK = GR_IF * S, STEP = BLK * (LANES / 32);
@@ -555,11 +556,14 @@ __device__ __forceinline__ void grid_rows(const int32_t* __restrict__ xpt, int n
     R a[GR_IF][2];
     cx<R> g[GR_IF][2];
     const cx<R>* pp[GR_IF];
+    auto point = [&](int u) { return pot + (int64_t)__shfl_sync(0xffffffffu, cur, u * S + slot) * NPOT; };
+    if constexpr (AHEAD)
 #pragma unroll
-    for (int u = 0; u < GR_IF; ++u) pp[u] = pot + (int64_t)__shfl_sync(0xffffffffu, cur, u * S + slot) * NPOT;
+      for (int u = 0; u < GR_IF; ++u) pp[u] = point(u);
 #pragma unroll
     for (int u = 0; u < GR_IF; ++u) {
       const int j = b + u * S + slot;
+      if constexpr (!AHEAD) pp[u] = point(u);
       a[u][0] = a[u][1] = R(0);
       g[u][0] = g[u][1] = czero<R>();
       if (j < n) {
@@ -620,7 +624,7 @@ struct RowTables {
 // form before (near records per triangle pair and target point, 706 MB per product
 // instead of 230, tested per triangle) took 145 us in complex64 and 5.0 ms in
 // complex128 on the 12 um guide; this one 62 and 321 us.
-template <typename R, int K, int LANES>
+template <typename R, int K, int LANES, bool AHEAD>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : K == 2 ? 7 : 6)
     k_rows(RowTables T, const cx<R>* __restrict__ nmv, const R* __restrict__ gval, const R* __restrict__ xw,
            const cx<R>* pot, int64_t cs_g, const cx<R>* __restrict__ x, int xst, cx<R>* __restrict__ y, int64_t ldy,
@@ -658,13 +662,13 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
     int i;
     if (r < nL) {
       const int h = lane & 7;
-      grid_rows<R, K, 8, 8, LANES>(T.xpt + x0, D.nx, xw + 8 * x0 + 2 * (h & 3), pot + 2 * h, cs_g, kc, lane, ga);
+      grid_rows<R, K, 8, 8, LANES, AHEAD>(T.xpt + x0, D.nx, xw + 8 * x0 + 2 * (h & 3), pot + 2 * h, cs_g, kc, lane, ga);
       i = h >> 2;  // groups 0, 1 -> E row; 2, 3 -> H row
     } else {
       const int h = lane & 15, g = h >> 1;
-      grid_rows<R, K, 16, 24, LANES>(T.xpt + x0, D.nx,
-                                     xw + 8 * T.nxl + 24 * (x0 - T.nxl) + 2 * (g < 4 ? h & 3 : h - 4), pot + 2 * h, cs_g,
-                                     kc, lane, ga);
+      grid_rows<R, K, 16, 24, LANES, AHEAD>(T.xpt + x0, D.nx,
+                                            xw + 8 * T.nxl + 24 * (x0 - T.nxl) + 2 * (g < 4 ? h & 3 : h - 4),
+                                            pot + 2 * h, cs_g, kc, lane, ga);
       i = (g + 2) >> 2;  // groups 0, 1 -> Eq. 3; 2 .. 5 -> Eq. 13; 6, 7 -> Eq. 14
       if (lane < 5) {
         const int g = T.gcol[5 * (r - nL) + lane];
@@ -704,7 +708,7 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 8 ? 1 : K == 1 ? 8 : 
 // The same for the transposed apply: x = near part (transposed matrix) +
 // projection transposed (the value blocks Q0 against the convolved adjoint
 // fields of J_e, M outside, J_i, M inside: groups 4 .. 7 of pot).
-template <typename R, int LANES>
+template <typename R, int LANES, bool AHEAD>
 __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
     k_rows_adj(RowTables T, const cx<R>* __restrict__ nmt, const R* __restrict__ gval, const R* __restrict__ xw,
                const cx<R>* pot, const cx<R>* __restrict__ y, cx<R>* __restrict__ x) {
@@ -723,10 +727,10 @@ __global__ void __launch_bounds__(NM_THREADS, sizeof(R) == 4 ? 8 : 1)
     const int h = lane & 7, grp = h >> 1;
     cx<R> gs[1] = {czero<R>()};
     if (r < nL)
-      grid_rows<R, 1, 8, 8, LANES>(T.xpt + x0, D.nx, xw + 8 * x0 + 2 * (h & 1), pot + 16 + 2 * h, 0, 1, lane, gs);
+      grid_rows<R, 1, 8, 8, LANES, AHEAD>(T.xpt + x0, D.nx, xw + 8 * x0 + 2 * (h & 1), pot + 16 + 2 * h, 0, 1, lane, gs);
     else
-      grid_rows<R, 1, 8, 24, LANES>(T.xpt + x0, D.nx, xw + 8 * T.nxl + 24 * (x0 - T.nxl) + 2 * (h & 1), pot + 16 + 2 * h,
-                                    0, 1, lane, gs);
+      grid_rows<R, 1, 8, 24, LANES, AHEAD>(T.xpt + x0, D.nx, xw + 8 * T.nxl + 24 * (x0 - T.nxl) + 2 * (h & 1),
+                                           pot + 16 + 2 * h, 0, 1, lane, gs);
     const cx<R> ga = gs[0];
     // groups J_e, M, J_i, -M; on plain edges J_i = -J_e
     if (r < nL) {
@@ -785,11 +789,21 @@ bool wide_rows(const scabem_op* op, int groups) {
   return op->ne * groups < 152 * (sizeof(R) == 4 ? 14 : 6) && op->nm_nnz > 64 * op->ne;
 }
 
+// Whether a warp's row of one complex128 column hands out its point indices ahead
+// of the loads: 104 registers and 16 rows per SM at a time, against 134 and 12.
+// Large operators gain by it (4368 rows 208 us against 216, 29,130 rows 755 and 778).
+// Up to about two rounds of rows the last round, nearly empty, decides, for either
+// form at its own sizes (1776 rows 151 and 148 us, 2208 rows 160 and 166, 3072 rows
+// 199 and 191, 3648 rows 204 and 202): there the form with fewer rows in flight stays.
+bool rows_ahead(const scabem_op* op) { return op->ne >= 152 * 28; }
+
 template <typename R, int K>
 int launch_rows(scabem_op* op, const cx<R>* x, cx<R>* y, int64_t ldy, int kc, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
   const bool wide = wide_rows<R>(op, (int)cdiv(kc, K));
-  auto fn = wide ? k_rows<R, K, NM_THREADS> : k_rows<R, K, 32>;
+  auto fn = wide ? k_rows<R, K, NM_THREADS, true> : k_rows<R, K, 32, true>;
+  if constexpr (sizeof(R) == 8 && K == 1)
+    if (!wide && !rows_ahead(op)) fn = k_rows<R, K, 32, false>;
   const int64_t units = op->ne * cdiv(kc, K);
   CK(launch_pdl(fn, dim3((unsigned)cdiv(units * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
                 row_tables(op, op->rdesc), pd.nmv, pd.gram, pd.xw, pd.grid, col_stride_pot(op), x, batch_stride(kc),
@@ -821,7 +835,9 @@ template <typename R>
 int rows_adjoint(scabem_op* op, const cx<R>* y, cx<R>* x, cudaStream_t s) {
   PrecData<R>& pd = pdata<R>(op);
   const bool wide = wide_rows<R>(op, 1);
-  auto fn = wide ? k_rows_adj<R, NM_THREADS> : k_rows_adj<R, 32>;
+  auto fn = wide ? k_rows_adj<R, NM_THREADS, true> : k_rows_adj<R, 32, true>;
+  if constexpr (sizeof(R) == 8)
+    if (!wide && !rows_ahead(op)) fn = k_rows_adj<R, 32, false>;
   CK(launch_pdl(fn, dim3((unsigned)cdiv(op->ne * (wide ? NM_THREADS : 32), NM_THREADS)), NM_THREADS, 0, s,
                 row_tables(op, op->rdesc_t), pd.nmt, pd.gram, pd.xw, pd.grid, y, x));
   return SCABEM_OK;
