@@ -792,7 +792,7 @@ bool wide_rows(const scabem_op* op, int groups) {
 // Whether a warp's row of one complex128 column hands out its point indices ahead
 // of the loads: 104 registers and 16 rows per SM at a time, against 134 and 12.
 // Large operators gain by it (4368 rows 208 us against 216, 29,130 rows 755 and 778).
-// Up to about two rounds of rows the last round, nearly empty, decides, for either
+// Up to about two waves of rows the last wave, nearly empty, decides, for either
 // form at its own sizes (1776 rows 151 and 148 us, 2208 rows 160 and 166, 3072 rows
 // 199 and 191, 3648 rows 204 and 202): there the form with fewer rows in flight stays.
 bool rows_ahead(const scabem_op* op) { return op->ne >= 152 * 28; }
